@@ -673,8 +673,9 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 if (lane == 0 && in_mask != 0u && co_tile * 128 + quarter * 32 < p.c_out) {
                     const int cw = c0 & (p.tw - 1), chh = (c0 >> p.tw_log) & (p.th - 1), cn = c0 >> (p.tw_log + p.th_log);
                     tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
-                    tma_store_commit();
                 }
+                // also for a chunk outside the tensor (an empty group): the wait above counts groups, one per chunk
+                if (lane == 0) tma_store_commit();
             }
             tc_fence_before();
             mbar_arrive(acc_empty0 + 8 * buf);

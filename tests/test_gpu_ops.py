@@ -112,6 +112,26 @@ def test_conv_cuda_core_kernels(case, dtype):
     assert TIGHT[dtype] <= TOL[dtype]
 
 
+@pytest.mark.parametrize("case", [(21, 42, 42, 256, 64, 1), (21, 14, 14, 128, 512, 1), (9, 13, 11, 256, 128, 3)])
+def test_conv_tiles_with_empty_chunks_are_reproducible(case):
+    """Pixel tiles that reach past the tensor leave whole store chunks of the role-swapped kernel out; the others' slabs
+    must not be rewritten before their stores have read them.  Many runs, compared bit for bit."""
+    import torch
+    dtype = ck.DTYPE_BF16
+    n, h, w, cin, cout, k = case
+    shape = ck.ConvShape(n, h, w, cin, cout, k, 1, k // 2)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    dz = torch.randn((n, h, w, cout), generator=gen, device="cuda").bfloat16()
+    wt = torch.randn((cout, k, k, cin), generator=gen, device="cuda").bfloat16()
+    scratch = torch.empty(max(ck.conv2d_scratch_bytes(shape, dtype), 256), dtype=torch.uint8, device="cuda")
+    first = None
+    for _ in range(200):
+        dx = torch.empty((n, h, w, cin), dtype=torch.bfloat16, device="cuda")
+        ck.conv2d_dgrad(shape, dtype, 2, dz, wt, dx, scratch)
+        first = dx if first is None else first
+        assert torch.equal(dx, first)
+
+
 @pytest.mark.parametrize("case", TC_CASES)
 def test_conv_tensor_core_kernels(case):
     """tcgen05 forward / dgrad / wgrad against the float64 oracle, and bit-reproducible."""
