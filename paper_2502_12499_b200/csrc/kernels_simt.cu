@@ -8,9 +8,11 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 
+#include "conv_simt.cuh"
 #include "internal.h"
 
 namespace ckpt {
@@ -36,121 +38,47 @@ template <> __device__ __forceinline__ float cvt<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 cvt<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 // ================================================================================================
-// Implicit GEMM  C[M][N] = sum_k A(m,k) * B(k,n), 64x64 tile, 16-deep k slices, 4x4 per thread.
-//   MODE 0 forward: M = pixels out, N = c_out, K = k*k*c_in
-//   MODE 1 dgrad  : M = pixels in,  N = c_in,  K = k*k*c_out
-//   MODE 2 wgrad  : M = c_out,      N = k*k*c_in, K = pixels out, split over gridDim.z
+// Convolutions on the CUDA cores (kernel and tile shapes: conv_simt.cuh)
 // ================================================================================================
-constexpr int TM = 64, TN = 64, TK = 16;
-
-template <typename T, int MODE>
-__device__ __forceinline__ float load_a(const ConvGeom& g, const T* A, int m, int kk, int M, int K) {
-    if (m >= M || kk >= K) return 0.f;
-    if (MODE == 0) {
-        int ci = kk % g.cin, tap = kk / g.cin, r = tap / g.k, s = tap % g.k;
-        int ow = m % g.wo, t = m / g.wo, oh = t % g.ho, n = t / g.ho;
-        int ih = oh * g.stride - g.pad + r, iw = ow * g.stride - g.pad + s;
-        if (ih < 0 || ih >= g.h || iw < 0 || iw >= g.w) return 0.f;
-        return ld(A + (((size_t)n * g.h + ih) * g.w + iw) * g.cin + ci);
-    } else if (MODE == 1) {
-        int co = kk % g.cout, tap = kk / g.cout, r = tap / g.k, s = tap % g.k;
-        int iw = m % g.w, t = m / g.w, ih = t % g.h, n = t / g.h;
-        int th = ih + g.pad - r, tw = iw + g.pad - s;
-        if (th < 0 || tw < 0 || th % g.stride || tw % g.stride) return 0.f;
-        int oh = th / g.stride, ow = tw / g.stride;
-        if (oh >= g.ho || ow >= g.wo) return 0.f;
-        return ld(A + (((size_t)n * g.ho + oh) * g.wo + ow) * g.cout + co);
-    } else {
-        return ld(A + (size_t)kk * g.cout + m);              // dz[pixel][c_out]
+namespace simt {
+// The tile shape, the CTAs of a cluster that share a tile's reduction and (wgrad) the slices whose partial sums a second
+// kernel adds: the cheapest by a model of clocks per SM.  FMA time is the tile volume over 128 lanes and the share of the
+// peak a tile shape reaches (narrower blocks per thread read more operand bytes per FMA); a cluster costs its exchange,
+// further slices a launch and a pass over the partial sums.
+Plan plan(int mode, int M, int N, int K, bool vectors) {
+    static const int tile_m[7] = {128, 128, 64, 128, 64, 128, 64}, tile_n[7] = {128, 64, 64, 32, 32, 16, 16};
+    static const double share[7] = {0.85, 0.8, 0.7, 0.6, 0.5, 0.4, 0.35};
+    Plan best{2, 1, 1, K};
+    double best_t = 1e300;
+    for (int t = 0; t < 7; ++t) {
+        if (!vectors && t != 2 && t != 4 && t != 6) continue;
+        const int bm = mode == 2 ? tile_n[t] : tile_m[t], bn = mode == 2 ? tile_m[t] : tile_n[t];
+        const int64_t tiles = (int64_t)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
+        for (int cluster = 1; cluster <= 8; cluster *= 2) {
+            for (int slices = 1; slices <= (mode == 2 ? 128 : 1); slices += slices < 16 ? 1 : slices / 8) {
+                const int parts = cluster * slices;
+                const int per = ((K + parts - 1) / parts + 31) / 32 * 32;
+                if (parts > 1 && (per < 64 || (int64_t)per * (parts - 1) >= K)) continue;
+                // CTAs per SM; one or two of 128 threads do not hide the latency of their shared-memory reads
+                const double load = std::ceil((double)(tiles * parts) / 148.0);
+                const double hidden = t == 0 ? (load < 2 ? 0.8 : 1.0) : (load < 2 ? 0.6 : load < 3 ? 0.8 : 1.0);
+                double clk = load * ((double)bm * bn * per / (128.0 * share[t] * hidden) + 300.0) + 2000.0;
+                if (cluster > 1) clk += 1000.0 + load * bm * bn / 32.0;
+                if (slices > 1) clk += 4000.0 + (double)slices * M * N * 8.0 / 2500.0;
+                if (clk < best_t) { best_t = clk; best = Plan{t, cluster, slices, per}; }
+            }
+        }
     }
+    return best;
 }
+}  // namespace simt
 
-template <typename T, int MODE>
-__device__ __forceinline__ float load_b(const ConvGeom& g, const T* B, int kk, int n, int K, int N) {
-    if (kk >= K || n >= N) return 0.f;
-    if (MODE == 0) {
-        return ld(B + (size_t)n * K + kk);                   // w[c_out][k][k][c_in]
-    } else if (MODE == 1) {
-        int co = kk % g.cout, tap = kk / g.cout;
-        return ld(B + ((size_t)co * g.k * g.k + tap) * g.cin + n);
-    } else {
-        int ci = n % g.cin, tap = n / g.cin, r = tap / g.k, s = tap % g.k;
-        int ow = kk % g.wo, t = kk / g.wo, oh = t % g.ho, img = t / g.ho;
-        int ih = oh * g.stride - g.pad + r, iw = ow * g.stride - g.pad + s;
-        if (ih < 0 || ih >= g.h || iw < 0 || iw >= g.w) return 0.f;
-        return ld(B + (((size_t)img * g.h + ih) * g.w + iw) * g.cin + ci);
-    }
-}
+static bool whole_chunks(int dtype, int channels, const void* p) { return channels % (dtype == CKPT_DTYPE_BF16 ? 8 : 4) == 0 && (uintptr_t)p % 16 == 0; }
 
-template <typename T, int MODE>
-__global__ void __launch_bounds__(256) conv_gemm_kernel(ConvGeom g, const T* __restrict__ A, const T* __restrict__ B,
-                                                        void* __restrict__ out, const float* __restrict__ bias,
-                                                        int relu, int M, int N, int K, int k_per_slice) {
-    __shared__ float As[TK][TM + 1];
-    __shared__ float Bs[TK][TN + 1];
-    const int tid = threadIdx.x;
-    const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-    const int k_begin = blockIdx.z * k_per_slice;
-    const int k_end = min(K, k_begin + k_per_slice);
-    const int tx = tid % 16, ty = tid / 16;
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-    for (int k0 = k_begin; k0 < k_end; k0 += TK) {
-        // operand tiles; the index that is contiguous in memory varies fastest across threads
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            if (MODE == 2) {
-                int mm = tid % TM, kk = tid / TM + 4 * p;
-                As[kk][mm] = (k0 + kk < k_end) ? load_a<T, MODE>(g, A, m0 + mm, k0 + kk, M, K) : 0.f;
-            } else {
-                int kk = tid % TK, mm = tid / TK + 16 * p;
-                As[kk][mm] = (k0 + kk < k_end) ? load_a<T, MODE>(g, A, m0 + mm, k0 + kk, M, K) : 0.f;
-            }
-            if (MODE == 0) {
-                int kk = tid % TK, nn = tid / TK + 16 * p;
-                Bs[kk][nn] = (k0 + kk < k_end) ? load_b<T, MODE>(g, B, k0 + kk, n0 + nn, K, N) : 0.f;
-            } else {
-                int nn = tid % TN, kk = tid / TN + 4 * p;
-                Bs[kk][nn] = (k0 + kk < k_end) ? load_b<T, MODE>(g, B, k0 + kk, n0 + nn, K, N) : 0.f;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < TK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int m = m0 + ty * 4 + i;
-        if (m >= M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int n = n0 + tx * 4 + j;
-            if (n >= N) continue;
-            float v = acc[i][j];
-            if (MODE == 2) {
-                ((float*)out)[((size_t)blockIdx.z * M + m) * N + n] = v;
-            } else {
-                if (bias) v += bias[n];
-                if (relu) v = fmaxf(v, 0.f);
-                ((T*)out)[(size_t)m * N + n] = cvt<T>(v);
-            }
-        }
-    }
+static int simt_conv(int mode, int dtype, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N,
+                     int K, bool va, bool vb, const simt::Plan& p, cudaStream_t st) {
+    return dtype == CKPT_DTYPE_BF16 ? simt::launch<__nv_bfloat16>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, st)
+                                    : simt::launch<float>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, st);
 }
 
 // out[e] = sum over slices (in slice order) of partial[slice][e]
@@ -162,72 +90,38 @@ __global__ void slice_sum_kernel(const float* __restrict__ partial, float* __res
     out[e] = s;
 }
 
-template <typename T>
-static int launch_fwd(const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, cudaStream_t st) {
-    int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
-    dim3 grid((M + TM - 1) / TM, (N + TN - 1) / TN, 1);
-    conv_gemm_kernel<T, 0><<<grid, 256, 0, st>>>(g, (const T*)x, (const T*)w, z, bias, relu, M, N, K, K);
-    CKPT_LAUNCH_CHECK("conv forward (CUDA cores)");
-    return CKPT_OK;
+int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, void* stream) {
+    if (!bias && !relu && small_conv_supported(dtype, g)) return small_conv_fwd(g, x, w, z, stream);
+    const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
+    const bool v = whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
+    return simt_conv(0, dtype, g, x, w, z, bias, relu, M, N, K, v, v, simt::plan(0, M, N, K, v), (cudaStream_t)stream);
 }
-template <typename T>
-static int launch_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, cudaStream_t st) {
-    int M = g.n * g.h * g.w, N = g.cin, K = g.k * g.k * g.cout;
-    dim3 grid((M + TM - 1) / TM, (N + TN - 1) / TN, 1);
-    conv_gemm_kernel<T, 1><<<grid, 256, 0, st>>>(g, (const T*)dz, (const T*)w, dx, nullptr, 0, M, N, K, K);
-    CKPT_LAUNCH_CHECK("conv dgrad (CUDA cores)");
-    return CKPT_OK;
-}
-
-static void wgrad_split(const ConvGeom& g, int* slices, int* k_per_slice) {
-    int M = g.cout, N = g.k * g.k * g.cin;
-    int64_t K = (int64_t)g.n * g.ho * g.wo;
-    int64_t tiles = (int64_t)((M + TM - 1) / TM) * ((N + TN - 1) / TN);
-    int64_t want = std::max<int64_t>(1, (148 * 4 + tiles - 1) / tiles);      // about four tiles per SM
-    int64_t max_by_k = std::max<int64_t>(1, K / 256);                        // at least 256 deep per slice
-    int64_t s = std::min<int64_t>(std::min<int64_t>(want, max_by_k), 512);
-    int64_t per = ((K + s - 1) / s + TK - 1) / TK * TK;
-    *slices = (int)((K + per - 1) / per);
-    *k_per_slice = (int)per;
+int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w, void* dx, void* stream) {
+    // (a strided layer's K splits over the parity classes of the input: the longest class has ceil(k / stride)^2 positions)
+    const int taps = (g.k + g.stride - 1) / g.stride;
+    const int M = g.n * g.h * g.w, N = g.cin, K = taps * taps * g.cout;
+    const bool va = whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, w);
+    return simt_conv(1, dtype, g, dz, w, dx, nullptr, 0, M, N, K, va, vb, simt::plan(1, M, N, K, va && vb), (cudaStream_t)stream);
 }
 
 int64_t simt_wgrad_scratch_bytes(const ConvGeom& g) {
-    int slices, per;
-    wgrad_split(g, &slices, &per);
-    if (slices <= 1) return 0;
-    return (int64_t)slices * g.cout * g.k * g.k * g.cin * (int64_t)sizeof(float);
+    const int M = g.cout, N = g.k * g.k * g.cin, K = g.n * g.ho * g.wo;
+    const int slices = std::max(simt::plan(2, M, N, K, true).slices, simt::plan(2, M, N, K, false).slices);
+    return slices <= 1 ? 0 : (int64_t)slices * M * N * (int64_t)sizeof(float);
 }
-
-template <typename T>
-static int launch_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes, cudaStream_t st) {
-    int M = g.cout, N = g.k * g.k * g.cin, K = g.n * g.ho * g.wo;
-    int slices, per;
-    wgrad_split(g, &slices, &per);
-    if (slices > 1 && scratch_bytes < simt_wgrad_scratch_bytes(g)) { set_error("wgrad scratch too small"); return CKPT_E_WORKSPACE; }
-    dim3 grid((M + TM - 1) / TM, (N + TN - 1) / TN, slices);
-    float* target = slices > 1 ? (float*)scratch : dw;
-    conv_gemm_kernel<T, 2><<<grid, 256, 0, st>>>(g, (const T*)dz, (const T*)x, target, nullptr, 0, M, N, K, per);
-    CKPT_LAUNCH_CHECK("conv wgrad (CUDA cores)");
-    if (slices > 1) {
-        int64_t elems = (int64_t)M * N;
-        slice_sum_kernel<<<(unsigned)((elems + 255) / 256), 256, 0, st>>>((const float*)scratch, dw, elems, slices);
+int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes, void* stream) {
+    const int M = g.cout, N = g.k * g.k * g.cin, K = g.n * g.ho * g.wo;
+    const bool va = whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, x);
+    const simt::Plan p = simt::plan(2, M, N, K, va && vb);
+    const int64_t elems = (int64_t)M * N;
+    if (p.slices > 1 && (!scratch || scratch_bytes < p.slices * elems * 4)) { set_error("wgrad scratch too small"); return CKPT_E_WORKSPACE; }
+    int rc = simt_conv(2, dtype, g, dz, x, p.slices > 1 ? scratch : dw, nullptr, 0, M, N, K, va, vb, p, (cudaStream_t)stream);
+    if (rc) return rc;
+    if (p.slices > 1) {
+        slice_sum_kernel<<<(unsigned)((elems + 255) / 256), 256, 0, (cudaStream_t)stream>>>((const float*)scratch, dw, elems, p.slices);
         CKPT_LAUNCH_CHECK("wgrad slice sum");
     }
     return CKPT_OK;
-}
-
-int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, void* stream) {
-    if (!bias && !relu && small_conv_supported(dtype, g)) return small_conv_fwd(g, x, w, z, stream);
-    return dtype == CKPT_DTYPE_BF16 ? launch_fwd<__nv_bfloat16>(g, x, w, z, bias, relu, (cudaStream_t)stream)
-                                    : launch_fwd<float>(g, x, w, z, bias, relu, (cudaStream_t)stream);
-}
-int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w, void* dx, void* stream) {
-    return dtype == CKPT_DTYPE_BF16 ? launch_dgrad<__nv_bfloat16>(g, dz, w, dx, (cudaStream_t)stream)
-                                    : launch_dgrad<float>(g, dz, w, dx, (cudaStream_t)stream);
-}
-int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes, void* stream) {
-    return dtype == CKPT_DTYPE_BF16 ? launch_wgrad<__nv_bfloat16>(g, dz, x, dw, scratch, scratch_bytes, (cudaStream_t)stream)
-                                    : launch_wgrad<float>(g, dz, x, dw, scratch, scratch_bytes, (cudaStream_t)stream);
 }
 
 // ================================================================================================

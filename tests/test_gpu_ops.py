@@ -39,6 +39,16 @@ CONV_CASES = [
     (5, 1, 1, 200, 70, 1, 1, 0),     # fully connected as a 1x1 convolution
     (3, 21, 18, 3, 64, 3, 1, 1),     # first-layer kernels (3 input channels, 64 outputs)
     (2, 40, 40, 3, 128, 3, 1, 1),
+    # tile shapes, edges and splits of the CUDA-core kernel
+    (1, 1, 1, 4, 8, 1, 1, 0),        # one pixel, one chunk of K
+    (32, 2, 2, 256, 256, 3, 1, 1),   # few tiles: the reduction split over a cluster
+    (7, 1, 1, 1000, 10, 1, 1, 0),    # classifier with fewer classes than a chunk, both operands of the dgrad mixed
+    (2, 19, 23, 48, 80, 3, 1, 1),    # ragged tiles in every dimension
+    (16, 28, 28, 128, 128, 3, 1, 1), # large tiles, weight gradient in slices
+    (2, 1, 9, 8, 12, 3, 2, 1),       # stride 2 on one row: empty parity classes
+    (3, 10, 11, 20, 36, 3, 3, 1),    # stride 3: nine classes of three sizes
+    (2, 12, 9, 16, 24, 1, 3, 0),     # classes that no filter position reaches: zero gradient
+    (2, 11, 13, 5, 16, 5, 2, 2),     # forward value by value, weight gradient with one chunked operand
 ]
 
 
