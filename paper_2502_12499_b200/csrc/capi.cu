@@ -25,9 +25,13 @@ int* op_status_word() {
     if (cudaGetSymbolAddress((void**)&word, g_op_status) != cudaSuccess) return nullptr;
     return word;
 }
-bool want_tc(int impl, int dtype, const ConvGeom& g, int* rc) {
+bool enough_scratch(int dtype, const ConvGeom& g, const void* scratch, int64_t bytes) {
+    return scratch && tc_conv_supported(dtype, g) && bytes >= tc_conv_scratch_bytes(g);
+}
+// a, b, c: the call's tensors.  Where a shape also has CUDA-core kernels these take any alignment and less scratch.
+bool want_tc(int impl, int dtype, const ConvGeom& g, const void* a, const void* b, const void* c, bool enough_scratch, int* rc) {
     *rc = CKPT_OK;
-    bool ok = tc_conv_supported(dtype, g);
+    bool ok = tc_conv_usable(dtype, g, a, b, c) && (enough_scratch || !tc_conv_ragged(g) || impl == 2);
     if (impl == 2 && !ok) { set_error("no tensor-core kernel for this shape"); *rc = CKPT_E_UNSUPPORTED; return false; }
     return impl != 1 && ok;
 }
@@ -56,7 +60,7 @@ int ckpt_conv2d_forward(const ckpt_conv_shape* s, int dtype, int impl, const voi
     ConvGeom g = make_geom(*s);
     if (impl != 1 && tc_first_conv_supported(dtype, g)) return tc_first_conv_fwd(g, x, w, z, op_status_word(), stream);
     if (impl != 1 && stem_conv_supported(dtype, g)) return stem_conv_fwd(g, x, w, z, op_status_word(), stream);
-    if (want_tc(impl, dtype, g, &rc)) return tc_conv_fwd(g, x, w, z, nullptr, 0, scratch, scratch_bytes, op_status_word(), stream);
+    if (want_tc(impl, dtype, g, x, w, z, true, &rc)) return tc_conv_fwd(g, x, w, z, nullptr, 0, scratch, scratch_bytes, op_status_word(), stream);
     if (rc) return rc;
     return simt_conv_fwd(dtype, g, x, w, z, nullptr, 0, stream);
 }
@@ -71,7 +75,7 @@ int ckpt_conv2d_bn_statistics(const ckpt_conv_shape* s, int dtype, const void* x
     const int64_t rows = (int64_t)g.n * g.ho * g.wo;
     if (scratch_bytes < bn_scratch_bytes(rows, g.cout)) { set_error("scratch too small for the statistics"); return CKPT_E_WORKSPACE; }
     if (fused) *fused = 0;
-    if (tc_conv_supported(dtype, g)) {
+    if (tc_conv_usable(dtype, g, x, w, z) && (!tc_conv_ragged(g) || scratch_bytes >= tc_conv_scratch_bytes(g))) {
         if (scratch_bytes < tc_conv_scratch_bytes(g)) { set_error("scratch too small for the convolution"); return CKPT_E_WORKSPACE; }
         int blocks = 0;
         if ((rc = tc_conv_fwd_stats(g, x, w, z, (float*)scratch, &blocks, op_status_word(), stream, scratch_bytes))) return rc;
@@ -104,7 +108,7 @@ int ckpt_conv2d_dgrad(const ckpt_conv_shape* s, int dtype, int impl, const void*
     if (rc) return rc;
     if (!dz || !w || !dx) { set_error("null tensor"); return CKPT_E_NULL; }
     ConvGeom g = make_geom(*s);
-    if (want_tc(impl, dtype, g, &rc)) return tc_conv_dgrad(g, dz, w, dx, scratch, scratch_bytes, op_status_word(), stream);
+    if (want_tc(impl, dtype, g, dz, w, dx, enough_scratch(dtype, g, scratch, scratch_bytes), &rc)) return tc_conv_dgrad(g, dz, w, dx, scratch, scratch_bytes, op_status_word(), stream);
     if (rc) return rc;
     return simt_conv_dgrad(dtype, g, dz, w, dx, stream);
 }
@@ -119,7 +123,7 @@ int ckpt_conv2d_wgrad(const ckpt_conv_shape* s, int dtype, int impl, const void*
         return small_conv_wgrad(g, dz, x, dw, scratch, scratch_bytes, op_status_word(), stream);
     if (impl != 1 && stem_conv_supported(dtype, g))
         return stem_conv_wgrad(g, dz, x, dw, scratch, scratch_bytes, op_status_word(), stream);
-    if (want_tc(impl, dtype, g, &rc)) return tc_conv_wgrad(g, dz, x, dw, scratch, scratch_bytes, op_status_word(), stream);
+    if (want_tc(impl, dtype, g, dz, x, nullptr, enough_scratch(dtype, g, scratch, scratch_bytes), &rc)) return tc_conv_wgrad(g, dz, x, dw, scratch, scratch_bytes, op_status_word(), stream);
     if (rc) return rc;
     return simt_conv_wgrad(dtype, g, dz, x, dw, scratch, scratch_bytes, stream);
 }

@@ -87,8 +87,8 @@ static int check_conv(const ckpt_unit_desc& u, const Shape& in, int64_t idx) {
     return CKPT_OK;
 }
 
-static bool use_tc(const ckpt_chain* ch, const ConvGeom& g) {
-    return ch->impl == 0 && tc_conv_supported(ch->dtype, g);
+static bool use_tc(const ckpt_chain* ch, const ConvGeom& g, const void* a, const void* b, const void* c) {
+    return ch->impl == 0 && tc_conv_usable(ch->dtype, g, a, b, c);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -128,7 +128,7 @@ static int64_t workspace_need(const ckpt_chain* ch, int policy) {
 
 static int conv_forward_any(StepCtx& c, const ConvGeom& g, const void* x, const void* w, void* z,
                             const float* bias, int relu) {
-    if (use_tc(c.ch, g))
+    if (use_tc(c.ch, g, x, w, z))
         return tc_conv_fwd(g, x, w, z, bias, relu, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
     if (c.ch->impl == 0 && !bias && !relu && tc_first_conv_supported(c.ch->dtype, g))
         return tc_first_conv_fwd(g, x, w, z, c.status(), c.stream);
@@ -137,7 +137,7 @@ static int conv_forward_any(StepCtx& c, const ConvGeom& g, const void* x, const 
     return simt_conv_fwd(c.ch->dtype, g, x, w, z, bias, relu, c.stream);
 }
 static int conv_dgrad_any(StepCtx& c, const ConvGeom& g, const void* dz, const void* w, void* dx) {
-    if (use_tc(c.ch, g))
+    if (use_tc(c.ch, g, dz, w, dx))
         return tc_conv_dgrad(g, dz, w, dx, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
     return simt_conv_dgrad(c.ch->dtype, g, dz, w, dx, c.stream);
 }
@@ -146,7 +146,7 @@ static int conv_wgrad_any(StepCtx& c, const ConvGeom& g, const void* dz, const v
         return small_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
     if (c.ch->impl == 0 && stem_conv_supported(c.ch->dtype, g))
         return stem_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
-    if (use_tc(c.ch, g))
+    if (use_tc(c.ch, g, dz, x, nullptr))
         return tc_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
     return simt_conv_wgrad(c.ch->dtype, g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.stream);
 }
@@ -168,7 +168,7 @@ static int conv_backward_pair(StepCtx& c, const ConvGeom& g, const void* dz, con
     const bool sgd = c.ch->sgd_lr != 0.f;
     if (sgd && dx && (rc = conv_dgrad_any(c, g, dz, w, dx))) return rc;
     const bool stem = c.ch->impl == 0 && stem_conv_supported(c.ch->dtype, g);
-    const bool tc_path = !(c.ch->impl == 0 && small_conv_supported(c.ch->dtype, g)) && !stem && use_tc(c.ch, g);
+    const bool tc_path = !(c.ch->impl == 0 && small_conv_supported(c.ch->dtype, g)) && !stem && use_tc(c.ch, g, dz, x, nullptr);
     if (sgd && stem) {
         rc = stem_conv_wgrad(g, dz, x, (float*)c.grads[param], c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream, sgd_of(c, param));
         if (rc) return rc;
@@ -191,9 +191,10 @@ static int conv_with_statistics(StepCtx& c, const ConvGeom& g, const void* x, co
     const int64_t rows = (int64_t)g.n * g.ho * g.wo;
     char* scr = c.ws + c.ch->off_scr;
     int rc;
-    if (use_tc(c.ch, g) || (c.ch->impl == 0 && (tc_first_conv_supported(dt, g) || stem_conv_supported(dt, g)))) {
+    const bool tc = use_tc(c.ch, g, x, w, z);
+    if (tc || (c.ch->impl == 0 && (tc_first_conv_supported(dt, g) || stem_conv_supported(dt, g)))) {
         int blocks = 0;
-        if (use_tc(c.ch, g)) rc = tc_conv_fwd_stats(g, x, w, z, (float*)scr, &blocks, c.status(), c.stream, c.ch->scr_bytes);
+        if (tc) rc = tc_conv_fwd_stats(g, x, w, z, (float*)scr, &blocks, c.status(), c.stream, c.ch->scr_bytes);
         else if (stem_conv_supported(dt, g)) rc = stem_conv_fwd(g, x, w, z, c.status(), c.stream, (float*)scr, &blocks);
         else rc = tc_first_conv_fwd(g, x, w, z, c.status(), c.stream, (float*)scr, &blocks);
         if (rc) return rc;

@@ -140,7 +140,7 @@ __global__ void take_paired_columns_kernel(const float* __restrict__ dwp, float*
 }  // namespace
 
 bool small_conv_supported(int dtype, const ConvGeom& g) {
-    return dtype == CKPT_DTYPE_BF16 && g.cin == 3 && g.k == 3 && g.stride == 1 && g.pad == 1 && g.cout % 64 == 0;
+    return dtype == CKPT_DTYPE_BF16 && g.cin == 3 && g.k == 3 && g.stride == 1 && g.pad == 1 && g.cout % 8 == 0 && g.cout >= 16;
 }
 
 static bool paired(const ConvGeom& g) { return g.w % 2 == 0; }
@@ -168,6 +168,9 @@ int small_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, voi
 
 int small_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes,
                      int* device_status, void* stream) {
+    // (16-byte rows for the TMA unit; a channel count that is no multiple of 64 also has the CUDA-core kernel)
+    if (g.cout % 64 && (((uintptr_t)dz & 15u) || !scratch || scratch_bytes < small_conv_scratch_bytes(g)))
+        return simt_conv_wgrad(CKPT_DTYPE_BF16, g, dz, x, dw, scratch, scratch_bytes, stream);
     if (!scratch || scratch_bytes < small_conv_scratch_bytes(g)) { set_error("first-layer wgrad scratch too small"); return CKPT_E_WORKSPACE; }
     cudaStream_t st = (cudaStream_t)stream;
     char* base = (char*)scratch;

@@ -199,8 +199,9 @@ __device__ __forceinline__ float warp_column_sum(float (&v)[32], int lane) {
 // Epilogue of one 32-column chunk: rounds the accumulators to bf16, stores the valid rows and, when the
 // batch-norm statistics are gathered here, adds the chunk's per-column sum and sum of squares (of
 // the rounded values, i.e. of what is stored) into the lane's running totals.
+// columns: how many of the chunk's 32 columns exist (a multiple of 8; more than 32 = all).
 __device__ __forceinline__ void store_chunk(const uint32_t (&v)[32], bool valid, __nv_bfloat16* dst, bool stats, int lane,
-                                            float& sum, float& sumsq) {
+                                            float& sum, float& sumsq, int columns = 32) {
     float r[32];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -213,7 +214,7 @@ __device__ __forceinline__ void store_chunk(const uint32_t (&v)[32], bool valid,
             r[8 * q + 2 * e] = valid ? f.x : 0.f;
             r[8 * q + 2 * e + 1] = valid ? f.y : 0.f;
         }
-        if (valid) *reinterpret_cast<uint4*>(dst + 8 * q) = pk;
+        if (valid && 8 * q + 8 <= columns) *reinterpret_cast<uint4*>(dst + 8 * q) = pk;
     }
     if (stats) {
         float sq[32];
@@ -356,7 +357,7 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         const int quarter = warp % 4;               // a warp may only touch its own 32 TMEM lanes
         const int row = quarter * 32 + lane;
         const int wl = row % p.tw, hl = (row / p.tw) % p.th, nl = row / (p.tw * p.th);
-        const bool stats = stat_partial != nullptr;   // the caller guarantees whole 32-column chunks and no bias/ReLU
+        const bool stats = stat_partial != nullptr;   // the caller guarantees no bias/ReLU
         float s_acc[8], q_acc[8];
 #pragma unroll
         for (int ci = 0; ci < 8; ++ci) { s_acc[ci] = 0.f; q_acc[ci] = 0.f; }
@@ -375,11 +376,11 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 if (c0 >= p.bn) break;
                 uint32_t v[32];
                 tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * p.bn + c0), v);
+                const int col0 = n_tile * p.bn + c0;          // first output channel of this chunk
                 if (stats) {
-                    store_chunk(v, valid, dst + c0, true, lane, s_acc[ci], q_acc[ci]);
+                    store_chunk(v, valid, dst + c0, true, lane, s_acc[ci], q_acc[ci], p.c_out - col0);
                     continue;
                 }
-                const int col0 = n_tile * p.bn + c0;          // first output channel of this chunk
                 if (valid && col0 < p.c_out) {
                     if (bias) {
 #pragma unroll
@@ -411,8 +412,10 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             for (int ci = 0; ci < 8; ++ci) {
                 if (ci * 32 < p.bn) {
                     const int ch = n_tile * p.bn + ci * 32 + lane;
-                    stat_partial[(blk * 2) * p.c_out + ch] = s_acc[ci];
-                    stat_partial[(blk * 2 + 1) * p.c_out + ch] = q_acc[ci];
+                    if (ch < p.c_out) {
+                        stat_partial[(blk * 2) * p.c_out + ch] = s_acc[ci];
+                        stat_partial[(blk * 2 + 1) * p.c_out + ch] = q_acc[ci];
+                    }
                 }
             }
         }
@@ -562,7 +565,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     const int co_tile = blockIdx.x % p.co_tiles;
     const int first = blockIdx.x / p.co_tiles;
     const int my_tiles = first < p.p_tiles ? (p.p_tiles - first + p.ctas_per_co - 1) / p.ctas_per_co : 0;
-    const int blocks = p.c_red / 64;
+    const int blocks = (p.c_red + 63) / 64;      // a ragged last block is zero-filled by the TMA unit
     const int iters = p.taps * blocks;
 
     auto full_bar = [&](int s) { return bars + 8u * s; };
@@ -743,7 +746,7 @@ tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const int co_tile = blockIdx.x % p.co_tiles;
     const int first = blockIdx.x / p.co_tiles;
     const int my_tiles = first < p.p_tiles ? (p.p_tiles - first + p.ctas_per_co - 1) / p.ctas_per_co : 0;
-    const int blocks = p.c_red / 64;
+    const int blocks = (p.c_red + 63) / 64;      // a ragged last block is zero-filled by the TMA unit
     const int cols = p.ncols * blocks;
 
     auto a_full = [&](int s) { return bars + 8u * s; };
@@ -1249,7 +1252,7 @@ struct WgradParams {
     int px;                      // pixels per operand box and stage: 64, 128 or 256
     int tiles_w, tiles_h, tiles_n;
     int nb;                      // column blocks per CTA (1..4)
-    int total_blocks;            // k*k*c_in/64
+    int total_blocks;            // k*k * 64-channel blocks of c_in (a ragged last block is zero-filled)
     int tiles_per_slice;         // pixel tiles per CTA along the reduction
     int total_tiles;
     int stages;
@@ -1277,7 +1280,7 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     const int slice = blockIdx.x, group = blockIdx.y, co_tile = blockIdx.z;
     const int blk_begin = group * p.nb;
     const int nb_here = min(p.nb, p.total_blocks - blk_begin);
-    const int cin_blocks = p.c_in / 64;
+    const int cin_blocks = (p.c_in + 63) / 64;
     const int tile_begin = slice * p.tiles_per_slice;
     const int tile_end = min(p.total_tiles, tile_begin + p.tiles_per_slice);
     const int iters = tile_end - tile_begin;
@@ -1367,22 +1370,27 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         if (iters > 0 && mbar_wait(accum_bar, 0, failed, status, 203)) {
             tc_fence_after();
             for (int j = 0; j < nb_here; ++j) {
+                const int tap = (blk_begin + j) / cin_blocks, ch0 = (blk_begin + j) % cin_blocks * 64;
                 for (int c0 = 0; c0 < 64; c0 += 32) {
+                    if (ch0 + c0 >= p.c_in) break;
                     uint32_t v[32];
                     tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(j * 64 + c0), v);
                     __syncwarp();
 #pragma unroll
                     for (int e = 0; e < 32; ++e) turn[quarter][lane][e] = __uint_as_float(v[e]);
                     __syncwarp();
-                    float* dst = dst_first + (size_t)(blk_begin + j) * 64 + c0 + lane;     // column (tap, c_in) = block*64 + c
+                    float* dst = dst_first + (size_t)tap * p.c_in + ch0 + c0 + lane;       // column (tap, c_in)
+                    const int rows = ch0 + c0 + lane < p.c_in ? p.c_out - co_first : 0;
 #pragma unroll 8
                     for (int r = 0; r < 32; ++r)
-                        if (co_first + r < p.c_out) dst[(size_t)r * row_elems] = turn[quarter][r][lane];
+                        if (r < rows) dst[(size_t)r * row_elems] = turn[quarter][r][lane];
                 }
             }
         } else if (iters == 0 && valid) {
-            for (int j = 0; j < nb_here; ++j)
-                for (int c = 0; c < 64; ++c) dst_row[(size_t)(blk_begin + j) * 64 + c] = 0.f;
+            for (int j = 0; j < nb_here; ++j) {
+                const int tap = (blk_begin + j) / cin_blocks, ch0 = (blk_begin + j) % cin_blocks * 64;
+                for (int c = ch0; c < min(ch0 + 64, p.c_in); ++c) dst_row[(size_t)tap * p.c_in + c] = 0.f;
+            }
         }
     }
     tc_fence_before();
@@ -1547,6 +1555,7 @@ struct WRowsParams {
     int pairview;
     int row_elems;               // floats per partial row: 9 * c_in, or 4 columns * 3 * 64 in the pair view
     int cols;                    // columns per CTA: 2, or 1 for short reductions (half the partial sums per CTA)
+    int total_cols;              // 3 horizontal offsets x 64-channel blocks (4 in the pair view); the last CTA may have one column only
 };
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -1564,9 +1573,8 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int slice = blockIdx.x, pair = blockIdx.y, co_tile = blockIdx.z;
-    const int ncols = p.cols;
+    const int ncols = min(p.cols, p.total_cols - p.cols * pair);
     const int my_tiles = slice < p.m_tiles ? (p.m_tiles - slice + p.slices - 1) / p.slices : 0;
-    const int cin_blocks = p.c_in / 64;
 
     if (threadIdx.x == 0) {
         failed_flag = 0;
@@ -1598,7 +1606,7 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             if (lane < 2) {
                 tma_load_4d(dst + lane * p.dz_box, &map_dz, full_bar(s), co_tile * 128 + 64 * lane, w0, h0, img);
             } else if (lane < 2 + ncols) {
-                const int col = ncols * pair + (lane - 2);
+                const int col = p.cols * pair + (lane - 2);
                 const int ch = p.pairview ? ((col + 1) & 1) * 64 : (col / 3) * 64;
                 const int shift = p.pairview ? (col + 1) / 2 - 1 : col % 3 - 1;
                 tma_load_4d(dst + 2 * p.dz_box + (lane - 2) * p.patch_bytes, &map_x, full_bar(s), ch, w0 + shift, h0 - 1, img);
@@ -1638,10 +1646,11 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         if (my_tiles > 0 && mbar_wait(accum_bar, 0, failed, status, 703)) {
             tc_fence_after();
             for (int c = 0; c < ncols; ++c) {
-                const int col = ncols * pair + c, cib = col / 3, dx = col % 3;
+                const int col = p.cols * pair + c, cib = col / 3, dx = col % 3;
                 for (int dy = 0; dy < 3; ++dy) {
                     float* dst = dst_row + (p.pairview ? (size_t)(col * 3 + dy) * 64
-                                                       : (size_t)((dy * 3 + dx) * cin_blocks + cib) * 64);   // column (tap, c_in)
+                                                       : (size_t)(dy * 3 + dx) * p.c_in + cib * 64);   // column (tap, c_in)
+                    const int here = p.pairview ? 64 : min(64, p.c_in - cib * 64);      // a multiple of 8
 #pragma unroll
                     for (int c0 = 0; c0 < 64; c0 += 32) {
                         uint32_t v[32];
@@ -1649,6 +1658,7 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
                         if (valid) {
 #pragma unroll
                             for (int e = 0; e < 8; ++e)
+                                if (c0 + 4 * e < here)
                                 *reinterpret_cast<float4*>(dst + c0 + 4 * e) =
                                     make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]), __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]));
                         }
@@ -1657,10 +1667,11 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             }
         } else if (my_tiles == 0 && valid) {
             for (int c = 0; c < ncols; ++c) {
-                const int col = ncols * pair + c, cib = col / 3, dx = col % 3;
+                const int col = p.cols * pair + c, cib = col / 3, dx = col % 3;
                 for (int dy = 0; dy < 3; ++dy) {
-                    float* dst = dst_row + (p.pairview ? (size_t)(col * 3 + dy) * 64 : (size_t)((dy * 3 + dx) * cin_blocks + cib) * 64);
-                    for (int e = 0; e < 64; ++e) dst[e] = 0.f;
+                    float* dst = dst_row + (p.pairview ? (size_t)(col * 3 + dy) * 64 : (size_t)(dy * 3 + dx) * p.c_in + cib * 64);
+                    const int here = p.pairview ? 64 : min(64, p.c_in - cib * 64);
+                    for (int e = 0; e < here; ++e) dst[e] = 0.f;
                 }
             }
         }
@@ -1739,7 +1750,7 @@ tc_conv_first_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* _
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int k = chunk * 8 + e, r = k / 10, tt = k % 10;      // filter row r in columns 10 r .. 10 r + 8
-            v[e] = (r < 3 && tt < 9) ? __ldg(reinterpret_cast<const uint16_t*>(w) + (size_t)(co0 + co) * 27 + r * 9 + tt) : (uint16_t)0;
+            v[e] = (r < 3 && tt < 9 && co0 + co < p.c_out) ? __ldg(reinterpret_cast<const uint16_t*>(w) + (size_t)(co0 + co) * 27 + r * 9 + tt) : (uint16_t)0;
         }
         *reinterpret_cast<uint4*>(b_tile + co * 128 + ((chunk ^ (co & 7)) * 16)) = *reinterpret_cast<const uint4*>(v);
     }
@@ -1905,6 +1916,7 @@ tc_conv_first_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* _
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int col = h * 32 + lane;
+                    if (co0 + col >= p.c_out) continue;
 #pragma unroll
                     for (int k = 0; k < 2; ++k)
                         stat_partial[((size_t)blockIdx.x * 2 + k) * p.c_out + co0 + col] =
@@ -2116,7 +2128,7 @@ tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int k = chunk * 8 + e, r = k / 24, tt = k % 24;
-            v[e] = (r < 7 && tt < 21) ? __ldg(reinterpret_cast<const uint16_t*>(w) + (size_t)(co0 + co) * 147 + r * 21 + tt) : (uint16_t)0;
+            v[e] = (r < 7 && tt < 21 && co0 + co < p.c_out) ? __ldg(reinterpret_cast<const uint16_t*>(w) + (size_t)(co0 + co) * 147 + r * 21 + tt) : (uint16_t)0;
         }
         *reinterpret_cast<uint4*>(b_tile + (chunk >> 3) * 8192 + co * 128 + (((chunk & 7) ^ (co & 7)) * 16)) = *reinterpret_cast<const uint4*>(v);
     }
@@ -2224,6 +2236,7 @@ tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int col = h * 32 + lane;
+                    if (co0 + col >= p.c_out) continue;
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
                         float acc = 0.f;
@@ -2343,6 +2356,7 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
         const int quarter = warp % 4;
         const int row = quarter * 32 + lane;
         float* const base = partial + ((size_t)slice * p.c_out + (size_t)co_tile * 64) * 147;
+        const int here = min(64, p.c_out - co_tile * 64);
         if (my_tiles > 0 && mbar_wait(accum_bar, 0, failed, status, 625)) {
             tc_fence_after();
 #pragma unroll
@@ -2356,12 +2370,13 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
                     tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 64 + c0), v);
                     if (valid) {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) dst[(size_t)(c0 + e) * 147] = __uint_as_float(v[e]);
+                        for (int e = 0; e < 32; ++e)
+                            if (c0 + e < here) dst[(size_t)(c0 + e) * 147] = __uint_as_float(v[e]);
                     }
                 }
             }
         } else if (my_tiles == 0) {
-            for (int i = threadIdx.x - (kStemGather + 64); i < 64 * 147; i += 128) base[i] = 0.f;
+            for (int i = threadIdx.x - (kStemGather + 64); i < here * 147; i += 128) base[i] = 0.f;
         }
     }
     tc_fence_before();
@@ -2660,7 +2675,11 @@ void choose_tile(int pixels, int W, int H, int N, int* tw, int* th, int* tn) {
     }
 }
 
-int pick_bn(int c_out) { return c_out % 256 == 0 ? 256 : (c_out % 128 == 0 ? 128 : 64); }
+// (whole 32-column chunks: what lies past c_out in the last chunk is zero-filled on the way in and never stored)
+int pick_bn(int c_out) {
+    if (c_out % 64 && c_out <= 256) return (c_out + 31) / 32 * 32;
+    return c_out % 256 == 0 ? 256 : (c_out % 128 == 0 ? 128 : 64);
+}
 
 int launch_c64(const void* x, const void* w_mat, void* out, float* stat_partial, int* stat_blocks, int N, int H, int W,
                int c_out, int* status, cudaStream_t st, const char* what, bool b_mn = false) {
@@ -2761,7 +2780,8 @@ int launch_generic(FwdParams p, const void* a, int a_n, int a_h, int a_w, const 
     {   // few pixel tiles (fully connected layers): narrower channel tiles give every SM a share of the matrix
         const int64_t m_tiles = (int64_t)p.tiles_w * p.tiles_h * p.tiles_n;
         const int floor_bn = b_mn ? 64 : 32;
-        while (p.bn > floor_bn && m_tiles * ((c_out + p.bn - 1) / p.bn) < 148) p.bn /= 2;
+        if (b_mn) p.bn = (p.bn + 63) / 64 * 64;
+        while (p.bn > floor_bn && m_tiles * ((c_out + p.bn - 1) / p.bn) < 148) p.bn = (p.bn / 2 + floor_bn - 1) / floor_bn * floor_bn;
     }
     p.n_tiles = (c_out + p.bn - 1) / p.bn;
     const uint32_t stage_bytes = 128 * 128 + p.bn * 128;
@@ -2788,7 +2808,7 @@ int launch_generic(FwdParams p, const void* a, int a_n, int a_h, int a_w, const 
     // statistics in the epilogue: whole 32-column chunks, plain stores, output written once per pixel
     // (a short reduction cannot hide the column sums behind its MMAs: a 64 -> 256 1x1 layer took 172 us with them
     // against 78 us without, more than the separate pass over the output costs; from 16 stages per tile on they are free)
-    const bool gather = stat_partial && stat_blocks && !bias && !relu && !b_mn && c_out % 64 == 0 && p.bn >= 32 && p.out_stride == 1 &&
+    const bool gather = stat_partial && stat_blocks && !bias && !relu && !b_mn && p.bn >= 32 && p.out_stride == 1 &&
                         p.taps * ((c_red + 63) / 64) >= 16;
     if (gather) *stat_blocks = 4 * p.ctas_per_n;
     if (b_mn) tc_conv_fwd_kernel<true><<<(unsigned)ctas, kThreads, smem, st>>>(mx, mw, (__nv_bfloat16*)out, bias, relu, nullptr, p, status);
@@ -2804,7 +2824,9 @@ int launch_generic(FwdParams p, const void* a, int a_n, int a_h, int a_w, const 
 // 0.124 -> 0.105, 256 -> 256 at 56x56 0.219 -> 0.195, 28x28 and 14x14 within 4 % either way; 64 -> 64 at 224x224 stays
 // with the 64-channel kernel (0.31 against 0.64 ms).
 bool t_applies(int c_red, int c_out, int k, int pad) {
-    return (c_out % 128 == 0 || (c_out == 64 && c_red >= 128)) && c_red % 64 == 0 && ((k == 3 && pad == 1) || (k == 1 && pad == 0));
+    if (!((k == 3 && pad == 1) || (k == 1 && pad == 0))) return false;
+    if (c_red % 64 || c_out % 64) return c_red % 8 == 0 && c_out % 8 == 0;
+    return c_out % 128 == 0 || (c_out == 64 && c_red >= 128);
 }
 // The role-swapped kernel on prepared terms (p.taps, p.tap_*, p.fold): input [N][H][W][x_channels], output
 // [N][H][W][c_out], filter matrix as given by its tensor map.
@@ -3065,7 +3087,7 @@ int launch_fc(const ConvGeom& g, const void* x, const void* w, void* z, const fl
 
 void wgrad_plan(const ConvGeom& g, WgradParams* p, int* slices, int* groups, int* co_tiles) {
     p->H = g.ho; p->W = g.wo; p->N = g.n; p->c_out = g.cout; p->c_in = g.cin; p->k = g.k; p->pad = g.pad; p->stride = g.stride;
-    p->total_blocks = g.k * g.k * g.cin / 64;
+    p->total_blocks = g.k * g.k * ((g.cin + 63) / 64);
     // column blocks per CTA: 4 when that divides evenly or the remainder is small, else 3
     p->nb = p->total_blocks % 4 == 0 ? 4 : (p->total_blocks % 3 == 0 ? 3 : (p->total_blocks >= 4 ? 4 : p->total_blocks));
     // pixels per stage: as many as leave two stages in shared memory (96 KB per stage at most), for reductions long
@@ -3130,7 +3152,7 @@ void wgrad_c64_plan(const ConvGeom& g, W64Params* p) {
 namespace {
 constexpr int WROWS_MIN_W = 14;
 bool wgrad_rows_applies(const ConvGeom& g) {
-    return g.k == 3 && g.pad == 1 && g.stride == 1 && g.cin % 128 == 0 && g.cout % 64 == 0 && g.w >= WROWS_MIN_W && g.h >= 8;
+    return g.k == 3 && g.pad == 1 && g.stride == 1 && (g.cin % 128 == 0 || g.cin % 64) && g.cin % 8 == 0 && g.cout % 8 == 0 && g.w >= WROWS_MIN_W && g.h >= 8;
 }
 void wgrad_rows_plan(const ConvGeom& g, WRowsParams* p, int* pairs, int* co_tiles) {
     p->H = g.h; p->W = g.w; p->N = g.n; p->c_out = g.cout; p->c_in = g.cin;
@@ -3139,7 +3161,8 @@ void wgrad_rows_plan(const ConvGeom& g, WRowsParams* p, int* pairs, int* co_tile
     p->tiles_h = (g.h + p->th - 1) / p->th;
     p->tiles_w = (g.w + 7) / 8;
     p->m_tiles = p->tiles_w * p->tiles_h * g.n;
-    *pairs = 3 * (g.cin / 64) / 2;
+    p->total_cols = 3 * ((g.cin + 63) / 64);
+    *pairs = (p->total_cols + 1) / 2;
     *co_tiles = (g.cout + 127) / 128;
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
@@ -3174,6 +3197,7 @@ void wgrad_pairview_plan(const ConvGeom& g, WRowsParams* p, int* co_tiles) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     p->slices = std::max(1, std::min(sms / (2 * *co_tiles), p->m_tiles));
     p->pairview = 1;
+    p->total_cols = 4;
     p->row_elems = 4 * 3 * 64;
     // A short reduction is dominated by what every CTA writes and the fold reads back (128 x 192 floats per column):
     // with one column per CTA and half as many slices the same SMs are busy with half the partial sums.
@@ -3186,17 +3210,29 @@ void wgrad_pairview_plan(const ConvGeom& g, WRowsParams* p, int* co_tiles) {
 }
 }  // namespace
 
+// Channel counts that leave part of a 64-channel block to zero fill run here too: the padding is cheaper than the
+// CUDA cores (16 images, us, CUDA cores -> here, forward / weight gradient: 48 -> 48 at 96 x 96 244 -> 27 / 332 -> 31,
+// 96 -> 96 at 48 x 48 229 -> 15 / 278 -> 27; 32 -> 32 at 112 x 112, 64 images 428 -> 131 / 869 -> 99).  Below 32
+// channels seven eighths of the products are padding: with many pixels the forward is level and the weight gradient
+// still wins (16 -> 16 at 56 x 56, 32 images 27 -> 27 / 59 -> 25), with few pixels nothing does (8 images of 14 x 14).
+constexpr int64_t TC_MIN_RAGGED_PIXELS = 4096;
+
+bool tc_conv_ragged(const ConvGeom& g) { return g.cin % 64 || g.cout % 64; }
+
 bool tc_conv_supported(int dtype, const ConvGeom& g) {
     if (dtype != CKPT_DTYPE_BF16) return false;
     if (g.stride != 1 && g.stride != 2) return false;
     if (!((g.k == 3 && g.pad == 1) || (g.k == 1 && g.pad == 0))) return false;
-    // the reduction runs over whole 64-channel blocks per tap; only a stride-1 1x1 filter may end in a
-    // ragged block (zero-filled), and stores are 8 channels wide
-    if (g.cin % 64) return false;
-    if (g.stride == 2) return g.cout % 64 == 0;
-    if (g.cout % 64 && !(g.k == 1 && g.cout % 8 == 0)) return false;
+    // 16-byte rows of channels for the TMA unit; blocks of 64 that a channel count does not fill are zero-filled
+    if (g.cin % 8 || g.cout % 8) return false;
+    if (tc_conv_ragged(g) && std::min(g.cin, g.cout) < 32 && (std::min(g.cin, g.cout) < 16 || (int64_t)g.n * g.ho * g.wo < TC_MIN_RAGGED_PIXELS)) return false;
+    if (g.stride == 2) return true;
     if (g.ho != g.h || g.wo != g.w) return false;
     return true;
+}
+
+bool tc_conv_usable(int dtype, const ConvGeom& g, const void* a, const void* b, const void* c) {
+    return tc_conv_supported(dtype, g) && (!tc_conv_ragged(g) || (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c) & 15u) == 0);
 }
 
 // batch-norm partial sums left by the forward kernel: one row pair per pixel tile
@@ -3238,7 +3274,7 @@ static int64_t tc_conv_work_bytes(const ConvGeom& g) {
 }
 
 bool tc_first_conv_supported(int dtype, const ConvGeom& g) {
-    return dtype == CKPT_DTYPE_BF16 && g.cin == 3 && g.k == 3 && g.stride == 1 && g.pad == 1 && g.cout % 64 == 0;
+    return dtype == CKPT_DTYPE_BF16 && g.cin == 3 && g.k == 3 && g.stride == 1 && g.pad == 1 && g.cout % 8 == 0 && g.cout >= 16;
 }
 
 // partial / blocks: null, or where the kernel leaves the batch-norm partial sums of its output
@@ -3254,11 +3290,11 @@ int tc_first_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, 
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if ((reinterpret_cast<uintptr_t>(x) & 15u) || p.pixels >= (1LL << 31)) {
+    if ((reinterpret_cast<uintptr_t>(x) & 15u) || p.pixels >= (1LL << 31) || (g.cout % 64 && (reinterpret_cast<uintptr_t>(z) & 15u))) {
         // the staged row segments are copied in 16-byte pieces and pixels are counted in 32 bits: an input that is not
         // 16-byte aligned, or larger than that, takes the CUDA-core kernel
         if (blocks) *blocks = 0;
-        return small_conv_fwd(g, x, w, z, stream);
+        return simt_conv_fwd(CKPT_DTYPE_BF16, g, x, w, z, nullptr, 0, stream);
     }
     CUtensorMap map_out;
     int rc = make_mat_map(&map_out, z, p.pixels, g.cout, 32);
@@ -3269,7 +3305,7 @@ int tc_first_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, 
         if (e != cudaSuccess) return cuda_fail(e, "shared-memory opt-in of the first-layer kernel");
         attr_set = true;
     }
-    dim3 grid((unsigned)std::min(p.m_tiles, kFirstCtasPerSm * sms), (unsigned)(g.cout / 64));
+    dim3 grid((unsigned)std::min(p.m_tiles, kFirstCtasPerSm * sms), (unsigned)((g.cout + 63) / 64));
     if (blocks) *blocks = partial ? (int)grid.x : 0;
     tc_conv_first_kernel<<<grid, kFirstThreads, kFirstSmem, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)w,
                                                                                    map_out, partial, p, device_status);
@@ -3281,7 +3317,7 @@ int tc_first_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, 
 // 7x7 stride-2 padding-3 stem on 3 input channels
 // ------------------------------------------------------------------------------------------------
 bool stem_conv_supported(int dtype, const ConvGeom& g) {
-    return dtype == CKPT_DTYPE_BF16 && g.cin == 3 && g.k == 7 && g.stride == 2 && g.pad == 3 && g.cout % 64 == 0;
+    return dtype == CKPT_DTYPE_BF16 && g.cin == 3 && g.k == 7 && g.stride == 2 && g.pad == 3 && g.cout % 8 == 0 && g.cout >= 16;
 }
 static int sm_count() {
     int sms = 148, dev = 0;
@@ -3304,7 +3340,7 @@ static bool stem_direct(const ConvGeom& g, const void* x) {
 }
 static int stem_wgrad_slices(const ConvGeom& g) {
     const StemParams p = stem_params(g);
-    return std::max(1, std::min(p.m_tiles, sm_count() / std::max(1, g.cout / 64)));
+    return std::max(1, std::min(p.m_tiles, sm_count() / ((g.cout + 63) / 64)));
 }
 int64_t stem_conv_scratch_bytes(const ConvGeom& g) {
     const int64_t partial = (int64_t)stem_wgrad_slices(g) * g.cout * 147 * 4;
@@ -3318,7 +3354,7 @@ int stem_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, int*
     if (!stem_conv_supported(CKPT_DTYPE_BF16, g)) { set_error("stem kernel: unsupported shape"); return CKPT_E_UNSUPPORTED; }
     if (!device_status) { set_error("device status word missing"); return CKPT_E_NULL; }
     if (blocks) *blocks = 0;
-    if (!stem_direct(g, x)) return simt_conv_fwd(CKPT_DTYPE_BF16, g, x, w, z, nullptr, 0, stream);
+    if (!stem_direct(g, x) || (g.cout % 64 && (reinterpret_cast<uintptr_t>(z) & 15u))) return simt_conv_fwd(CKPT_DTYPE_BF16, g, x, w, z, nullptr, 0, stream);
     const StemParams p = stem_params(g);
     CUtensorMap map_out;
     int rc = make_act_map(&map_out, z, g.n, g.ho, g.wo, g.cout, 32, 1, 1);
@@ -3329,7 +3365,7 @@ int stem_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, int*
         if (e != cudaSuccess) return cuda_fail(e, "shared-memory opt-in of the stem kernel");
         attr_set = true;
     }
-    const int co_tiles = g.cout / 64;
+    const int co_tiles = (g.cout + 63) / 64;
     dim3 grid((unsigned)std::min(p.m_tiles, std::max(1, sm_count() / co_tiles)), (unsigned)co_tiles);
     if (blocks) *blocks = partial ? (int)grid.x : 0;
     tc_conv_stem_kernel<<<grid, kStemFwdThreads, kStemFwdSmem, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)w,
@@ -3342,9 +3378,10 @@ int stem_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw,
                     int* device_status, void* stream, const SgdUpdate& upd) {
     if (!stem_conv_supported(CKPT_DTYPE_BF16, g)) { set_error("stem kernel: unsupported shape"); return CKPT_E_UNSUPPORTED; }
     if (!device_status) { set_error("device status word missing"); return CKPT_E_NULL; }
-    if (!scratch || scratch_bytes < stem_conv_scratch_bytes(g)) { set_error("stem wgrad scratch too small"); return CKPT_E_WORKSPACE; }
+    const bool simt = !stem_direct(g, x) || (g.cout % 64 && ((reinterpret_cast<uintptr_t>(dz) & 15u) || !scratch || scratch_bytes < stem_conv_scratch_bytes(g)));
+    if (!simt && (!scratch || scratch_bytes < stem_conv_scratch_bytes(g))) { set_error("stem wgrad scratch too small"); return CKPT_E_WORKSPACE; }
     cudaStream_t st = (cudaStream_t)stream;
-    if (!stem_direct(g, x)) {
+    if (simt) {
         int rc = simt_conv_wgrad(CKPT_DTYPE_BF16, g, dz, x, dw, scratch, scratch_bytes, stream);
         if (rc == CKPT_OK && upd.w) rc = sgd_update(upd, dw, (int64_t)g.cout * 147, stream);
         return rc;
@@ -3360,7 +3397,7 @@ int stem_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw,
         if (e != cudaSuccess) return cuda_fail(e, "shared-memory opt-in of the stem wgrad kernel");
         attr_set = true;
     }
-    dim3 grid((unsigned)p.slices, (unsigned)(g.cout / 64));
+    dim3 grid((unsigned)p.slices, (unsigned)((g.cout + 63) / 64));
     tc_wgrad_stem_kernel<<<grid, kStemWgradThreads, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_stem_kernel", "stem conv wgrad (tensor cores)");
     launch_slice_sum((const float*)scratch, dw, (int64_t)g.cout * 147, p.slices, st, upd);

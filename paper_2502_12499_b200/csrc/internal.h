@@ -113,6 +113,10 @@ int tc_first_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, 
 
 // Tensor-core (tcgen05) implicit-GEMM kernels; *_supported tells whether the shape has one.
 bool tc_conv_supported(int dtype, const ConvGeom& g);
+// Channel counts that do not fill 64-channel blocks.  Such a shape also has CUDA-core kernels to fall back on, which
+// take any alignment: tc_conv_usable is tc_conv_supported for the tensors of one call (null = not looked at).
+bool tc_conv_ragged(const ConvGeom& g);
+bool tc_conv_usable(int dtype, const ConvGeom& g, const void* a, const void* b, const void* c);
 int64_t tc_conv_scratch_bytes(const ConvGeom& g);
 int tc_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu,
                 void* scratch, int64_t scratch_bytes, int* device_status, void* stream);

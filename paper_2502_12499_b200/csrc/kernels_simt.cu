@@ -91,7 +91,7 @@ __global__ void slice_sum_kernel(const float* __restrict__ partial, float* __res
 }
 
 int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, void* stream) {
-    if (!bias && !relu && small_conv_supported(dtype, g)) return small_conv_fwd(g, x, w, z, stream);
+    if (!bias && !relu && small_conv_supported(dtype, g) && g.cout % 64 == 0) return small_conv_fwd(g, x, w, z, stream);
     const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
     const bool v = whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
     return simt_conv(0, dtype, g, x, w, z, bias, relu, M, N, K, v, v, simt::plan(0, M, N, K, v), (cudaStream_t)stream);

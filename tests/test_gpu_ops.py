@@ -404,3 +404,52 @@ def test_softmax_cross_entropy(dtype):
     torch.cuda.synchronize()
     assert abs(loss.item() - loss_ref) <= 1e-5 * abs(loss_ref)
     assert max_rel_err(to_host(g), g_ref) <= TIGHT[dtype]
+
+
+@pytest.mark.parametrize("case", [
+    # channel counts that leave part of a 64-channel block (reduction) or of a tile (output) to zero fill
+    (2, 19, 23, 48, 80, 3, 1),       # ragged tiles in every dimension as well
+    (6, 24, 32, 16, 16, 3, 1),       # the narrowest served
+    (2, 40, 56, 96, 48, 3, 1),       # halo-patch strips; reduction of one and a half blocks, odd column count in wgrad
+    (3, 14, 14, 72, 200, 3, 1),      # stacked strips, two output tiles, the second a partial one
+    (2, 9, 11, 136, 40, 1, 0),       # 1x1, reduction ending in 8 channels
+    (6, 30, 30, 64, 96, 1, 0),       # 1x1 with whole reduction blocks
+    (3, 15, 13, 48, 96, 3, 1, 2),    # stride 2: ragged parity classes
+    (3, 9, 11, 96, 40, 1, 0, 2),     # stride-2 projection: filter read in place, classes without a term
+])
+def test_conv_ragged_channels_on_tensor_cores(case):
+    test_conv_tensor_core_kernels(case)
+
+
+@pytest.mark.parametrize("case,expect_fused", [
+    ((2, 40, 56, 96, 48, 3, 1), True),       # halo-patch kernel
+    ((3, 13, 19, 48, 72, 3, 1), True),       # role-swapped kernel
+    ((3, 31, 33, 136, 40, 3, 1, 2), True),   # generic kernel: the last 32-column chunk is a partial one
+])
+def test_conv_bn_statistics_ragged_channels(case, expect_fused):
+    test_conv_bn_statistics(case, expect_fused)
+
+
+def test_conv_ragged_channels_without_alignment():
+    """48 channels at addresses the TMA unit cannot take: the CUDA-core kernels run."""
+    import torch
+    shape, dtype = ck.ConvShape(2, 16, 17, 48, 48, 3, 1, 1), ck.DTYPE_BF16
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    x, wt = (torch.randn(s, generator=gen, device="cuda").bfloat16() for s in ((2, 16, 17, 48), (48, 3, 3, 48)))
+    scratch = torch.empty(max(ck.conv2d_scratch_bytes(shape, dtype), 256), dtype=torch.uint8, device="cuda")
+    off = torch.empty(x.numel() + 1, dtype=torch.bfloat16, device="cuda")[1:].view(x.shape)
+    off.copy_(x)
+    a, b = torch.empty_like(x), torch.empty_like(x)
+    ck.conv2d_forward(shape, dtype, 0, x, wt, a, scratch)
+    ck.conv2d_forward(shape, dtype, 0, off, wt, b, scratch)
+    assert max_rel_err(to_host(b), to_host(a)) <= TIGHT[dtype]
+
+
+@pytest.mark.parametrize("n,h,w,cout", [(3, 21, 18, 48), (2, 40, 41, 96), (40, 32, 32, 16)])
+def test_first_layer_kernels_ragged_channels(n, h, w, cout):
+    test_first_layer_kernels(n, h, w, cout)
+
+
+@pytest.mark.parametrize("n,h,w,cout", [(2, 23, 19, 32), (2, 30, 37, 72)])
+def test_stem_kernels_ragged_channels(n, h, w, cout):
+    test_stem_kernels(n, h, w, cout)
