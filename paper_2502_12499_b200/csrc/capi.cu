@@ -164,7 +164,15 @@ int ckpt_bn_relu_backward(int dtype, int64_t rows, int32_t c, const void* dy, co
                           const float* stats, int relu, void* dz, float* dgamma, float* dbeta, void* scratch, void* stream) {
     if (!dy || !z || !gamma || !stats || !dz || !dgamma || !dbeta || !scratch) { set_error("null pointer"); return CKPT_E_NULL; }
     if (rows < 1 || c < 1) { set_error("bad shape"); return CKPT_E_BAD_ARG; }
-    return bn_relu_backward(dtype, rows, c, dy, z, gamma, stats, relu, dz, dgamma, dbeta, scratch, stream);
+    // the counters of the cooperative kernel sit at the end of the caller's scratch, behind the rows it uses of it
+    BnBackwardExtra ex;
+    if (bn_backward_fused_applies(dtype, rows, c, dy, z, nullptr, dz) && (uintptr_t)scratch % 16 == 0) {
+        ex.counters = (unsigned*)((char*)scratch + (bn_scratch_bytes(rows, c) & ~(int64_t)15)) - 2 * kBnSyncGroups;
+        ex.status = op_status_word();
+        cudaError_t e = cudaMemsetAsync(ex.counters, 0, 2 * kBnSyncGroups * sizeof(unsigned), (cudaStream_t)stream);
+        if (e != cudaSuccess) return cuda_fail(e, "clearing the batch-norm counters");
+    }
+    return bn_relu_backward(dtype, rows, c, const_cast<void*>(dy), z, stats, relu, dz, dgamma, dbeta, scratch, stream, ex);
 }
 
 int ckpt_maxpool_forward(int dtype, int32_t n, int32_t h, int32_t w, int32_t c, int32_t k, int32_t stride, int32_t pad,

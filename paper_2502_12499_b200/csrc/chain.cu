@@ -115,6 +115,10 @@ struct StepCtx {
     int* status() const { return (int*)(ws + ch->off_misc + 64); }
 };
 
+// The misc region: result (16 bytes), status word (at 64), batch-norm counters (at 128) - cleared before every step - and
+// the labels.
+static const int64_t kMiscCleared = 128 + 2 * kBnSyncGroups * 4, kMiscLabels = kMiscCleared + 256;
+
 static const int64_t kGradId = 1000000007;   // arena id of the per-segment gradient buffer
 
 // Workspace layout per schedule: Algorithm 4's schedule stops before the tail of the block region and the buffer of
@@ -181,6 +185,17 @@ static int conv_backward_pair(StepCtx& c, const ConvGeom& g, const void* dz, con
     }
     if (!sgd && dx && (rc = conv_dgrad_any(c, g, dz, w, dx))) return rc;
     return CKPT_OK;
+}
+
+// What goes along with the batch-norm backward whose scale is parameter `first` (and its shift the next one): the
+// update of both (nothing in the step reads them again: the saved statistics hold what forward and backward need of them).
+static BnBackwardExtra bn_extra(StepCtx& c, int first, const void* mask = nullptr) {
+    BnBackwardExtra ex;
+    ex.mask = mask;
+    ex.gamma = sgd_of(c, first); ex.beta = sgd_of(c, first + 1);
+    ex.counters = (unsigned*)(c.ws + c.ch->off_misc + 128);
+    ex.status = c.status();
+    return ex;
 }
 
 // Convolution followed by the batch statistics of its stored output.  The tensor-core kernels gather the
@@ -310,23 +325,20 @@ static int block_backward(StepCtx& c, const Unit& u, const void* x, const void* 
     int rc;
     // the interiors are re-derived from x, unless every block kept its own since the forward pass (store-all, literally)
     if (!keeps_interiors(c.ch, c.policy) && (rc = block_interiors(c, u, x, B, true))) return rc;
-    // through the final ReLU: g_in <- dL/d(bn3 + shortcut)
-    if ((rc = relu_mask_inplace(dt, out_px * co, g_in, y, c.stream))) return rc;
+    // through the final ReLU: g_in <- dL/d(bn3 + shortcut), by the first batch-norm backward that reads it
+    const void* mask = y;
     const void* dx_shortcut = g_in;                       // identity shortcut: the same gradient flows to x
     if (project) {
-        if ((rc = bn_relu_backward(dt, out_px, co, g_in, B.zp, (const float*)p[10], B.sp, 0, B.t0, (float*)g[10], (float*)g[11], scr, c.stream))) return rc;
-        if ((rc = sgd_step(c, pf + 10)) || (rc = sgd_step(c, pf + 11))) return rc;
+        if ((rc = bn_relu_backward(dt, out_px, co, g_in, B.zp, B.sp, 0, B.t0, (float*)g[10], (float*)g[11], scr, c.stream, bn_extra(c, pf + 10, mask)))) return rc;
+        mask = nullptr;
         if ((rc = conv_backward_pair(c, u.gp, B.t0, x, p[9], pf + 9, g_out ? B.dxs : nullptr))) return rc;
         dx_shortcut = B.dxs;
     }
-    if ((rc = bn_relu_backward(dt, out_px, co, g_in, B.z3, (const float*)p[7], B.s3, 0, B.t1, (float*)g[7], (float*)g[8], scr, c.stream))) return rc;
-    if ((rc = sgd_step(c, pf + 7)) || (rc = sgd_step(c, pf + 8))) return rc;
+    if ((rc = bn_relu_backward(dt, out_px, co, g_in, B.z3, B.s3, 0, B.t1, (float*)g[7], (float*)g[8], scr, c.stream, bn_extra(c, pf + 7, mask)))) return rc;
     if ((rc = conv_backward_pair(c, u.g3, B.t1, B.b, p[6], pf + 6, B.db))) return rc;
-    if ((rc = bn_relu_backward(dt, out_px, mid, B.db, B.z2, (const float*)p[4], B.s2, 1, B.db, (float*)g[4], (float*)g[5], scr, c.stream))) return rc;
-    if ((rc = sgd_step(c, pf + 4)) || (rc = sgd_step(c, pf + 5))) return rc;
+    if ((rc = bn_relu_backward(dt, out_px, mid, B.db, B.z2, B.s2, 1, B.db, (float*)g[4], (float*)g[5], scr, c.stream, bn_extra(c, pf + 4)))) return rc;
     if ((rc = conv_backward_pair(c, u.g2, B.db, B.a, p[3], pf + 3, B.da))) return rc;
-    if ((rc = bn_relu_backward(dt, in_px, mid, B.da, B.z1, (const float*)p[1], B.s1, 1, B.da, (float*)g[1], (float*)g[2], scr, c.stream))) return rc;
-    if ((rc = sgd_step(c, pf + 1)) || (rc = sgd_step(c, pf + 2))) return rc;
+    if ((rc = bn_relu_backward(dt, in_px, mid, B.da, B.z1, B.s1, 1, B.da, (float*)g[1], (float*)g[2], scr, c.stream, bn_extra(c, pf + 1)))) return rc;
     if ((rc = conv_backward_pair(c, u.g1, B.da, x, p[0], pf, g_out))) return rc;
     if (!g_out) return CKPT_OK;
     return add_tensors(dt, in_px * u.in.c, g_out, dx_shortcut, g_out, c.stream);
@@ -390,19 +402,15 @@ static int unit_forward(StepCtx& c, int64_t i, const void* x_raw, void* y, bool 
 static int through_pending_act(StepCtx& c, int64_t j, const void* d_j, void* g, int sum_blocks = 0) {
     if (!pending_act(c.ch, j)) return CKPT_OK;
     const Unit& uj = c.ch->units[j - 1];
-    void* const* p = c.params + uj.param_first;
     void* const* gr = c.grads + uj.param_first;
     int rc;
+    const BnBackwardExtra ex = bn_extra(c, uj.param_first + 1);
     if (sum_blocks > 0)
         rc = bn_relu_backward_from_partials(c.ch->dtype, rows_of(c.ch, j), uj.out.c, g, d_j, stats_of(c, j), 1, g,
-                                            (float*)gr[1], (float*)gr[2], c.ws + c.ch->off_scr, sum_blocks, c.stream);
+                                            (float*)gr[1], (float*)gr[2], c.ws + c.ch->off_scr, sum_blocks, c.stream, ex);
     else
-        rc = bn_relu_backward(c.ch->dtype, rows_of(c.ch, j), uj.out.c, g, d_j, (const float*)p[1], stats_of(c, j), 1, g,
-                              (float*)gr[1], (float*)gr[2], c.ws + c.ch->off_scr, c.stream);
-    // scale and shift of unit j are not read again in this step: the saved statistics block holds what forward and
-    // backward need of them
-    if (!rc) rc = sgd_step(c, uj.param_first + 1);
-    if (!rc) rc = sgd_step(c, uj.param_first + 2);
+        rc = bn_relu_backward(c.ch->dtype, rows_of(c.ch, j), uj.out.c, g, d_j, stats_of(c, j), 1, g,
+                              (float*)gr[1], (float*)gr[2], c.ws + c.ch->off_scr, c.stream, ex);
     return rc;
 }
 
@@ -424,9 +432,8 @@ static int unit_backward(StepCtx& c, int64_t i, const void* x_raw, const void* y
         case CKPT_UNIT_BN:
             // the statistics saved by this unit's (re)computed forward are those of its input
             if ((rc = activated(c, i - 1, x_raw, &x))) return rc;
-            if ((rc = bn_relu_backward(dt, rows_of(c.ch, i), u.out.c, g_in, x, (const float*)p[0], stats_of(c, i), 0,
-                                       g_out ? g_out : g_in, (float*)g[0], (float*)g[1], c.ws + c.ch->off_scr, c.stream))) return rc;
-            if ((rc = sgd_step(c, u.param_first)) || (rc = sgd_step(c, u.param_first + 1))) return rc;
+            if ((rc = bn_relu_backward(dt, rows_of(c.ch, i), u.out.c, g_in, x, stats_of(c, i), 0, g_out ? g_out : g_in, (float*)g[0],
+                                       (float*)g[1], c.ws + c.ch->off_scr, c.stream, bn_extra(c, u.param_first)))) return rc;
             break;
         case CKPT_UNIT_RELU:
             if (g_out && (rc = relu_backward(dt, rows_of(c.ch, i) * u.out.c, g_in, y, g_out, c.stream))) return rc;
@@ -553,7 +560,7 @@ static int run_step(StepCtx& c, double* loss_out) {
         const void* out_act = nullptr;
         if ((rc = activated(c, n, ptr(n), &out_act))) return rc;
         if (ch->loss == CKPT_LOSS_SOFTMAX_CE) {
-            const int32_t* lab = (const int32_t*)(c.ws + ch->off_misc + 128 + 256);
+            const int32_t* lab = (const int32_t*)(c.ws + ch->off_misc + kMiscLabels);
             cudaError_t e = cudaMemcpyAsync((void*)lab, c.labels, ch->batch * sizeof(int32_t), cudaMemcpyDefault, c.stream);
             if (e != cudaSuccess) return cuda_fail(e, "copy of the labels");
             rc = softmax_ce(ch->dtype, (int)ch->batch, so.h * so.w * so.c, out_act, lab,
@@ -733,7 +740,7 @@ static int capture_step(ckpt_chain* ch, StepCtx c, uint64_t key, const std::vect
     const int64_t launches0 = g_launches;
     double unused = 0;
     int rc = CKPT_OK;
-    e = cudaMemsetAsync(c.ws + ch->off_misc, 0, 128, c.stream);
+    e = cudaMemsetAsync(c.ws + ch->off_misc, 0, kMiscCleared, c.stream);
     if (e != cudaSuccess) rc = cuda_fail(e, "clearing the status words");
     if (!rc) rc = run_step(c, &unused);
     StepGraph g;
@@ -970,7 +977,7 @@ int ckpt_chain_create(const ckpt_unit_desc* units, int64_t n, int64_t batch, int
     ch->off_g1 = o; o += ch->max_d;
     ch->off_scr = o; ch->scr_bytes = align_up(scr, 256); o += ch->scr_bytes;
     ch->off_stats = o; o += align_up(std::max<int64_t>(stats_floats, 1) * 4, 256);
-    ch->off_misc = o; o += align_up(128 + 256 + batch * 4, 256);
+    ch->off_misc = o; o += align_up(kMiscLabels + batch * 4, 256);
     ch->off_blk = o; o += ch->blk_bytes;
     // last: the buffer of the activated copy.  Algorithm 4's schedule never needs it (see run_step) and takes a
     // workspace that ends here
@@ -1132,7 +1139,7 @@ int ckpt_train_step(ckpt_chain* chain, const uint8_t* is_ckpt, int policy, const
         chain->seen_keys.push_back(key);       // first step with these arguments runs launch by launch
         if (chain->seen_keys.size() > 64) chain->seen_keys.erase(chain->seen_keys.begin());
     }
-    cudaError_t e = cudaMemsetAsync(c.ws + chain->off_misc, 0, 128, c.stream);
+    cudaError_t e = cudaMemsetAsync(c.ws + chain->off_misc, 0, kMiscCleared, c.stream);
     if (e != cudaSuccess) return cuda_fail(e, "clearing the status words");
     const int64_t launches0 = g_launches;
     rc = run_step(c, &loss);

@@ -138,9 +138,22 @@ int tc_selftest_wait(long long limit_cycles, int* device_status, void* stream);
 int64_t bn_scratch_bytes(int64_t rows, int c);
 int bn_relu_forward(int dtype, int64_t rows, int c, const void* z, const float* gamma, const float* beta,
                     int relu, void* y, float* stats, void* scratch, void* stream);
-int bn_relu_backward(int dtype, int64_t rows, int c, const void* dy, const void* z, const float* gamma,
-                     const float* stats, int relu, void* dz, float* dgamma, float* dbeta, void* scratch,
-                     void* stream);
+// What a batch-norm backward may do besides: mask dy by mask > 0 first (in place: the ReLU behind a residual join), update
+// scale and shift, and, with zeroed counters (2 * kBnSyncGroups words, left zeroed) and a status word, run as one
+// cooperative kernel.
+constexpr int kBnSyncGroups = 64;
+struct BnBackwardExtra {
+    const void* mask = nullptr;
+    SgdUpdate gamma, beta;
+    unsigned* counters = nullptr;
+    int* status = nullptr;
+};
+int bn_relu_backward(int dtype, int64_t rows, int c, void* dy, const void* z, const float* stats, int relu, void* dz, float* dgamma,
+                     float* dbeta, void* scratch, void* stream, const BnBackwardExtra& extra);
+// The cooperative kernel (bn_fused.cu) and the tensors it takes.
+bool bn_backward_fused_applies(int dtype, int64_t rows, int c, const void* dy, const void* z, const void* mask, const void* dz);
+int bn_backward_fused(int dtype, int64_t rows, int c, void* dy, const void* z, const float* stats, int relu, void* dz, float* dgamma,
+                      float* dbeta, float* partial, const BnBackwardExtra& extra, void* stream);
 
 // stats = the 4*c floats written by bn_statistics (mean, 1/std, scale, shift).
 int bn_statistics(int dtype, int64_t rows, int c, const void* z, const float* gamma, const float* beta, float* stats,
@@ -168,7 +181,8 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
 // bytes of scratch with which the general (not 2x2) backward runs in two light passes (0: no such path)
 int64_t maxpool_backward_scratch_bytes(int dtype, int n, int h, int w, int c, int k, int stride, int pad);
 int bn_relu_backward_from_partials(int dtype, int64_t rows, int c, const void* dy, const void* z, const float* stats, int relu,
-                                   void* dz, float* dgamma, float* dbeta, void* scratch, int blocks, void* stream);
+                                   void* dz, float* dgamma, float* dbeta, void* scratch, int blocks, void* stream,
+                                   const BnBackwardExtra& extra);
 int avgpool_forward(int dtype, int n, int h, int w, int c, const void* x, void* y, void* stream);
 int avgpool_backward(int dtype, int n, int h, int w, int c, const void* dy, void* dx, void* stream);
 

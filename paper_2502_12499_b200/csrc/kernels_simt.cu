@@ -14,6 +14,7 @@
 
 #include "conv_simt.cuh"
 #include "internal.h"
+#include "vec.cuh"
 
 namespace ckpt {
 
@@ -30,12 +31,6 @@ ConvGeom make_geom(const ckpt_conv_shape& s) {
     return g;
 }
 
-template <typename T> __device__ __forceinline__ float ld(const T* p);
-template <> __device__ __forceinline__ float ld<float>(const float* p) { return *p; }
-template <> __device__ __forceinline__ float ld<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-template <typename T> __device__ __forceinline__ T cvt(float v);
-template <> __device__ __forceinline__ float cvt<float>(float v) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 cvt<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 // ================================================================================================
 // Convolutions on the CUDA cores (kernel and tile shapes: conv_simt.cuh)
@@ -137,61 +132,6 @@ static unsigned elementwise_grid(int64_t items) {
 constexpr int BN_THREADS = 256;
 constexpr int BN_MAX_BLOCKS = 148 * 8;
 constexpr float BN_EPS = 1e-5f;
-
-template <typename T, int VEC>
-__device__ __forceinline__ void load_vec(const T* p, float (&v)[VEC]) {
-    if constexpr (VEC == 1) {
-        v[0] = ld(p);
-    } else if constexpr (sizeof(T) == 4) {
-        float4 t = *reinterpret_cast<const float4*>(p);
-        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-    } else {
-        uint4 t = *reinterpret_cast<const uint4*>(p);
-        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&t);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { float2 f = __bfloat1622float2(h[i]); v[2 * i] = f.x; v[2 * i + 1] = f.y; }
-    }
-}
-template <typename T, int VEC>
-__device__ __forceinline__ void store_vec(T* p, const float (&v)[VEC]) {
-    if constexpr (VEC == 1) {
-        *p = cvt<T>(v[0]);
-    } else if constexpr (sizeof(T) == 4) {
-        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    } else {
-        uint4 t;
-        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&t);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-        *reinterpret_cast<uint4*>(p) = t;
-    }
-}
-
-// A vector as loaded: kept packed in registers until it is used, so that many loads can be in flight
-// per thread without the register cost of their unpacked form.
-template <typename T, int VEC> struct RawVec { T e[VEC]; };
-template <> struct RawVec<__nv_bfloat16, 8> { uint4 q; };
-template <> struct RawVec<float, 4> { float4 q; };
-template <typename T, int VEC>
-__device__ __forceinline__ RawVec<T, VEC> load_raw(const T* p) {
-    RawVec<T, VEC> r;
-    if constexpr (VEC == 1) r.e[0] = *p;
-    else if constexpr (sizeof(T) == 4) r.q = *reinterpret_cast<const float4*>(p);
-    else r.q = *reinterpret_cast<const uint4*>(p);
-    return r;
-}
-template <typename T, int VEC>
-__device__ __forceinline__ void unpack(const RawVec<T, VEC>& r, float (&v)[VEC]) {
-    if constexpr (VEC == 1) {
-        v[0] = (float)r.e[0];
-    } else if constexpr (sizeof(T) == 4) {
-        v[0] = r.q.x; v[1] = r.q.y; v[2] = r.q.z; v[3] = r.q.w;
-    } else {
-        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&r.q);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { float2 f = __bfloat1622float2(h[i]); v[2 * i] = f.x; v[2 * i + 1] = f.y; }
-    }
-}
 
 // Launch shape of the streaming element-wise kernels: a block works through `per_block` consecutive
 // chunks of THREADS*U vectors.  Few chunks per block on large tensors (many short-lived blocks keep
@@ -342,7 +282,7 @@ __global__ void __launch_bounds__(32) bn_finalize_fwd_kernel(const float* __rest
 //   dz = scale*g - k1 - xhat*k2,  k1 = scale*dbeta/rows, k2 = scale*dgamma/rows
 __global__ void __launch_bounds__(32) bn_finalize_bwd_kernel(const float* __restrict__ partial, int blocks, int c, double inv_rows,
                                        const float* __restrict__ stats, float* __restrict__ dgamma, float* __restrict__ dbeta,
-                                       float* __restrict__ coef) {
+                                       float* __restrict__ coef, SgdUpdate gamma, SgdUpdate beta) {
     const int ch = blockIdx.x;
     double s, q;
     warp_channel_sums(partial, blocks, c, ch, s, q);
@@ -351,6 +291,8 @@ __global__ void __launch_bounds__(32) bn_finalize_bwd_kernel(const float* __rest
     const double gx = (double)stats[c + ch] * (q - (double)stats[ch] * s);
     dbeta[ch] = (float)s;
     dgamma[ch] = (float)gx;
+    if (gamma.w) { float* w = (float*)gamma.w + ch; *w = fmaf(-gamma.lr, (float)gx, *w); }
+    if (beta.w) { float* w = (float*)beta.w + ch; *w = fmaf(-beta.lr, (float)s, *w); }
     double scale = stats[2 * c + ch];
     // dz = scale*g - k1 - xhat*k2 with k1 = scale*dbeta/rows, k2 = scale*dgamma/rows and
     // xhat = (z - mean)*inv_std, regrouped as  dz = scale*g - A - z*B
@@ -592,7 +534,7 @@ static int bn_apply_t(int64_t rows, int c, const void* z, const float* stats, in
 
 template <typename T, int VEC>
 static int bn_backward_t(int64_t rows, int c, const void* dy, const void* z, const float* stats, int relu, void* dz,
-                         float* dgamma, float* dbeta, void* scratch, cudaStream_t st) {
+                         float* dgamma, float* dbeta, void* scratch, const BnBackwardExtra& ex, cudaStream_t st) {
     BnLayout L = bn_layout(rows, c, VEC);
     float* partial = (float*)scratch;
     float* coef = partial + (size_t)BN_MAX_BLOCKS * c * 2;
@@ -607,7 +549,7 @@ static int bn_backward_t(int64_t rows, int c, const void* dy, const void* z, con
                                                                           L.rows_per_iter, L.rows_per_block, partial);
     }
     CKPT_LAUNCH_CHECK("batch-norm backward sums");
-    bn_finalize_bwd_kernel<<<c, 32, 0, st>>>(partial, blocks, c, 1.0 / (double)rows, stats, dgamma, dbeta, coef);
+    bn_finalize_bwd_kernel<<<c, 32, 0, st>>>(partial, blocks, c, 1.0 / (double)rows, stats, dgamma, dbeta, coef, ex.gamma, ex.beta);
     CKPT_LAUNCH_CHECK("batch-norm backward finalize");
     int64_t vecs = rows * c / VEC;
     const StreamGrid sg = stream_grid(vecs, 256, BN_BWD_U);
@@ -778,26 +720,31 @@ int add_tensors(int dtype, int64_t elems, const void* a, const void* b, void* ou
     return CKPT_OK;
 }
 
-int bn_relu_backward(int dtype, int64_t rows, int c, const void* dy, const void* z, const float* gamma, const float* stats,
-                     int relu, void* dz, float* dgamma, float* dbeta, void* scratch, void* stream) {
-    (void)gamma;   // scale = gamma * inv_std is part of the saved statistics
+int bn_relu_backward(int dtype, int64_t rows, int c, void* dy, const void* z, const float* stats, int relu, void* dz, float* dgamma,
+                     float* dbeta, void* scratch, void* stream, const BnBackwardExtra& ex) {
     cudaStream_t st = (cudaStream_t)stream;
+    if (ex.counters && ex.status && bn_backward_fused_applies(dtype, rows, c, dy, z, ex.mask, dz))
+        return bn_backward_fused(dtype, rows, c, dy, z, stats, relu, dz, dgamma, dbeta, (float*)scratch, ex, stream);
+    if (ex.mask) {
+        int rc = relu_mask_inplace(dtype, rows * c, dy, ex.mask, stream);
+        if (rc) return rc;
+    }
     int vec = bn_vec(dtype, c);
     if (dtype == CKPT_DTYPE_BF16)
-        return vec == 8 ? bn_backward_t<__nv_bfloat16, 8>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, st)
-                        : bn_backward_t<__nv_bfloat16, 1>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, st);
-    return vec == 4 ? bn_backward_t<float, 4>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, st)
-                    : bn_backward_t<float, 1>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, st);
+        return vec == 8 ? bn_backward_t<__nv_bfloat16, 8>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, ex, st)
+                        : bn_backward_t<__nv_bfloat16, 1>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, ex, st);
+    return vec == 4 ? bn_backward_t<float, 4>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, ex, st)
+                    : bn_backward_t<float, 1>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, ex, st);
 }
 
 // Batch-norm backward whose per-channel sums (sum g, sum g*z over `blocks` partial row pairs at the start of
 // `scratch`) were left by the kernel that produced dy: finalize and apply only.
 template <typename T, int VEC>
 static int bn_backward_tail_t(int64_t rows, int c, const void* dy, const void* z, const float* stats, int relu, void* dz,
-                              float* dgamma, float* dbeta, void* scratch, int blocks, cudaStream_t st) {
+                              float* dgamma, float* dbeta, void* scratch, int blocks, const BnBackwardExtra& ex, cudaStream_t st) {
     float* partial = (float*)scratch;
     float* coef = partial + (size_t)BN_MAX_BLOCKS * c * 2;
-    bn_finalize_bwd_kernel<<<c, 32, 0, st>>>(partial, blocks, c, 1.0 / (double)rows, stats, dgamma, dbeta, coef);
+    bn_finalize_bwd_kernel<<<c, 32, 0, st>>>(partial, blocks, c, 1.0 / (double)rows, stats, dgamma, dbeta, coef, ex.gamma, ex.beta);
     CKPT_LAUNCH_CHECK("batch-norm backward finalize");
     const int64_t vecs = rows * c / VEC;
     const StreamGrid sg = stream_grid(vecs, 256, BN_BWD_U);
@@ -807,15 +754,16 @@ static int bn_backward_tail_t(int64_t rows, int c, const void* dy, const void* z
     return CKPT_OK;
 }
 int bn_relu_backward_from_partials(int dtype, int64_t rows, int c, const void* dy, const void* z, const float* stats, int relu,
-                                   void* dz, float* dgamma, float* dbeta, void* scratch, int blocks, void* stream) {
+                                   void* dz, float* dgamma, float* dbeta, void* scratch, int blocks, void* stream,
+                                   const BnBackwardExtra& ex) {
     cudaStream_t st = (cudaStream_t)stream;
     if (blocks < 1 || blocks > BN_MAX_BLOCKS) { set_error("batch-norm backward: %d partial rows", blocks); return CKPT_E_BAD_ARG; }
     int vec = bn_vec(dtype, c);
     if (dtype == CKPT_DTYPE_BF16)
-        return vec == 8 ? bn_backward_tail_t<__nv_bfloat16, 8>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, blocks, st)
-                        : bn_backward_tail_t<__nv_bfloat16, 1>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, blocks, st);
-    return vec == 4 ? bn_backward_tail_t<float, 4>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, blocks, st)
-                    : bn_backward_tail_t<float, 1>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, blocks, st);
+        return vec == 8 ? bn_backward_tail_t<__nv_bfloat16, 8>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, blocks, ex, st)
+                        : bn_backward_tail_t<__nv_bfloat16, 1>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, blocks, ex, st);
+    return vec == 4 ? bn_backward_tail_t<float, 4>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, blocks, ex, st)
+                    : bn_backward_tail_t<float, 1>(rows, c, dy, z, stats, relu, dz, dgamma, dbeta, scratch, blocks, ex, st);
 }
 
 // ================================================================================================

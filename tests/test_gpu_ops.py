@@ -453,3 +453,49 @@ def test_first_layer_kernels_ragged_channels(n, h, w, cout):
 @pytest.mark.parametrize("n,h,w,cout", [(2, 23, 19, 32), (2, 30, 37, 72)])
 def test_stem_kernels_ragged_channels(n, h, w, cout):
     test_stem_kernels(n, h, w, cout)
+
+
+@pytest.mark.parametrize("dtype", [ck.DTYPE_F32, ck.DTYPE_BF16])
+@pytest.mark.parametrize("rows,c,relu", [(1, 8, 1), (63, 64, 1), (65, 64, 0), (1000, 48, 1), (257, 72, 1), (129, 2048, 1), (30000, 256, 1), (120011, 64, 1),
+                                         (1031, 1000, 0)])
+def test_bn_backward_in_one_kernel(rows, c, relu, dtype):
+    """The cooperative batch-norm backward at the edges of its split: a single row, less and more than a step of a CTA,
+    channel groups of every width (lanes that do and do not divide a warp), tensors that fit its ring and tensors that
+    are walked back through global memory.  Against float64 on the stored tensors."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(rows + c)
+    store = torch.bfloat16 if dtype == ck.DTYPE_BF16 else torch.float32
+    z, dy = ((torch.randn((rows, c), generator=gen, device="cuda") * 1.3 + 0.2).to(store) for _ in range(2))
+    gamma = torch.rand(c, generator=gen, device="cuda") + 0.5
+    beta = torch.randn(c, generator=gen, device="cuda") * 0.3
+    mean, inv = z.double().mean(0), (z.double().var(0, unbiased=False) + 1e-5).rsqrt()
+    stats = torch.stack((mean, inv, gamma * inv, beta - mean * gamma * inv)).float()
+    scratch = torch.full((ck.bn_scratch_bytes(rows, c),), 0xFF, dtype=torch.uint8, device="cuda")
+    outs = []
+    for rep in range(2):
+        dz, dg, db = torch.full_like(z, float("nan")), torch.empty(c, device="cuda"), torch.empty(c, device="cuda")
+        ck.bn_relu_backward(dtype, rows, c, dy, z, gamma, stats, relu, dz, dg, db, scratch)
+        outs.append((dz, dg, db))
+    torch.cuda.synchronize()
+    assert ck.op_status() == 0
+    for a, b in zip(outs[0], outs[1]):
+        assert torch.equal(a, b)
+    s = stats.double()
+    t = z.double() * s[2] + s[3]
+    g = dy.double() * (t > 0) if relu else dy.double()
+    # columns with a value whose sign float32 may round the other way are left out of the comparison of dz
+    sure = ~(t.abs() < 2.0 ** -22 * ((z.double() * s[2]).abs() + s[3].abs())).any(0)
+    assert sure.double().mean() > 0.5
+    xhat = (z.double() - s[0]) * s[1]
+    dbeta, dgamma = g.sum(0), (g * xhat).sum(0)
+    want = s[2] * (g - dbeta / rows - xhat * dgamma / rows)
+    dz, dg, db = (t.double() for t in outs[0])
+    # float32 sums of `rows` terms (one of them more or less where a sign was not sure)
+    scale = float(g.abs().sum(0).max()) + 1e-30
+    assert float((db - dbeta).abs().max()) <= 1e-5 * scale and float((dg - dgamma).abs().max()) <= 1e-5 * scale * float(xhat.abs().max() + 1)
+    # the result is scale*g - A - z*B; A and B carry the float32 rounding of sums over |g| and |g z|, and there is one rounding
+    # to the storage type
+    absg, absgz = g.abs().sum(0), (g * z.double()).abs().sum(0)
+    terms = s[2].abs() * (g.abs() + (absg + s[1] ** 2 * (absgz + s[0].abs() * absg) * (s[0].abs() + z.double().abs())) / rows)
+    off = (dz - want).abs() > 2.0 ** -20 * terms + (2.0 ** -8 * want.abs() if dtype == ck.DTYPE_BF16 else 0.0)
+    assert not (off & sure).any()
