@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "internal.h"
@@ -133,6 +134,18 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// The same with the descriptors in halves: only the low words (address and leading offset) change along a reduction, and
+// the thread that issues the MMAs has 30 to 130 clocks for each.
+__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                          uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
 // The mbarrier is signalled once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -163,6 +176,8 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     d |= (uint64_t)2 << 61;     // 128-byte swizzle
     return d;
 }
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return ((addr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16); }
+__device__ __forceinline__ uint32_t desc_hi(uint32_t sbo) { return ((sbo >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29); }
 // Instruction descriptor: f32 accumulator, bf16 A and B, M x N tile, operand majors (0 = K, 1 = MN).
 __host__ __device__ inline uint32_t instr_desc(int M, int N, int a_mn_major, int b_mn_major) {
     uint32_t d = 0;
@@ -174,6 +189,27 @@ __host__ __device__ inline uint32_t instr_desc(int M, int N, int a_mn_major, int
     d |= (uint32_t)(N >> 3) << 17;
     d |= (uint32_t)(M >> 4) << 24;
     return d;
+}
+
+// Cluster rank, cluster-wide barrier (every thread of every CTA, also after a failed wait) and loads from a peer's shared memory.
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_address(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float4 peer_load(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
@@ -505,7 +541,7 @@ struct TParams {
     // matrix, i.e. zeros)
     int pair;
     int tap_col2[12];
-    int tw_log, th_log;          // pixel tile tw x th x tn = 256, powers of two
+    int tw_log, th_log;          // pixel tile tw x th x tn = tile_cols: powers of two, or one row of tile_cols pixels (tw_log = 8)
     int tw, th, tn;
     int tiles_w, tiles_h, tiles_n;
     int co_tiles, p_tiles, ctas_per_co;
@@ -514,7 +550,8 @@ struct TParams {
     int patch_ok;                // the caller filled ncols / col_term
     int ncols;                   // columns per 64-channel block: (horizontal offset, channel offset) pairs
     int col_term[4][3];          // term (index into the tap tables) of column c at vertical tap dy; tap_dh = dy - 1
-    int tile_cols;               // pixels per tile = 8 * th * stack
+    int tile_cols;               // pixels per tile: a multiple of 32, at most 256; 8 * th * stack for the halo-patch kernel
+    int split;                   // CTAs of a cluster that share the reduction of a tile
     uint32_t patch_bytes;        // 8 x (th + 2) pixels x 128 bytes; stacked: 8 x th x stack
     // stacked form for small images (tc_conv_tp_kernel): a tile is the strip of `stack` whole images, each taking th
     // rows of the accumulator (its H rows and th - H idle ones) and th rows of the patch (rows -1 .. th - 2: the image,
@@ -523,38 +560,49 @@ struct TParams {
     int stack;                   // 0 = one image per tile with a halo of its own (th + 2 patch rows)
 };
 
+// Coordinates of filter box `box` (0 or 1) of a term: one box of 128 output channels x 64 reduction channels, or two of
+// 64 output channels each (filter read in place, pixel pairs).
+template <bool A_MN>
+__device__ __forceinline__ void filter_box(const TParams& p, int tap, int blk, int co_tile, int box, int& c0, int& c1) {
+    if (p.pair) {
+        const int col = box ? p.tap_col2[tap] : p.tap_col[tap];
+        if (A_MN) {     // forward filter [c_red][9][64]: 64 reduction rows x the 64 output channels of a position
+            c0 = (col < 0 ? 9 : col) * 64; c1 = blk * 64;
+        } else {        // filter [64][9][c_red]: the 64 output channels x 64 reduction channels of a position
+            c0 = col < 0 ? 9 * p.c_red : col * p.c_red + blk * 64; c1 = 0;
+        }
+    } else if (A_MN) {
+        // (with 64 output channels the second box lies past them: it is sent outside the matrix, i.e. zero fill)
+        const int ch = co_tile * 128 + box * 64;
+        c0 = box == 0 || ch < p.c_out ? p.tap_col[tap] * p.c_out + ch : p.taps * p.c_out; c1 = blk * 64;
+    } else {
+        c0 = p.tap_col[tap] * p.c_red + blk * 64; c1 = co_tile * 128;
+    }
+}
 template <bool A_MN>
 __device__ __forceinline__ void load_filter_boxes(const TParams& p, const CUtensorMap* map_w, uint32_t a_dst, uint32_t bar, int tap, int blk,
                                                   int co_tile) {
-    if (p.pair) {
-        const int c0 = p.tap_col[tap], c1 = p.tap_col2[tap];
-        if (A_MN) {     // forward filter [c_red][9][64]: 64 reduction rows x the 64 output channels of a position
-            tma_load_2d(a_dst, map_w, bar, (c0 < 0 ? 9 : c0) * 64, blk * 64);
-            tma_load_2d(a_dst + 8192, map_w, bar, (c1 < 0 ? 9 : c1) * 64, blk * 64);
-        } else {        // filter [64][9][c_red]: the 64 output channels x 64 reduction channels of a position
-            tma_load_2d(a_dst, map_w, bar, c0 < 0 ? 9 * p.c_red : c0 * p.c_red + blk * 64, 0);
-            tma_load_2d(a_dst + 8192, map_w, bar, c1 < 0 ? 9 * p.c_red : c1 * p.c_red + blk * 64, 0);
-        }
-    } else if (A_MN) {
-        tma_load_2d(a_dst, map_w, bar, p.tap_col[tap] * p.c_out + co_tile * 128, blk * 64);
-        // (with 64 output channels the second box lies past them: it is sent outside the matrix, i.e. zero fill)
-        tma_load_2d(a_dst + 8192, map_w, bar,
-                    co_tile * 128 + 64 < p.c_out ? p.tap_col[tap] * p.c_out + co_tile * 128 + 64 : p.taps * p.c_out, blk * 64);
-    } else {
-        tma_load_2d(a_dst, map_w, bar, p.tap_col[tap] * p.c_red + blk * 64, co_tile * 128);
+    for (int box = 0; box < (A_MN || p.pair ? 2 : 1); ++box) {
+        int c0, c1;
+        filter_box<A_MN>(p, tap, blk, co_tile, box, c0, c1);
+        tma_load_4d(a_dst + box * 8192, map_w, bar, c0, c1, 0, 0);
     }
 }
 
 // A_MN (dgrad): the M operand is the forward filter [c_red][taps][c_out] read in place, output channels contiguous:
 // two boxes of 64 reduction rows x 64 output channels per stage (at the column block of the mirrored filter
 // position), an MN-major operand for the tensor core.  No transposed copy of the filter is made.
-template <bool A_MN>
+// SPLIT: few tiles with a long reduction (small images, small batches).  The p.split CTAs of a cluster take a share of
+// the terms of one tile each, leave their float32 accumulators in shared memory and add them up in rank order, every
+// 32 x 32 block by one warp of the cluster, which finishes it as usual.
+template <bool A_MN, bool SPLIT>
 __global__ void __launch_bounds__(kThreadsT, 1)
 tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                  const __grid_constant__ CUtensorMap map_out, float* __restrict__ stat_partial, TParams p, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    constexpr uint32_t a_bytes = 128 * 128, b_bytes = 256 * 128, stage_bytes = a_bytes + b_bytes;
+    constexpr uint32_t a_bytes = 128 * 128;
+    const uint32_t stage_bytes = a_bytes + (uint32_t)p.tile_cols * 128;
     const uint32_t bars = base + (uint32_t)p.stages * stage_bytes;           // full[s], empty[s], acc_full[2], acc_empty[2]
     const uint32_t out_stage = bars + 256;                                   // [8 warps][2][32 pixels x 32 channels] bf16
     __shared__ uint32_t tmem_base_slot;
@@ -562,11 +610,14 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     volatile int* failed = &failed_flag;
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int co_tile = blockIdx.x % p.co_tiles;
-    const int first = blockIdx.x / p.co_tiles;
+    const int rank = SPLIT ? (int)cluster_rank() : 0;
+    const int work = SPLIT ? blockIdx.x / p.split : blockIdx.x;
+    const int co_tile = work % p.co_tiles;
+    const int first = work / p.co_tiles;
     const int my_tiles = first < p.p_tiles ? (p.p_tiles - first + p.ctas_per_co - 1) / p.ctas_per_co : 0;
     const int blocks = (p.c_red + 63) / 64;      // a ragged last block is zero-filled by the TMA unit
-    const int iters = p.taps * blocks;
+    const int terms = p.taps * blocks;
+    const int it0 = SPLIT ? terms * rank / p.split : 0, it1 = SPLIT ? terms * (rank + 1) / p.split : terms;
 
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (kMaxStages + s); };
@@ -593,49 +644,84 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
 
-    if (warp == 0 && lane == 0) {
-        // ---------------- TMA producer: filter box (M operand) and pixel box (N operand) per stage
-        int g = 0;
+    if (warp == 0) {
+        // ---------------- TMA producer: pixel box (N operand, lane 0) and filter box or boxes (M operand, lanes 1 and 2)
+        // of a stage leave as one instruction, the lanes differing in tensor map, coordinates and target.  One thread
+        // issuing them in turn took about 790 clocks per stage, whatever the tile: more than the MMAs of a stage.
+        const bool two = A_MN || p.pair;
+        const uint32_t lane_dst = lane == 0 ? a_bytes : (lane == 2 ? 8192u : 0u);
+        const CUtensorMap* const map = lane == 0 ? &map_x : &map_w;
+        int g = 0, s = 0;
+        uint32_t phase = 1u, dst = base + lane_dst;
         bool ok = true;
         for (int j = 0; j < my_tiles && ok; ++j) {
             int w0, h0, n0;
             tile_origin(j, w0, h0, n0);
-            for (int it = 0; it < iters; ++it, ++g) {
-                const int s = g % p.stages;
-                if (!mbar_wait(empty_bar(s), ((uint32_t)(g / p.stages) & 1u) ^ 1u, failed, status, 901)) { ok = false; break; }
-                const int tap = it / blocks, blk = it % blocks;
-                const uint32_t a_dst = base + (uint32_t)s * stage_bytes;
-                mbar_expect_tx(full_bar(s), stage_bytes);
-                load_filter_boxes<A_MN>(p, &map_w, a_dst, full_bar(s), tap, blk, co_tile);
-                tma_load_4d(a_dst + a_bytes, &map_x, full_bar(s), blk * 64 + p.tap_xc[tap], w0 + p.tap_dw[tap], h0 + p.tap_dh[tap], n0);
+            int tap = it0 / blocks, blk = it0 % blocks, left = it1 - it0;
+            while (left > 0 && ok) {
+                // one term: its reduction blocks move along one coordinate
+                int c0 = 0, c1 = 0, c2 = 0, c3 = 0, step0 = 64, step1 = 0;
+                if (lane == 0) {
+                    c0 = blk * 64 + p.tap_xc[tap]; c1 = w0 + p.tap_dw[tap]; c2 = h0 + p.tap_dh[tap]; c3 = n0;
+                } else {
+                    filter_box<A_MN>(p, tap, blk, co_tile, lane == 2, c0, c1);
+                    if (A_MN) { step0 = 0; step1 = 64; }
+                    else if (p.pair && (lane == 2 ? p.tap_col2[tap] : p.tap_col[tap]) < 0) step0 = 0;
+                }
+                const int here = min(blocks - blk, left);
+                for (int q = 0; q < here; ++q, ++g) {
+                    if (!mbar_wait(empty_bar(s), phase, failed, status, 901)) { ok = false; break; }
+                    if (lane == 0) mbar_expect_tx(full_bar(s), stage_bytes);
+                    __syncwarp();
+                    if (lane < (two ? 3 : 2)) tma_load_4d(dst, map, full_bar(s), c0, c1, c2, c3);
+                    c0 += step0; c1 += step1; dst += stage_bytes;
+                    if (++s == p.stages) { s = 0; phase ^= 1u; dst = base + lane_dst; }
+                }
+                left -= here; blk = 0; ++tap;
             }
         }
-        if (*failed) {
+        if (*failed && lane == 0) {
             for (int q = max(0, g - p.stages); q < g; ++q) mbar_drain(full_bar(q % p.stages), (uint32_t)(q / p.stages) & 1u);
         }
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer
-        const uint32_t idesc = instr_desc(128, 256, A_MN ? 1 : 0, 0);
-        constexpr uint32_t a_step = A_MN ? 2048u : 32u, a_lbo = A_MN ? 8192u : 0u;
+        const uint32_t idesc = instr_desc(128, p.tile_cols, A_MN ? 1 : 0, 0);
+        constexpr uint32_t a_step = (A_MN ? 2048u : 32u) / 16, b_step = 32u / 16;
+        const uint32_t a_lo0 = desc_lo(base, A_MN ? 8192u : 0u), b_lo0 = desc_lo(base + a_bytes, 0u), hi = desc_hi(1024u), lo_step = stage_bytes / 16;
         bool ok = true;
-        int g = 0;
+        int s = 0;
+        uint32_t phase = 0u, a_lo = a_lo0, b_lo = b_lo0;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int buf = j & 1;
             if (!mbar_wait(acc_empty0 + 8 * buf, ((uint32_t)(j >> 1) & 1u) ^ 1u, failed, status, 904)) { ok = false; break; }
             const uint32_t acc = tmem_base + (uint32_t)(buf * 256);
-            for (int it = 0; it < iters; ++it, ++g) {
-                const int s = g % p.stages;
-                if (!mbar_wait(full_bar(s), (uint32_t)(g / p.stages) & 1u, failed, status, 902)) { ok = false; break; }
+            uint32_t more = 0u;
+            for (int it = it0; it < it1; ++it) {
+                if (!mbar_wait(full_bar(s), phase, failed, status, 902)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t a_addr = base + (uint32_t)s * stage_bytes;
-                const uint32_t b_addr = a_addr + a_bytes;
+                umma_bf16(acc, a_lo, hi, b_lo, hi, idesc, more);
+                more = 1u;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma_bf16(acc, smem_desc(a_addr + kk * a_step, a_lbo, 1024), smem_desc(b_addr + kk * 32, 0, 1024), idesc,
-                              (it > 0 || kk > 0) ? 1u : 0u);
+                for (int kk = 1; kk < 4; ++kk) umma_bf16(acc, a_lo + kk * a_step, hi, b_lo + kk * b_step, hi, idesc, 1u);
                 umma_commit(empty_bar(s));
+                a_lo += lo_step; b_lo += lo_step;
+                if (++s == p.stages) { s = 0; phase ^= 1u; a_lo = a_lo0; b_lo = b_lo0; }
             }
             if (ok) umma_commit(acc_full0 + 8 * buf);
+        }
+    } else if (SPLIT && warp >= 2) {
+        // ---------------- accumulator to shared memory, [pixel][channel] floats over the operand stages (all of them read)
+        const int quarter = warp % 4;
+        if (mbar_wait(acc_full0, 0, failed, status, 905)) {
+            tc_fence_after();
+            for (int c0 = (warp - 2) / 4 * 32; c0 < p.tile_cols; c0 += 32 * kTEpi) {
+                uint32_t v[32];
+                tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
+                const uint32_t dst = base + (uint32_t)(c0 * 512 + (quarter * 32 + lane) * 4);
+#pragma unroll
+                for (int e = 0; e < 32; ++e) asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + (uint32_t)(e * 512)), "r"(v[e]) : "memory");
+            }
+            tc_fence_before();
         }
     } else if (warp >= 2) {
         // ---------------- epilogue: lane of the accumulator = output channel, column = pixel of the tile.  A chunk
@@ -659,10 +745,10 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             int w0, h0, n0;
             tile_origin(j, w0, h0, n0);
 #pragma unroll 1
-            for (int c0 = half * 32; c0 < 256; c0 += 32 * kTEpi, ++chunk_count) {
+            for (int c0 = half * 32; c0 < p.tile_cols; c0 += 32 * kTEpi, ++chunk_count) {
                 // lane e works out whether pixel c0 + e of the tile lies inside the tensor (for the sums)
                 const int idx = c0 + lane;
-                const int wl = idx & (p.tw - 1), hl = (idx >> p.tw_log) & (p.th - 1), nl = idx >> (p.tw_log + p.th_log);
+                const int wl = idx & ((1 << p.tw_log) - 1), hl = (idx >> p.tw_log) & (p.th - 1), nl = idx >> (p.tw_log + p.th_log);
                 const bool inside = (w0 + wl < p.W) && (h0 + hl < p.H) && (n0 + nl < p.N);
                 const uint32_t in_mask = __ballot_sync(0xffffffffu, inside);
                 uint32_t v[32];
@@ -674,7 +760,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0 && in_mask != 0u && co_tile * 128 + quarter * 32 < p.c_out) {
-                    const int cw = c0 & (p.tw - 1), chh = (c0 >> p.tw_log) & (p.th - 1), cn = c0 >> (p.tw_log + p.th_log);
+                    const int cw = c0 & ((1 << p.tw_log) - 1), chh = (c0 >> p.tw_log) & (p.th - 1), cn = c0 >> (p.tw_log + p.th_log);
                     tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
                 }
                 // also for a chunk outside the tensor (an empty group): the wait above counts groups, one per chunk
@@ -697,6 +783,64 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 stat_partial[(row * 2 + 1) * p.c_out + co] = s2;
             }
         }
+    }
+    if (SPLIT) {
+        __syncwarp();
+        cluster_sync();
+        if (warp >= 2 && !*failed) {
+            int w0, h0, n0;
+            tile_origin(0, w0, h0, n0);
+            const int blocks32 = p.tile_cols / 32 * 4;              // (pixel chunk, channel quarter)
+            for (int b = rank + p.split * (warp - 2); b < blocks32; b += p.split * 4 * kTEpi) {
+                const int c0 = b / 4 * 32, quarter = b % 4, co = co_tile * 128 + quarter * 32 + lane;
+                const int idx = c0 + lane;
+                const int wl = idx & ((1 << p.tw_log) - 1), hl = (idx >> p.tw_log) & (p.th - 1), nl = idx >> (p.tw_log + p.th_log);
+                const bool inside = (w0 + wl < p.W) && (h0 + hl < p.H) && (n0 + nl < p.N);
+                const uint32_t in_mask = __ballot_sync(0xffffffffu, inside);
+                // 16-byte pieces of the block (four pixels per load of the warp) from every rank, the sums back into this
+                // CTA's copy - no one else reads this block - and from there one channel per lane
+                const uint32_t block = base + (uint32_t)(c0 * 512 + quarter * 128), piece = block + (uint32_t)((lane / 8) * 512 + (lane % 8) * 16);
+                float4 acc[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int r = 0; r < p.split; ++r) {
+                    const uint32_t src = peer_address(piece, (uint32_t)r);
+                    float4 x[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) x[e] = peer_load(src + (uint32_t)(e * 2048));
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) { acc[e].x += x[e].x; acc[e].y += x[e].y; acc[e].z += x[e].z; acc[e].w += x[e].w; }
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(piece + (uint32_t)(e * 2048)), "f"(acc[e].x), "f"(acc[e].y), "f"(acc[e].z), "f"(acc[e].w) : "memory");
+                __syncwarp();
+                uint32_t v[32];
+#pragma unroll
+                for (int e = 0; e < 32; ++e) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v[e]) : "r"(block + (uint32_t)(e * 512 + lane * 4)) : "memory");
+                float sum[4] = {0.f, 0.f, 0.f, 0.f}, sumsq[4] = {0.f, 0.f, 0.f, 0.f};
+                const uint32_t slab = out_stage + (uint32_t)((warp - 2) * kTSlabs * 2048);
+                if (lane == 0) tma_store_wait_read<0>();
+                __syncwarp();
+                t_chunk_to_slab<true>(v, in_mask, slab + (uint32_t)(lane * 2), stat_partial != nullptr, sum, sumsq);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0 && in_mask != 0u && co_tile * 128 + quarter * 32 < p.c_out) {
+                    const int cw = c0 & ((1 << p.tw_log) - 1), chh = (c0 >> p.tw_log) & (p.th - 1), cn = c0 >> (p.tw_log + p.th_log);
+                    tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
+                    tma_store_commit();
+                }
+                if (stat_partial && co < p.c_out) {
+                    // one partial row pair per pixel chunk
+                    const size_t row = (size_t)first * (p.tile_cols / 32) + c0 / 32;
+                    stat_partial[(row * 2) * p.c_out + co] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+                    stat_partial[(row * 2 + 1) * p.c_out + co] = (sumsq[0] + sumsq[1]) + (sumsq[2] + sumsq[3]);
+                }
+            }
+            if (lane == 0) tma_store_wait_all();
+        }
+        __syncwarp();
+        cluster_sync();                                              // no CTA leaves while a peer reads its shared memory
     }
     tc_fence_before();
     __syncthreads();
@@ -779,27 +923,29 @@ tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer: per column one patch, then the filter boxes of its three vertical taps
-        int ga = 0, gp = 0;
+        int ga = 0, gp = 0, sa = 0, sp = 0;
+        uint32_t a_phase = 1u, p_phase = 1u;
         bool ok = true;
         for (int j = 0; j < my_tiles && ok; ++j) {
             int w0, h0, n0;
             tile_origin(j, w0, h0, n0);
+            int col = 0, blk = 0;
             for (int c = 0; c < cols && ok; ++c, ++gp) {
-                const int col = c / blocks, blk = c % blocks;
-                const int sp = gp % kTpPatches;
-                if (!mbar_wait(p_empty(sp), ((uint32_t)(gp / kTpPatches) & 1u) ^ 1u, failed, status, 911)) { ok = false; break; }
                 const int t0 = p.col_term[col][0];
+                const int x0 = blk * 64 + p.tap_xc[t0], x1 = w0 + p.tap_dw[t0];
+                if (!mbar_wait(p_empty(sp), p_phase, failed, status, 911)) { ok = false; break; }
                 mbar_expect_tx(p_full(sp), p.patch_bytes);
-                tma_load_4d(patches + (uint32_t)sp * kTpPatchSlot, &map_x, p_full(sp), blk * 64 + p.tap_xc[t0], w0 + p.tap_dw[t0], h0 - 1, n0);
+                tma_load_4d(patches + (uint32_t)sp * kTpPatchSlot, &map_x, p_full(sp), x0, x1, h0 - 1, n0);
                 for (int dy = 0; dy < 3; ++dy, ++ga) {
-                    const int sa = ga % kTpBoxes;
-                    if (!mbar_wait(a_empty(sa), ((uint32_t)(ga / kTpBoxes) & 1u) ^ 1u, failed, status, 912)) { ok = false; break; }
                     const int tap = p.col_term[col][dy];
-                    const uint32_t a_dst = base + (uint32_t)sa * a_bytes;
+                    if (!mbar_wait(a_empty(sa), a_phase, failed, status, 912)) { ok = false; break; }
                     mbar_expect_tx(a_full(sa), a_bytes);
-                    load_filter_boxes<A_MN>(p, &map_w, a_dst, a_full(sa), tap, blk, co_tile);
+                    load_filter_boxes<A_MN>(p, &map_w, base + (uint32_t)sa * a_bytes, a_full(sa), tap, blk, co_tile);
+                    if (++sa == kTpBoxes) { sa = 0; a_phase ^= 1u; }
                 }
                 if (!ok) { ++gp; break; }       // this column's patch is in flight: count it for the drain below
+                if (++sp == kTpPatches) { sp = 0; p_phase ^= 1u; }
+                if (++blk == blocks) { blk = 0; ++col; }
             }
         }
         if (*failed) {
@@ -809,30 +955,33 @@ tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer
         const uint32_t idesc = instr_desc(128, p.tile_cols, A_MN ? 1 : 0, 0);
-        constexpr uint32_t a_step = A_MN ? 2048u : 32u, a_lbo = A_MN ? 8192u : 0u;
+        constexpr uint32_t a_step = (A_MN ? 2048u : 32u) / 16, a_lbo = A_MN ? 8192u : 0u;
+        const uint32_t hi = desc_hi(1024u);
         bool ok = true;
-        int ga = 0, gp = 0;
+        int sa = 0, sp = 0;
+        uint32_t a_phase = 0u, p_phase = 0u;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int buf = j & 1;
             if (!mbar_wait(acc_empty0 + 8 * buf, ((uint32_t)(j >> 1) & 1u) ^ 1u, failed, status, 914)) { ok = false; break; }
             const uint32_t acc = tmem_base + (uint32_t)(buf * 256);
-            for (int c = 0; c < cols && ok; ++c, ++gp) {
-                const int sp = gp % kTpPatches;
-                if (!mbar_wait(p_full(sp), (uint32_t)(gp / kTpPatches) & 1u, failed, status, 915)) { ok = false; break; }
-                const uint32_t patch = patches + (uint32_t)sp * kTpPatchSlot;
-                for (int dy = 0; dy < 3; ++dy, ++ga) {
-                    const int sa = ga % kTpBoxes;
-                    if (!mbar_wait(a_full(sa), (uint32_t)(ga / kTpBoxes) & 1u, failed, status, 916)) { ok = false; break; }
+            uint32_t more = 0u;
+            for (int c = 0; c < cols && ok; ++c) {
+                if (!mbar_wait(p_full(sp), p_phase, failed, status, 915)) { ok = false; break; }
+                uint32_t b_lo = desc_lo(patches + (uint32_t)sp * kTpPatchSlot, 0u);
+                for (int dy = 0; dy < 3; ++dy) {
+                    if (!mbar_wait(a_full(sa), a_phase, failed, status, 916)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t a_addr = base + (uint32_t)sa * a_bytes;
-                    const uint32_t b_addr = patch + (uint32_t)dy * 1024u;
+                    const uint32_t a_lo = desc_lo(base + (uint32_t)sa * a_bytes, a_lbo);
+                    umma_bf16(acc, a_lo, hi, b_lo, hi, idesc, more);
+                    more = 1u;
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma_bf16(acc, smem_desc(a_addr + kk * a_step, a_lbo, 1024), smem_desc(b_addr + kk * 32, 0, 1024), idesc,
-                                  (c > 0 || dy > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 1; kk < 4; ++kk) umma_bf16(acc, a_lo + kk * a_step, hi, b_lo + kk * 2u, hi, idesc, 1u);
                     umma_commit(a_empty(sa));
+                    b_lo += 1024u / 16;
+                    if (++sa == kTpBoxes) { sa = 0; a_phase ^= 1u; }
                 }
                 if (ok) umma_commit(p_empty(sp));
+                if (++sp == kTpPatches) { sp = 0; p_phase ^= 1u; }
             }
             if (ok) umma_commit(acc_full0 + 8 * buf);
         }
@@ -1253,6 +1402,7 @@ struct WgradParams {
     int tiles_w, tiles_h, tiles_n;
     int nb;                      // column blocks per CTA (1..4)
     int total_blocks;            // k*k * 64-channel blocks of c_in (a ragged last block is zero-filled)
+    int tile_store;              // the target takes tile stores (16-byte aligned)
     int tiles_per_slice;         // pixel tiles per CTA along the reduction
     int total_tiles;
     int stages;
@@ -1260,7 +1410,7 @@ struct WgradParams {
 
 __global__ void __launch_bounds__(kThreads, 1)
 tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
-                     float* __restrict__ partial, WgradParams p, int* status) {
+                     const __grid_constant__ CUtensorMap map_out, float* __restrict__ partial, WgradParams p, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     // One copy brings px pixels x 64 channels (px = 64, 128 or 256: as many as leave two stages in shared memory, so
@@ -1273,7 +1423,6 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     const uint32_t bars = base + (uint32_t)p.stages * stage_bytes;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int failed_flag;
-    __shared__ float turn[4][32][33];                             // per epilogue warp: a 32 x 32 block on its way out
     volatile int* failed = &failed_flag;
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -1346,46 +1495,62 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             if (!mbar_wait(full_bar(s), phase, failed, status, 202)) { ok = false; break; }
             tc_fence_after();
             const uint32_t a_addr = base + (uint32_t)s * stage_bytes;
-            const uint32_t b_addr = a_addr + 2 * box_bytes;
+            const uint32_t a_lo = desc_lo(a_addr, box_bytes), b_lo = desc_lo(a_addr + 2 * box_bytes, box_bytes), hi = desc_hi(1024u);
             const int k_steps = p.px / 16;
 #pragma unroll 4
             for (int kk = 0; kk < k_steps; ++kk) {  // K = 16 pixels = 2 groups of 8 rows = 2048 bytes per step
-                umma_bf16(tmem_base, smem_desc(a_addr + kk * 2048, box_bytes, 1024), smem_desc(b_addr + kk * 2048, box_bytes, 1024),
-                          idesc, (it > 0 || kk > 0) ? 1u : 0u);
+                umma_bf16(tmem_base, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, (it > 0 || kk > 0) ? 1u : 0u);
             }
             umma_commit(empty_bar(s));
         }
         if (ok) umma_commit(accum_bar);
     } else if (warp >= 2) {
-        // Thread l of a warp holds row l of each 32 x 32 block; the block is turned through shared memory so
-        // that every store instruction writes 32 consecutive floats of one row (a full line) instead of 16-byte
-        // pieces of 32 rows: the fully connected gradients are hundreds of megabytes of such rows.
+        // Thread l of a warp holds row l of each 32 x 32 block; the block goes to shared memory (swizzled rows of 128
+        // bytes, over operand stages that the tensor core has read) and leaves as one tile store, clipped at the last
+        // input channel of the tap and the last output channel.  (Turned blocks stored by the lanes, 128 bytes per
+        // instruction, kept the last 10 us of short reductions: 256 -> 1024 at 13 x 11, 21 images 22.6 -> 15.3 us with the slice sum.)
         const int quarter = warp % 4;
         const int co_first = co_tile * 128 + quarter * 32;
         const int co = co_first + lane;
         const bool valid = co < p.c_out;
         const size_t row_elems = (size_t)p.k * p.k * p.c_in;
         float* dst_row = partial + ((size_t)slice * p.c_out + (valid ? co : 0)) * row_elems;
-        float* dst_first = partial + ((size_t)slice * p.c_out + co_first) * row_elems;
         if (iters > 0 && mbar_wait(accum_bar, 0, failed, status, 203)) {
             tc_fence_after();
+            const int slabs = min(8, (int)((uint32_t)p.stages * stage_bytes / (4u * 4096u)));
+            int count = 0;
             for (int j = 0; j < nb_here; ++j) {
                 const int tap = (blk_begin + j) / cin_blocks, ch0 = (blk_begin + j) % cin_blocks * 64;
-                for (int c0 = 0; c0 < 64; c0 += 32) {
+                for (int c0 = 0; c0 < 64; c0 += 32, ++count) {
                     if (ch0 + c0 >= p.c_in) break;
                     uint32_t v[32];
                     tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(j * 64 + c0), v);
-                    __syncwarp();
+                    if (!p.tile_store) {
+                        if (valid) {
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) turn[quarter][lane][e] = __uint_as_float(v[e]);
+                            for (int e = 0; e < 32; ++e)
+                                if (ch0 + c0 + e < p.c_in) dst_row[(size_t)tap * p.c_in + ch0 + c0 + e] = __uint_as_float(v[e]);
+                        }
+                        continue;
+                    }
+                    const uint32_t slab = base + (uint32_t)(quarter * slabs + count % slabs) * 4096u;
+                    if (count >= slabs) {
+                        if (lane == 0) tma_store_wait_read<0>();
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                                     ::"r"(slab + (uint32_t)(lane * 128 + ((e ^ (lane & 7)) * 16))), "r"(v[4 * e]), "r"(v[4 * e + 1]), "r"(v[4 * e + 2]), "r"(v[4 * e + 3]) : "memory");
+                    fence_proxy_async();
                     __syncwarp();
-                    float* dst = dst_first + (size_t)tap * p.c_in + ch0 + c0 + lane;       // column (tap, c_in)
-                    const int rows = ch0 + c0 + lane < p.c_in ? p.c_out - co_first : 0;
-#pragma unroll 8
-                    for (int r = 0; r < 32; ++r)
-                        if (r < rows) dst[(size_t)r * row_elems] = turn[quarter][r][lane];
+                    if (lane == 0 && co_first < p.c_out) {
+                        tma_store_4d(&map_out, slab, ch0 + c0, tap, co_first, slice);
+                        tma_store_commit();
+                    }
                 }
             }
+            if (lane == 0) tma_store_wait_all();
         } else if (iters == 0 && valid) {
             for (int j = 0; j < nb_here; ++j) {
                 const int tap = (blk_begin + j) / cin_blocks, ch0 = (blk_begin + j) % cin_blocks * 64;
@@ -1627,9 +1792,10 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
 #pragma unroll 1
             for (int c = 0; c < ncols; ++c) {
                 const uint32_t x_addr = dz_addr + 2 * p.dz_box + (uint32_t)c * p.patch_bytes;
+                const uint32_t a_lo = desc_lo(dz_addr, p.dz_box), b_lo = desc_lo(x_addr, 1024u), hi = desc_hi(1024u);
+#pragma unroll 2
                 for (int kk = 0; kk < ksteps; ++kk)
-                    umma_bf16(tmem_base + (uint32_t)c * 192, smem_desc(dz_addr + kk * 2048, p.dz_box, 1024),
-                              smem_desc(x_addr + kk * 2048, 1024, 1024), idesc, (j > 0 || kk > 0) ? 1u : 0u);
+                    umma_bf16(tmem_base + (uint32_t)c * 192, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, (j > 0 || kk > 0) ? 1u : 0u);
             }
             umma_commit(empty_bar(s));
         }
@@ -2649,17 +2815,33 @@ int make_act_map(CUtensorMap* map, const void* ptr, int N, int H, int W, int C, 
 }
 
 // Row-major [rows][cols] bf16 matrix as (cols, rows); box = 64 columns x box_rows.
-int make_mat_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int box_rows) {
+// rank 4: the same with two dimensions of one element behind (for copies that share an instruction with 4-D ones).
+int make_mat_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int box_rows, int rank = 2) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return CKPT_E_CUDA; }
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
-    cuuint32_t es[2] = {1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, es,
+    cuuint64_t dims[4] = {(cuuint64_t)cols, (cuuint64_t)rows, 1, 1};
+    cuuint64_t strides[3] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * rows * 2, (cuuint64_t)cols * rows * 2};
+    cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, 1};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(ptr), dims, strides, box, es,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled failed for a weight matrix (code %d)", (int)r); return CKPT_E_CUDA; }
+    return CKPT_OK;
+}
+
+// Weight gradients, float32 [slices][c_out][taps][c_in]; box = 32 input channels x 32 output channels of one tap, 128-byte
+// swizzle, for stores.
+int make_partial_map(CUtensorMap* map, float* ptr, int c_in, int taps, int c_out, int slices) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return CKPT_E_CUDA; }
+    cuuint64_t dims[4] = {(cuuint64_t)c_in, (cuuint64_t)taps, (cuuint64_t)c_out, (cuuint64_t)slices};
+    cuuint64_t strides[3] = {(cuuint64_t)c_in * 4, (cuuint64_t)c_in * taps * 4, (cuuint64_t)c_in * taps * c_out * 4};
+    cuuint32_t box[4] = {32, 1, 32, 1};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, ptr, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled failed for a weight gradient (code %d)", (int)r); return CKPT_E_CUDA; }
     return CKPT_OK;
 }
 
@@ -2861,10 +3043,42 @@ bool tp_stack(int H, int W, int N, int co_tiles, int* th_out, int* stack_out) {
     return true;
 }
 
+// Pixel tile and reduction split of the plain role-swapped kernel, by a model of clocks fitted to a sweep of both over
+// 26 shapes: a stage (64 reduction channels of one term) takes its four MMAs - 430 however few pixels, 2 per pixel above
+// 215 - or its bytes from the L2; the epilogue of a tile takes about 16 per pixel and runs under the next tile's stages; a
+// cluster that shares a reduction costs its launch and exchange.  us, one 256-pixel tile per CTA -> chosen: 512 -> 512 at
+// 2 x 2, 128 images 25.5 -> 11.8 (64 pixels, 4 CTAs each), 512 -> 512 at 20 x 12, 13 images 26.2 -> 20.2 (256, 2),
+// 256 -> 256 at 13 x 11, 21 images 16.0 -> 12.6 (128, 2), 1x1 1024 -> 256 at 14 x 14, 128 images 17.1 -> 15.1 (192, 1).
+// 1x1 filters see the pixels as one row (tiles of any multiple of 32, no ragged edges but the last).
+void t_plan(TParams* p, int* W, int* H, int* N) {
+    const bool flat = p->taps == 1 && !p->fold;
+    if (flat) { p->W = *W = *W * *H * *N; p->H = *H = 1; p->N = *N = 1; }
+    int sms = 148, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int co = (p->c_out + 127) / 128, terms = p->taps * ((p->c_red + 63) / 64);
+    double best = 1e30;
+    for (int cols = 256; cols >= 64; cols -= 32) {
+        if (!flat && (cols & (cols - 1))) continue;
+        if (p->fold && cols != 256) continue;
+        int tw = cols, th = 1, tn = 1;
+        if (!flat) choose_tile(cols, *W, *H, *N, &tw, &th, &tn);
+        const int64_t tiles = (int64_t)((*W + tw - 1) / tw) * ((*H + th - 1) / th) * ((*N + tn - 1) / tn);
+        for (int split = 1; split <= 8; split *= 2) {
+            if (split > 1 && (p->fold || terms < 2 * split || (int64_t)tiles * co * split > sms - 4 * split)) break;
+            const double active = std::min<double>(sms, (double)tiles * co * split);
+            const double bytes = 16384.0 + 128.0 * cols, stage = std::max(std::max(2.0 * cols, 430.0), bytes / std::min(100.0, 9000.0 / active));
+            const double loop = std::ceil((double)terms / split) * stage, out = 16.0 * cols;
+            const int64_t per_co = std::max<int64_t>(1, std::min<int64_t>(tiles, sms / co)), rounds = (tiles + per_co - 1) / per_co;
+            const double t = split == 1 ? rounds * std::max(loop, out) + std::min(loop, out) : loop + out + 2000.0 + 10.0 * cols + 300.0 * split;
+            if (t < best) { best = t; p->tile_cols = cols; p->split = split; p->tw = tw; p->th = th; p->tn = tn; }
+        }
+    }
+}
+
 int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& mw, void* out, float* stat_partial, int* stat_blocks,
                   int N, int H, int W, int c_red, int c_out, int* status, cudaStream_t st, const char* what, bool a_mn) {
     p.H = H; p.W = W; p.N = N; p.c_red = c_red; p.c_out = c_out;
-    choose_tile(256, W, H, N, &p.tw, &p.th, &p.tn);
     bool patch = false;
     int strip_h = 0, stack = 0;
     p.stack = 0;
@@ -2880,6 +3094,8 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
         p.tile_cols = 8 * strip_h * stack;
         p.patch_bytes = (uint32_t)(8 * strip_h * stack) * 128;
     }
+    p.split = 1;
+    if (!patch) t_plan(&p, &W, &H, &N);
     p.tw_log = 0; while ((1 << p.tw_log) < p.tw) ++p.tw_log;
     p.th_log = 0; while ((1 << p.th_log) < p.th) ++p.th_log;
     p.tiles_w = (W + p.tw - 1) / p.tw; p.tiles_h = (H + p.th - 1) / p.th; p.tiles_n = (N + p.tn - 1) / p.tn;
@@ -2890,7 +3106,8 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     p.ctas_per_co = std::max(1, std::min(p.p_tiles, sms / p.co_tiles));
-    constexpr uint32_t stage_bytes = 128 * 128 + 256 * 128;
+    if (p.split > 1) p.ctas_per_co = p.p_tiles;
+    const uint32_t stage_bytes = 128 * 128 + (uint32_t)p.tile_cols * 128;
     constexpr uint32_t t_slabs = 4 * kTEpi * kTSlabs * 2048;
     p.stages = std::min<int>(kMaxStages, (227 * 1024 - 1024 - 256 - t_slabs - 64) / stage_bytes);
     CUtensorMap mx;
@@ -2913,14 +3130,15 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 256 + t_slabs;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_conv_t_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 64);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_conv_t_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 64);
+        cudaError_t e = cudaSuccess;
+        for (auto kernel : {tc_conv_t_kernel<false, false>, tc_conv_t_kernel<true, false>, tc_conv_t_kernel<false, true>, tc_conv_t_kernel<true, true>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 64);
         if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
         attr_set = true;
     }
     // partial row pairs per CTA: one per epilogue warp of a channel's quarter (the plain kernel has two), twice that
-    // in the pixel-pair form
-    if (stat_blocks) *stat_blocks = stat_partial ? (p.fold ? 2 : 1) * (patch ? kTpEpi : kTEpi) * p.ctas_per_co : 0;
+    // in the pixel-pair form; one per chunk of 32 pixels where a cluster shares a tile
+    if (stat_blocks) *stat_blocks = !stat_partial ? 0 : p.split > 1 ? p.p_tiles * (p.tile_cols / 32) : (p.fold ? 2 : 1) * (patch ? kTpEpi : kTEpi) * p.ctas_per_co;
     if (patch) {
         static bool tp_attr_set = false;
         if (!tp_attr_set) {
@@ -2934,8 +3152,23 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
         CKPT_LAUNCH_CHECK_NAMED("tc_conv_tp_kernel", what);
         return CKPT_OK;
     }
-    if (a_mn) tc_conv_t_kernel<true><<<p.ctas_per_co * p.co_tiles, kThreadsT, smem, st>>>(mx, mw, mo, stat_blocks ? stat_partial : nullptr, p, status);
-    else tc_conv_t_kernel<false><<<p.ctas_per_co * p.co_tiles, kThreadsT, smem, st>>>(mx, mw, mo, stat_blocks ? stat_partial : nullptr, p, status);
+    float* const stats = stat_blocks ? stat_partial : nullptr;
+    const unsigned grid = (unsigned)(p.ctas_per_co * p.co_tiles * p.split);
+    if (p.split > 1) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreadsT); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)p.split; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr; cfg.numAttrs = 1;
+        const cudaError_t e = a_mn ? cudaLaunchKernelEx(&cfg, tc_conv_t_kernel<true, true>, mx, mw, mo, stats, p, status)
+                                   : cudaLaunchKernelEx(&cfg, tc_conv_t_kernel<false, true>, mx, mw, mo, stats, p, status);
+        if (e != cudaSuccess) return cuda_fail(e, what);
+    } else if (a_mn) {
+        tc_conv_t_kernel<true, false><<<grid, kThreadsT, smem, st>>>(mx, mw, mo, stats, p, status);
+    } else {
+        tc_conv_t_kernel<false, false><<<grid, kThreadsT, smem, st>>>(mx, mw, mo, stats, p, status);
+    }
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_t_kernel", what);
     return CKPT_OK;
 }
@@ -2954,7 +3187,7 @@ int launch_t(const void* x, const void* w_mat, void* out, float* stat_partial, i
         p.tap_dh[t] = t / k - pad; p.tap_dw[t] = t % k - pad; p.tap_col[t] = a_mn ? k * k - 1 - t : t; p.tap_xc[t] = 0;
     }
     CUtensorMap mw;
-    int rc = a_mn ? make_mat_map(&mw, w_mat, c_red, (int64_t)k * k * c_out, 64) : make_mat_map(&mw, w_mat, c_out, (int64_t)k * k * c_red, 128);
+    int rc = a_mn ? make_mat_map(&mw, w_mat, c_red, (int64_t)k * k * c_out, 64, 4) : make_mat_map(&mw, w_mat, c_out, (int64_t)k * k * c_red, 128, 4);
     if (rc) return rc;
     return launch_t_core(p, x, c_red, mw, out, stat_partial, stat_blocks, N, H, W, c_red, c_out, status, st, what, a_mn);
 }
@@ -2997,7 +3230,7 @@ int launch_t_paired(const void* x, const void* w, int flip, void* out, float* st
         p.tap_col2[t] = position(sp - 1);
     }
     CUtensorMap mw;
-    int rc = flip ? make_mat_map(&mw, w, c_red, 9 * 64, 64) : make_mat_map(&mw, w, 64, (int64_t)9 * c_red, 64);
+    int rc = flip ? make_mat_map(&mw, w, c_red, 9 * 64, 64, 4) : make_mat_map(&mw, w, 64, (int64_t)9 * c_red, 64, 4);
     if (rc) return rc;
     return launch_t_core(p, x, 2 * c_red, mw, out, stat_partial, stat_blocks, N, H, W / 2, c_red, 128, status, st, what, flip != 0);
 }
@@ -3617,8 +3850,12 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
     }
     const size_t smem = (size_t)p.stages * (2 + p.nb) * p.px * 128 + 1024 + 256;
     float* target = slices > 1 ? (float*)scratch : dw;
+    CUtensorMap mo;
+    memset(&mo, 0, sizeof(mo));
+    p.tile_store = (uintptr_t)target % 16 == 0 && g.cin % 4 == 0;
+    if (p.tile_store && (rc = make_partial_map(&mo, target, g.cin, g.k * g.k, g.cout, slices))) return rc;
     dim3 grid(slices, groups, co_tiles);
-    tc_conv_wgrad_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, target, p, device_status);
+    tc_conv_wgrad_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, target, p, device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_wgrad_kernel", "conv wgrad (tensor cores)");
     if (slices > 1) {
         launch_slice_sum((const float*)scratch, dw, elems, slices, st, upd);

@@ -499,3 +499,32 @@ def test_bn_backward_in_one_kernel(rows, c, relu, dtype):
     terms = s[2].abs() * (g.abs() + (absg + s[1] ** 2 * (absgz + s[0].abs() * absg) * (s[0].abs() + z.double().abs())) / rows)
     off = (dz - want).abs() > 2.0 ** -20 * terms + (2.0 ** -8 * want.abs() if dtype == ck.DTYPE_BF16 else 0.0)
     assert not (off & sure).any()
+
+
+@pytest.mark.parametrize("case", [
+    (3, 2, 2, 512, 512, 3, 1),       # reduction shared by a cluster, smallest pixel tile
+    (13, 10, 6, 512, 200, 3, 1),     # the same with partial pixel and channel tiles
+    (5, 13, 11, 1024, 136, 1, 0),    # 1x1 on one row of pixels, shared reduction, partial last tile
+    (64, 14, 14, 512, 256, 1, 0),    # 1x1, pixel tiles that are no power of two
+    (40, 15, 13, 128, 128, 3, 1),    # one CTA per tile, 128 pixels
+])
+def test_conv_tile_and_split_choices(case):
+    test_conv_tensor_core_kernels(case)
+
+
+@pytest.mark.parametrize("case,expect_fused", [((13, 10, 6, 512, 200, 3, 1), True), ((5, 13, 11, 1024, 136, 1, 0), True)])
+def test_conv_bn_statistics_shared_reduction(case, expect_fused):
+    test_conv_bn_statistics(case, expect_fused)
+
+
+def test_conv_wgrad_into_unaligned_gradient():
+    """A gradient buffer the tile stores cannot take gets the same values by plain stores."""
+    import torch
+    shape, dtype = ck.ConvShape(2, 6, 6, 64, 64, 1, 1, 0), ck.DTYPE_BF16
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    x, dz = (torch.randn((2, 6, 6, 64), generator=gen, device="cuda").bfloat16() for _ in range(2))
+    scratch = torch.empty(max(ck.conv2d_scratch_bytes(shape, dtype), 256), dtype=torch.uint8, device="cuda")
+    a, b = torch.empty(64 * 64, device="cuda"), torch.empty(64 * 64 + 1, device="cuda")[1:]
+    ck.conv2d_wgrad(shape, dtype, 0, dz, x, a, scratch)
+    ck.conv2d_wgrad(shape, dtype, 0, dz, x, b, scratch)
+    assert torch.equal(a, b)
