@@ -745,26 +745,27 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             int w0, h0, n0;
             tile_origin(j, w0, h0, n0);
 #pragma unroll 1
-            for (int c0 = half * 32; c0 < p.tile_cols; c0 += 32 * kTEpi, ++chunk_count) {
+            for (int c0 = half * 32; c0 < p.tile_cols; c0 += 32 * kTEpi) {
                 // lane e works out whether pixel c0 + e of the tile lies inside the tensor (for the sums)
                 const int idx = c0 + lane;
                 const int wl = idx & ((1 << p.tw_log) - 1), hl = (idx >> p.tw_log) & (p.th - 1), nl = idx >> (p.tw_log + p.th_log);
                 const bool inside = (w0 + wl < p.W) && (h0 + hl < p.H) && (n0 + nl < p.N);
                 const uint32_t in_mask = __ballot_sync(0xffffffffu, inside);
+                if (in_mask == 0u || co_tile * 128 + quarter * 32 >= p.c_out) continue;       // nothing of it inside the tensor
                 uint32_t v[32];
                 tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + c0), v);
-                const uint32_t slab = out_stage + (uint32_t)(((warp - 2) * kTSlabs + (chunk_count % kTSlabs)) * 2048);
+                const uint32_t slab = out_stage + (uint32_t)(((warp - 2) * kTSlabs + (chunk_count++ % kTSlabs)) * 2048);
                 if (lane == 0) tma_store_wait_read<kTSlabs - 1>();    // the store that last read this slab has left it
                 __syncwarp();
                 t_chunk_to_slab<true>(v, in_mask, slab + (uint32_t)(lane * 2), stats, sum, sumsq);
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0 && in_mask != 0u && co_tile * 128 + quarter * 32 < p.c_out) {
+                // (one branch for store and commit: a commit in a branch of its own made 64 -> 256 at 56 x 56 15 % slower)
+                if (lane == 0) {
                     const int cw = c0 & ((1 << p.tw_log) - 1), chh = (c0 >> p.tw_log) & (p.th - 1), cn = c0 >> (p.tw_log + p.th_log);
                     tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
+                    tma_store_commit();
                 }
-                // also for a chunk outside the tensor (an empty group): the wait above counts groups, one per chunk
-                if (lane == 0) tma_store_commit();
             }
             tc_fence_before();
             mbar_arrive(acc_empty0 + 8 * buf);
@@ -3045,7 +3046,7 @@ bool tp_stack(int H, int W, int N, int co_tiles, int* th_out, int* stack_out) {
 
 // Pixel tile and reduction split of the plain role-swapped kernel, by a model of clocks fitted to a sweep of both over
 // 26 shapes: a stage (64 reduction channels of one term) takes its four MMAs - 430 however few pixels, 2 per pixel above
-// 215 - or its bytes from the L2; the epilogue of a tile takes about 16 per pixel and runs under the next tile's stages; a
+// 215 - or its bytes from the L2; the epilogue of a tile takes about 1100 and 15 per pixel and runs under the next tile's stages; a
 // cluster that shares a reduction costs its launch and exchange.  us, one 256-pixel tile per CTA -> chosen: 512 -> 512 at
 // 2 x 2, 128 images 25.5 -> 11.8 (64 pixels, 4 CTAs each), 512 -> 512 at 20 x 12, 13 images 26.2 -> 20.2 (256, 2),
 // 256 -> 256 at 13 x 11, 21 images 16.0 -> 12.6 (128, 2), 1x1 1024 -> 256 at 14 x 14, 128 images 17.1 -> 15.1 (192, 1).
@@ -3068,7 +3069,7 @@ void t_plan(TParams* p, int* W, int* H, int* N) {
             if (split > 1 && (p->fold || terms < 2 * split || (int64_t)tiles * co * split > sms - 4 * split)) break;
             const double active = std::min<double>(sms, (double)tiles * co * split);
             const double bytes = 16384.0 + 128.0 * cols, stage = std::max(std::max(2.0 * cols, 430.0), bytes / std::min(100.0, 9000.0 / active));
-            const double loop = std::ceil((double)terms / split) * stage, out = 16.0 * cols;
+            const double loop = std::ceil((double)terms / split) * stage, out = 1100.0 + 15.0 * cols;
             const int64_t per_co = std::max<int64_t>(1, std::min<int64_t>(tiles, sms / co)), rounds = (tiles + per_co - 1) / per_co;
             const double t = split == 1 ? rounds * std::max(loop, out) + std::min(loop, out) : loop + out + 2000.0 + 10.0 * cols + 300.0 * split;
             if (t < best) { best = t; p->tile_cols = cols; p->split = split; p->tw = tw; p->th = th; p->tn = tn; }
