@@ -1391,6 +1391,16 @@ tc_conv_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     }
 }
 
+// A 32 x 32 float block, row `lane` in this thread, to a slab in the layout of a 128-byte swizzled tile store.
+__device__ __forceinline__ void block_to_slab(const uint32_t (&v)[32], uint32_t slab, int lane) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                     ::"r"(slab + (uint32_t)(lane * 128 + ((e ^ (lane & 7)) * 16))), "r"(v[4 * e]), "r"(v[4 * e + 1]), "r"(v[4 * e + 2]), "r"(v[4 * e + 3]) : "memory");
+    fence_proxy_async();
+    __syncwarp();
+}
+
 // ------------------------------------------------------------------------------------------------
 // wgrad kernel: D[c_out tile of 128][up to 4 blocks of 64 (tap, c_in) columns], K = pixels
 // ------------------------------------------------------------------------------------------------
@@ -1539,12 +1549,7 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
                         if (lane == 0) tma_store_wait_read<0>();
                         __syncwarp();
                     }
-#pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
-                                     ::"r"(slab + (uint32_t)(lane * 128 + ((e ^ (lane & 7)) * 16))), "r"(v[4 * e]), "r"(v[4 * e + 1]), "r"(v[4 * e + 2]), "r"(v[4 * e + 3]) : "memory");
-                    fence_proxy_async();
-                    __syncwarp();
+                    block_to_slab(v, slab, lane);
                     if (lane == 0 && co_first < p.c_out) {
                         tma_store_4d(&map_out, slab, ch0 + c0, tap, co_first, slice);
                         tma_store_commit();
@@ -1726,7 +1731,7 @@ struct WRowsParams {
 
 __global__ void __launch_bounds__(kThreads, 1)
 tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
-                     float* __restrict__ partial, WRowsParams p, int* status) {
+                     const __grid_constant__ CUtensorMap map_out, float* __restrict__ partial, WRowsParams p, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t bars = base + (uint32_t)p.stages * p.stage_bytes;
@@ -1802,36 +1807,40 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         }
         if (ok) umma_commit(accum_bar);
     } else if (warp >= 2) {
-        // Thread l of a warp holds row l (an output channel) of the accumulator and writes its 64 floats of a (column,
-        // dy) block as 16-byte pieces.  (Turning 32 x 32 blocks through shared memory for full-line stores, as the
-        // generic wgrad kernel does for its much wider rows, measured 10-25 % slower here.)
+        // Blocks of 32 output channels x 32 input channels of a tap leave as tile stores through the operand stages, as in
+        // tc_conv_wgrad_kernel (rows stored by the lanes in 16-byte pieces: 21.9 us with the fold at 64 -> 64, 56 x 56, 32
+        // images, against 17.5; 128 -> 128 at 16 x 16, 128 images 26.9 against 17.6).
         const int quarter = warp % 4;
-        const int co = co_tile * 128 + quarter * 32 + lane;
+        const int co_first = co_tile * 128 + quarter * 32, co = co_first + lane;
         const bool valid = co < p.c_out;
         const size_t row_elems = (size_t)p.row_elems;
         float* dst_row = partial + ((size_t)slice * p.c_out + (valid ? co : 0)) * row_elems;
         if (my_tiles > 0 && mbar_wait(accum_bar, 0, failed, status, 703)) {
             tc_fence_after();
+            const int slabs = min(12, (int)((uint32_t)p.stages * p.stage_bytes / (4u * 4096u)));
+            int count = 0;
             for (int c = 0; c < ncols; ++c) {
                 const int col = p.cols * pair + c, cib = col / 3, dx = col % 3;
                 for (int dy = 0; dy < 3; ++dy) {
-                    float* dst = dst_row + (p.pairview ? (size_t)(col * 3 + dy) * 64
-                                                       : (size_t)(dy * 3 + dx) * p.c_in + cib * 64);   // column (tap, c_in)
-                    const int here = p.pairview ? 64 : min(64, p.c_in - cib * 64);      // a multiple of 8
-#pragma unroll
-                    for (int c0 = 0; c0 < 64; c0 += 32) {
+                    const int tap = p.pairview ? col * 3 + dy : dy * 3 + dx, ch0 = p.pairview ? 0 : cib * 64;
+                    const int here = p.pairview ? 64 : p.c_in - ch0;
+                    for (int c0 = 0; c0 < 64 && c0 < here; c0 += 32, ++count) {
                         uint32_t v[32];
                         tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * 192 + dy * 64 + c0), v);
-                        if (valid) {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                if (c0 + 4 * e < here)
-                                *reinterpret_cast<float4*>(dst + c0 + 4 * e) =
-                                    make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]), __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]));
+                        const uint32_t slab = base + (uint32_t)(quarter * slabs + count % slabs) * 4096u;
+                        if (count >= slabs) {
+                            if (lane == 0) tma_store_wait_read<0>();
+                            __syncwarp();
+                        }
+                        block_to_slab(v, slab, lane);
+                        if (lane == 0 && co_first < p.c_out) {
+                            tma_store_4d(&map_out, slab, ch0 + c0, tap, co_first, slice);
+                            tma_store_commit();
                         }
                     }
                 }
             }
+            if (lane == 0) tma_store_wait_all();
         } else if (my_tiles == 0 && valid) {
             for (int c = 0; c < ncols; ++c) {
                 const int col = p.cols * pair + c, cib = col / 3, dx = col % 3;
@@ -3779,7 +3788,9 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         if (rc) return rc;
         const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
         dim3 grid(p.slices, 4 / p.cols, co_tiles);
-        tc_wgrad_rows_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, (float*)scratch, p, device_status);
+        CUtensorMap mo;
+        if ((rc = make_partial_map(&mo, (float*)scratch, 64, 12, 2 * g.cout, p.slices))) return rc;
+        tc_wgrad_rows_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_rows_kernel (pixel pairs)", "conv wgrad, 64 input channels as pixel pairs (tensor cores)");
         pairview_fold_kernel<8><<<(unsigned)((g.cout * 144 + 31) / 32), dim3(32, 8), 0, st>>>((const float*)scratch, dw, g.cout, p.slices, upd);
         CKPT_LAUNCH_CHECK_NAMED("pairview_fold_kernel", "wgrad pair fold");
@@ -3826,7 +3837,9 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         if (rc) return rc;
         const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
         dim3 grid(p.slices, pairs, co_tiles);
-        tc_wgrad_rows_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, (float*)scratch, p, device_status);
+        CUtensorMap mo;
+        if ((rc = make_partial_map(&mo, (float*)scratch, g.cin, 9, g.cout, p.slices))) return rc;
+        tc_wgrad_rows_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_rows_kernel", "conv wgrad, shared vertical taps (tensor cores)");
         launch_slice_sum((const float*)scratch, dw, elems, p.slices, st, upd);
         CKPT_LAUNCH_CHECK_NAMED("slice_sum_kernel", "wgrad slice sum");
