@@ -110,6 +110,7 @@ struct StepCtx {
     int64_t recomputed = 0;
     int64_t* stage_trace = nullptr;     // optional: live arena bytes at the end of each of the 2n+2 stages
     void* host_result = nullptr;        // capture: pinned destination of the loss and the status word (no wait)
+    bool masked = false;                // the current gradient has been through the ReLU that ends the unit it enters (a residual block)
     char* act_buf = nullptr;            // where the activated copy of a unit's input goes (null: the workspace's own buffer)
     int64_t act_cap = 0;                // its capacity in bytes
     int* status() const { return (int*)(ws + ch->off_misc + 64); }
@@ -140,9 +141,9 @@ static int conv_forward_any(StepCtx& c, const ConvGeom& g, const void* x, const 
         return stem_conv_fwd(g, x, w, z, c.status(), c.stream);
     return simt_conv_fwd(c.ch->dtype, g, x, w, z, bias, relu, c.stream);
 }
-static int conv_dgrad_any(StepCtx& c, const ConvGeom& g, const void* dz, const void* w, void* dx) {
+static int conv_dgrad_any(StepCtx& c, const ConvGeom& g, const void* dz, const void* w, void* dx, const GradientJoin& join = GradientJoin()) {
     if (use_tc(c.ch, g, dz, w, dx))
-        return tc_conv_dgrad(g, dz, w, dx, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
+        return tc_conv_dgrad(g, dz, w, dx, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream, join);
     return simt_conv_dgrad(c.ch->dtype, g, dz, w, dx, c.stream);
 }
 static int conv_wgrad_any(StepCtx& c, const ConvGeom& g, const void* dz, const void* x, float* dw) {
@@ -167,10 +168,11 @@ static int sgd_step(StepCtx& c, int param) {
 }
 // Weight gradient and input gradient of one convolution.  Without an update: wgrad, then dgrad.  With one the filter
 // changes as soon as its gradient is summed, so the input gradient (which reads the filter) runs first.
-static int conv_backward_pair(StepCtx& c, const ConvGeom& g, const void* dz, const void* x, const void* w, int param, void* dx) {
+static int conv_backward_pair(StepCtx& c, const ConvGeom& g, const void* dz, const void* x, const void* w, int param, void* dx,
+                              const GradientJoin& join = GradientJoin()) {
     int rc;
     const bool sgd = c.ch->sgd_lr != 0.f;
-    if (sgd && dx && (rc = conv_dgrad_any(c, g, dz, w, dx))) return rc;
+    if (sgd && dx && (rc = conv_dgrad_any(c, g, dz, w, dx, join))) return rc;
     const bool stem = c.ch->impl == 0 && stem_conv_supported(c.ch->dtype, g);
     const bool tc_path = !(c.ch->impl == 0 && small_conv_supported(c.ch->dtype, g)) && !stem && use_tc(c.ch, g, dz, x, nullptr);
     if (sgd && stem) {
@@ -183,7 +185,7 @@ static int conv_backward_pair(StepCtx& c, const ConvGeom& g, const void* dz, con
         if ((rc = conv_wgrad_any(c, g, dz, x, (float*)c.grads[param]))) return rc;
         if ((rc = sgd_step(c, param))) return rc;
     }
-    if (!sgd && dx && (rc = conv_dgrad_any(c, g, dz, w, dx))) return rc;
+    if (!sgd && dx && (rc = conv_dgrad_any(c, g, dz, w, dx, join))) return rc;
     return CKPT_OK;
 }
 
@@ -311,8 +313,9 @@ static int block_forward(StepCtx& c, const Unit& u, const void* x, void* y, bool
                        project ? B.sp : nullptr, y, c.stream);
 }
 
-// g_in = dL/dy (overwritten), g_out = dL/dx or null.
-static int block_backward(StepCtx& c, const Unit& u, const void* x, const void* y, void* g_in, void* g_out) {
+// g_in = dL/dy (overwritten), g_out = dL/dx or null.  c.masked: g_in has been through the final ReLU already; on return it
+// says whether g_out has been through the ReLU that ends the block before (mask_out: there is one, its output is x).
+static int block_backward(StepCtx& c, const Unit& u, const void* x, const void* y, void* g_in, void* g_out, bool mask_out) {
     const int dt = c.ch->dtype;
     const BlockBuffers B = block_buffers(c, u);
     void* const* p = c.params + u.param_first;
@@ -326,7 +329,8 @@ static int block_backward(StepCtx& c, const Unit& u, const void* x, const void* 
     // the interiors are re-derived from x, unless every block kept its own since the forward pass (store-all, literally)
     if (!keeps_interiors(c.ch, c.policy) && (rc = block_interiors(c, u, x, B, true))) return rc;
     // through the final ReLU: g_in <- dL/d(bn3 + shortcut), by the first batch-norm backward that reads it
-    const void* mask = y;
+    const void* mask = c.masked ? nullptr : y;
+    c.masked = false;
     const void* dx_shortcut = g_in;                       // identity shortcut: the same gradient flows to x
     if (project) {
         if ((rc = bn_relu_backward(dt, out_px, co, g_in, B.zp, B.sp, 0, B.t0, (float*)g[10], (float*)g[11], scr, c.stream, bn_extra(c, pf + 10, mask)))) return rc;
@@ -339,6 +343,12 @@ static int block_backward(StepCtx& c, const Unit& u, const void* x, const void* 
     if ((rc = bn_relu_backward(dt, out_px, mid, B.db, B.z2, B.s2, 1, B.db, (float*)g[4], (float*)g[5], scr, c.stream, bn_extra(c, pf + 4)))) return rc;
     if ((rc = conv_backward_pair(c, u.g2, B.db, B.a, p[3], pf + 3, B.da))) return rc;
     if ((rc = bn_relu_backward(dt, in_px, mid, B.da, B.z1, B.s1, 1, B.da, (float*)g[1], (float*)g[2], scr, c.stream, bn_extra(c, pf + 1)))) return rc;
+    if (g_out && use_tc(c.ch, u.g1, B.da, p[0], g_out) && tc_dgrad_joins(u.g1)) {
+        GradientJoin join;
+        join.add = dx_shortcut;
+        if (mask_out) { join.mask = x; c.masked = true; }
+        return conv_backward_pair(c, u.g1, B.da, x, p[0], pf, g_out, join);
+    }
     if ((rc = conv_backward_pair(c, u.g1, B.da, x, p[0], pf, g_out))) return rc;
     if (!g_out) return CKPT_OK;
     return add_tensors(dt, in_px * u.in.c, g_out, dx_shortcut, g_out, c.stream);
@@ -466,7 +476,7 @@ static int unit_backward(StepCtx& c, int64_t i, const void* x_raw, const void* y
         }
         case CKPT_UNIT_BOTTLENECK:
             if ((rc = activated(c, i - 1, x_raw, &x))) return rc;
-            if ((rc = block_backward(c, u, x, y, g_in, g_out))) return rc;
+            if ((rc = block_backward(c, u, x, y, g_in, g_out, i > 1 && c.ch->units[i - 2].desc.kind == CKPT_UNIT_BOTTLENECK && !c.ch->tap))) return rc;
             break;
         default:
             set_error("unit kind %d has no backward kernel", u.desc.kind);

@@ -38,6 +38,7 @@ constexpr int kThreads = 192;
 // and every launch without sums 5-14 % slower, with one slab or two; two warps per quarter stay.
 constexpr int kTEpi = 2;
 constexpr int kTSlabs = 2;
+constexpr int kJoinSlots = 3;
 constexpr int kThreadsT = 64 + 128 * kTEpi;           // TMA warp, MMA warp, 4 * kTEpi epilogue warps
 constexpr int kMaxStages = 8;
 constexpr uint32_t kSmemBudget = 200 * 1024;          // operand stages; barriers live behind them
@@ -552,6 +553,8 @@ struct TParams {
     int col_term[4][3];          // term (index into the tap tables) of column c at vertical tap dy; tap_dh = dy - 1
     int tile_cols;               // pixels per tile: a multiple of 32, at most 256; 8 * th * stack for the halo-patch kernel
     int split;                   // CTAs of a cluster that share the reduction of a tile
+    // gradient join (1x1 input gradients, pixels as one row): what is stored is (sum + join_add) where join_mask > 0
+    const __nv_bfloat16 *join_add, *join_mask;    // join_mask may be null
     uint32_t patch_bytes;        // 8 x (th + 2) pixels x 128 bytes; stacked: 8 x th x stack
     // stacked form for small images (tc_conv_tp_kernel): a tile is the strip of `stack` whole images, each taking th
     // rows of the accumulator (its H rows and th - H idle ones) and th rows of the patch (rows -1 .. th - 2: the image,
@@ -589,22 +592,42 @@ __device__ __forceinline__ void load_filter_boxes(const TParams& p, const CUtens
     }
 }
 
+// The join by plain loads: channel `co` of 32 consecutive pixels from `pixel` on.
+__device__ __forceinline__ void join_chunk(const TParams& p, size_t pixel, int co, uint32_t in_mask, uint32_t (&v)[32]) {
+    const size_t at = pixel * p.c_out + co;
+    const uint16_t *const add = reinterpret_cast<const uint16_t*>(p.join_add) + at, *const mask = reinterpret_cast<const uint16_t*>(p.join_mask) + at;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+        if (!((in_mask >> e) & 1u) || co >= p.c_out) continue;
+        const float sum = __uint_as_float(v[e]) + __uint_as_float((uint32_t)__ldg(add + (size_t)e * p.c_out) << 16);
+        v[e] = !p.join_mask || __uint_as_float((uint32_t)__ldg(mask + (size_t)e * p.c_out) << 16) > 0.f ? __float_as_uint(sum) : 0u;
+    }
+}
+
 // A_MN (dgrad): the M operand is the forward filter [c_red][taps][c_out] read in place, output channels contiguous:
 // two boxes of 64 reduction rows x 64 output channels per stage (at the column block of the mirrored filter
 // position), an MN-major operand for the tensor core.  No transposed copy of the filter is made.
 // SPLIT: few tiles with a long reduction (small images, small batches).  The p.split CTAs of a cluster take a share of
 // the terms of one tile each, leave their float32 accumulators in shared memory and add them up in rank order, every
 // 32 x 32 block by one warp of the cluster, which finishes it as usual.
-template <bool A_MN, bool SPLIT>
+//
+// JOIN: the input gradient of a residual block's first convolution takes the shortcut's gradient, and the mask of the ReLU
+// that ends the block before, on its way out: a separate addition and masking would write, read twice and write the tensor
+// again.  Every epilogue warp has three slots; the chunk's values of both tensors arrive in one by tile loads while the
+// chunk before is finished, and the result leaves from the slot.  (Values loaded by the lanes, 64 bytes per instruction,
+// made 256 -> 1024 at 14 x 14, 128 images 70 us; JOINUS with the slots, HBM takes 27.)
+template <bool A_MN, bool SPLIT, bool JOIN>
 __global__ void __launch_bounds__(kThreadsT, 1)
 tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                 const __grid_constant__ CUtensorMap map_out, float* __restrict__ stat_partial, TParams p, int* status) {
+                 const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_add,
+                 const __grid_constant__ CUtensorMap map_mask, float* __restrict__ stat_partial, TParams p, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     constexpr uint32_t a_bytes = 128 * 128;
     const uint32_t stage_bytes = a_bytes + (uint32_t)p.tile_cols * 128;
     const uint32_t bars = base + (uint32_t)p.stages * stage_bytes;           // full[s], empty[s], acc_full[2], acc_empty[2]
-    const uint32_t out_stage = bars + 256;                                   // [8 warps][2][32 pixels x 32 channels] bf16
+    // [8 warps][2][32 pixels x 32 channels] bf16; with a join [8 warps][3][add, then the result | mask]
+    const uint32_t out_stage = bars + 512;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int failed_flag;
     volatile int* failed = &failed_flag;
@@ -633,6 +656,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         failed_flag = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full0 + 8 * b, 1); mbar_init(acc_empty0 + 8 * b, 128 * kTEpi); }
+        if (JOIN) for (int s = 0; s < 4 * kTEpi * kJoinSlots; ++s) mbar_init(bars + 256u + 8u * s, 1);
         fence_barrier_init();
         tma_prefetch_desc(&map_x);
         tma_prefetch_desc(&map_w);
@@ -722,6 +746,68 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 for (int e = 0; e < 32; ++e) asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + (uint32_t)(e * 512)), "r"(v[e]) : "memory");
             }
             tc_fence_before();
+        }
+    } else if (JOIN && warp >= 2) {
+        // ---------------- epilogue with a gradient join (pixels as one row, see above)
+        const int quarter = warp % 4, half = (warp - 2) / 4, ch = co_tile * 128 + quarter * 32;
+        const bool mine = ch < p.c_out, masked = p.join_mask != nullptr;
+        const int per_tile = (p.tile_cols / 32 - half + kTEpi - 1) / kTEpi, total = mine ? my_tiles * per_tile : 0;
+        const uint32_t slots = out_stage + (uint32_t)((warp - 2) * kJoinSlots) * 4096u, slot_bars = bars + 256u + (uint32_t)((warp - 2) * kJoinSlots) * 8u;
+        auto column = [&](int n) { return (first + n / per_tile * p.ctas_per_co) * p.tile_cols + (half + n % per_tile * kTEpi) * 32; };
+        int fetched = 0, done = 0;
+        auto fetch = [&]() {                          // lane 0: chunk `fetched` into its slot
+            const int s = fetched % kJoinSlots;
+            mbar_expect_tx(slot_bars + 8u * s, masked ? 4096u : 2048u);
+            tma_load_4d(slots + (uint32_t)s * 4096u, &map_add, slot_bars + 8u * s, ch, column(fetched), 0, 0);
+            if (masked) tma_load_4d(slots + (uint32_t)s * 4096u + 2048u, &map_mask, slot_bars + 8u * s, ch, column(fetched), 0, 0);
+            ++fetched;
+        };
+        if (lane == 0 && total > 0) fetch();
+        bool ok = true;
+        for (int j = 0; j < my_tiles && ok; ++j) {
+            const int buf = j & 1;
+            if (!mbar_wait(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 906)) break;
+            tc_fence_after();
+            if (mine) {
+#pragma unroll 1
+                for (int m = 0; m < per_tile; ++m, ++done) {
+                    // the next chunk's slot: a store read it two chunks ago
+                    if (lane == 0 && fetched < total) { tma_store_wait_read<kJoinSlots - 2>(); fetch(); }
+                    const int s = done % kJoinSlots, w0 = column(done);
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + (half + m * kTEpi) * 32), v);
+                    if (!mbar_wait(slot_bars + 8u * s, (uint32_t)(done / kJoinSlots) & 1u, failed, status, 907)) { ok = false; break; }
+                    const uint32_t slab = slots + (uint32_t)s * 4096u + (uint32_t)(lane * 2);
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2) {
+                        uint16_t a0, a1, m0, m1;
+                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(a0) : "r"(slab + (uint32_t)(e * 64)) : "memory");
+                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(a1) : "r"(slab + (uint32_t)((e + 1) * 64)) : "memory");
+                        float f0 = __uint_as_float(v[e]) + __uint_as_float((uint32_t)a0 << 16), f1 = __uint_as_float(v[e + 1]) + __uint_as_float((uint32_t)a1 << 16);
+                        if (masked) {
+                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(m0) : "r"(slab + (uint32_t)(2048 + e * 64)) : "memory");
+                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(m1) : "r"(slab + (uint32_t)(2048 + (e + 1) * 64)) : "memory");
+                            f0 = __uint_as_float((uint32_t)m0 << 16) > 0.f ? f0 : 0.f;
+                            f1 = __uint_as_float((uint32_t)m1 << 16) > 0.f ? f1 : 0.f;
+                        }
+                        const __nv_bfloat162 r = __floats2bfloat162_rn(f0, f1);
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(slab + (uint32_t)(e * 64)), "h"(__bfloat16_as_ushort(r.x)) : "memory");
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(slab + (uint32_t)((e + 1) * 64)), "h"(__bfloat16_as_ushort(r.y)) : "memory");
+                    }
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (w0 < p.W) tma_store_4d(&map_out, slots + (uint32_t)s * 4096u, ch, w0, 0, 0);
+                        tma_store_commit();
+                    }
+                }
+            }
+            tc_fence_before();
+            mbar_arrive(acc_empty0 + 8 * buf);
+        }
+        if (lane == 0) {
+            for (int n = done; n < fetched; ++n) mbar_drain(slot_bars + 8u * (n % kJoinSlots), (uint32_t)(n / kJoinSlots) & 1u);
+            tma_store_wait_all();
         }
     } else if (warp >= 2) {
         // ---------------- epilogue: lane of the accumulator = output channel, column = pixel of the tile.  A chunk
@@ -819,6 +905,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 uint32_t v[32];
 #pragma unroll
                 for (int e = 0; e < 32; ++e) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v[e]) : "r"(block + (uint32_t)(e * 512 + lane * 4)) : "memory");
+                if constexpr (JOIN) join_chunk(p, (size_t)w0 + c0, co, in_mask, v);
                 float sum[4] = {0.f, 0.f, 0.f, 0.f}, sumsq[4] = {0.f, 0.f, 0.f, 0.f};
                 const uint32_t slab = out_stage + (uint32_t)((warp - 2) * kTSlabs * 2048);
                 if (lane == 0) tma_store_wait_read<0>();
@@ -3053,6 +3140,20 @@ bool tp_stack(int H, int W, int N, int co_tiles, int* th_out, int* stack_out) {
     return true;
 }
 
+// 32 channels x bw x bh x bn pixels of an NHWC bf16 tensor without swizzle.
+int make_chunk_map(CUtensorMap* map, const void* ptr, int N, int H, int W, int C, int bw, int bh, int bn) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return CKPT_E_CUDA; }
+    cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
+    cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
+    cuuint32_t box[4] = {32, (cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bn};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled failed for an output tensor (code %d)", (int)r); return CKPT_E_CUDA; }
+    return CKPT_OK;
+}
+
 // Pixel tile and reduction split of the plain role-swapped kernel, by a model of clocks fitted to a sweep of both over
 // 26 shapes: a stage (64 reduction channels of one term) takes its four MMAs - 430 however few pixels, 2 per pixel above
 // 215 - or its bytes from the L2; the epilogue of a tile takes about 1100 and 15 per pixel and runs under the next tile's stages; a
@@ -3119,29 +3220,24 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     if (p.split > 1) p.ctas_per_co = p.p_tiles;
     const uint32_t stage_bytes = 128 * 128 + (uint32_t)p.tile_cols * 128;
     constexpr uint32_t t_slabs = 4 * kTEpi * kTSlabs * 2048;
-    p.stages = std::min<int>(kMaxStages, (227 * 1024 - 1024 - 256 - t_slabs - 64) / stage_bytes);
+    const uint32_t slabs = p.join_add ? 4 * kTEpi * kJoinSlots * 4096 : t_slabs;
+    p.stages = std::min<int>(kMaxStages, (227 * 1024 - 1024 - 512 - slabs - 64) / stage_bytes);
     CUtensorMap mx;
     int rc = make_act_map(&mx, x, N, H, W, x_channels, p.tw, patch && !p.stack ? p.th + 2 : p.th, p.tn);
     if (rc) return rc;
-    // the box of one epilogue chunk: 32 consecutive pixels of the tile (w fastest) x 32 channels, no swizzle
-    CUtensorMap mo;
-    {
-        const int bw = std::min(p.tw, 32), bh = std::min(p.th, 32 / bw), bnn = 32 / (bw * bh);
-        EncodeTiledFn fn = encode_fn();
-        if (!fn) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return CKPT_E_CUDA; }
-        cuuint64_t dims[4] = {(cuuint64_t)c_out, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
-        cuuint64_t strides[3] = {(cuuint64_t)c_out * 2, (cuuint64_t)W * c_out * 2, (cuuint64_t)H * W * c_out * 2};
-        cuuint32_t box[4] = {32, (cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bnn};
-        cuuint32_t es[4] = {1, 1, 1, 1};
-        CUresult r = fn(&mo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, out, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled failed for an output tensor (code %d)", (int)r); return CKPT_E_CUDA; }
-    }
-    const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 256 + t_slabs;
+    // the box of one epilogue chunk: 32 consecutive pixels of the tile (w fastest) x 32 channels
+    CUtensorMap mo, madd, mmask;
+    const int bw = std::min(p.tw, 32), bh = std::min(p.th, 32 / bw), bnn = 32 / (bw * bh);
+    if ((rc = make_chunk_map(&mo, out, N, H, W, c_out, bw, bh, bnn))) return rc;
+    madd = mmask = mo;
+    if (p.join_add && (rc = make_chunk_map(&madd, p.join_add, N, H, W, c_out, bw, bh, bnn))) return rc;
+    if (p.join_mask && (rc = make_chunk_map(&mmask, p.join_mask, N, H, W, c_out, bw, bh, bnn))) return rc;
+    const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 512 + slabs;
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaSuccess;
-        for (auto kernel : {tc_conv_t_kernel<false, false>, tc_conv_t_kernel<true, false>, tc_conv_t_kernel<false, true>, tc_conv_t_kernel<true, true>})
+        for (auto kernel : {tc_conv_t_kernel<false, false, false>, tc_conv_t_kernel<true, false, false>, tc_conv_t_kernel<false, true, false>,
+                            tc_conv_t_kernel<true, true, false>, tc_conv_t_kernel<true, false, true>, tc_conv_t_kernel<true, true, true>})
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 64);
         if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
         attr_set = true;
@@ -3171,21 +3267,21 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
         attr.id = cudaLaunchAttributeClusterDimension;
         attr.val.clusterDim.x = (unsigned)p.split; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
         cfg.attrs = &attr; cfg.numAttrs = 1;
-        const cudaError_t e = a_mn ? cudaLaunchKernelEx(&cfg, tc_conv_t_kernel<true, true>, mx, mw, mo, stats, p, status)
-                                   : cudaLaunchKernelEx(&cfg, tc_conv_t_kernel<false, true>, mx, mw, mo, stats, p, status);
+        const auto kernel = p.join_add ? tc_conv_t_kernel<true, true, true> : a_mn ? tc_conv_t_kernel<true, true, false> : tc_conv_t_kernel<false, true, false>;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mx, mw, mo, madd, mmask, stats, p, status);
         if (e != cudaSuccess) return cuda_fail(e, what);
-    } else if (a_mn) {
-        tc_conv_t_kernel<true, false><<<grid, kThreadsT, smem, st>>>(mx, mw, mo, stats, p, status);
     } else {
-        tc_conv_t_kernel<false, false><<<grid, kThreadsT, smem, st>>>(mx, mw, mo, stats, p, status);
+        const auto kernel = p.join_add ? tc_conv_t_kernel<true, false, true> : a_mn ? tc_conv_t_kernel<true, false, false> : tc_conv_t_kernel<false, false, false>;
+        kernel<<<grid, kThreadsT, smem, st>>>(mx, mw, mo, madd, mmask, stats, p, status);
     }
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_t_kernel", what);
     return CKPT_OK;
 }
 
 int launch_t(const void* x, const void* w_mat, void* out, float* stat_partial, int* stat_blocks, int N, int H, int W, int c_red,
-             int c_out, int k, int pad, int* status, cudaStream_t st, const char* what, bool a_mn = false) {
+             int c_out, int k, int pad, int* status, cudaStream_t st, const char* what, bool a_mn = false, const GradientJoin& join = GradientJoin()) {
     TParams p;
+    p.join_add = (const __nv_bfloat16*)join.add; p.join_mask = (const __nv_bfloat16*)join.mask;
     p.taps = k * k;
     p.fold = 0;
     p.pair = 0;
@@ -3223,6 +3319,7 @@ int launch_t_paired(const void* x, const void* w, int flip, void* out, float* st
     // pair sees column sp through filter column s = sp - q.  flip: w is the forward filter [c_red][9][64] and the
     // input gradient takes the mirrored position.
     TParams p;
+    p.join_add = p.join_mask = nullptr;
     p.taps = 12;
     p.fold = 64;
     p.pair = 1;
@@ -3685,8 +3782,12 @@ int tc_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, const 
                            "conv forward (tensor cores)");
 }
 
+bool tc_dgrad_joins(const ConvGeom& g) {
+    return tc_conv_supported(CKPT_DTYPE_BF16, g) && g.k == 1 && g.stride == 1 && t_applies(g.cout, g.cin, 1, 0) && (int64_t)g.n * g.h * g.w >= 256;
+}
+
 int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, void* scratch, int64_t scratch_bytes,
-                  int* device_status, void* stream) {
+                  int* device_status, void* stream, const GradientJoin& join) {
     if (!device_status) { set_error("no status word"); return CKPT_E_NULL; }
     const int taps = g.k * g.k;
     cudaStream_t st = (cudaStream_t)stream;
@@ -3735,6 +3836,10 @@ int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, vo
             }
         }
         return CKPT_OK;
+    }
+    if (join.add) {
+        if (!tc_dgrad_joins(g)) { set_error("this input gradient has no join"); return CKPT_E_UNSUPPORTED; }
+        return launch_t(dz, w, dx, nullptr, nullptr, g.n, g.h, g.w, g.cout, g.cin, 1, 0, device_status, st, "conv dgrad with join (tensor cores)", true, join);
     }
     if (taps == 1) {
         // [c_out][c_in] is already the dgrad's B operand with the reduction (c_out) as rows: the tensor core reads

@@ -125,8 +125,12 @@ int tc_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, const 
 int tc_conv_fwd_stats(const ConvGeom& g, const void* x, const void* w, void* z, float* partial, int* blocks,
                       int* device_status, void* stream,
                       int64_t partial_bytes = 0);
+// Gradient join of a residual block: dx = (input gradient + add) where mask > 0 (add, mask: bf16 tensors of dx's shape,
+// mask may be null); 1x1 stride-1 filters for which tc_dgrad_joins holds.
+struct GradientJoin { const void *add = nullptr, *mask = nullptr; };
+bool tc_dgrad_joins(const ConvGeom& g);
 int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, void* scratch,
-                  int64_t scratch_bytes, int* device_status, void* stream);
+                  int64_t scratch_bytes, int* device_status, void* stream, const GradientJoin& join = GradientJoin());
 // upd: optional parameter update applied together with the gradient (the filter must no longer be needed by this step)
 int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch,
                   int64_t scratch_bytes, int* device_status, void* stream, const SgdUpdate& upd = SgdUpdate());

@@ -434,3 +434,23 @@ def test_store_all_that_keeps_block_interiors(dtype):
     assert rep_c["launches"] == rep_d["launches"] and rep_c["peak_bytes"] == rep_d["peak_bytes"]
     for a, b in zip(g_a, g_c):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_joined_gradients_equal_separate_ones(graph):
+    """The input gradient of a residual block takes the shortcut's gradient and the previous block's ReLU on its way out.
+    With the gradient tap on, that ReLU is applied by the block it ends instead: the same bits."""
+    import torch
+    spec = wl.resnet_chain([2, 2, 1, 1], 5, hw=(70, 90), classes=24)
+    params = wl.make_params(spec, seed=5, bn_affine="random")
+    x, labels = wl.make_batch(spec, seed=6)
+    runner = StepRunner(spec, params)
+    runner.chain.set_graph(graph)
+    mask = ck.plan(ck.ALGO_DYNAMIC_N, runner.d)[0]
+    _, plain = runner.run(ck.POLICY_DYNAMIC, mask, x, labels)
+    tap = torch.empty(int(sum(runner.d[1:])), dtype=torch.uint8, device="cuda")
+    runner.chain.set_gradient_tap(tap)
+    _, tapped = runner.run(ck.POLICY_DYNAMIC, mask, x, labels)
+    runner.chain.set_gradient_tap(None)
+    for a, b in zip(plain, tapped):
+        assert np.array_equal(a, b)
