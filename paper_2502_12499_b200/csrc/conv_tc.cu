@@ -38,7 +38,7 @@ constexpr int kThreads = 192;
 // and every launch without sums 5-14 % slower, with one slab or two; two warps per quarter stay.
 constexpr int kTEpi = 2;
 constexpr int kTSlabs = 2;
-constexpr int kJoinSlots = 3;
+constexpr int kJoinSlots = 4;
 constexpr int kThreadsT = 64 + 128 * kTEpi;           // TMA warp, MMA warp, 4 * kTEpi epilogue warps
 constexpr int kMaxStages = 8;
 constexpr uint32_t kSmemBudget = 200 * 1024;          // operand stages; barriers live behind them
@@ -613,9 +613,9 @@ __device__ __forceinline__ void join_chunk(const TParams& p, size_t pixel, int c
 //
 // JOIN: the input gradient of a residual block's first convolution takes the shortcut's gradient, and the mask of the ReLU
 // that ends the block before, on its way out: a separate addition and masking would write, read twice and write the tensor
-// again.  Every epilogue warp has three slots; the chunk's values of both tensors arrive in one by tile loads while the
-// chunk before is finished, and the result leaves from the slot.  (Values loaded by the lanes, 64 bytes per instruction,
-// made 256 -> 1024 at 14 x 14, 128 images 70 us; JOINUS with the slots, HBM takes 27.)
+// again.  Every epilogue warp has four slots; the chunk's values of both tensors arrive in one by tile loads two chunks ahead
+// of their turn, and the result leaves from the slot.  (Values loaded by the lanes, 64 bytes per instruction,
+// made 256 -> 1024 at 14 x 14, 128 images 70 us; 35 with the slots, HBM takes 27.)
 template <bool A_MN, bool SPLIT, bool JOIN>
 __global__ void __launch_bounds__(kThreadsT, 1)
 tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
@@ -626,7 +626,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     constexpr uint32_t a_bytes = 128 * 128;
     const uint32_t stage_bytes = a_bytes + (uint32_t)p.tile_cols * 128;
     const uint32_t bars = base + (uint32_t)p.stages * stage_bytes;           // full[s], empty[s], acc_full[2], acc_empty[2]
-    // [8 warps][2][32 pixels x 32 channels] bf16; with a join [8 warps][3][add, then the result | mask]
+    // [8 warps][2][32 pixels x 32 channels] bf16; with a join [8 warps][4][add, then the result | mask]
     const uint32_t out_stage = bars + 512;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int failed_flag;
@@ -762,7 +762,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             if (masked) tma_load_4d(slots + (uint32_t)s * 4096u + 2048u, &map_mask, slot_bars + 8u * s, ch, column(fetched), 0, 0);
             ++fetched;
         };
-        if (lane == 0 && total > 0) fetch();
+        if (lane == 0) while (fetched < min(total, kJoinSlots - 2)) fetch();
         bool ok = true;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int buf = j & 1;
@@ -771,28 +771,34 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             if (mine) {
 #pragma unroll 1
                 for (int m = 0; m < per_tile; ++m, ++done) {
-                    // the next chunk's slot: a store read it two chunks ago
-                    if (lane == 0 && fetched < total) { tma_store_wait_read<kJoinSlots - 2>(); fetch(); }
+                    // two chunks ahead, into the slot that a store read two chunks ago
+                    if (lane == 0 && fetched < total) { tma_store_wait_read<1>(); fetch(); }
                     const int s = done % kJoinSlots, w0 = column(done);
                     uint32_t v[32];
                     tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + (half + m * kTEpi) * 32), v);
                     if (!mbar_wait(slot_bars + 8u * s, (uint32_t)(done / kJoinSlots) & 1u, failed, status, 907)) { ok = false; break; }
                     const uint32_t slab = slots + (uint32_t)s * 4096u + (uint32_t)(lane * 2);
+                    // (all loads of a half chunk before its stores: in turn each pair would wait for its loads)
 #pragma unroll
-                    for (int e = 0; e < 32; e += 2) {
-                        uint16_t a0, a1, m0, m1;
-                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(a0) : "r"(slab + (uint32_t)(e * 64)) : "memory");
-                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(a1) : "r"(slab + (uint32_t)((e + 1) * 64)) : "memory");
-                        float f0 = __uint_as_float(v[e]) + __uint_as_float((uint32_t)a0 << 16), f1 = __uint_as_float(v[e + 1]) + __uint_as_float((uint32_t)a1 << 16);
-                        if (masked) {
-                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(m0) : "r"(slab + (uint32_t)(2048 + e * 64)) : "memory");
-                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(m1) : "r"(slab + (uint32_t)(2048 + (e + 1) * 64)) : "memory");
-                            f0 = __uint_as_float((uint32_t)m0 << 16) > 0.f ? f0 : 0.f;
-                            f1 = __uint_as_float((uint32_t)m1 << 16) > 0.f ? f1 : 0.f;
+                    for (int h = 0; h < 32; h += 16) {
+                        uint16_t add[16], mask[16];
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(add[e]) : "r"(slab + (uint32_t)((h + e) * 64)));
+                            if (masked) asm volatile("ld.shared.u16 %0, [%1];" : "=h"(mask[e]) : "r"(slab + (uint32_t)(2048 + (h + e) * 64)));
                         }
-                        const __nv_bfloat162 r = __floats2bfloat162_rn(f0, f1);
-                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(slab + (uint32_t)(e * 64)), "h"(__bfloat16_as_ushort(r.x)) : "memory");
-                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(slab + (uint32_t)((e + 1) * 64)), "h"(__bfloat16_as_ushort(r.y)) : "memory");
+#pragma unroll
+                        for (int e = 0; e < 16; e += 2) {
+                            float f0 = __uint_as_float(v[h + e]) + __uint_as_float((uint32_t)add[e] << 16);
+                            float f1 = __uint_as_float(v[h + e + 1]) + __uint_as_float((uint32_t)add[e + 1] << 16);
+                            if (masked) {
+                                f0 = __uint_as_float((uint32_t)mask[e] << 16) > 0.f ? f0 : 0.f;
+                                f1 = __uint_as_float((uint32_t)mask[e + 1] << 16) > 0.f ? f1 : 0.f;
+                            }
+                            const __nv_bfloat162 r = __floats2bfloat162_rn(f0, f1);
+                            asm volatile("st.shared.b16 [%0], %1;" ::"r"(slab + (uint32_t)((h + e) * 64)), "h"(__bfloat16_as_ushort(r.x)) : "memory");
+                            asm volatile("st.shared.b16 [%0], %1;" ::"r"(slab + (uint32_t)((h + e + 1) * 64)), "h"(__bfloat16_as_ushort(r.y)) : "memory");
+                        }
                     }
                     fence_proxy_async();
                     __syncwarp();
