@@ -552,6 +552,7 @@ struct TParams {
     int ncols;                   // columns per 64-channel block: (horizontal offset, channel offset) pairs
     int col_term[4][3];          // term (index into the tap tables) of column c at vertical tap dy; tap_dh = dy - 1
     int tile_cols;               // pixels per tile: a multiple of 32, at most 256; 8 * th * stack for the halo-patch kernel
+    int in_stride;               // pixel box origin = tile origin * in_stride + tap offset (tensor map of the same stride)
     int split;                   // CTAs of a cluster that share the reduction of a tile
     // gradient join (1x1 input gradients, pixels as one row): what is stored is (sum + join_add) where join_mask > 0
     const __nv_bfloat16 *join_add, *join_mask;    // join_mask may be null
@@ -686,7 +687,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 // one term: its reduction blocks move along one coordinate
                 int c0 = 0, c1 = 0, c2 = 0, c3 = 0, step0 = 64, step1 = 0;
                 if (lane == 0) {
-                    c0 = blk * 64 + p.tap_xc[tap]; c1 = w0 + p.tap_dw[tap]; c2 = h0 + p.tap_dh[tap]; c3 = n0;
+                    c0 = blk * 64 + p.tap_xc[tap]; c1 = w0 * p.in_stride + p.tap_dw[tap]; c2 = h0 * p.in_stride + p.tap_dh[tap]; c3 = n0;
                 } else {
                     filter_box<A_MN>(p, tap, blk, co_tile, lane == 2, c0, c1);
                     if (A_MN) { step0 = 0; step1 = 64; }
@@ -3146,12 +3147,15 @@ bool tp_stack(int H, int W, int N, int co_tiles, int* th_out, int* stack_out) {
     return true;
 }
 
-// 32 channels x bw x bh x bn pixels of an NHWC bf16 tensor without swizzle.
-int make_chunk_map(CUtensorMap* map, const void* ptr, int N, int H, int W, int C, int bw, int bh, int bn) {
+// 32 channels x bw x bh x bn pixels of an NHWC bf16 tensor without swizzle; rows and images `row` and `image` pixels apart,
+// neighbouring pixels `pixel` (0: a dense tensor).
+int make_chunk_map(CUtensorMap* map, const void* ptr, int N, int H, int W, int C, int bw, int bh, int bn, int64_t pixel = 0, int64_t row = 0,
+                   int64_t image = 0) {
+    if (!pixel) { pixel = 1; row = W; image = (int64_t)H * W; }
     EncodeTiledFn fn = encode_fn();
     if (!fn) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return CKPT_E_CUDA; }
     cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
-    cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
+    cuuint64_t strides[3] = {(cuuint64_t)(pixel * C * 2), (cuuint64_t)(row * C * 2), (cuuint64_t)(image * C * 2)};
     cuuint32_t box[4] = {32, (cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bn};
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -3167,8 +3171,8 @@ int make_chunk_map(CUtensorMap* map, const void* ptr, int N, int H, int W, int C
 // 2 x 2, 128 images 25.5 -> 11.8 (64 pixels, 4 CTAs each), 512 -> 512 at 20 x 12, 13 images 26.2 -> 20.2 (256, 2),
 // 256 -> 256 at 13 x 11, 21 images 16.0 -> 12.6 (128, 2), 1x1 1024 -> 256 at 14 x 14, 128 images 17.1 -> 15.1 (192, 1).
 // 1x1 filters see the pixels as one row (tiles of any multiple of 32, no ragged edges but the last).
-void t_plan(TParams* p, int* W, int* H, int* N) {
-    const bool flat = p->taps == 1 && !p->fold;
+void t_plan(TParams* p, int* W, int* H, int* N, bool dense) {
+    const bool flat = p->taps == 1 && !p->fold && dense;
     if (flat) { p->W = *W = *W * *H * *N; p->H = *H = 1; p->N = *N = 1; }
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
@@ -3180,6 +3184,7 @@ void t_plan(TParams* p, int* W, int* H, int* N) {
         if (p->fold && cols != 256) continue;
         int tw = cols, th = 1, tn = 1;
         if (!flat) choose_tile(cols, *W, *H, *N, &tw, &th, &tn);
+        if (tw * p->in_stride > 256 || th * p->in_stride > 256) continue;       // the box of a strided tensor map
         const int64_t tiles = (int64_t)((*W + tw - 1) / tw) * ((*H + th - 1) / th) * ((*N + tn - 1) / tn);
         for (int split = 1; split <= 8; split *= 2) {
             if (split > 1 && (p->fold || terms < 2 * split || (int64_t)tiles * co * split > sms - 4 * split)) break;
@@ -3193,8 +3198,13 @@ void t_plan(TParams* p, int* W, int* H, int* N) {
     }
 }
 
+// Strided convolutions on the plain role-swapped kernel: the grid N x H x W is that of the output (forward), read from an
+// input of x_h x x_w, or one parity class of the input gradient, written to every out_stride-th pixel of rows of out_w.
+struct TView { int in_stride, x_h, x_w, out_stride, out_h, out_w; };
+
 int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& mw, void* out, float* stat_partial, int* stat_blocks,
-                  int N, int H, int W, int c_red, int c_out, int* status, cudaStream_t st, const char* what, bool a_mn) {
+                  int N, int H, int W, int c_red, int c_out, int* status, cudaStream_t st, const char* what, bool a_mn, const TView* view = nullptr) {
+    p.in_stride = view ? view->in_stride : 1;
     p.H = H; p.W = W; p.N = N; p.c_red = c_red; p.c_out = c_out;
     bool patch = false;
     int strip_h = 0, stack = 0;
@@ -3212,7 +3222,7 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
         p.patch_bytes = (uint32_t)(8 * strip_h * stack) * 128;
     }
     p.split = 1;
-    if (!patch) t_plan(&p, &W, &H, &N);
+    if (!patch) t_plan(&p, &W, &H, &N, !view);
     p.tw_log = 0; while ((1 << p.tw_log) < p.tw) ++p.tw_log;
     p.th_log = 0; while ((1 << p.th_log) < p.th) ++p.th_log;
     p.tiles_w = (W + p.tw - 1) / p.tw; p.tiles_h = (H + p.th - 1) / p.th; p.tiles_n = (N + p.tn - 1) / p.tn;
@@ -3229,12 +3239,14 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     const uint32_t slabs = p.join_add ? 4 * kTEpi * kJoinSlots * 4096 : t_slabs;
     p.stages = std::min<int>(kMaxStages, (227 * 1024 - 1024 - 512 - slabs - 64) / stage_bytes);
     CUtensorMap mx;
-    int rc = make_act_map(&mx, x, N, H, W, x_channels, p.tw, patch && !p.stack ? p.th + 2 : p.th, p.tn);
+    int rc = view ? make_act_map(&mx, x, N, view->x_h, view->x_w, x_channels, p.tw, p.th, p.tn, view->in_stride)
+                  : make_act_map(&mx, x, N, H, W, x_channels, p.tw, patch && !p.stack ? p.th + 2 : p.th, p.tn);
     if (rc) return rc;
     // the box of one epilogue chunk: 32 consecutive pixels of the tile (w fastest) x 32 channels
     CUtensorMap mo, madd, mmask;
     const int bw = std::min(p.tw, 32), bh = std::min(p.th, 32 / bw), bnn = 32 / (bw * bh);
-    if ((rc = make_chunk_map(&mo, out, N, H, W, c_out, bw, bh, bnn))) return rc;
+    const int64_t os = view ? view->out_stride : 0;
+    if ((rc = make_chunk_map(&mo, out, N, H, W, c_out, bw, bh, bnn, os, view ? os * view->out_w : 0, view ? (int64_t)view->out_h * view->out_w : 0))) return rc;
     madd = mmask = mo;
     if (p.join_add && (rc = make_chunk_map(&madd, p.join_add, N, H, W, c_out, bw, bh, bnn))) return rc;
     if (p.join_mask && (rc = make_chunk_map(&mmask, p.join_mask, N, H, W, c_out, bw, bh, bnn))) return rc;
@@ -3751,9 +3763,31 @@ int stem_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw,
     return CKPT_OK;
 }
 
+static TParams strided_terms() {
+    TParams q;
+    q.fold = 0; q.pair = 0; q.patch_ok = 0; q.ncols = 0;
+    q.join_add = q.join_mask = nullptr;
+    return q;
+}
+
+// Both strided directions take the role-swapped kernel where it serves the channel counts: its outputs leave as tile stores
+// and carry the batch-norm sums for nothing (128 images, us, generic kernel -> here: 3x3 128 -> 128 at 56 x 56 with sums
+// 54.7 -> 36.3, input gradient 76.5 -> 51.0; 1x1 512 -> 1024 at 28 x 28 with sums 50.8 -> 29.9; 3x3 512 -> 512 at 14 x 14
+// 60.1 -> 27.0; 1x1 1024 -> 2048 at 14 x 14 alone is slower, 29.4 -> 34.0, with sums 39.1 -> 37.1).
 // Strided forward: the operand boxes take every stride-th input pixel, the tiles walk the output grid.
 static int launch_strided_fwd(const ConvGeom& g, const void* x, const void* w, void* z, int* status, cudaStream_t st,
                               float* stat_partial = nullptr, int* stat_blocks = nullptr) {
+    if (t_applies(g.cin, g.cout, g.k, g.pad)) {
+        TParams q = strided_terms();
+        q.taps = g.k * g.k;
+        for (int t = 0; t < q.taps; ++t) { q.tap_dh[t] = t / g.k - g.pad; q.tap_dw[t] = t % g.k - g.pad; q.tap_col[t] = t; q.tap_xc[t] = 0; }
+        CUtensorMap mw;
+        int rc = make_mat_map(&mw, w, g.cout, (int64_t)q.taps * g.cin, 128, 4);
+        if (rc) return rc;
+        const TView view = {g.stride, g.h, g.w, 1, g.ho, g.wo};
+        return launch_t_core(q, x, g.cin, mw, z, stat_partial, stat_blocks, g.n, g.ho, g.wo, g.cin, g.cout, status, st,
+                             "strided conv forward (tensor cores)", false, &view);
+    }
     FwdParams p;
     p.taps = g.k * g.k;
     for (int t = 0; t < p.taps; ++t) { p.tap_dh[t] = t / g.k - g.pad; p.tap_dw[t] = t % g.k - g.pad; p.tap_col[t] = t; }
@@ -3803,7 +3837,8 @@ int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, vo
         // a + (ph + pad - r)/stride (likewise along the width): one stride-1 sum over dz per class.
         const int sd = g.stride;
         const void* w_mat = w;
-        if (taps > 1) {
+        const bool in_place = t_applies(g.cout, g.cin, g.k, g.pad);      // role-swapped kernel: the filter is read where it is
+        if (taps > 1 && !in_place) {
             const int64_t elems = (int64_t)g.cout * taps * g.cin;
             if (!scratch || scratch_bytes < elems * 2) { set_error("dgrad scratch too small"); return CKPT_E_WORKSPACE; }
             const unsigned grid = (unsigned)std::min<int64_t>((elems + 255) / 256, 148 * 8);
@@ -3834,6 +3869,25 @@ int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, vo
                 const int gh = (g.h - ph + sd - 1) / sd, gw = (g.w - pw + sd - 1) / sd;
                 if (gh <= 0 || gw <= 0) continue;
                 if (p.taps == 0) continue;          // cleared above
+                if (in_place) {
+                    TParams q = strided_terms();
+                    q.taps = p.taps;
+                    int t = 0;
+                    for (int r = 0; r < g.k; ++r)
+                        for (int c = 0; c < g.k; ++c) {
+                            if ((ph + g.pad - r) % sd != 0 || (pw + g.pad - c) % sd != 0) continue;
+                            q.tap_dh[t] = p.tap_dh[t]; q.tap_dw[t] = p.tap_dw[t]; q.tap_col[t] = r * g.k + c; q.tap_xc[t] = 0;
+                            ++t;
+                        }
+                    CUtensorMap mw;
+                    int rc = make_mat_map(&mw, w, g.cout, (int64_t)taps * g.cin, 64, 4);
+                    if (rc) return rc;
+                    const TView view = {1, g.ho, g.wo, sd, g.h, g.w};
+                    rc = launch_t_core(q, dz, g.cout, mw, (__nv_bfloat16*)dx + ((int64_t)ph * g.w + pw) * g.cin, nullptr, nullptr, g.n, gh, gw, g.cout, g.cin,
+                                       device_status, st, "strided conv dgrad (tensor cores)", true, &view);
+                    if (rc) return rc;
+                    continue;
+                }
                 p.in_stride = 1;
                 p.out_H = g.h; p.out_W = g.w; p.out_stride = sd; p.out_oh = ph; p.out_ow = pw;
                 int rc = launch_generic(p, dz, g.n, g.ho, g.wo, w_mat, taps, dx, nullptr, 0, g.n, gh, gw, g.cout, g.cin,

@@ -528,3 +528,24 @@ def test_conv_wgrad_into_unaligned_gradient():
     ck.conv2d_wgrad(shape, dtype, 0, dz, x, a, scratch)
     ck.conv2d_wgrad(shape, dtype, 0, dz, x, b, scratch)
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("channels,hw", [(64, (56, 56)), (24, (9, 7)), (1000, (2, 3)), (13, (5, 4))])
+def test_average_pool_in_a_chain(channels, hw):
+    """Global average pooling forward and backward at vector and odd channel counts: gradients of a pooled sum loss."""
+    import torch
+    spec = dict(units=[{"kind": "avgpool"}], input_hwc=(hw[0], hw[1], channels), batch=3, dtype="f32", loss="sum", name="pool")
+    spec["units"].insert(0, {"kind": "relu"})
+    chain = ck.Chain(spec)
+    gen = torch.Generator(device="cuda").manual_seed(channels)
+    x = torch.randn((3, hw[0], hw[1], channels), generator=gen, device="cuda")
+    arena = torch.empty(ck.eval(ck.MODEL_STORE_ALL, chain.sizes(), None), dtype=torch.uint8, device="cuda")
+    tap = torch.empty(int(sum(chain.sizes()[1:])), dtype=torch.uint8, device="cuda")
+    chain.set_gradient_tap(tap)
+    report = ck.train_step(chain, None, ck.POLICY_STORE_ALL, x, None, [], [], arena,
+                           torch.empty(chain.workspace_bytes_for(ck.POLICY_STORE_ALL), dtype=torch.uint8, device="cuda"))
+    want = torch.relu(x).double().mean((1, 2))
+    assert abs(report["loss"] - float(want.sum())) <= 1e-4 * float(want.abs().sum())
+    n = x.numel()
+    g = tap[:n * 4].view(torch.float32)
+    assert torch.allclose(g, torch.full_like(g, 1.0 / (hw[0] * hw[1])), rtol=1e-6)
