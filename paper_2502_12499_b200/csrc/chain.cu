@@ -146,26 +146,22 @@ static int conv_dgrad_any(StepCtx& c, const ConvGeom& g, const void* dz, const v
         return tc_conv_dgrad(g, dz, w, dx, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream, join);
     return simt_conv_dgrad(c.ch->dtype, g, dz, w, dx, c.stream);
 }
-static int conv_wgrad_any(StepCtx& c, const ConvGeom& g, const void* dz, const void* x, float* dw) {
-    if (c.ch->impl == 0 && small_conv_supported(c.ch->dtype, g))
-        return small_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
-    if (c.ch->impl == 0 && stem_conv_supported(c.ch->dtype, g))
-        return stem_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
-    if (use_tc(c.ch, g, dz, x, nullptr))
-        return tc_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream);
-    return simt_conv_wgrad(c.ch->dtype, g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.stream);
-}
-
 // "Update w_i with g_i" (Algorithms 1, 2, 4), when a learning rate is set.  param = index of the parameter tensor.
 static SgdUpdate sgd_of(StepCtx& c, int param) {
     SgdUpdate u;
     if (c.ch->sgd_lr != 0.f) { u.w = c.params[param]; u.lr = c.ch->sgd_lr; u.dtype = c.ch->params[param].dtype; }
     return u;
 }
-static int sgd_step(StepCtx& c, int param) {
-    if (c.ch->sgd_lr == 0.f) return CKPT_OK;
-    return sgd_update(sgd_of(c, param), (const float*)c.grads[param], c.ch->params[param].elems, c.stream);
+static int conv_wgrad_any(StepCtx& c, const ConvGeom& g, const void* dz, const void* x, float* dw, const SgdUpdate& upd) {
+    if (c.ch->impl == 0 && small_conv_supported(c.ch->dtype, g))
+        return small_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream, upd);
+    if (c.ch->impl == 0 && stem_conv_supported(c.ch->dtype, g))
+        return stem_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream, upd);
+    if (use_tc(c.ch, g, dz, x, nullptr))
+        return tc_conv_wgrad(g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream, upd);
+    return simt_conv_wgrad(c.ch->dtype, g, dz, x, dw, c.ws + c.ch->off_scr, c.ch->scr_bytes, c.stream, upd);
 }
+
 // Weight gradient and input gradient of one convolution.  Without an update: wgrad, then dgrad.  With one the filter
 // changes as soon as its gradient is summed, so the input gradient (which reads the filter) runs first.
 static int conv_backward_pair(StepCtx& c, const ConvGeom& g, const void* dz, const void* x, const void* w, int param, void* dx,
@@ -173,18 +169,7 @@ static int conv_backward_pair(StepCtx& c, const ConvGeom& g, const void* dz, con
     int rc;
     const bool sgd = c.ch->sgd_lr != 0.f;
     if (sgd && dx && (rc = conv_dgrad_any(c, g, dz, w, dx, join))) return rc;
-    const bool stem = c.ch->impl == 0 && stem_conv_supported(c.ch->dtype, g);
-    const bool tc_path = !(c.ch->impl == 0 && small_conv_supported(c.ch->dtype, g)) && !stem && use_tc(c.ch, g, dz, x, nullptr);
-    if (sgd && stem) {
-        rc = stem_conv_wgrad(g, dz, x, (float*)c.grads[param], c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream, sgd_of(c, param));
-        if (rc) return rc;
-    } else if (sgd && tc_path) {
-        rc = tc_conv_wgrad(g, dz, x, (float*)c.grads[param], c.ws + c.ch->off_scr, c.ch->scr_bytes, c.status(), c.stream, sgd_of(c, param));
-        if (rc) return rc;
-    } else {
-        if ((rc = conv_wgrad_any(c, g, dz, x, (float*)c.grads[param]))) return rc;
-        if ((rc = sgd_step(c, param))) return rc;
-    }
+    if ((rc = conv_wgrad_any(c, g, dz, x, (float*)c.grads[param], sgd_of(c, param)))) return rc;
     if (!sgd && dx && (rc = conv_dgrad_any(c, g, dz, w, dx, join))) return rc;
     return CKPT_OK;
 }
@@ -469,8 +454,7 @@ static int unit_backward(StepCtx& c, int64_t i, const void* x_raw, const void* y
             if ((rc = activated(c, i - 1, x_raw, &x))) return rc;
             if (u.desc.flags & 1)
                 if ((rc = relu_mask_inplace(dt, elems, g_in, y, c.stream))) return rc;
-            if ((rc = column_sums(dt, c.ch->batch, u.out.c, g_in, (float*)g[1], c.stream))) return rc;
-            if ((rc = sgd_step(c, u.param_first + 1))) return rc;
+            if ((rc = column_sums(dt, c.ch->batch, u.out.c, g_in, (float*)g[1], c.stream, sgd_of(c, u.param_first + 1)))) return rc;
             if ((rc = conv_backward_pair(c, u.geom, g_in, x, p[0], u.param_first, g_out))) return rc;
             break;
         }

@@ -102,7 +102,7 @@ struct Pixel {
 template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 conv_gemm_kernel(ConvGeom g, const T* __restrict__ A, const T* __restrict__ B, void* __restrict__ out, const float* __restrict__ bias,
-                 int relu, int M, int N, int K, int k_per_slice, int cluster) {
+                 int relu, int M, int N, int K, int k_per_slice, int cluster, SgdUpdate upd) {
     using L = Tile<T, MODE, BM, BN, TM, TN>;
     constexpr int NT = L::threads, V = L::V, BK = L::BK;
     extern __shared__ __align__(16) uint8_t smem[];
@@ -327,6 +327,10 @@ conv_gemm_kernel(ConvGeom g, const T* __restrict__ A, const T* __restrict__ B, v
         if (m >= M || n >= N) return;
         if (MODE == 2) {
             ((float*)out)[((int64_t)z * M + m) * N + n] = v;
+            if (upd.w) {                                       // (one slice only) the filter is of the storage type
+                T* const w = (T*)upd.w + (int64_t)m * N + n;
+                *w = from_f<T>(fmaf(-upd.lr, v, to_f(*w)));
+            }
         } else {
             if (bias) v += bias[n];
             if (relu) v = fmaxf(v, 0.f);
@@ -381,7 +385,7 @@ Plan plan(int mode, int M, int N, int K, bool vectors);
 
 template <typename T>
 int launch(int mode, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K,
-           bool va, bool vb, const Plan& p, cudaStream_t st);
+           bool va, bool vb, const Plan& p, const SgdUpdate& upd, cudaStream_t st);
 
 }  // namespace simt
 }  // namespace ckpt

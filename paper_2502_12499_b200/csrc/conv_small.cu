@@ -123,17 +123,22 @@ __global__ void __launch_bounds__(256) unfold3x3_rows_kernel(const __nv_bfloat16
 // column of filter value k = (r, s, c) in an unfolded row
 __device__ __forceinline__ int unfolded_column(int k) { return (k / 9) * 10 + k % 9; }
 
+// One gradient value, and the update of its (bf16) filter value.
+__device__ __forceinline__ void take(float v, float* dw, int i, const SgdUpdate& upd) {
+    dw[i] = v;
+    if (upd.w) { __nv_bfloat16* w = (__nv_bfloat16*)upd.w + i; *w = __float2bfloat16_rn(fmaf(-upd.lr, v, __bfloat162float(*w))); }
+}
 // dw[co][0..K) out of the padded [c_out][64] result
-__global__ void take_columns_kernel(const float* __restrict__ dwp, float* __restrict__ dw, int cout, int k) {
+__global__ void take_columns_kernel(const float* __restrict__ dwp, float* __restrict__ dw, int cout, int k, SgdUpdate upd) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < cout * k) dw[i] = dwp[(i / k) * 64 + unfolded_column(i % k)];
+    if (i < cout * k) take(dwp[(i / k) * 64 + unfolded_column(i % k)], dw, i, upd);
 }
 // Paired pixels: dwp is [(parity, co)][(parity, column)]; the gradient is the sum of its two diagonal blocks.
-__global__ void take_paired_columns_kernel(const float* __restrict__ dwp, float* __restrict__ dw, int cout, int k) {
+__global__ void take_paired_columns_kernel(const float* __restrict__ dwp, float* __restrict__ dw, int cout, int k, SgdUpdate upd) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < cout * k) {
         const int co = i / k, col = unfolded_column(i % k);
-        dw[i] = dwp[(size_t)co * 64 + col] + dwp[(size_t)(cout + co) * 64 + 32 + col];
+        take(dwp[(size_t)co * 64 + col] + dwp[(size_t)(cout + co) * 64 + 32 + col], dw, i, upd);
     }
 }
 
@@ -167,10 +172,10 @@ int small_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, voi
 }
 
 int small_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes,
-                     int* device_status, void* stream) {
+                     int* device_status, void* stream, const SgdUpdate& upd) {
     // (16-byte rows for the TMA unit; a channel count that is no multiple of 64 also has the CUDA-core kernel)
     if (g.cout % 64 && (((uintptr_t)dz & 15u) || !scratch || scratch_bytes < small_conv_scratch_bytes(g)))
-        return simt_conv_wgrad(CKPT_DTYPE_BF16, g, dz, x, dw, scratch, scratch_bytes, stream);
+        return simt_conv_wgrad(CKPT_DTYPE_BF16, g, dz, x, dw, scratch, scratch_bytes, stream, upd);
     if (!scratch || scratch_bytes < small_conv_scratch_bytes(g)) { set_error("first-layer wgrad scratch too small"); return CKPT_E_WORKSPACE; }
     cudaStream_t st = (cudaStream_t)stream;
     char* base = (char*)scratch;
@@ -186,8 +191,8 @@ int small_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw
     const ConvGeom u = unfolded_geom(g);
     int rc = tc_conv_wgrad(u, dz, xcol, dwp, tc_scratch, scratch_bytes - xcol_bytes(g) - dwp_bytes(g), device_status, stream);
     if (rc) return rc;
-    if (paired(g)) take_paired_columns_kernel<<<(g.cout * 27 + 255) / 256, 256, 0, st>>>(dwp, dw, g.cout, 27);
-    else take_columns_kernel<<<(g.cout * 27 + 255) / 256, 256, 0, st>>>(dwp, dw, g.cout, 27);
+    if (paired(g)) take_paired_columns_kernel<<<(g.cout * 27 + 255) / 256, 256, 0, st>>>(dwp, dw, g.cout, 27, upd);
+    else take_columns_kernel<<<(g.cout * 27 + 255) / 256, 256, 0, st>>>(dwp, dw, g.cout, 27, upd);
     CKPT_LAUNCH_CHECK("first-layer wgrad column pick");
     return CKPT_OK;
 }

@@ -1515,7 +1515,7 @@ struct WgradParams {
 
 __global__ void __launch_bounds__(kThreads, 1)
 tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
-                     const __grid_constant__ CUtensorMap map_out, float* __restrict__ partial, WgradParams p, int* status) {
+                     const __grid_constant__ CUtensorMap map_out, float* __restrict__ partial, WgradParams p, SgdUpdate upd, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     // One copy brings px pixels x 64 channels (px = 64, 128 or 256: as many as leave two stages in shared memory, so
@@ -1628,8 +1628,30 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
                 const int tap = (blk_begin + j) / cin_blocks, ch0 = (blk_begin + j) % cin_blocks * 64;
                 for (int c0 = 0; c0 < 64; c0 += 32, ++count) {
                     if (ch0 + c0 >= p.c_in) break;
+                    // a gradient that is complete here updates its filter at once: 64 bytes of a row per lane (the update in a
+                    // pass of its own reads the gradient again: 64 us more for a 25088 x 4096 matrix)
+                    __nv_bfloat16* const w_row = upd.w && valid ? (__nv_bfloat16*)upd.w + (size_t)co * row_elems + (size_t)tap * p.c_in + ch0 + c0 : nullptr;
+                    uint4 w_old[4];
+                    if (w_row) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (ch0 + c0 + 8 * q < p.c_in) w_old[q] = reinterpret_cast<const uint4*>(w_row)[q];
+                    }
                     uint32_t v[32];
                     tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(j * 64 + c0), v);
+                    if (w_row) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            if (ch0 + c0 + 8 * q >= p.c_in) break;
+                            __nv_bfloat162* const pr = reinterpret_cast<__nv_bfloat162*>(&w_old[q]);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float2 o = __bfloat1622float2(pr[e]);
+                                pr[e] = __floats2bfloat162_rn(fmaf(-upd.lr, __uint_as_float(v[8 * q + 2 * e]), o.x), fmaf(-upd.lr, __uint_as_float(v[8 * q + 2 * e + 1]), o.y));
+                            }
+                            reinterpret_cast<uint4*>(w_row)[q] = w_old[q];
+                        }
+                    }
                     if (!p.tile_store) {
                         if (valid) {
 #pragma unroll
@@ -2868,19 +2890,25 @@ __global__ void slice_sum_tc_kernel(const float* __restrict__ partial, float* __
 }
 
 // sum of the `slices` partial results of a split wgrad into the caller's gradient
-static void launch_slice_sum(const float* partial, float* out, int64_t elems, int slices, cudaStream_t st,
-                             const SgdUpdate& upd = SgdUpdate()) {
+}  // namespace
+
+int slice_sum(const float* partial, float* out, int64_t elems, int slices, void* stream, const SgdUpdate& upd) {
+    cudaStream_t st = (cudaStream_t)stream;
     if (elems % 4 || ((uintptr_t)partial | (uintptr_t)out) % 16 || (upd.w && (uintptr_t)upd.w % 16)) {
         slice_sum_tc_kernel<<<(unsigned)((elems + 255) / 256), 256, 0, st>>>(partial, out, elems, slices);
-        if (upd.w) sgd_update(upd, out, elems, st);
-        return;
+        CKPT_LAUNCH_CHECK_NAMED("slice_sum_kernel", "wgrad slice sum");
+        return sgd_update(upd, out, elems, st);
     }
     const int64_t elems4 = elems / 4;
     const unsigned blocks = (unsigned)((elems4 + 31) / 32);
     if (slices >= 16) slice_sum4_kernel<32, 8><<<blocks, dim3(32, 8), 0, st>>>((const float4*)partial, (float4*)out, elems4, slices, upd);
     else if (slices >= 4) slice_sum4_kernel<32, 4><<<blocks, dim3(32, 4), 0, st>>>((const float4*)partial, (float4*)out, elems4, slices, upd);
     else slice_sum4_kernel<256, 1><<<(unsigned)((elems4 + 255) / 256), dim3(256, 1), 0, st>>>((const float4*)partial, (float4*)out, elems4, slices, upd);
+    CKPT_LAUNCH_CHECK_NAMED("slice_sum_kernel", "wgrad slice sum");
+    return CKPT_OK;
 }
+
+namespace {
 
 // ------------------------------------------------------------------------------------------------
 // Host side
@@ -3740,9 +3768,7 @@ int stem_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw,
     if (!simt && (!scratch || scratch_bytes < stem_conv_scratch_bytes(g))) { set_error("stem wgrad scratch too small"); return CKPT_E_WORKSPACE; }
     cudaStream_t st = (cudaStream_t)stream;
     if (simt) {
-        int rc = simt_conv_wgrad(CKPT_DTYPE_BF16, g, dz, x, dw, scratch, scratch_bytes, stream);
-        if (rc == CKPT_OK && upd.w) rc = sgd_update(upd, dw, (int64_t)g.cout * 147, stream);
-        return rc;
+        return simt_conv_wgrad(CKPT_DTYPE_BF16, g, dz, x, dw, scratch, scratch_bytes, stream, upd);
     }
     StemParams p = stem_params(g);
     p.slices = stem_wgrad_slices(g);
@@ -3758,9 +3784,7 @@ int stem_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw,
     dim3 grid((unsigned)p.slices, (unsigned)((g.cout + 63) / 64));
     tc_wgrad_stem_kernel<<<grid, kStemWgradThreads, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_stem_kernel", "stem conv wgrad (tensor cores)");
-    launch_slice_sum((const float*)scratch, dw, (int64_t)g.cout * 147, p.slices, st, upd);
-    CKPT_LAUNCH_CHECK("stem wgrad slice sum");
-    return CKPT_OK;
+    return slice_sum((const float*)scratch, dw, (int64_t)g.cout * 147, p.slices, st, upd);
 }
 
 static TParams strided_terms() {
@@ -3982,9 +4006,7 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         dim3 grid(p.slices, g.cout / 64);
         tc_wgrad_c64_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_c64_kernel", "conv wgrad, 64 input channels (tensor cores)");
-        launch_slice_sum((const float*)scratch, dw, elems, p.slices, st, upd);
-        CKPT_LAUNCH_CHECK_NAMED("slice_sum_kernel", "wgrad slice sum");
-        return CKPT_OK;
+        return slice_sum((const float*)scratch, dw, elems, p.slices, st, upd);
     }
     if (wgrad_rows_applies(g)) {
         WRowsParams p;
@@ -4006,9 +4028,7 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         if ((rc = make_partial_map(&mo, (float*)scratch, g.cin, 9, g.cout, p.slices))) return rc;
         tc_wgrad_rows_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_rows_kernel", "conv wgrad, shared vertical taps (tensor cores)");
-        launch_slice_sum((const float*)scratch, dw, elems, p.slices, st, upd);
-        CKPT_LAUNCH_CHECK_NAMED("slice_sum_kernel", "wgrad slice sum");
-        return CKPT_OK;
+        return slice_sum((const float*)scratch, dw, elems, p.slices, st, upd);
     }
     WgradParams p;
     int slices, groups, co_tiles;
@@ -4034,14 +4054,11 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
     p.tile_store = (uintptr_t)target % 16 == 0 && g.cin % 4 == 0;
     if (p.tile_store && (rc = make_partial_map(&mo, target, g.cin, g.k * g.k, g.cout, slices))) return rc;
     dim3 grid(slices, groups, co_tiles);
-    tc_conv_wgrad_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, target, p, device_status);
+    const bool update = slices == 1 && upd.w && upd.dtype == CKPT_DTYPE_BF16 && (uintptr_t)upd.w % 16 == 0;
+    tc_conv_wgrad_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, target, p, update ? upd : SgdUpdate(), device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_wgrad_kernel", "conv wgrad (tensor cores)");
-    if (slices > 1) {
-        launch_slice_sum((const float*)scratch, dw, elems, slices, st, upd);
-        CKPT_LAUNCH_CHECK_NAMED("slice_sum_kernel", "wgrad slice sum");
-    } else if (upd.w) {
-        return sgd_update(upd, dw, elems, st);       // the gradient went straight to the caller's buffer
-    }
+    if (slices > 1) return slice_sum((const float*)scratch, dw, elems, slices, st, upd);
+    if (upd.w && !update) return sgd_update(upd, dw, elems, st);
     return CKPT_OK;
 }
 

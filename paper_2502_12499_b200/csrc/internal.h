@@ -75,6 +75,8 @@ struct SgdUpdate {
     int dtype = CKPT_DTYPE_F32;
 };
 int sgd_update(const SgdUpdate& u, const float* g, int64_t elems, void* stream);
+// Sum of the `slices` partial results of a split weight gradient into the caller's gradient, with the update.
+int slice_sum(const float* partial, float* out, int64_t elems, int slices, void* stream, const SgdUpdate& upd = SgdUpdate());
 
 // ------------------------------------------------------------------ kernel launchers (kernels_simt.cu)
 struct ConvGeom {
@@ -88,14 +90,14 @@ int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, vo
 int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w, void* dx, void* stream);
 int64_t simt_wgrad_scratch_bytes(const ConvGeom& g);
 int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw,
-                    void* scratch, int64_t scratch_bytes, void* stream);
+                    void* scratch, int64_t scratch_bytes, void* stream, const SgdUpdate& upd = SgdUpdate());
 
 // First layer (3 input channels, 3x3, stride 1, padding 1, bf16): CUDA-core kernels of their own.
 bool small_conv_supported(int dtype, const ConvGeom& g);
 int64_t small_conv_scratch_bytes(const ConvGeom& g);
 int small_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, void* stream);
 int small_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch,
-                     int64_t scratch_bytes, int* device_status, void* stream);
+                     int64_t scratch_bytes, int* device_status, void* stream, const SgdUpdate& upd = SgdUpdate());
 
 // 7x7 stride-2 padding-3 stem on 3 input channels (bf16): operand tiles gathered by threads from staged input rows,
 // forward with the batch-norm partial sums of its output (partial / blocks as for the first layer), weight gradient
@@ -194,8 +196,8 @@ int avgpool_backward(int dtype, int n, int h, int w, int c, const void* dy, void
 int relu_mask_inplace(int dtype, int64_t elems, void* g, const void* y, void* stream);
 int relu_forward(int dtype, int64_t elems, const void* x, void* y, void* stream);
 int relu_backward(int dtype, int64_t elems, const void* dy, const void* y, void* dx, void* stream);
-// out[c] (f32) = sum over rows of g[row][c], rows summed in index order.
-int column_sums(int dtype, int64_t rows, int c, const void* g, float* out, void* stream);
+// out[c] (f32) = sum over rows of g[row][c], in a fixed order.
+int column_sums(int dtype, int64_t rows, int c, const void* g, float* out, void* stream, const SgdUpdate& upd = SgdUpdate());
 int softmax_ce(int dtype, int batch, int classes, const void* logits, const int32_t* labels,
                float* loss, void* dlogits, float* row_scratch, void* stream);
 // loss (device double) = sum of all elements; grad filled with ones.

@@ -71,18 +71,9 @@ Plan plan(int mode, int M, int N, int K, bool vectors) {
 static bool whole_chunks(int dtype, int channels, const void* p) { return channels % (dtype == CKPT_DTYPE_BF16 ? 8 : 4) == 0 && (uintptr_t)p % 16 == 0; }
 
 static int simt_conv(int mode, int dtype, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N,
-                     int K, bool va, bool vb, const simt::Plan& p, cudaStream_t st) {
-    return dtype == CKPT_DTYPE_BF16 ? simt::launch<__nv_bfloat16>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, st)
-                                    : simt::launch<float>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, st);
-}
-
-// out[e] = sum over slices (in slice order) of partial[slice][e]
-__global__ void slice_sum_kernel(const float* __restrict__ partial, float* __restrict__ out, int64_t elems, int slices) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= elems) return;
-    float s = 0.f;
-    for (int z = 0; z < slices; ++z) s += partial[(size_t)z * elems + e];
-    out[e] = s;
+                     int K, bool va, bool vb, const simt::Plan& p, cudaStream_t st, const SgdUpdate& upd = SgdUpdate()) {
+    return dtype == CKPT_DTYPE_BF16 ? simt::launch<__nv_bfloat16>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, upd, st)
+                                    : simt::launch<float>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, upd, st);
 }
 
 int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, void* stream) {
@@ -104,19 +95,17 @@ int64_t simt_wgrad_scratch_bytes(const ConvGeom& g) {
     const int slices = std::max(simt::plan(2, M, N, K, true).slices, simt::plan(2, M, N, K, false).slices);
     return slices <= 1 ? 0 : (int64_t)slices * M * N * (int64_t)sizeof(float);
 }
-int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes, void* stream) {
+int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes, void* stream,
+                    const SgdUpdate& upd) {
     const int M = g.cout, N = g.k * g.k * g.cin, K = g.n * g.ho * g.wo;
     const bool va = whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, x);
     const simt::Plan p = simt::plan(2, M, N, K, va && vb);
     const int64_t elems = (int64_t)M * N;
     if (p.slices > 1 && (!scratch || scratch_bytes < p.slices * elems * 4)) { set_error("wgrad scratch too small"); return CKPT_E_WORKSPACE; }
-    int rc = simt_conv(2, dtype, g, dz, x, p.slices > 1 ? scratch : dw, nullptr, 0, M, N, K, va, vb, p, (cudaStream_t)stream);
-    if (rc) return rc;
-    if (p.slices > 1) {
-        slice_sum_kernel<<<(unsigned)((elems + 255) / 256), 256, 0, (cudaStream_t)stream>>>((const float*)scratch, dw, elems, p.slices);
-        CKPT_LAUNCH_CHECK("wgrad slice sum");
-    }
-    return CKPT_OK;
+    int rc = simt_conv(2, dtype, g, dz, x, p.slices > 1 ? scratch : dw, nullptr, 0, M, N, K, va, vb, p, (cudaStream_t)stream,
+                       p.slices > 1 ? SgdUpdate() : upd);
+    if (rc || p.slices <= 1) return rc;
+    return slice_sum((const float*)scratch, dw, elems, p.slices, stream, upd);
 }
 
 // ================================================================================================
@@ -1435,17 +1424,26 @@ int relu_backward(int dtype, int64_t elems, const void* dy, const void* y, void*
     return CKPT_OK;
 }
 
+// A block sums 32 columns, eight threads each.
 template <typename T>
-__global__ void column_sum_kernel(const T* __restrict__ g, float* __restrict__ out, int64_t rows, int c) {
-    int ch = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ch >= c) return;
+__global__ void __launch_bounds__(256) column_sum_kernel(const T* __restrict__ g, float* __restrict__ out, int64_t rows, int c, SgdUpdate upd) {
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x % 32, part = threadIdx.x / 32, ch = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int64_t r = 0; r < rows; ++r) s += ld(g + r * c + ch);
+    if (ch < c) {
+#pragma unroll 4
+        for (int64_t r = part; r < rows; r += 8) s += ld(g + r * c + ch);
+    }
+    red[part][lane] = s;
+    __syncthreads();
+    if (part != 0 || ch >= c) return;
+    for (int q = 1; q < 8; ++q) s += red[q][lane];
     out[ch] = s;
+    if (upd.w) { float* w = (float*)upd.w + ch; *w = fmaf(-upd.lr, s, *w); }
 }
-int column_sums(int dtype, int64_t rows, int c, const void* g, float* out, void* stream) {
-    if (dtype == CKPT_DTYPE_BF16) column_sum_kernel<__nv_bfloat16><<<(c + 127) / 128, 128, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)g, out, rows, c);
-    else column_sum_kernel<float><<<(c + 127) / 128, 128, 0, (cudaStream_t)stream>>>((const float*)g, out, rows, c);
+int column_sums(int dtype, int64_t rows, int c, const void* g, float* out, void* stream, const SgdUpdate& upd) {
+    if (dtype == CKPT_DTYPE_BF16) column_sum_kernel<__nv_bfloat16><<<(c + 31) / 32, 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)g, out, rows, c, upd);
+    else column_sum_kernel<float><<<(c + 31) / 32, 256, 0, (cudaStream_t)stream>>>((const float*)g, out, rows, c, upd);
     CKPT_LAUNCH_CHECK("column sums");
     return CKPT_OK;
 }
