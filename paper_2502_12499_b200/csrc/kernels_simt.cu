@@ -50,10 +50,12 @@ Plan plan(int mode, int M, int N, int K, bool vectors) {
         const int bm = mode == 2 ? tile_n[t] : tile_m[t], bn = mode == 2 ? tile_m[t] : tile_n[t];
         const int64_t tiles = (int64_t)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
         for (int cluster = 1; cluster <= 8; cluster *= 2) {
-            for (int slices = 1; slices <= (mode == 2 ? 128 : 1); slices += slices < 16 ? 1 : slices / 8) {
+            // 1, 2, 3, 4, 6, 8, 12, ... slices: a finer search costs the host 17 us per layer and gains nothing
+            for (int slices = 1; slices <= (mode == 2 ? 128 : 1); slices = slices < 3 ? slices + 1 : (slices & (slices - 1)) ? slices / 3 * 4 : slices / 2 * 3) {
                 const int parts = cluster * slices;
                 const int per = ((K + parts - 1) / parts + 31) / 32 * 32;
-                if (parts > 1 && (per < 64 || (int64_t)per * (parts - 1) >= K)) continue;
+                if (parts > 1 && per < 64) break;
+                if (parts > 1 && (int64_t)per * (parts - 1) >= K) continue;
                 // CTAs per SM; one or two of 128 threads do not hide the latency of their shared-memory reads
                 const double load = std::ceil((double)(tiles * parts) / 148.0);
                 const double hidden = t == 0 ? (load < 2 ? 0.8 : 1.0) : (load < 2 ? 0.6 : load < 3 ? 0.8 : 1.0);
