@@ -993,9 +993,184 @@ __global__ void __launch_bounds__(256) maxpool2x2_bwd_sums_kernel(const T* __res
     }
 }
 
-bool maxpool_fuses_activation(int dtype, int h, int w, int c, int k, int stride, int pad) {
+static bool pool_2x2(int dtype, int h, int w, int c, int k, int stride, int pad) {
     const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
     return k == 2 && stride == 2 && pad == 0 && h % 2 == 0 && w % 2 == 0 && c % vec == 0;
+}
+// The residual networks' 3x3 pooling with stride 2 and padding 1 behind the stem.
+static bool pool_3x3(int dtype, int c, int k, int stride, int pad) {
+    return dtype == CKPT_DTYPE_BF16 && k == 3 && stride == 2 && pad == 1 && c % 8 == 0 && c <= 1024 && 256 % (c / 8) == 0;
+}
+bool maxpool_fuses_activation(int dtype, int h, int w, int c, int k, int stride, int pad) {
+    return pool_2x2(dtype, h, w, c, k, stride, pad) || pool_3x3(dtype, c, k, stride, pad);
+}
+
+// 3x3 pooling, stride 2, padding 1, of a pre-normalisation tensor: what is pooled is bf16(max(z*scale + shift, 0)), which
+// grows with z where the scale is positive and falls where it is negative, so the forward takes the maximum of z (its sign
+// flipped for negative scales) in packed pairs and normalises nine times less.  A thread owns eight channels of a window,
+// its nine loads in flight at once.
+__device__ __forceinline__ void pool3_load(const __nv_bfloat16* __restrict__ z, int64_t img, int oh, int ow, int h, int w, int c, int ch, uint4 (&r)[9], uint32_t& valid) {
+    valid = 0u;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+        const int ih = 2 * oh - 1 + t / 3, iw = 2 * ow - 1 + t % 3;
+        if (ih >= 0 && ih < h && iw >= 0 && iw < w) {
+            r[t] = *reinterpret_cast<const uint4*>(z + ((img * h + ih) * w + iw) * c + ch);
+            valid |= 1u << t;
+        }
+    }
+}
+__device__ __forceinline__ uint32_t& word(uint4& v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
+__global__ void __launch_bounds__(256) maxpool3_fwd_act_kernel(const __nv_bfloat16* __restrict__ z, __nv_bfloat16* __restrict__ y, int64_t items, int h, int w,
+                                                               int c, int ho, int wo, const float* __restrict__ act) {
+    const int lanes = c / 8;
+    const int ch = (int)(threadIdx.x % lanes) * 8;              // 256 and the grid stride are multiples of `lanes`
+    float sc[8], sh[8];
+    uint32_t flip[4];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { sc[k] = act[2 * c + ch + k]; sh[k] = act[3 * c + ch + k]; }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) flip[k] = (sc[2 * k] < 0.f ? 0x8000u : 0u) | (sc[2 * k + 1] < 0.f ? 0x80000000u : 0u);
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < items; i += (int64_t)gridDim.x * 256) {
+        const uint32_t t = (uint32_t)(i / lanes);
+        const int ow = (int)(t % (uint32_t)wo), oh = (int)(t / (uint32_t)wo % (uint32_t)ho);
+        const int64_t img = t / ((uint32_t)wo * (uint32_t)ho);
+        uint4 r[9];
+        uint32_t valid;
+        pool3_load(z, img, oh, ow, h, w, c, ch, r, valid);
+        uint4 best = make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);      // -infinity
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            if (!((valid >> q) & 1u)) continue;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t v = word(r[q], k) ^ flip[k];
+                const __nv_bfloat162 m = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&word(best, k)), *reinterpret_cast<const __nv_bfloat162*>(&v));
+                word(best, k) = *reinterpret_cast<const uint32_t*>(&m);
+            }
+        }
+        float o[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t v = word(best, k) ^ flip[k];
+            o[2 * k] = fmaxf(fmaf(__uint_as_float(v << 16), sc[2 * k], sh[2 * k]), 0.f);
+            o[2 * k + 1] = fmaxf(fmaf(__uint_as_float(v & 0xffff0000u), sc[2 * k + 1], sh[2 * k + 1]), 0.f);
+        }
+        store_vec<__nv_bfloat16, 8>(y + i * 8, o);
+    }
+}
+// Position (0..8) of the first maximum of the normalised values, one byte per channel.
+__global__ void __launch_bounds__(256) maxpool3_arg_act_kernel(const __nv_bfloat16* __restrict__ z, uint8_t* __restrict__ arg, int64_t items, int h, int w,
+                                                               int c, int ho, int wo, const float* __restrict__ act) {
+    const int lanes = c / 8;
+    const int ch = (int)(threadIdx.x % lanes) * 8;
+    float sc[8], sh[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { sc[k] = act[2 * c + ch + k]; sh[k] = act[3 * c + ch + k]; }
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < items; i += (int64_t)gridDim.x * 256) {
+        const uint32_t t = (uint32_t)(i / lanes);
+        const int ow = (int)(t % (uint32_t)wo), oh = (int)(t / (uint32_t)wo % (uint32_t)ho);
+        const int64_t img = t / ((uint32_t)wo * (uint32_t)ho);
+        uint4 r[9];
+        uint32_t valid;
+        pool3_load(z, img, oh, ow, h, w, c, ch, r, valid);
+        uint4 best = make_uint4(0xbf80bf80u, 0xbf80bf80u, 0xbf80bf80u, 0xbf80bf80u);      // -1: below every normalised value
+        uint4 pos = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            if (!((valid >> q) & 1u)) continue;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t v = word(r[q], k);
+                const __nv_bfloat162 a = __floats2bfloat162_rn(fmaxf(fmaf(__uint_as_float(v << 16), sc[2 * k], sh[2 * k]), 0.f),
+                                                               fmaxf(fmaf(__uint_as_float(v & 0xffff0000u), sc[2 * k + 1], sh[2 * k + 1]), 0.f));
+                const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&word(best, k));
+                const uint32_t more = __hgt2_mask(a, b);                                  // strict: the first maximum stays
+                word(pos, k) = (word(pos, k) & ~more) | ((uint32_t)(q * 0x10001) & more);
+                const __nv_bfloat162 m = __hmax2(a, b);
+                word(best, k) = *reinterpret_cast<const uint32_t*>(&m);
+            }
+        }
+        *reinterpret_cast<uint2*>(arg + i * 8) = make_uint2(__byte_perm(pos.x, pos.y, 0x6420), __byte_perm(pos.z, pos.w, 0x6420));
+    }
+}
+// Gradient of a 2 x 2 quad of inputs (rows 2a, 2a + 1; columns 2b, 2b + 1) from the recorded positions: an even row belongs
+// to window a only (its middle row), an odd one to windows a (last row) and a + 1 (first row).  With `act` the producer's
+// batch-norm backward sums (sum g, sum g*z over the values its ReLU passes) go to `partial` as in the 2x2 kernel.
+template <bool SUMS>
+__global__ void __launch_bounds__(256) maxpool3_bwd_kernel(const uint8_t* __restrict__ arg, const __nv_bfloat16* __restrict__ dy, __nv_bfloat16* __restrict__ dx,
+                                                           int64_t items, int h, int w, int c, int ho, int wo, const __nv_bfloat16* __restrict__ z,
+                                                           const float* __restrict__ act, float* __restrict__ partial) {
+    __shared__ float red[SUMS ? 256 : 1][17];
+    const int lanes = c / 8;
+    const int ch = (int)(threadIdx.x % lanes) * 8;
+    float sc[8], sh[8], s0[8], s1[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { sc[k] = SUMS ? act[2 * c + ch + k] : 0.f; sh[k] = SUMS ? act[3 * c + ch + k] : 0.f; s0[k] = 0.f; s1[k] = 0.f; }
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < items; i += (int64_t)gridDim.x * 256) {
+        const uint32_t t = (uint32_t)(i / lanes);
+        const int b = (int)(t % (uint32_t)wo), a = (int)(t / (uint32_t)wo % (uint32_t)ho);
+        const int64_t img = t / ((uint32_t)wo * (uint32_t)ho);
+        uint2 pos[4];
+        uint4 raw[4], zr[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {                            // windows (a + q/2, b + q%2)
+            const bool in = a + q / 2 < ho && b + q % 2 < wo;
+            const int64_t o = ((img * ho + a + q / 2) * wo + b + q % 2) * c + ch;
+            pos[q] = in ? *reinterpret_cast<const uint2*>(arg + o) : make_uint2(0xffffffffu, 0xffffffffu);
+            raw[q] = in ? *reinterpret_cast<const uint4*>(dy + o) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (SUMS && 2 * a + q / 2 < h && 2 * b + q % 2 < w)
+                zr[q] = *reinterpret_cast<const uint4*>(z + ((img * h + 2 * a + q / 2) * w + 2 * b + q % 2) * c + ch);
+        float g[4][8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) unpack<__nv_bfloat16, 8>(from_uint4<__nv_bfloat16, 8>(raw[q]), g[q]);
+        auto at = [&](int q, int k) { return (int)((k < 4 ? pos[q].x >> (8 * k) : pos[q].y >> (8 * (k - 4))) & 0xffu); };
+#pragma unroll
+        for (int in = 0; in < 4; ++in) {
+            if (2 * a + in / 2 >= h || 2 * b + in % 2 >= w) continue;
+            float o[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                o[k] = 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (q / 2 > in / 2 || q % 2 > in % 2) continue;                      // an even row or column has one window
+                    const int r = in / 2 ? (q / 2 ? 0 : 2) : 1, s = in % 2 ? (q % 2 ? 0 : 2) : 1;
+                    o[k] += at(q, k) == r * 3 + s ? g[q][k] : 0.f;
+                }
+            }
+            const uint4 packed = as_uint4(pack_raw<__nv_bfloat16, 8>(o));
+            *reinterpret_cast<uint4*>(dx + ((img * h + 2 * a + in / 2) * w + 2 * b + in % 2) * c + ch) = packed;
+            if (SUMS) {
+                float v[8], stored[8];
+                unpack<__nv_bfloat16, 8>(from_uint4<__nv_bfloat16, 8>(zr[in]), v);
+                unpack<__nv_bfloat16, 8>(from_uint4<__nv_bfloat16, 8>(packed), stored);
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (fmaf(v[k], sc[k], sh[k]) > 0x1p-134f) { s0[k] += stored[k]; s1[k] = fmaf(stored[k], v[k], s1[k]); }
+            }
+        }
+    }
+    if (!SUMS) return;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { red[threadIdx.x][k] = s0[k]; red[threadIdx.x][8 + k] = s1[k]; }
+    __syncthreads();
+    for (int off = 128; off >= lanes; off >>= 1) {               // `lanes` divides 256: threads t and t + off hold the same group
+        if ((int)threadIdx.x < off)
+#pragma unroll
+            for (int k = 0; k < 16; ++k) red[threadIdx.x][k] += red[threadIdx.x + off][k];
+        __syncthreads();
+    }
+    if ((int)threadIdx.x < lanes) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            partial[((size_t)blockIdx.x * 2 + 0) * c + ch + k] = red[threadIdx.x][k];
+            partial[((size_t)blockIdx.x * 2 + 1) * c + ch + k] = red[threadIdx.x][8 + k];
+        }
+    }
 }
 
 // Vector forms of the two general pooling kernels: one thread handles VEC consecutive channels of a
@@ -1147,16 +1322,17 @@ __global__ void __launch_bounds__(256) maxpool_bwd_arg_kernel(const uint8_t* __r
 }
 
 int64_t maxpool_backward_scratch_bytes(int dtype, int n, int h, int w, int c, int k, int stride, int pad) {
-    if (maxpool_fuses_activation(dtype, h, w, c, k, stride, pad) || k * k > 250) return 0;
+    if (pool_2x2(dtype, h, w, c, k, stride, pad) || k * k > 250) return 0;
     const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
     if (c % vec) return 0;
     const int ho = (h + 2 * pad - k) / stride + 1, wo = (w + 2 * pad - k) / stride + 1;
-    return (int64_t)n * ho * wo * c;
+    // (behind the positions, room for the batch-norm sums of the 3x3 kernel)
+    return align_up((int64_t)n * ho * wo * c, 256) + (pool_3x3(dtype, c, k, stride, pad) ? bn_scratch_bytes(0, c) : 0);
 }
 
 int maxpool_forward(int dtype, int n, int h, int w, int c, int k, int stride, int pad, const void* x, void* y, const float* act, void* stream) {
     int ho = (h + 2 * pad - k) / stride + 1, wo = (w + 2 * pad - k) / stride + 1;
-    if (maxpool_fuses_activation(dtype, h, w, c, k, stride, pad)) {
+    if (pool_2x2(dtype, h, w, c, k, stride, pad)) {
         const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
         const int64_t items = (int64_t)n * ho * wo * (c / vec);
         if (dtype == CKPT_DTYPE_BF16)
@@ -1164,6 +1340,12 @@ int maxpool_forward(int dtype, int n, int h, int w, int c, int k, int stride, in
         else
             maxpool2x2_fwd_kernel<float, 4><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const float*)x, (float*)y, items, wo, ho, c / vec, c, act);
         CKPT_LAUNCH_CHECK("max-pool 2x2 forward");
+        return CKPT_OK;
+    }
+    if (act && pool_3x3(dtype, c, k, stride, pad)) {
+        const int64_t items = (int64_t)n * ho * wo * (c / 8);
+        maxpool3_fwd_act_kernel<<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)y, items, h, w, c, ho, wo, act);
+        CKPT_LAUNCH_CHECK("max-pool 3x3 forward");
         return CKPT_OK;
     }
     if (act) { set_error("the general pooling kernel takes an activated input"); return CKPT_E_BAD_ARG; }
@@ -1189,7 +1371,7 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
                      float* bn_partial, int* bn_blocks, void* scratch, int64_t scratch_bytes) {
     int ho = (h + 2 * pad - k) / stride + 1, wo = (w + 2 * pad - k) / stride + 1;
     if (bn_blocks) *bn_blocks = 0;
-    if (maxpool_fuses_activation(dtype, h, w, c, k, stride, pad)) {
+    if (pool_2x2(dtype, h, w, c, k, stride, pad)) {
         const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
         const int64_t items = (int64_t)n * ho * wo * (c / vec);
         const int cv = c / vec;
@@ -1211,6 +1393,24 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
         CKPT_LAUNCH_CHECK("max-pool 2x2 backward");
         return CKPT_OK;
     }
+    if (act && pool_3x3(dtype, c, k, stride, pad)) {
+        // batch-norm sums first in the scratch region (the batch-norm backward reads them there), positions behind them
+        const int64_t sums = align_up(bn_scratch_bytes(0, c), 256), windows = (int64_t)n * ho * wo * (c / 8);
+        if (!scratch || scratch_bytes < sums + windows * 8 || (uintptr_t)scratch % 16) { set_error("pooling scratch too small"); return CKPT_E_WORKSPACE; }
+        uint8_t* const arg = (uint8_t*)scratch + sums;
+        cudaStream_t st = (cudaStream_t)stream;
+        maxpool3_arg_act_kernel<<<elementwise_grid(windows), 256, 0, st>>>((const __nv_bfloat16*)x, arg, windows, h, w, c, ho, wo, act);
+        CKPT_LAUNCH_CHECK("max-pool 3x3 arg-max");
+        const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((windows + 255) / 256, BN_MAX_BLOCKS));
+        if (bn_partial && bn_blocks) {
+            maxpool3_bwd_kernel<true><<<grid, 256, 0, st>>>(arg, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, (const __nv_bfloat16*)x, act, bn_partial);
+            *bn_blocks = (int)grid;
+        } else {
+            maxpool3_bwd_kernel<false><<<grid, 256, 0, st>>>(arg, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, nullptr, nullptr, nullptr);
+        }
+        CKPT_LAUNCH_CHECK("max-pool 3x3 backward");
+        return CKPT_OK;
+    }
     if (act) { set_error("the general pooling kernel takes an activated input"); return CKPT_E_BAD_ARG; }
     const int64_t arg_bytes = maxpool_backward_scratch_bytes(dtype, n, h, w, c, k, stride, pad);
     if (arg_bytes > 0 && scratch && scratch_bytes >= arg_bytes && ((uintptr_t)scratch & 7u) == 0) {
@@ -1220,7 +1420,8 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
         if (dtype == CKPT_DTYPE_BF16) {
             maxpool_argmax_kernel<__nv_bfloat16, 8><<<elementwise_grid(windows), 256, 0, st>>>((const __nv_bfloat16*)x, (uint8_t*)scratch, windows, h, w, c, ho, wo, k, stride, pad);
             CKPT_LAUNCH_CHECK("max-pool arg-max");
-            maxpool_bwd_arg_kernel<__nv_bfloat16, 8><<<elementwise_grid(pixels), 256, 0, st>>>((const uint8_t*)scratch, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, pixels, h, w, c, ho, wo, k, stride, pad);
+            if (pool_3x3(dtype, c, k, stride, pad)) maxpool3_bwd_kernel<false><<<elementwise_grid(windows), 256, 0, st>>>((const uint8_t*)scratch, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, nullptr, nullptr, nullptr);
+            else maxpool_bwd_arg_kernel<__nv_bfloat16, 8><<<elementwise_grid(pixels), 256, 0, st>>>((const uint8_t*)scratch, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, pixels, h, w, c, ho, wo, k, stride, pad);
         } else {
             maxpool_argmax_kernel<float, 4><<<elementwise_grid(windows), 256, 0, st>>>((const float*)x, (uint8_t*)scratch, windows, h, w, c, ho, wo, k, stride, pad);
             CKPT_LAUNCH_CHECK("max-pool arg-max");

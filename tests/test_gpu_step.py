@@ -454,3 +454,24 @@ def test_joined_gradients_equal_separate_ones(graph):
     runner.chain.set_gradient_tap(None)
     for a, b in zip(plain, tapped):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("hw,channels", [((9, 12), 16), ((22, 17), 64), ((5, 6), 24), ((40, 40), 64)])
+def test_pooling_reads_the_pending_normalisation(hw, channels):
+    """3x3 pooling behind a convolution + batch norm + ReLU: the pooled values, the routed gradient and the batch-norm
+    gradients equal those of the same layers as units of their own (which pool a stored, normalised tensor)."""
+    units = [wl.conv_unit(3, channels), {"kind": "maxpool", "k": 3, "stride": 2, "pad": 1}, {"kind": "avgpool"},
+             {"kind": "fc", "cin": channels, "cout": 7, "relu": False}]
+    spec = dict(units=units, input_hwc=(hw[0], hw[1], 3), batch=4, dtype="bf16", loss="softmax_ce", name="pool")
+    params = wl.make_params(spec, seed=3, bn_affine="random")
+    split, origin = wl.split_units(spec)
+    x, labels = wl.make_batch(spec, seed=4)
+    a = StepRunner(spec, params)
+    b = StepRunner(split, wl.split_params(origin, params))
+    rep_a, g_a = a.run(ck.POLICY_STORE_ALL, None, x, labels)
+    rep_b, g_b = b.run(ck.POLICY_STORE_ALL, None, x, labels)
+    # the same bf16 tensors; the batch-norm sums add the same terms in another order
+    assert abs(rep_a["loss"] - rep_b["loss"]) <= 1e-3 * abs(rep_b["loss"])
+    for u, v in zip(g_a, g_b):
+        assert u.shape == v.shape
+        assert np.linalg.norm(u - v) <= 2e-2 * np.linalg.norm(v) + 1e-6
