@@ -263,12 +263,15 @@ static BlockBuffers block_buffers(StepCtx& c, const Unit& u) {
     return B;
 }
 
-// z1, a, z2, b, z3 (and zp) with their statistics; the residual join is left to the caller.
+// z1, a, z2, b, z3 (and zp) with their statistics; the residual join is left to the caller, unless y is given.
 // have_stats: the block's four statistics blocks are those of this very input (they were written by the unit's last
-// forward, original or recomputed, and every unit has a block of its own), so the backward's re-derivation of the
-// interior tensors runs the convolutions without gathering sums and skips the finalize steps; the tensors come out
-// bit-identical (same kernels, same reduction order).
-static int block_interiors(StepCtx& c, const Unit& u, const void* x, const BlockBuffers& B, bool have_stats = false) {
+// forward, original or recomputed, and every unit has a block of its own), so the convolutions gather no sums, no finalize
+// step runs, and their epilogues write the activated tensors (bit-identical to those of the stand-alone pass); the tensors
+// come out as before (same products, and sums in the same order).
+// y (with have_stats): the block's output is all that is wanted; z1, z2 and z3 are not stored where the epilogues can do
+// without, and *joined says whether y has been written.
+static int block_interiors(StepCtx& c, const Unit& u, const void* x, const BlockBuffers& B, bool have_stats = false, void* y = nullptr,
+                           bool* joined = nullptr) {
     const int dt = c.ch->dtype;
     void* const* p = c.params + u.param_first;
     const int64_t in_px = c.ch->batch * u.in.h * u.in.w, out_px = c.ch->batch * u.out.h * u.out.w;
@@ -278,21 +281,33 @@ static int block_interiors(StepCtx& c, const Unit& u, const void* x, const Block
         if (have_stats) return conv_forward_any(c, g, in, p[w_index], z, nullptr, 0);
         return conv_with_statistics(c, g, in, p[w_index], z, (const float*)p[w_index + 1], (const float*)p[w_index + 2], stats);
     };
-    if ((rc = conv(u.g1, x, 0, B.z1, B.s1))) return rc;
-    if ((rc = bn_apply(dt, in_px, mid, B.z1, B.s1, 1, B.a, c.stream))) return rc;
-    if ((rc = conv(u.g2, B.a, 3, B.z2, B.s2))) return rc;
-    if ((rc = bn_apply(dt, out_px, mid, B.z2, B.s2, 1, B.b, c.stream))) return rc;
-    if ((rc = conv(u.g3, B.b, 6, B.z3, B.s3))) return rc;
-    if (u.desc.flags & 2) {
-        if ((rc = conv(u.gp, x, 9, B.zp, B.sp))) return rc;
+    auto conv_act = [&](const ConvGeom& g, const void* in, int w_index, void* z, float* stats, int64_t rows, void* act) {
+        if (have_stats && use_tc(c.ch, g, in, p[w_index], z) && tc_fwd_takes_known_stats(g, false)) {
+            KnownStats known;
+            known.stats = stats; known.act = act;
+            return tc_conv_fwd_known_stats(g, in, p[w_index], y ? nullptr : z, known, c.status(), c.stream);
+        }
+        int e = conv(g, in, w_index, z, stats);
+        return e ? e : bn_apply(dt, rows, mid, z, stats, 1, act, c.stream);
+    };
+    if ((rc = conv_act(u.g1, x, 0, B.z1, B.s1, in_px, B.a))) return rc;
+    if ((rc = conv_act(u.g2, B.a, 3, B.z2, B.s2, out_px, B.b))) return rc;
+    const bool project = (u.desc.flags & 2) != 0;
+    if (project && (rc = conv(u.gp, x, 9, B.zp, B.sp))) return rc;
+    if (y && use_tc(c.ch, u.g3, B.b, p[6], y) && tc_fwd_takes_known_stats(u.g3, true)) {
+        KnownStats known;
+        known.stats = B.s3; known.shortcut = project ? B.zp : x; known.shortcut_stats = project ? B.sp : nullptr;
+        *joined = true;
+        return tc_conv_fwd_known_stats(u.g3, B.b, p[6], y, known, c.status(), c.stream);
     }
-    return CKPT_OK;
+    return conv(u.g3, B.b, 6, B.z3, B.s3);
 }
 
 static int block_forward(StepCtx& c, const Unit& u, const void* x, void* y, bool have_stats = false) {
     const BlockBuffers B = block_buffers(c, u);
-    int rc = block_interiors(c, u, x, B, have_stats);
-    if (rc) return rc;
+    bool joined = false;
+    int rc = block_interiors(c, u, x, B, have_stats, have_stats ? y : nullptr, &joined);
+    if (rc || joined) return rc;
     const bool project = (u.desc.flags & 2) != 0;
     return bn_add_relu(c.ch->dtype, c.ch->batch * u.out.h * u.out.w, u.out.c, B.z3, B.s3, project ? (const void*)B.zp : x,
                        project ? B.sp : nullptr, y, c.stream);

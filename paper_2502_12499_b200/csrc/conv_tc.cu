@@ -556,6 +556,11 @@ struct TParams {
     int split;                   // CTAs of a cluster that share the reduction of a tile
     // gradient join (1x1 input gradients, pixels as one row): what is stored is (sum + join_add) where join_mask > 0
     const __nv_bfloat16 *join_add, *join_mask;    // join_mask may be null
+    // known batch statistics (segment recomputation): scale and shift at 2c and 3c of a block of 4c floats, c = act_channels
+    // (an output channel's are at channel % c).  The activated form goes out beside the convolution's (act_raw) or alone,
+    // or the residual join of the block: max(z*scale + shift + shortcut, 0), the shortcut with statistics of its own or none.
+    const float *act_stats, *shortcut_stats;
+    int act_raw, act_channels;
     uint32_t patch_bytes;        // 8 x (th + 2) pixels x 128 bytes; stacked: 8 x th x stack
     // stacked form for small images (tc_conv_tp_kernel): a tile is the strip of `stack` whole images, each taking th
     // rows of the accumulator (its H rows and th - H idle ones) and th rows of the patch (rows -1 .. th - 2: the image,
@@ -593,6 +598,39 @@ __device__ __forceinline__ void load_filter_boxes(const TParams& p, const CUtens
     }
 }
 
+// Activated form of a chunk: the lane's channel rounded to bf16 as the stored convolution, normalised, clamped, rounded.
+__device__ __forceinline__ void act_chunk_to_slab(const uint32_t (&v)[32], uint32_t slab_lane, float scale, float shift) {
+#pragma unroll
+    for (int e = 0; e < 32; e += 2) {
+        const __nv_bfloat162 z = __floats2bfloat162_rn(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+        const uint32_t bits = *reinterpret_cast<const uint32_t*>(&z);
+        const __nv_bfloat162 r = __floats2bfloat162_rn(fmaxf(fmaf(__uint_as_float(bits << 16), scale, shift), 0.f),
+                                                       fmaxf(fmaf(__uint_as_float(bits & 0xffff0000u), scale, shift), 0.f));
+        asm volatile("st.shared.b16 [%0], %1;" ::"r"(slab_lane + (uint32_t)(e * 64)), "h"(__bfloat16_as_ushort(r.x)) : "memory");
+        asm volatile("st.shared.b16 [%0], %1;" ::"r"(slab_lane + (uint32_t)((e + 1) * 64)), "h"(__bfloat16_as_ushort(r.y)) : "memory");
+    }
+}
+struct ActCoef { float scale, shift, scale2, shift2; };
+__device__ __forceinline__ ActCoef act_coef(const TParams& p, int co) {
+    const int c = p.act_channels, ch = min(co, p.c_out - 1) % c;
+    ActCoef a = {p.act_stats[2 * c + ch], p.act_stats[3 * c + ch], 1.f, 0.f};
+    if (p.shortcut_stats) { a.scale2 = p.shortcut_stats[2 * c + ch]; a.shift2 = p.shortcut_stats[3 * c + ch]; }
+    return a;
+}
+__device__ __forceinline__ float residual(const TParams& p, const ActCoef& a, float acc, uint16_t shortcut) {
+    const float z = __bfloat162float(__float2bfloat16_rn(acc)), s = __uint_as_float((uint32_t)shortcut << 16);
+    return fmaxf(fmaf(z, a.scale, a.shift) + (p.shortcut_stats ? fmaf(s, a.scale2, a.shift2) : s), 0.f);
+}
+// The residual join by plain loads.
+__device__ __forceinline__ void residual_chunk(const TParams& p, size_t pixel, int co, uint32_t in_mask, uint32_t (&v)[32]) {
+    const uint16_t* const add = reinterpret_cast<const uint16_t*>(p.join_add) + pixel * p.c_out + co;
+    const ActCoef a = act_coef(p, co);
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+        if (!((in_mask >> e) & 1u) || co >= p.c_out) continue;
+        v[e] = __float_as_uint(residual(p, a, __uint_as_float(v[e]), __ldg(add + (size_t)e * p.c_out)));
+    }
+}
 // The join by plain loads: channel `co` of 32 consecutive pixels from `pixel` on.
 __device__ __forceinline__ void join_chunk(const TParams& p, size_t pixel, int co, uint32_t in_mask, uint32_t (&v)[32]) {
     const size_t at = pixel * p.c_out + co;
@@ -617,11 +655,16 @@ __device__ __forceinline__ void join_chunk(const TParams& p, size_t pixel, int c
 // again.  Every epilogue warp has four slots; the chunk's values of both tensors arrive in one by tile loads two chunks ahead
 // of their turn, and the result leaves from the slot.  (Values loaded by the lanes, 64 bytes per instruction,
 // made 256 -> 1024 at 14 x 14, 128 images 70 us; 35 with the slots, HBM takes 27.)
-template <bool A_MN, bool SPLIT, bool JOIN>
+//
+// EPI_ACT, EPI_RESIDUAL: the batch statistics of the output are known (see TParams): normalisation and ReLU, or the whole
+// residual join, in the epilogue instead of a pass that reads the tensor again.
+enum { EPI_PLAIN = 0, EPI_JOIN = 1, EPI_ACT = 2, EPI_RESIDUAL = 3 };
+template <bool A_MN, bool SPLIT, int EPI>
 __global__ void __launch_bounds__(kThreadsT, 1)
 tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_add,
                  const __grid_constant__ CUtensorMap map_mask, float* __restrict__ stat_partial, TParams p, int* status) {
+    constexpr bool LOADS = EPI == EPI_JOIN || EPI == EPI_RESIDUAL;         // the epilogue reads tensors of its own
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     constexpr uint32_t a_bytes = 128 * 128;
@@ -657,7 +700,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         failed_flag = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full0 + 8 * b, 1); mbar_init(acc_empty0 + 8 * b, 128 * kTEpi); }
-        if (JOIN) for (int s = 0; s < 4 * kTEpi * kJoinSlots; ++s) mbar_init(bars + 256u + 8u * s, 1);
+        if (LOADS) for (int s = 0; s < 4 * kTEpi * kJoinSlots; ++s) mbar_init(bars + 256u + 8u * s, 1);
         fence_barrier_init();
         tma_prefetch_desc(&map_x);
         tma_prefetch_desc(&map_w);
@@ -748,10 +791,11 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             }
             tc_fence_before();
         }
-    } else if (JOIN && warp >= 2) {
+    } else if (LOADS && warp >= 2) {
         // ---------------- epilogue with a gradient join (pixels as one row, see above)
         const int quarter = warp % 4, half = (warp - 2) / 4, ch = co_tile * 128 + quarter * 32;
-        const bool mine = ch < p.c_out, masked = p.join_mask != nullptr;
+        const bool mine = ch < p.c_out, masked = EPI == EPI_JOIN && p.join_mask != nullptr;
+        const ActCoef coef = EPI == EPI_RESIDUAL ? act_coef(p, ch + lane) : ActCoef();
         const int per_tile = (p.tile_cols / 32 - half + kTEpi - 1) / kTEpi, total = mine ? my_tiles * per_tile : 0;
         const uint32_t slots = out_stage + (uint32_t)((warp - 2) * kJoinSlots) * 4096u, slot_bars = bars + 256u + (uint32_t)((warp - 2) * kJoinSlots) * 8u;
         auto column = [&](int n) { return (first + n / per_tile * p.ctas_per_co) * p.tile_cols + (half + n % per_tile * kTEpi) * 32; };
@@ -790,8 +834,14 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         }
 #pragma unroll
                         for (int e = 0; e < 16; e += 2) {
-                            float f0 = __uint_as_float(v[h + e]) + __uint_as_float((uint32_t)add[e] << 16);
-                            float f1 = __uint_as_float(v[h + e + 1]) + __uint_as_float((uint32_t)add[e + 1] << 16);
+                            float f0, f1;
+                            if (EPI == EPI_RESIDUAL) {
+                                f0 = residual(p, coef, __uint_as_float(v[h + e]), add[e]);
+                                f1 = residual(p, coef, __uint_as_float(v[h + e + 1]), add[e + 1]);
+                            } else {
+                                f0 = __uint_as_float(v[h + e]) + __uint_as_float((uint32_t)add[e] << 16);
+                                f1 = __uint_as_float(v[h + e + 1]) + __uint_as_float((uint32_t)add[e + 1] << 16);
+                            }
                             if (masked) {
                                 f0 = __uint_as_float((uint32_t)mask[e] << 16) > 0.f ? f0 : 0.f;
                                 f1 = __uint_as_float((uint32_t)mask[e + 1] << 16) > 0.f ? f1 : 0.f;
@@ -831,6 +881,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         const bool stats = stat_partial != nullptr;
         float sum[4] = {0.f, 0.f, 0.f, 0.f}, sumsq[4] = {0.f, 0.f, 0.f, 0.f};
         int chunk_count = 0;
+        const ActCoef coef = EPI == EPI_ACT ? act_coef(p, co) : ActCoef();
         for (int j = 0; j < my_tiles; ++j) {
             const int buf = j & 1;
             if (!mbar_wait(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 903)) break;
@@ -847,16 +898,20 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 if (in_mask == 0u || co_tile * 128 + quarter * 32 >= p.c_out) continue;       // nothing of it inside the tensor
                 uint32_t v[32];
                 tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + c0), v);
-                const uint32_t slab = out_stage + (uint32_t)(((warp - 2) * kTSlabs + (chunk_count++ % kTSlabs)) * 2048);
-                if (lane == 0) tma_store_wait_read<kTSlabs - 1>();    // the store that last read this slab has left it
+                // (EPI_ACT: two slabs per chunk, the stored form and the activated one)
+                constexpr int kPer = EPI == EPI_ACT ? 2 : 1;
+                const uint32_t slab = out_stage + (uint32_t)(((warp - 2) * kTSlabs + (chunk_count++ % kTSlabs)) * kPer * 2048);
+                if (lane == 0) tma_store_wait_read<kTSlabs - 1>();    // the stores that last read this slab have left it
                 __syncwarp();
-                t_chunk_to_slab<true>(v, in_mask, slab + (uint32_t)(lane * 2), stats, sum, sumsq);
+                if (EPI != EPI_ACT || p.act_raw) t_chunk_to_slab<true>(v, in_mask, slab + (uint32_t)(lane * 2), stats, sum, sumsq);
+                if constexpr (EPI == EPI_ACT) act_chunk_to_slab(v, slab + 2048u + (uint32_t)(lane * 2), coef.scale, coef.shift);
                 fence_proxy_async();
                 __syncwarp();
                 // (one branch for store and commit: a commit in a branch of its own made 64 -> 256 at 56 x 56 15 % slower)
                 if (lane == 0) {
                     const int cw = c0 & ((1 << p.tw_log) - 1), chh = (c0 >> p.tw_log) & (p.th - 1), cn = c0 >> (p.tw_log + p.th_log);
-                    tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
+                    if (EPI != EPI_ACT || p.act_raw) tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
+                    if (EPI == EPI_ACT) tma_store_4d(&map_add, slab + 2048u, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
                     tma_store_commit();
                 }
             }
@@ -912,17 +967,23 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 uint32_t v[32];
 #pragma unroll
                 for (int e = 0; e < 32; ++e) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v[e]) : "r"(block + (uint32_t)(e * 512 + lane * 4)) : "memory");
-                if constexpr (JOIN) join_chunk(p, (size_t)w0 + c0, co, in_mask, v);
+                if constexpr (EPI == EPI_JOIN) join_chunk(p, (size_t)w0 + c0, co, in_mask, v);
+                if constexpr (EPI == EPI_RESIDUAL) residual_chunk(p, (size_t)w0 + c0, co, in_mask, v);
                 float sum[4] = {0.f, 0.f, 0.f, 0.f}, sumsq[4] = {0.f, 0.f, 0.f, 0.f};
                 const uint32_t slab = out_stage + (uint32_t)((warp - 2) * kTSlabs * 2048);
                 if (lane == 0) tma_store_wait_read<0>();
                 __syncwarp();
-                t_chunk_to_slab<true>(v, in_mask, slab + (uint32_t)(lane * 2), stat_partial != nullptr, sum, sumsq);
+                if (EPI != EPI_ACT || p.act_raw) t_chunk_to_slab<true>(v, in_mask, slab + (uint32_t)(lane * 2), stat_partial != nullptr, sum, sumsq);
+                if constexpr (EPI == EPI_ACT) {
+                    const ActCoef a = act_coef(p, co);
+                    act_chunk_to_slab(v, slab + 2048u + (uint32_t)(lane * 2), a.scale, a.shift);
+                }
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0 && in_mask != 0u && co_tile * 128 + quarter * 32 < p.c_out) {
                     const int cw = c0 & ((1 << p.tw_log) - 1), chh = (c0 >> p.tw_log) & (p.th - 1), cn = c0 >> (p.tw_log + p.th_log);
-                    tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
+                    if (EPI != EPI_ACT || p.act_raw) tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
+                    if (EPI == EPI_ACT) tma_store_4d(&map_add, slab + 2048u, co_tile * 128 + quarter * 32, w0 + cw, h0 + chh, n0 + cn);
                     tma_store_commit();
                 }
                 if (stat_partial && co < p.c_out) {
@@ -967,10 +1028,12 @@ constexpr int kTpEpi = 2;                          // epilogue warps per quarter
 constexpr int kTpThreads = 64 + 128 * kTpEpi;
 constexpr uint32_t kTpSmem = kTpBoxes * 16384 + kTpPatches * kTpPatchSlot + 256 + 4 * kTpEpi * 2048 + 1024;
 
-template <bool A_MN>
+// ACT: as EPI_ACT of the plain kernel; the chunk's two forms leave from one slab in turn.
+template <bool A_MN, bool ACT>
 __global__ void __launch_bounds__(kTpThreads, 1)
 tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                  const __grid_constant__ CUtensorMap map_out, float* __restrict__ stat_partial, TParams p, int* status) {
+                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_act, float* __restrict__ stat_partial, TParams p,
+                  int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     constexpr uint32_t a_bytes = 128 * 128;
@@ -1086,6 +1149,7 @@ tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         const int co = co_tile * 128 + quarter * 32 + lane;
         const bool stats = stat_partial != nullptr;
         float sum[4] = {0.f, 0.f, 0.f, 0.f}, sumsq[4] = {0.f, 0.f, 0.f, 0.f};
+        const ActCoef coef = ACT ? act_coef(p, co) : ActCoef();
         for (int j = 0; j < my_tiles; ++j) {
             const int buf = j & 1;
             if (!mbar_wait(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 913)) break;
@@ -1104,14 +1168,30 @@ tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
                 const uint32_t slab = out_stage + (uint32_t)((warp - 2) * 2048);
                 if (lane == 0) tma_store_wait_read<0>();          // the store that last read this slab has left it
                 __syncwarp();
-                t_chunk_to_slab<false>(v, in_mask, slab + (uint32_t)(lane * 2), stats, sum, sumsq);
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0 && in_mask != 0u && co_tile * 128 + quarter * 32 < p.c_out) {
-                    const int crow = c0 >> 3;                    // a chunk is four accumulator rows of one image (th % 4 == 0)
-                    tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0, p.stack ? crow % p.th : h0 + crow,
-                                 p.stack ? n0 + crow / p.th : n0);
-                    tma_store_commit();
+                const int crow = c0 >> 3;                        // a chunk is four accumulator rows of one image (th % 4 == 0)
+                const int sh = p.stack ? crow % p.th : h0 + crow, sn = p.stack ? n0 + crow / p.th : n0;
+                const bool leaves = lane == 0 && in_mask != 0u && co_tile * 128 + quarter * 32 < p.c_out;
+                if (!ACT || p.act_raw) {
+                    t_chunk_to_slab<false>(v, in_mask, slab + (uint32_t)(lane * 2), stats, sum, sumsq);
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (leaves) {
+                        tma_store_4d(&map_out, slab, co_tile * 128 + quarter * 32, w0, sh, sn);
+                        tma_store_commit();
+                    }
+                }
+                if constexpr (ACT) {
+                    if (p.act_raw) {
+                        if (lane == 0) tma_store_wait_read<0>();
+                        __syncwarp();
+                    }
+                    act_chunk_to_slab(v, slab + (uint32_t)(lane * 2), coef.scale, coef.shift);
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (leaves) {
+                        tma_store_4d(&map_act, slab, co_tile * 128 + quarter * 32, w0, sh, sn);
+                        tma_store_commit();
+                    }
                 }
             }
             tc_fence_before();
@@ -3231,7 +3311,7 @@ void t_plan(TParams* p, int* W, int* H, int* N, bool dense) {
 struct TView { int in_stride, x_h, x_w, out_stride, out_h, out_w; };
 
 int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& mw, void* out, float* stat_partial, int* stat_blocks,
-                  int N, int H, int W, int c_red, int c_out, int* status, cudaStream_t st, const char* what, bool a_mn, const TView* view = nullptr) {
+                  int N, int H, int W, int c_red, int c_out, int* status, cudaStream_t st, const char* what, bool a_mn, const TView* view = nullptr, void* act_out = nullptr) {
     p.in_stride = view ? view->in_stride : 1;
     p.H = H; p.W = W; p.N = N; p.c_red = c_red; p.c_out = c_out;
     bool patch = false;
@@ -3264,7 +3344,7 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     if (p.split > 1) p.ctas_per_co = p.p_tiles;
     const uint32_t stage_bytes = 128 * 128 + (uint32_t)p.tile_cols * 128;
     constexpr uint32_t t_slabs = 4 * kTEpi * kTSlabs * 2048;
-    const uint32_t slabs = p.join_add ? 4 * kTEpi * kJoinSlots * 4096 : t_slabs;
+    const uint32_t slabs = p.join_add ? 4 * kTEpi * kJoinSlots * 4096 : p.act_stats ? 2 * t_slabs : t_slabs;
     p.stages = std::min<int>(kMaxStages, (227 * 1024 - 1024 - 512 - slabs - 64) / stage_bytes);
     CUtensorMap mx;
     int rc = view ? make_act_map(&mx, x, N, view->x_h, view->x_w, x_channels, p.tw, p.th, p.tn, view->in_stride)
@@ -3274,16 +3354,19 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     CUtensorMap mo, madd, mmask;
     const int bw = std::min(p.tw, 32), bh = std::min(p.th, 32 / bw), bnn = 32 / (bw * bh);
     const int64_t os = view ? view->out_stride : 0;
-    if ((rc = make_chunk_map(&mo, out, N, H, W, c_out, bw, bh, bnn, os, view ? os * view->out_w : 0, view ? (int64_t)view->out_h * view->out_w : 0))) return rc;
+    if ((rc = make_chunk_map(&mo, out ? out : act_out, N, H, W, c_out, bw, bh, bnn, os, view ? os * view->out_w : 0, view ? (int64_t)view->out_h * view->out_w : 0))) return rc;
     madd = mmask = mo;
     if (p.join_add && (rc = make_chunk_map(&madd, p.join_add, N, H, W, c_out, bw, bh, bnn))) return rc;
+    if (act_out && (rc = make_chunk_map(&madd, act_out, N, H, W, c_out, bw, bh, bnn))) return rc;
     if (p.join_mask && (rc = make_chunk_map(&mmask, p.join_mask, N, H, W, c_out, bw, bh, bnn))) return rc;
     const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 512 + slabs;
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaSuccess;
-        for (auto kernel : {tc_conv_t_kernel<false, false, false>, tc_conv_t_kernel<true, false, false>, tc_conv_t_kernel<false, true, false>,
-                            tc_conv_t_kernel<true, true, false>, tc_conv_t_kernel<true, false, true>, tc_conv_t_kernel<true, true, true>})
+        for (auto kernel : {tc_conv_t_kernel<false, false, EPI_PLAIN>, tc_conv_t_kernel<true, false, EPI_PLAIN>, tc_conv_t_kernel<false, true, EPI_PLAIN>,
+                            tc_conv_t_kernel<true, true, EPI_PLAIN>, tc_conv_t_kernel<true, false, EPI_JOIN>, tc_conv_t_kernel<true, true, EPI_JOIN>,
+                            tc_conv_t_kernel<false, false, EPI_ACT>, tc_conv_t_kernel<false, true, EPI_ACT>, tc_conv_t_kernel<false, false, EPI_RESIDUAL>,
+                            tc_conv_t_kernel<false, true, EPI_RESIDUAL>})
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 64);
         if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
         attr_set = true;
@@ -3294,13 +3377,14 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     if (patch) {
         static bool tp_attr_set = false;
         if (!tp_attr_set) {
-            cudaError_t e = cudaFuncSetAttribute(tc_conv_tp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTpSmem);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_conv_tp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTpSmem);
+            cudaError_t e = cudaSuccess;
+            for (auto kernel : {tc_conv_tp_kernel<false, false>, tc_conv_tp_kernel<true, false>, tc_conv_tp_kernel<false, true>})
+                if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTpSmem);
             if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
             tp_attr_set = true;
         }
-        if (a_mn) tc_conv_tp_kernel<true><<<p.ctas_per_co * p.co_tiles, kTpThreads, kTpSmem, st>>>(mx, mw, mo, stat_blocks ? stat_partial : nullptr, p, status);
-        else tc_conv_tp_kernel<false><<<p.ctas_per_co * p.co_tiles, kTpThreads, kTpSmem, st>>>(mx, mw, mo, stat_blocks ? stat_partial : nullptr, p, status);
+        const auto kernel = act_out ? tc_conv_tp_kernel<false, true> : a_mn ? tc_conv_tp_kernel<true, false> : tc_conv_tp_kernel<false, false>;
+        kernel<<<p.ctas_per_co * p.co_tiles, kTpThreads, kTpSmem, st>>>(mx, mw, mo, madd, stat_blocks ? stat_partial : nullptr, p, status);
         CKPT_LAUNCH_CHECK_NAMED("tc_conv_tp_kernel", what);
         return CKPT_OK;
     }
@@ -3313,21 +3397,32 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
         attr.id = cudaLaunchAttributeClusterDimension;
         attr.val.clusterDim.x = (unsigned)p.split; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
         cfg.attrs = &attr; cfg.numAttrs = 1;
-        const auto kernel = p.join_add ? tc_conv_t_kernel<true, true, true> : a_mn ? tc_conv_t_kernel<true, true, false> : tc_conv_t_kernel<false, true, false>;
+        const auto kernel = p.join_add ? (a_mn ? tc_conv_t_kernel<true, true, EPI_JOIN> : tc_conv_t_kernel<false, true, EPI_RESIDUAL>)
+                            : act_out ? tc_conv_t_kernel<false, true, EPI_ACT>
+                            : a_mn ? tc_conv_t_kernel<true, true, EPI_PLAIN> : tc_conv_t_kernel<false, true, EPI_PLAIN>;
         const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mx, mw, mo, madd, mmask, stats, p, status);
         if (e != cudaSuccess) return cuda_fail(e, what);
     } else {
-        const auto kernel = p.join_add ? tc_conv_t_kernel<true, false, true> : a_mn ? tc_conv_t_kernel<true, false, false> : tc_conv_t_kernel<false, false, false>;
+        const auto kernel = p.join_add ? (a_mn ? tc_conv_t_kernel<true, false, EPI_JOIN> : tc_conv_t_kernel<false, false, EPI_RESIDUAL>)
+                            : act_out ? tc_conv_t_kernel<false, false, EPI_ACT>
+                            : a_mn ? tc_conv_t_kernel<true, false, EPI_PLAIN> : tc_conv_t_kernel<false, false, EPI_PLAIN>;
         kernel<<<grid, kThreadsT, smem, st>>>(mx, mw, mo, madd, mmask, stats, p, status);
     }
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_t_kernel", what);
     return CKPT_OK;
 }
 
+void set_known(TParams* p, const KnownStats& known, int channels) {
+    p->act_stats = known.stats; p->act_channels = channels; p->act_raw = known.raw; p->shortcut_stats = known.shortcut_stats;
+    if (known.shortcut) p->join_add = (const __nv_bfloat16*)known.shortcut;
+}
+
 int launch_t(const void* x, const void* w_mat, void* out, float* stat_partial, int* stat_blocks, int N, int H, int W, int c_red,
-             int c_out, int k, int pad, int* status, cudaStream_t st, const char* what, bool a_mn = false, const GradientJoin& join = GradientJoin()) {
+             int c_out, int k, int pad, int* status, cudaStream_t st, const char* what, bool a_mn = false, const GradientJoin& join = GradientJoin(),
+             const KnownStats& known = KnownStats()) {
     TParams p;
     p.join_add = (const __nv_bfloat16*)join.add; p.join_mask = (const __nv_bfloat16*)join.mask;
+    set_known(&p, known, c_out);
     p.taps = k * k;
     p.fold = 0;
     p.pair = 0;
@@ -3341,7 +3436,7 @@ int launch_t(const void* x, const void* w_mat, void* out, float* stat_partial, i
     CUtensorMap mw;
     int rc = a_mn ? make_mat_map(&mw, w_mat, c_red, (int64_t)k * k * c_out, 64, 4) : make_mat_map(&mw, w_mat, c_out, (int64_t)k * k * c_red, 128, 4);
     if (rc) return rc;
-    return launch_t_core(p, x, c_red, mw, out, stat_partial, stat_blocks, N, H, W, c_red, c_out, status, st, what, a_mn);
+    return launch_t_core(p, x, c_red, mw, out, stat_partial, stat_blocks, N, H, W, c_red, c_out, status, st, what, a_mn, nullptr, known.act);
 }
 
 // 3x3, padding 1, 64 output channels, even width: two horizontally adjacent pixels are treated as one pixel with
@@ -3360,12 +3455,13 @@ bool paired_applies(int c_red, int c_out, int k, int pad, int N, int H, int W) {
     return pixels >= PAIR_MIN_PIXELS || (pixels >= PAIR_MIN_PIXELS_STRIPS && tp_strip(H, W / 2, N, 1, &th));
 }
 int launch_t_paired(const void* x, const void* w, int flip, void* out, float* stat_partial, int* stat_blocks, int N, int H, int W,
-                    int c_red, int* status, cudaStream_t st, const char* what) {
+                    int c_red, int* status, cudaStream_t st, const char* what, const KnownStats& known = KnownStats()) {
     // term t = (filter row r, column sp of the four input columns 2j-1 .. 2j+2 that pair j reaches); pixel q of the
     // pair sees column sp through filter column s = sp - q.  flip: w is the forward filter [c_red][9][64] and the
     // input gradient takes the mirrored position.
     TParams p;
     p.join_add = p.join_mask = nullptr;
+    set_known(&p, known, 64);
     p.taps = 12;
     p.fold = 64;
     p.pair = 1;
@@ -3385,7 +3481,7 @@ int launch_t_paired(const void* x, const void* w, int flip, void* out, float* st
     CUtensorMap mw;
     int rc = flip ? make_mat_map(&mw, w, c_red, 9 * 64, 64, 4) : make_mat_map(&mw, w, 64, (int64_t)9 * c_red, 64, 4);
     if (rc) return rc;
-    return launch_t_core(p, x, 2 * c_red, mw, out, stat_partial, stat_blocks, N, H, W / 2, c_red, 128, status, st, what, flip != 0);
+    return launch_t_core(p, x, 2 * c_red, mw, out, stat_partial, stat_blocks, N, H, W / 2, c_red, 128, status, st, what, flip != 0, nullptr, known.act);
 }
 
 // stat_partial / stat_blocks: null, or where the kernel leaves the batch-norm partial sums of its output
@@ -3791,6 +3887,7 @@ static TParams strided_terms() {
     TParams q;
     q.fold = 0; q.pair = 0; q.patch_ok = 0; q.ncols = 0;
     q.join_add = q.join_mask = nullptr;
+    q.act_stats = q.shortcut_stats = nullptr; q.act_raw = 0; q.act_channels = 1;
     return q;
 }
 
@@ -3800,9 +3897,10 @@ static TParams strided_terms() {
 // 60.1 -> 27.0; 1x1 1024 -> 2048 at 14 x 14 alone is slower, 29.4 -> 34.0, with sums 39.1 -> 37.1).
 // Strided forward: the operand boxes take every stride-th input pixel, the tiles walk the output grid.
 static int launch_strided_fwd(const ConvGeom& g, const void* x, const void* w, void* z, int* status, cudaStream_t st,
-                              float* stat_partial = nullptr, int* stat_blocks = nullptr) {
+                              float* stat_partial = nullptr, int* stat_blocks = nullptr, const KnownStats& known = KnownStats()) {
     if (t_applies(g.cin, g.cout, g.k, g.pad)) {
         TParams q = strided_terms();
+        set_known(&q, known, g.cout);
         q.taps = g.k * g.k;
         for (int t = 0; t < q.taps; ++t) { q.tap_dh[t] = t / g.k - g.pad; q.tap_dw[t] = t % g.k - g.pad; q.tap_col[t] = t; q.tap_xc[t] = 0; }
         CUtensorMap mw;
@@ -3810,7 +3908,7 @@ static int launch_strided_fwd(const ConvGeom& g, const void* x, const void* w, v
         if (rc) return rc;
         const TView view = {g.stride, g.h, g.w, 1, g.ho, g.wo};
         return launch_t_core(q, x, g.cin, mw, z, stat_partial, stat_blocks, g.n, g.ho, g.wo, g.cin, g.cout, status, st,
-                             "strided conv forward (tensor cores)", false, &view);
+                             "strided conv forward (tensor cores)", false, &view, known.act);
     }
     FwdParams p;
     p.taps = g.k * g.k;
@@ -3831,6 +3929,25 @@ int tc_conv_fwd_stats(const ConvGeom& g, const void* x, const void* w, void* z, 
     if (g.stride != 1) return launch_strided_fwd(g, x, w, z, device_status, (cudaStream_t)stream, partial, blocks);
     return launch_fwd_like(x, w, z, nullptr, 0, g.n, g.h, g.w, g.cin, g.cout, g.k, g.pad, device_status, (cudaStream_t)stream,
                            "conv forward (tensor cores)", partial, blocks);
+}
+
+bool tc_fwd_takes_known_stats(const ConvGeom& g, bool residual) {
+    if (!tc_conv_supported(CKPT_DTYPE_BF16, g) || fc_applies(g)) return false;
+    if (residual) return g.k == 1 && g.stride == 1 && t_applies(g.cin, g.cout, 1, 0);
+    return t_applies(g.cin, g.cout, g.k, g.pad) || (g.stride == 1 && paired_applies(g.cin, g.cout, g.k, g.pad, g.n, g.h, g.w));
+}
+
+int tc_conv_fwd_known_stats(const ConvGeom& g, const void* x, const void* w, void* z, const KnownStats& known, int* device_status, void* stream) {
+    if (!device_status) { set_error("no status word"); return CKPT_E_NULL; }
+    if (!tc_fwd_takes_known_stats(g, known.shortcut != nullptr)) { set_error("this convolution does not take known statistics"); return CKPT_E_UNSUPPORTED; }
+    cudaStream_t st = (cudaStream_t)stream;
+    KnownStats k = known;
+    k.raw = z && known.act ? 1 : 0;
+    if (g.stride != 1) return launch_strided_fwd(g, x, w, z, device_status, st, nullptr, nullptr, k);
+    if (!k.shortcut && paired_applies(g.cin, g.cout, g.k, g.pad, g.n, g.h, g.w))
+        return launch_t_paired(x, w, 0, z, nullptr, nullptr, g.n, g.h, g.w, g.cin, device_status, st, "conv forward with known statistics (tensor cores)", k);
+    return launch_t(x, w, z, nullptr, nullptr, g.n, g.h, g.w, g.cin, g.cout, g.k, g.pad, device_status, st,
+                    "conv forward with known statistics (tensor cores)", false, GradientJoin(), k);
 }
 
 int tc_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, void* scratch,

@@ -131,6 +131,18 @@ int tc_conv_fwd_stats(const ConvGeom& g, const void* x, const void* w, void* z, 
 // mask may be null); 1x1 stride-1 filters for which tc_dgrad_joins holds.
 struct GradientJoin { const void *add = nullptr, *mask = nullptr; };
 bool tc_dgrad_joins(const ConvGeom& g);
+// Forward convolution whose output's batch statistics (4 * c_out floats) are known: writes the activated form `act`, beside
+// the convolution's own output where z is not null; with a shortcut (1x1 filters) z takes the residual join
+// max(conv*scale + shift + shortcut, 0) instead, the shortcut normalised by statistics of its own if given.
+struct KnownStats {
+    const float* stats = nullptr;
+    void* act = nullptr;
+    const void* shortcut = nullptr;
+    const float* shortcut_stats = nullptr;
+    int raw = 0;                         // (set by the launcher)
+};
+bool tc_fwd_takes_known_stats(const ConvGeom& g, bool residual);
+int tc_conv_fwd_known_stats(const ConvGeom& g, const void* x, const void* w, void* z, const KnownStats& known, int* device_status, void* stream);
 int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, void* scratch,
                   int64_t scratch_bytes, int* device_status, void* stream, const GradientJoin& join = GradientJoin());
 // upd: optional parameter update applied together with the gradient (the filter must no longer be needed by this step)
