@@ -3580,18 +3580,23 @@ void wgrad_plan(const ConvGeom& g, WgradParams* p, int* slices, int* groups, int
     choose_tile(p->px, g.wo, g.ho, g.n, &p->tw, &p->th, &p->tn);
     p->tiles_w = (g.wo + p->tw - 1) / p->tw; p->tiles_h = (g.ho + p->th - 1) / p->th; p->tiles_n = (g.n + p->tn - 1) / p->tn;
     p->total_tiles = p->tiles_w * p->tiles_h * p->tiles_n;
+    // Short reductions of few columns do not fill the SMs with 256-column CTAs: half as wide for 1x1 filters and for fewer
+    // than 800 pixels, and slices down to 256 pixels below (us with the slice sum, four blocks and 512 pixels -> chosen:
+    // 256 -> 1024 at 13 x 11, 21 images 15.4 -> 12.3, at 14 x 14, 32 images 14.4 -> 12.2; 3x3 512 -> 512 at 2 x 2, 128 images
+    // 12.5 -> 10.8; 3x3 256 -> 256 at 13 x 11 keeps four blocks, 16.6 against 19.9).
+    if (p->nb > 2 && ((g.k == 1 && pixels <= 65536) || pixels <= 800)) p->nb = 2;
     // a reduction of one or two pixel tiles is all stores: narrower CTAs (128 accumulator columns) fit four to an SM
     if (p->total_tiles <= 2 && p->total_blocks >= 2) p->nb = 2;
     *groups = (p->total_blocks + p->nb - 1) / p->nb;
     *co_tiles = (g.cout + 127) / 128;
     // slices of the pixel range: one wave of equally long CTAs that fills the SMs as far as it can (every CTA pays
     // for its accumulator's way out - 128 KB of partial sums - once, so fewer and longer CTAs win: 256 -> 1024 at
-    // 14 x 14, batch 128: 35 us in one wave of 144 against 49 us in two waves of 288), at least 512 pixels per slice
+    // 14 x 14, batch 128: 35 us in one wave of 144 against 49 us in two waves of 288), at least 256 pixels per slice
     const int64_t base_ctas = (int64_t)*groups * *co_tiles;
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int64_t by_k = std::max<int64_t>(1, (int64_t)p->total_tiles * p->px / 512);
+    int64_t by_k = std::max<int64_t>(1, (int64_t)p->total_tiles * p->px / 256);
     int64_t s = 1;
     double best_eff = -1.0;
     for (int64_t cand = 1; cand <= std::min<int64_t>(by_k, 256); ++cand) {
