@@ -1408,7 +1408,7 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
         } else {
             maxpool3_bwd_kernel<false><<<grid, 256, 0, st>>>(arg, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, nullptr, nullptr, nullptr);
         }
-        CKPT_LAUNCH_CHECK("max-pool 3x3 backward");
+        CKPT_LAUNCH_CHECK("max-pool backward from arg-max");
         return CKPT_OK;
     }
     if (act) { set_error("the general pooling kernel takes an activated input"); return CKPT_E_BAD_ARG; }

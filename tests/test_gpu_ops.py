@@ -456,7 +456,7 @@ def test_stem_kernels_ragged_channels(n, h, w, cout):
 
 
 @pytest.mark.parametrize("dtype", [ck.DTYPE_F32, ck.DTYPE_BF16])
-@pytest.mark.parametrize("rows,c,relu", [(1, 8, 1), (63, 64, 1), (65, 64, 0), (1000, 48, 1), (257, 72, 1), (129, 2048, 1), (30000, 256, 1), (120011, 64, 1),
+@pytest.mark.parametrize("rows,c,relu", [(1, 8, 1), (63, 64, 1), (65, 64, 0), (1000, 48, 1), (257, 72, 1), (129, 2048, 1), (30000, 256, 1), (120011, 64, 1), (3003, 512, 1), (7300, 256, 0), (900, 1024, 1),
                                          (1031, 1000, 0)])
 def test_bn_backward_in_one_kernel(rows, c, relu, dtype):
     """The cooperative batch-norm backward at the edges of its split: a single row, less and more than a step of a CTA,
