@@ -371,6 +371,11 @@ CKPT_API int ckpt_op_status(int32_t* status);
  * cycles, recording its code (9001) in the status word that ckpt_op_status reads: the failure path of the bounded
  * waits, exercised without a fault.  Asynchronous on `stream`. */
 CKPT_API int ckpt_selftest_bounded_wait(int64_t limit_cycles, void* stream);
+/* The tile that the role-swapped convolution kernel takes for a bf16 shape of stride 1 (host only, no device needed), for
+ * tests of its limits.  epilogue: 0 plain, 1 joining another tensor, 2 writing the activated form.  plan (host, 6 values):
+ * pixels per tile, CTAs that share a reduction, operand stages, bytes of the stages, bytes of the accumulators that are
+ * exchanged in place of the stages (0 without sharing), shared memory in all.  CKPT_E_UNSUPPORTED: another kernel runs. */
+CKPT_API int ckpt_selftest_conv_plan(const ckpt_conv_shape* s, int epilogue, int32_t* plan);
 
 CKPT_API int ckpt_conv2d_scratch_bytes(const ckpt_conv_shape* s, int dtype, int64_t* bytes);
 CKPT_API int ckpt_conv2d_forward(const ckpt_conv_shape* s, int dtype, int impl, const void* x, const void* w,

@@ -396,6 +396,13 @@ def selftest_bounded_wait(limit_cycles, stream=None):
     _check(lib().ckpt_selftest_bounded_wait(C.c_int64(limit_cycles), _stream(stream)))
 
 
+def selftest_conv_plan(shape, epilogue):
+    """Tile of the role-swapped kernel: dict of pixels, split, stages, stage_bytes, exchange_bytes, smem (host only)."""
+    out = (C.c_int32 * 6)()
+    _check(lib().ckpt_selftest_conv_plan(C.byref(shape), C.c_int(epilogue), out))
+    return dict(zip(("pixels", "split", "stages", "stage_bytes", "exchange_bytes", "smem"), out))
+
+
 # ------------------------------------------------------------------------------------------------
 # single operations
 # ------------------------------------------------------------------------------------------------

@@ -146,6 +146,14 @@ int ckpt_selftest_bounded_wait(int64_t limit_cycles, void* stream) {
     return tc_selftest_wait((long long)limit_cycles, op_status_word(), stream);
 }
 
+int ckpt_selftest_conv_plan(const ckpt_conv_shape* s, int epilogue, int32_t* plan) {
+    int rc = check_shape(s, CKPT_DTYPE_BF16);
+    if (rc) return rc;
+    if (!plan) { set_error("plan is null"); return CKPT_E_NULL; }
+    if (epilogue < 0 || epilogue > 2) { set_error("unknown epilogue %d", epilogue); return CKPT_E_BAD_ARG; }
+    return tc_selftest_t_plan(make_geom(*s), epilogue, plan);
+}
+
 int ckpt_bn_scratch_bytes(int64_t rows, int32_t c, int64_t* bytes) {
     if (!bytes) { set_error("bytes is null"); return CKPT_E_NULL; }
     if (rows < 1 || c < 1) { set_error("bad shape"); return CKPT_E_BAD_ARG; }

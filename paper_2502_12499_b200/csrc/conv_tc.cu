@@ -3048,6 +3048,25 @@ int make_chunk_map(CUtensorMap* map, const void* ptr, int N, int H, int W, int C
     return CKPT_OK;
 }
 
+// Shared memory of the plain role-swapped kernel: barriers, the epilogue's slabs, and operand stages in the rest.  Slabs: a
+// pair of chunk slabs per epilogue warp; two pairs where the activated form leaves beside the convolution's; slots for the
+// tensors that a join reads.  The CTAs of a shared reduction finish through one pair whatever the epilogue (plain loads),
+// and leave their accumulators ([pixel][128 channels] floats) over the stages, which therefore have to hold them.
+constexpr uint32_t kTSmem = 227 * 1024 - 64, kTBars = 512;
+static_assert(kTSlabs >= 2, "a shared reduction keeps both forms of a chunk in its slabs");
+uint32_t t_slab_bytes(const TParams& p, int split) {
+    constexpr uint32_t pair = 4 * kTEpi * kTSlabs * 2048;
+    return split > 1 ? pair : p.join_add ? 4 * kTEpi * kJoinSlots * 4096 : p.act_stats ? 2 * pair : pair;
+}
+uint32_t t_stage_bytes(int cols) { return 128 * 128 + (uint32_t)cols * 128; }
+int t_stages(const TParams& p, int cols, int split) {
+    return std::min<int>(kMaxStages, (kTSmem - 1024 - kTBars - t_slab_bytes(p, split)) / t_stage_bytes(cols));
+}
+bool t_fits(const TParams& p, int cols, int split) {
+    const int stages = t_stages(p, cols, split);
+    return stages >= 2 && (split == 1 || (uint32_t)cols * 512 <= (uint32_t)stages * t_stage_bytes(cols));
+}
+
 // Pixel tile and reduction split of the plain role-swapped kernel, by a model of clocks fitted to a sweep of both over
 // 26 shapes: a stage (64 reduction channels of one term) takes its four MMAs - 430 however few pixels, 2 per pixel above
 // 215 - or its bytes from the L2; the epilogue of a tile takes about 1100 and 15 per pixel and runs under the next tile's stages; a
@@ -3072,6 +3091,7 @@ void t_plan(TParams* p, int* W, int* H, int* N, bool dense) {
         const int64_t tiles = (int64_t)((*W + tw - 1) / tw) * ((*H + th - 1) / th) * ((*N + tn - 1) / tn);
         for (int split = 1; split <= 8; split *= 2) {
             if (split > 1 && (p->fold || terms < 2 * split || (int64_t)tiles * co * split > sms - 4 * split)) break;
+            if (!t_fits(*p, cols, split)) continue;
             const double active = std::min<double>(sms, (double)tiles * co * split);
             const double bytes = 16384.0 + 128.0 * cols, stage = std::max(std::max(2.0 * cols, 430.0), bytes / std::min(100.0, 9000.0 / active));
             const double loop = std::ceil((double)terms / split) * stage, out = 1100.0 + 15.0 * cols;
@@ -3118,10 +3138,8 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     p.ctas_per_co = std::max(1, std::min(p.p_tiles, sms / p.co_tiles));
     if (p.split > 1) p.ctas_per_co = p.p_tiles;
-    const uint32_t stage_bytes = 128 * 128 + (uint32_t)p.tile_cols * 128;
-    constexpr uint32_t t_slabs = 4 * kTEpi * kTSlabs * 2048;
-    const uint32_t slabs = p.join_add ? 4 * kTEpi * kJoinSlots * 4096 : p.act_stats ? 2 * t_slabs : t_slabs;
-    p.stages = std::min<int>(kMaxStages, (227 * 1024 - 1024 - 512 - slabs - 64) / stage_bytes);
+    p.stages = t_stages(p, p.tile_cols, p.split);
+    if (!patch && !t_fits(p, p.tile_cols, p.split)) { set_error("role-swapped convolution: a tile that shared memory does not hold"); return CKPT_E_UNSUPPORTED; }
     CUtensorMap mx;
     int rc = view ? make_act_map(&mx, x, N, view->x_h, view->x_w, x_channels, p.tw, p.th, p.tn, view->in_stride)
                   : make_act_map(&mx, x, N, H, W, x_channels, p.tw, patch && !p.stack ? p.th + 2 : p.th, p.tn);
@@ -3135,7 +3153,7 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     if (p.join_add && (rc = make_chunk_map(&madd, p.join_add, N, H, W, c_out, bw, bh, bnn))) return rc;
     if (act_out && (rc = make_chunk_map(&madd, act_out, N, H, W, c_out, bw, bh, bnn))) return rc;
     if (p.join_mask && (rc = make_chunk_map(&mmask, p.join_mask, N, H, W, c_out, bw, bh, bnn))) return rc;
-    const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 512 + slabs;
+    const size_t smem = (size_t)p.stages * t_stage_bytes(p.tile_cols) + 1024 + kTBars + t_slab_bytes(p, p.split);
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaSuccess;
@@ -3143,7 +3161,7 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
                             tc_conv_t_kernel<true, true, EPI_PLAIN>, tc_conv_t_kernel<true, false, EPI_JOIN>, tc_conv_t_kernel<true, true, EPI_JOIN>,
                             tc_conv_t_kernel<false, false, EPI_ACT>, tc_conv_t_kernel<false, true, EPI_ACT>, tc_conv_t_kernel<false, false, EPI_RESIDUAL>,
                             tc_conv_t_kernel<false, true, EPI_RESIDUAL>})
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 64);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTSmem);
         if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
         attr_set = true;
     }
@@ -3963,6 +3981,22 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_wgrad_kernel", "conv wgrad (tensor cores)");
     if (slices > 1) return slice_sum((const float*)scratch, dw, elems, slices, st, upd);
     if (upd.w && !update) return sgd_update(upd, dw, elems, st);
+    return CKPT_OK;
+}
+
+int tc_selftest_t_plan(const ConvGeom& g, int epilogue, int* plan) {
+    if (!tc_conv_supported(CKPT_DTYPE_BF16, g) || g.stride != 1 || !t_applies(g.cin, g.cout, g.k, g.pad)) { set_error("the role-swapped kernel does not take this shape"); return CKPT_E_UNSUPPORTED; }
+    static const float some = 0.f;
+    TParams p = strided_terms();
+    p.taps = g.k * g.k; p.c_red = g.cin; p.c_out = g.cout; p.in_stride = 1;
+    if (epilogue == 1) p.join_add = reinterpret_cast<const __nv_bfloat16*>(&some);
+    if (epilogue == 2) p.act_stats = &some;
+    int W = g.w, H = g.h, N = g.n;
+    t_plan(&p, &W, &H, &N, true);
+    const int stages = t_stages(p, p.tile_cols, p.split);
+    plan[0] = p.tile_cols; plan[1] = p.split; plan[2] = stages; plan[3] = stages * (int)t_stage_bytes(p.tile_cols);
+    plan[4] = p.split > 1 ? p.tile_cols * 512 : 0;
+    plan[5] = plan[3] + 1024 + (int)kTBars + (int)t_slab_bytes(p, p.split);
     return CKPT_OK;
 }
 

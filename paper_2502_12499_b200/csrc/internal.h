@@ -151,6 +151,9 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
 
 // One tiny kernel whose only wait has no producer and gives up after `limit_cycles` (1 .. 2e9), writing its code
 // into the status word: the bounded-wait path, run to its limit on purpose.
+// Tile of the plain role-swapped kernel for a shape (epilogue: 0 plain, 1 join, 2 activated form): pixels, CTAs that share a
+// reduction, stages, their bytes, bytes of the accumulators that go over them, all shared memory.  No device needed.
+int tc_selftest_t_plan(const ConvGeom& g, int epilogue, int* plan);
 int tc_selftest_wait(long long limit_cycles, int* device_status, void* stream);
 
 int64_t bn_scratch_bytes(int64_t rows, int c);

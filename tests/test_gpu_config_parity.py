@@ -33,6 +33,7 @@ import numpy as np
 import pytest
 
 from oracle import numeric_oracle as no
+from paper_2502_12499_b200 import binding as ck
 from paper_2502_12499_b200 import workloads as wl
 from tests import parity_util as pu
 from tests.gpu_util import StepRunner
@@ -168,3 +169,22 @@ def test_resnet_blocks_at_benchmark_dispatch(stage, batch, expected):
     params, x, labels, step = run_case(spec, seed=5)
     assert_tensor_core_dispatch(step, expected)
     assert_units_match_locally(step, params, labels)
+
+
+@pytest.mark.parametrize("batch", [6, 13])
+def test_wide_blocks_share_long_reductions(batch):
+    """Residual blocks of 2048 channels on few pixels: the joined input gradient and the residual join of a recomputed
+    output share one tile's 2048-channel reduction among the CTAs of a cluster, in tiles of 160 pixels.  The store-all
+    step against the oracle, and the checkpointed step (which recomputes the first block) bit for bit against it."""
+    plan = ck.selftest_conv_plan(ck.ConvShape(batch, 7, 7, 2048, 2048, 1, 1, 0), 1)
+    assert plan["split"] > 1 and plan["pixels"] >= 160, plan
+    block = {"kind": "bottleneck", "cin": 2048, "mid": 2048, "cout": 2048, "stride": 1, "project": False}
+    spec = dict(units=[block, dict(block)], input_hwc=(7, 7, 2048), batch=batch, dtype="bf16", loss="sum", name="wide_blocks")
+    params, x, labels, step = run_case(spec, seed=9)
+    assert_tensor_core_dispatch(step, ["tc_conv_t_kernel"])
+    assert_units_match_locally(step, params, labels)
+    _, kept = step.runner.run(ck.POLICY_STORE_ALL, None, x, labels)
+    report, grads = step.runner.run(ck.POLICY_DYNAMIC, ck.mask_from_set(2, [0, 2]), x, labels)
+    assert report["device_status"] == 0 and report["recomputed_units"] > 0
+    for a, b in zip(kept, grads):
+        assert np.array_equal(a, b)
