@@ -301,7 +301,7 @@ CKPT_API int ckpt_chain_set_gradient_tap(ckpt_chain* chain, void* tap, int64_t t
 CKPT_API int ckpt_chain_set_sgd(ckpt_chain* chain, double learning_rate);
 
 /* Failure-path self-test (off by default).  With wait_runs_out = 1 every following step launches, after its loss,
- * one extra single-warp kernel whose only wait has no producer and a limit of 2e5 clock cycles: the wait gives up,
+ * one extra small kernel with a wait that nothing satisfies in time and a limit of 2e5 clock cycles: the wait gives up,
  * writes its code into the step's status word and the kernel returns, as every bounded wait of the tensor-core
  * kernels does when its producer never arrives.  The step then finishes normally on the device and returns
  * CKPT_E_DEVICE_TIMEOUT with report->device_status = 1; the context stays usable.  Nothing faults or spins without
@@ -367,9 +367,10 @@ typedef struct ckpt_conv_shape {
  * satisfied), clears it, and returns CKPT_E_DEVICE_TIMEOUT when it was not 0.  Call it after a batch of single
  * operations whose results matter.  (ckpt_train_step has its own status word and checks it itself.) */
 CKPT_API int ckpt_op_status(int32_t* status);
-/* Launches one single-warp kernel whose only wait has no producer and gives up after limit_cycles (1 .. 2e9) clock
- * cycles, recording its code (9001) in the status word that ckpt_op_status reads: the failure path of the bounded
- * waits, exercised without a fault.  Asynchronous on `stream`. */
+/* Launches one small kernel in which one lane of a waiting warp gives up after limit_cycles (1 .. 2e9) clock cycles,
+ * recording its code (9001) in the status word that ckpt_op_status reads, while the other lanes may still see the
+ * barrier complete: the failure path of the bounded waits, exercised without a fault.  A warp whose lanes left the wait
+ * with different answers records 9002.  Asynchronous on `stream`. */
 CKPT_API int ckpt_selftest_bounded_wait(int64_t limit_cycles, void* stream);
 /* The tile that the role-swapped convolution kernel takes for a bf16 shape of stride 1 (host only, no device needed), for
  * tests of its limits.  epilogue: 0 plain, 1 joining another tensor, 2 writing the activated form.  plan (host, 6 values):

@@ -81,6 +81,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         }
     }
 }
+// The same for a whole warp whose lanes have work in common behind the wait (a __syncwarp, a collective load): every lane
+// watches the barrier itself, and all go on or none does - a lane that gave up alone would leave the others waiting for it.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* failed, int* status, int code,
+                                               long long limit = kWaitCycles) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, failed, status, code, limit)) != 0;
+}
 // After a failure: give copies that are still in flight a bounded time to land.
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
     const long long t0 = clock64();
@@ -342,7 +348,7 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             for (int it = 0; it < iters; ++it, ++g) {
                 const int s = g % p.stages;
                 const uint32_t phase = (uint32_t)(g / p.stages) & 1u;
-                if (!mbar_wait(empty_bar(s), phase ^ 1u, failed, status, 101)) { ok = false; break; }
+                if (!(B_MN ? mbar_wait_warp(empty_bar(s), phase ^ 1u, failed, status, 101) : mbar_wait(empty_bar(s), phase ^ 1u, failed, status, 101))) { ok = false; break; }
                 const int tap = it / blocks, blk = it % blocks;
                 const uint32_t a_dst = base + (uint32_t)s * stage_bytes;
                 if (lane == 0) {
@@ -400,7 +406,7 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         for (int ci = 0; ci < 8; ++ci) { s_acc[ci] = 0.f; q_acc[ci] = 0.f; }
         for (int j = 0; j < my_tiles; ++j) {
             const int buf = j & 1;
-            if (!mbar_wait(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 103)) break;
+            if (!mbar_wait_warp(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 103)) break;
             tc_fence_after();
             int w0, h0, n0;
             tile_origin(j, w0, h0, n0);
@@ -738,7 +744,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 }
                 const int here = min(blocks - blk, left);
                 for (int q = 0; q < here; ++q, ++g) {
-                    if (!mbar_wait(empty_bar(s), phase, failed, status, 901)) { ok = false; break; }
+                    if (!mbar_wait_warp(empty_bar(s), phase, failed, status, 901)) { ok = false; break; }
                     if (lane == 0) mbar_expect_tx(full_bar(s), stage_bytes);
                     __syncwarp();
                     if (lane < (two ? 3 : 2)) tma_load_4d(dst, map, full_bar(s), c0, c1, c2, c3);
@@ -780,7 +786,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     } else if (SPLIT && warp >= 2) {
         // ---------------- accumulator to shared memory, [pixel][channel] floats over the operand stages (all of them read)
         const int quarter = warp % 4;
-        if (mbar_wait(acc_full0, 0, failed, status, 905)) {
+        if (mbar_wait_warp(acc_full0, 0, failed, status, 905)) {
             tc_fence_after();
             for (int c0 = (warp - 2) / 4 * 32; c0 < p.tile_cols; c0 += 32 * kTEpi) {
                 uint32_t v[32];
@@ -811,7 +817,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         bool ok = true;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int buf = j & 1;
-            if (!mbar_wait(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 906)) break;
+            if (!mbar_wait_warp(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 906)) break;
             tc_fence_after();
             if (mine) {
 #pragma unroll 1
@@ -821,7 +827,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                     const int s = done % kJoinSlots, w0 = column(done);
                     uint32_t v[32];
                     tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + (half + m * kTEpi) * 32), v);
-                    if (!mbar_wait(slot_bars + 8u * s, (uint32_t)(done / kJoinSlots) & 1u, failed, status, 907)) { ok = false; break; }
+                    if (!mbar_wait_warp(slot_bars + 8u * s, (uint32_t)(done / kJoinSlots) & 1u, failed, status, 907)) { ok = false; break; }
                     const uint32_t slab = slots + (uint32_t)s * 4096u + (uint32_t)(lane * 2);
                     // (all loads of a half chunk before its stores: in turn each pair would wait for its loads)
 #pragma unroll
@@ -884,7 +890,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         const ActCoef coef = EPI == EPI_ACT ? act_coef(p, co) : ActCoef();
         for (int j = 0; j < my_tiles; ++j) {
             const int buf = j & 1;
-            if (!mbar_wait(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 903)) break;
+            if (!mbar_wait_warp(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 903)) break;
             tc_fence_after();
             int w0, h0, n0;
             tile_origin(j, w0, h0, n0);
@@ -1152,7 +1158,7 @@ tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         const ActCoef coef = ACT ? act_coef(p, co) : ActCoef();
         for (int j = 0; j < my_tiles; ++j) {
             const int buf = j & 1;
-            if (!mbar_wait(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 913)) break;
+            if (!mbar_wait_warp(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 913)) break;
             tc_fence_after();
             int w0, h0, n0;
             tile_origin(j, w0, h0, n0);
@@ -1348,7 +1354,7 @@ tc_conv_c64_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         float s_acc[2] = {0.f, 0.f}, q_acc[2] = {0.f, 0.f};
         for (int j = 0; j < my_tiles; ++j) {
             const int b = j & 1;
-            if (!mbar_wait(acc_full0 + 8 * b, (uint32_t)(j >> 1) & 1u, failed, status, 305)) break;
+            if (!mbar_wait_warp(acc_full0 + 8 * b, (uint32_t)(j >> 1) & 1u, failed, status, 305)) break;
             tc_fence_after();
             int w0, h0, img;
             tile_origin(j, w0, h0, img);
@@ -1464,7 +1470,7 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             const int s = it % p.stages;
             const uint32_t phase = (uint32_t)(it / p.stages) & 1u;
             // every lane watches the barrier itself: measured faster than one lane polling for the warp
-            if (!mbar_wait(empty_bar(s), phase ^ 1u, failed, status, 201)) break;
+            if (!mbar_wait_warp(empty_bar(s), phase ^ 1u, failed, status, 201)) break;
             if (lane == 0) mbar_expect_tx(full_bar(s), (2 + (uint32_t)nb_here) * box_bytes);
             __syncwarp();
             int t = tile_begin + it;
@@ -1518,7 +1524,7 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         const bool valid = co < p.c_out;
         const size_t row_elems = (size_t)p.k * p.k * p.c_in;
         float* dst_row = partial + ((size_t)slice * p.c_out + (valid ? co : 0)) * row_elems;
-        if (iters > 0 && mbar_wait(accum_bar, 0, failed, status, 203)) {
+        if (iters > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 203)) {
             tc_fence_after();
             const int slabs = min(8, (int)((uint32_t)p.stages * stage_bytes / (4u * 4096u)));
             int count = 0;
@@ -1644,7 +1650,7 @@ tc_wgrad_c64_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_con
         for (int j = 0; j < my_tiles; ++j) {
             const int s = j % p.stages;
             const uint32_t phase = (uint32_t)(j / p.stages) & 1u;
-            if (!mbar_wait(empty_bar(s), phase ^ 1u, failed, status, 401)) break;
+            if (!mbar_wait_warp(empty_bar(s), phase ^ 1u, failed, status, 401)) break;
             int t = slice + j * p.slices;
             const int w0 = (t % p.tiles_w) * 8; t /= p.tiles_w;
             const int h0 = (t % p.tiles_h) * p.th;
@@ -1687,7 +1693,7 @@ tc_wgrad_c64_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_con
         const int quarter = warp % 4;
         const int row = quarter * 32 + lane;         // (tap of the pair) * 64 + c_in
         const int half = row / 64, ci = row % 64;
-        if (my_tiles > 0 && mbar_wait(accum_bar, 0, failed, status, 403)) {
+        if (my_tiles > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 403)) {
             tc_fence_after();
             for (int pair = 0; pair < 5; ++pair) {
                 const int tap = pair < 3 ? pair * 3 + half : (pair == 3 ? 2 + 3 * half : 8);
@@ -1780,7 +1786,7 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         int issued = 0;
         for (int j = 0; j < my_tiles; ++j) {
             const int s = j % p.stages;
-            if (!mbar_wait(empty_bar(s), (((uint32_t)(j / p.stages)) & 1u) ^ 1u, failed, status, 701)) break;
+            if (!mbar_wait_warp(empty_bar(s), (((uint32_t)(j / p.stages)) & 1u) ^ 1u, failed, status, 701)) break;
             int t = slice + j * p.slices;
             const int w0 = (t % p.tiles_w) * 8; t /= p.tiles_w;
             const int h0 = (t % p.tiles_h) * p.th;
@@ -1829,7 +1835,7 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         const bool valid = co < p.c_out;
         const size_t row_elems = (size_t)p.row_elems;
         float* dst_row = partial + ((size_t)slice * p.c_out + (valid ? co : 0)) * row_elems;
-        if (my_tiles > 0 && mbar_wait(accum_bar, 0, failed, status, 703)) {
+        if (my_tiles > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 703)) {
             tc_fence_after();
             const int slabs = min(12, (int)((uint32_t)p.stages * p.stage_bytes / (4u * 4096u)));
             int count = 0;
@@ -2053,7 +2059,7 @@ tc_conv_first_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* _
         float s_acc[2] = {0.f, 0.f}, q_acc[2] = {0.f, 0.f};
         for (int j = 0; j < my_tiles; ++j) {
             const int buf = j & 1;
-            if (!mbar_wait(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 604)) break;
+            if (!mbar_wait_warp(acc_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 604)) break;
             tc_fence_after();
             if (lane == 0) tma_store_wait_read<0>();          // the store of the previous tile has left this warp's slab
             __syncwarp();
@@ -2340,7 +2346,7 @@ tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
         int issued = 0;
         for (int j = 0; j < my_tiles; ++j) {
             const int st = j % kStemStages;
-            if (!mbar_wait(seg_empty0 + 8 * st, ((uint32_t)(j / kStemStages) & 1u) ^ 1u, failed, status, 611)) break;
+            if (!mbar_wait_warp(seg_empty0 + 8 * st, ((uint32_t)(j / kStemStages) & 1u) ^ 1u, failed, status, 611)) break;
             stem_stage_tile(p, x, stage + st * kStemStage, stem_tile(p, (int)blockIdx.x + j * (int)gridDim.x), seg_full0 + 8 * st, lane);
             issued = j + 1;
         }
@@ -2374,7 +2380,7 @@ tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
         uint8_t* const o_tile = o_tiles + group * 16384;
         float s_acc[2] = {0.f, 0.f}, q_acc[2] = {0.f, 0.f};
         for (int j = group; j < my_tiles; j += 2) {
-            if (!mbar_wait(acc_full0 + 8 * group, (uint32_t)(j >> 1) & 1u, failed, status, 614)) break;
+            if (!mbar_wait_warp(acc_full0 + 8 * group, (uint32_t)(j >> 1) & 1u, failed, status, 614)) break;
             tc_fence_after();
             if (lane == 0) tma_store_wait_read<0>();          // the store of this group's previous tile has left the warp's slab
             __syncwarp();
@@ -2504,8 +2510,8 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
         for (int j = 0; j < my_tiles; ++j) {
             const int st = j % kStemStages;
             const uint32_t phase = (uint32_t)(j / kStemStages) & 1u;
-            if (!mbar_wait(seg_empty0 + 8 * st, phase ^ 1u, failed, status, 621)) break;
-            if (!mbar_wait(dz_empty0 + 8 * st, phase ^ 1u, failed, status, 622)) break;
+            if (!mbar_wait_warp(seg_empty0 + 8 * st, phase ^ 1u, failed, status, 621)) break;
+            if (!mbar_wait_warp(dz_empty0 + 8 * st, phase ^ 1u, failed, status, 622)) break;
             const StemTile tile = stem_tile(p, slice + j * p.slices);
             stem_stage_tile(p, x, stage + st * kStemStage, tile, seg_full0 + 8 * st, lane);
             if (lane == 0) {
@@ -2547,7 +2553,7 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
         const int row = quarter * 32 + lane;
         float* const base = partial + ((size_t)slice * p.c_out + (size_t)co_tile * 64) * 147;
         const int here = min(64, p.c_out - co_tile * 64);
-        if (my_tiles > 0 && mbar_wait(accum_bar, 0, failed, status, 625)) {
+        if (my_tiles > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 625)) {
             tc_fence_after();
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
@@ -2661,7 +2667,7 @@ tc_fc_fwd_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         const int quarter = warp % 4;
         const int co = m_tile * 128 + quarter * 32 + lane;
         float* dst = partial + (size_t)slice * p.batch * p.c_out + co;
-        const bool have = iters > 0 && mbar_wait(accum_bar, 0, failed, status, 703);
+        const bool have = iters > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 703);
         if (have) tc_fence_after();
         for (int c0 = 0; c0 < p.bnb; c0 += 32) {
             uint32_t v[32];
@@ -4000,28 +4006,39 @@ int tc_selftest_t_plan(const ConvGeom& g, int epilogue, int* plan) {
     return CKPT_OK;
 }
 
-// A wait that nothing will ever satisfy, with a short limit: the barrier is initialised for one arrival and no
-// thread arrives.  The wait gives up after `limit_cycles`, records its code in the status word like every other
-// bounded wait of this file, and the kernel returns.  Used to exercise the status path end to end.
+// A wait that runs out, with a short limit: one lane of a warp gives up after `limit_cycles`, records its code in the status
+// word like every other bounded wait of this file, and the kernel returns.  The other lanes have twice the time, and another
+// warp completes the phase as soon as the first one has given up: they may see either, and still have to leave with it (mixed
+// answers are recorded as kSelftestMixed).  Used to exercise the failure path end to end.
 namespace {
-constexpr int kSelftestCode = 9001;
-__global__ void selftest_wait_kernel(long long limit_cycles, int* status) {
+constexpr int kSelftestCode = 9001, kSelftestMixed = 9002;
+__global__ void __launch_bounds__(64) selftest_wait_kernel(long long limit_cycles, int* status) {
     __shared__ __align__(8) uint64_t bar;
-    __shared__ int failed;
+    __shared__ int failed_flag;
+    volatile int* failed = &failed_flag;
+    const uint32_t b = smem_u32(&bar);
     if (threadIdx.x == 0) {
-        failed = 0;
-        mbar_init(smem_u32(&bar), 1);
+        failed_flag = 0;
+        mbar_init(b, 1);
         fence_barrier_init();
     }
     __syncthreads();
-    if (threadIdx.x == 0) mbar_wait(smem_u32(&bar), 0, &failed, status, kSelftestCode, limit_cycles);
+    if (threadIdx.x < 32) {
+        const bool arrived = mbar_wait_warp(b, 0, failed, status, kSelftestCode, threadIdx.x == 7 ? limit_cycles : 2 * limit_cycles);
+        const uint32_t answers = __ballot_sync(0xffffffffu, arrived);
+        if (threadIdx.x == 0 && answers != 0u) atomicExch(status, kSelftestMixed);
+    } else if (threadIdx.x == 32) {
+        const long long t0 = clock64();
+        while (!*failed && clock64() - t0 < 4 * limit_cycles + kDrainCycles) {}
+        mbar_arrive(b);
+    }
 }
 }  // namespace
 
 int tc_selftest_wait(long long limit_cycles, int* device_status, void* stream) {
     if (!device_status) { set_error("no status word"); return CKPT_E_NULL; }
     if (limit_cycles < 1 || limit_cycles > 2000000000LL) { set_error("wait limit must be 1 .. 2e9 cycles"); return CKPT_E_BAD_ARG; }
-    selftest_wait_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(limit_cycles, device_status);
+    selftest_wait_kernel<<<1, 64, 0, (cudaStream_t)stream>>>(limit_cycles, device_status);
     CKPT_LAUNCH_CHECK_NAMED("selftest_wait_kernel", "bounded-wait self-test");
     return CKPT_OK;
 }

@@ -31,6 +31,17 @@ def test_single_operation_status_word():
     assert float((z.float() - ref).abs().max()) <= 6e-3 * float(ref.abs().max())
 
 
+@pytest.mark.parametrize("limit", [1, 2000, 200000])
+def test_a_warp_leaves_a_failed_wait_together(limit):
+    """One lane gives up and the barrier completes right behind it: lanes that saw the completion may not go on alone (a
+    warp that parted there would wait for itself).  9002 would mean that the lanes left with different answers."""
+    for _ in range(20):
+        ck.selftest_bounded_wait(limit)
+        with pytest.raises(ck.CkptError) as e:
+            ck.op_status()
+        assert e.value.code == -10 and e.value.status == 9001
+
+
 @pytest.mark.parametrize("graph", [False, True])
 def test_train_step_reports_a_wait_that_ran_out(graph):
     spec = wl.plain_chain(3, 64, 64, (12, 12), 4, "bf16", "sum", name="status_chain")
