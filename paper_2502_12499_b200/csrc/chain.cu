@@ -111,6 +111,7 @@ struct StepCtx {
     int64_t* stage_trace = nullptr;     // optional: live arena bytes at the end of each of the 2n+2 stages
     void* host_result = nullptr;        // capture: pinned destination of the loss and the status word (no wait)
     bool masked = false;                // the current gradient has been through the ReLU that ends the unit it enters (a residual block)
+    const void* mask_after_tap = nullptr;   // ... will have been, once the tap has its copy: the output of that unit
     char* act_buf = nullptr;            // where the activated copy of a unit's input goes (null: the workspace's own buffer)
     int64_t act_cap = 0;                // its capacity in bytes
     int* status() const { return (int*)(ws + ch->off_misc + 64); }
@@ -346,7 +347,13 @@ static int block_backward(StepCtx& c, const Unit& u, const void* x, const void* 
     if (g_out && use_tc(c.ch, u.g1, B.da, p[0], g_out) && tc_dgrad_joins(u.g1)) {
         GradientJoin join;
         join.add = dx_shortcut;
-        if (mask_out) { join.mask = x; c.masked = true; }
+        if (mask_out) {
+            // (the tap takes the gradient in front of that ReLU, which then follows as a pass of its own: the batch-norm
+            // backward behind it runs as without a tap, on the same bits)
+            if (c.ch->tap) c.mask_after_tap = x;
+            else join.mask = x;
+            c.masked = true;
+        }
         return conv_backward_pair(c, u.g1, B.da, x, p[0], pf, g_out, join);
     }
     if ((rc = conv_backward_pair(c, u.g1, B.da, x, p[0], pf, g_out))) return rc;
@@ -475,7 +482,7 @@ static int unit_backward(StepCtx& c, int64_t i, const void* x_raw, const void* y
         }
         case CKPT_UNIT_BOTTLENECK:
             if ((rc = activated(c, i - 1, x_raw, &x))) return rc;
-            if ((rc = block_backward(c, u, x, y, g_in, g_out, i > 1 && c.ch->units[i - 2].desc.kind == CKPT_UNIT_BOTTLENECK && !c.ch->tap))) return rc;
+            if ((rc = block_backward(c, u, x, y, g_in, g_out, i > 1 && c.ch->units[i - 2].desc.kind == CKPT_UNIT_BOTTLENECK))) return rc;
             break;
         default:
             set_error("unit kind %d has no backward kernel", u.desc.kind);
@@ -647,6 +654,10 @@ static int run_step(StepCtx& c, double* loss_out) {
         if (need_dx) {
             g_cur = g_next; g_in_r = next_in_r;
             if ((rc = tap_gradient(c, i - 1, g_cur))) return rc;
+            if (c.mask_after_tap) {
+                if ((rc = relu_mask_inplace(ch->dtype, rows_of(ch, i - 1) * ch->units[i - 2].out.c, g_cur, c.mask_after_tap, c.stream))) return rc;
+                c.mask_after_tap = nullptr;
+            }
         }
         if (c.policy == CKPT_POLICY_DYNAMIC) if ((rc = A.release(i))) return rc;
         if (c.stage_trace) c.stage_trace[2 * n + 1 - i] = A.live_bytes();

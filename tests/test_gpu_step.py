@@ -475,3 +475,22 @@ def test_pooling_reads_the_pending_normalisation(hw, channels):
     for u, v in zip(g_a, g_b):
         assert u.shape == v.shape
         assert np.linalg.norm(u - v) <= 2e-2 * np.linalg.norm(v) + 1e-6
+
+
+@pytest.mark.parametrize("channels,hw,batch", [(256, 14, 30), (512, 7, 70), (2048, 7, 13)])
+def test_gradient_tap_changes_no_bits(channels, hw, batch):
+    """The tap takes the gradient in front of the ReLU that ends a residual block; the batch-norm backward behind it adds
+    up as without a tap.  Tensors at which that kernel divides its rows differently when it has a mask to apply."""
+    import torch
+    block = {"kind": "bottleneck", "cin": channels, "mid": 64, "cout": channels, "stride": 1, "project": False}
+    spec = dict(units=[block, dict(block), dict(block)], input_hwc=(hw, hw, channels), batch=batch, dtype="bf16", loss="sum", name="tap")
+    params = wl.make_params(spec, seed=7, bn_affine="random")
+    x, _ = wl.make_batch(spec, seed=8)
+    runner = StepRunner(spec, params)
+    _, plain = runner.run(ck.POLICY_STORE_ALL, None, x, None)
+    tap = torch.empty(int(sum(runner.d[1:])), dtype=torch.uint8, device="cuda")
+    runner.chain.set_gradient_tap(tap)
+    _, tapped = runner.run(ck.POLICY_STORE_ALL, None, x, None)
+    runner.chain.set_gradient_tap(None)
+    for a, b in zip(plain, tapped):
+        assert np.array_equal(a, b)
