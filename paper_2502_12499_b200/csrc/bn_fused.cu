@@ -107,6 +107,8 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
     auto slot = [&](int s) { return ring + (size_t)(s % Rg::slots) * (Rg::step_bytes / 16) + tid; };
     // the forward output, rounded to its type, is positive: for bf16 above half of the smallest subnormal
     constexpr float kPositive = sizeof(T) == 2 ? 0x1p-134f : 0.f;
+    const bool all = !p.relu;
+    auto passes = [&](float v, float scale, float shift) { return all || fmaf(v, scale, shift) > kPositive; };
 
 #pragma unroll 1
     for (int s = 0; s < Rg::slots; ++s) fetch(s, true);
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
 #pragma unroll
     for (int k = 0; k < VEC; ++k) {
         sc[k] = p.stats[2 * c + ch + k];
-        sh[k] = p.relu ? p.stats[3 * c + ch + k] : INFINITY;         // without a ReLU everything passes
+        sh[k] = p.stats[3 * c + ch + k];
         s0[k] = 0.f; s1[k] = 0.f;
     }
 #pragma unroll 1
@@ -137,8 +139,12 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
                     *reinterpret_cast<uint4*>(dy + (st + u) * hop) = packed;
                 }
 #pragma unroll
-                for (int k = 0; k < VEC; ++k)
-                    if (fmaf(v[k], sc[k], sh[k]) > kPositive) { s0[k] += g[k]; s1[k] = fmaf(g[k], v[k], s1[k]); }
+                for (int k = 0; k < VEC; ++k) {
+                    // (a blocked gradient still meets its z: a NaN or an infinity there reaches the sums)
+                    const float gi = passes(v[k], sc[k], sh[k]) ? g[k] : 0.f;
+                    s0[k] += gi;
+                    s1[k] = fmaf(gi, v[k], s1[k]);
+                }
             }
         }
 #pragma unroll
@@ -294,7 +300,7 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
                 unpack<T, VEC>(from_uint4<T, VEC>(held[kThreads]), v);
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) {
-                    const float gi = fmaf(v[k], sc[k], sh[k]) > kPositive ? g[k] : 0.f;
+                    const float gi = passes(v[k], sc[k], sh[k]) ? g[k] : 0.f;
                     o[k] = fmaf(-v[k], cb[k], fmaf(sc[k], gi, -ca[k]));
                 }
                 store_vec<T, VEC>(dz + s * hop, o);

@@ -501,6 +501,35 @@ def test_bn_backward_in_one_kernel(rows, c, relu, dtype):
     assert not (off & sure).any()
 
 
+@pytest.mark.parametrize("relu", [0, 1])
+@pytest.mark.parametrize("dtype", [ck.DTYPE_F32, ck.DTYPE_BF16])
+@pytest.mark.parametrize("rows,c", [(500, 3), (70, 64), (3003, 40), (30000, 256)])
+def test_bn_backward_passes_on_nan_and_infinity(rows, c, dtype, relu):
+    """NaN and infinite values of z under finite statistics reach dgamma (also where the ReLU blocks them: 0 * inf) and dz, on
+    every path alike: separate kernels (3 channels), one cluster per channel group, co-operative launch."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(c)
+    store = torch.bfloat16 if dtype == ck.DTYPE_BF16 else torch.float32
+    z, dy = ((torch.randn((rows, c), generator=gen, device="cuda") * 1.3 + 0.2).to(store) for _ in range(2))
+    gamma = torch.rand(c, generator=gen, device="cuda") + 0.5
+    mean, inv = z.double().mean(0), (z.double().var(0, unbiased=False) + 1e-5).rsqrt()
+    stats = torch.stack((mean, inv, gamma * inv, 0.1 - mean * gamma * inv)).float()
+    z[rows // 3, 0], z[rows // 2, 1], z[rows - 1, 2] = float("nan"), float("inf"), float("-inf")
+    s, v = stats.double(), z.double()
+    g = torch.where((v * s[2] + s[3] > 0) | (relu == 0), dy.double(), torch.zeros_like(v))
+    dbeta, dgamma = g.sum(0), s[1] * ((g * v).sum(0) - s[0] * g.sum(0))
+    dz, dg, db = torch.empty_like(z), torch.empty(c, device="cuda"), torch.empty(c, device="cuda")
+    scratch = torch.empty(ck.bn_scratch_bytes(rows, c), dtype=torch.uint8, device="cuda")
+    ck.bn_relu_backward(dtype, rows, c, dy, z, gamma, stats, relu, dz, dg, db, scratch)
+    assert ck.op_status() == 0
+    assert torch.equal(torch.isfinite(dg), torch.isfinite(dgamma)) and not torch.isfinite(dg[:3]).any()
+    assert torch.isfinite(db).all()
+    scale = float(g.abs().sum(0).max())               # float32 sums of `rows` terms
+    assert float((db.double() - dbeta).abs().max()) <= 1e-5 * scale
+    assert float((dg.double() - dgamma)[3:].abs().max()) <= 1e-4 * scale if c > 3 else True
+    assert torch.isfinite(dz[:, 3:]).all() and not torch.isfinite(dz[:, :3]).any()
+
+
 @pytest.mark.parametrize("case", [
     (3, 2, 2, 512, 512, 3, 1),       # reduction shared by a cluster, smallest pixel tile
     (13, 10, 6, 512, 200, 3, 1),     # the same with partial pixel and channel tiles
