@@ -75,5 +75,11 @@ __device__ __forceinline__ RawVec<T, VEC> pack_raw(const float (&v)[VEC]) {
 // 16-byte vectors as plain words (to keep them in shared memory)
 template <typename R> __device__ __forceinline__ uint4 as_uint4(const R& r) { return *reinterpret_cast<const uint4*>(&r); }
 template <typename T, int VEC> __device__ __forceinline__ RawVec<T, VEC> from_uint4(const uint4& u) { return *reinterpret_cast<const RawVec<T, VEC>*>(&u); }
+// value k of a vector (k known at compile time)
+template <typename T> __device__ __forceinline__ float element(const uint4& u, int k) {
+    const int w = sizeof(T) == 2 ? k / 2 : k;
+    const uint32_t x = w == 0 ? u.x : w == 1 ? u.y : w == 2 ? u.z : u.w;
+    return __uint_as_float(sizeof(T) == 4 ? x : k % 2 ? x & 0xffff0000u : x << 16);
+}
 
 }  // namespace ckpt

@@ -578,3 +578,24 @@ def test_average_pool_in_a_chain(channels, hw):
     n = x.numel()
     g = tap[:n * 4].view(torch.float32)
     assert torch.allclose(g, torch.full_like(g, 1.0 / (hw[0] * hw[1])), rtol=1e-6)
+
+
+@pytest.mark.parametrize("dtype,rows,c", [(ck.DTYPE_F32, 25088, 128), (ck.DTYPE_F32, 36960, 96), (ck.DTYPE_BF16, 24156, 512), (ck.DTYPE_BF16, 100352, 64)])
+def test_bn_backward_sums_keep_their_accuracy(dtype, rows, c):
+    """dgamma and dbeta against float64.  A float32 addition errs by 2.5e-8 of its result (rms): sums of a CTA's rows by chains
+    of a few additions per thread, the rest as two floats, come to 7e-8 of the result for float32 values and 4e-8 for bfloat16
+    ones (whose products add up exactly at first); added up in float32 throughout they came to 1.1e-7 and 9e-8."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(rows)
+    store = torch.bfloat16 if dtype == ck.DTYPE_BF16 else torch.float32
+    z, dy = ((torch.randn((rows, c), generator=gen, device="cuda") * 1.4 + shift).to(store) for shift in (0.3, 0.0))
+    gamma = torch.rand(c, generator=gen, device="cuda") + 0.5
+    mean, inv = z.double().mean(0), (z.double().var(0, unbiased=False) + 1e-5).rsqrt()
+    stats = torch.stack((mean, inv, gamma * inv, 0.1 - mean * gamma * inv)).float()
+    s = stats.double()
+    dbeta, dgamma = dy.double().sum(0), ((z.double() - s[0]) * s[1] * dy.double()).sum(0)
+    dz, dg, db = torch.empty_like(z), torch.empty(c, device="cuda"), torch.empty(c, device="cuda")
+    ck.bn_relu_backward(dtype, rows, c, dy, z, gamma, stats, 0, dz, dg, db, torch.empty(ck.bn_scratch_bytes(rows, c), dtype=torch.uint8, device="cuda"))
+    bound = 9e-8 if dtype == ck.DTYPE_F32 else 6e-8
+    errors = [float((got.double() - want).norm() / want.norm()) for got, want in ((dg, dgamma), (db, dbeta))]
+    assert max(errors) <= bound, errors
