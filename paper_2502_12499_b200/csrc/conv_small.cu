@@ -189,7 +189,7 @@ int small_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw
     else unfold3x3_rows_kernel<64><<<ugrid, 256, 0, st>>>((const __nv_bfloat16*)x, (uint4*)xcol, g.n, g.h, g.w, word_aligned);
     CKPT_LAUNCH_CHECK("first-layer unfold");
     const ConvGeom u = unfolded_geom(g);
-    int rc = tc_conv_wgrad(u, dz, xcol, dwp, tc_scratch, scratch_bytes - xcol_bytes(g) - dwp_bytes(g), device_status, stream);
+    int rc = tc_conv_wgrad(u, dz, xcol, dwp, tc_scratch, scratch_bytes - xcol_bytes(g) - dwp_bytes(g), device_status, stream, SgdUpdate(), g.cout % 64 != 0);
     if (rc) return rc;
     if (paired(g)) take_paired_columns_kernel<<<(g.cout * 27 + 255) / 256, 256, 0, st>>>(dwp, dw, g.cout, 27, upd);
     else take_columns_kernel<<<(g.cout * 27 + 255) / 256, 256, 0, st>>>(dwp, dw, g.cout, 27, upd);

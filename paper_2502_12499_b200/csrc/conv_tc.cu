@@ -40,6 +40,9 @@ constexpr int kTEpi = 2;
 constexpr int kTSlabs = 2;
 constexpr int kJoinSlots = 4;
 constexpr int kThreadsT = 64 + 128 * kTEpi;           // TMA warp, MMA warp, 4 * kTEpi epilogue warps
+// Weight gradients with short accumulation chains: two epilogue warps per quarter, MMAs per chain.
+constexpr int kThreadsShort = 64 + 256;
+constexpr int kChain = 4;
 constexpr int kMaxStages = 8;
 constexpr uint32_t kSmemBudget = 200 * 1024;          // operand stages; barriers live behind them
 constexpr long long kWaitCycles = 4000000000LL;       // ~2 s at 2 GHz: far beyond any legitimate wait
@@ -1417,7 +1420,14 @@ struct WgradParams {
     int stages;
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
+// SHORT: the tensor core cuts its running sum off at every MMA, toward zero, so that the error of a sum grows with the
+// number of MMAs behind it (relative, in norm: 2.6e-7 after 256 pixels, 2e-6 after 4000), where float32 additions that round
+// to nearest stay at 1e-7 to 4e-7.  Shapes whose weight gradient the CUDA cores used to sum keep that accuracy: after
+// kChain MMAs (64 pixels) the accumulator is added to registers of the epilogue warps, under the MMAs of the next 64 pixels
+// into the other half of tensor memory (48 -> 48 at 96 x 96, 16 images 2.1e-6 -> 1.6e-7, CUDA cores 3.9e-7; 96 -> 512 at
+// 36 x 61, 11 images 2.1e-6 -> 1.9e-7, CUDA cores 6e-7; the training step of a 48-channel VGG-16 on 96 x 96 pixels 2.7 %).
+template <bool SHORT>
+__global__ void __launch_bounds__(SHORT ? kThreadsShort : kThreads, 1)
 tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
                      const __grid_constant__ CUtensorMap map_out, float* __restrict__ partial, WgradParams p, SgdUpdate upd, int* status) {
     extern __shared__ uint8_t smem_raw[];
@@ -1443,16 +1453,18 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     const int tile_end = min(p.total_tiles, tile_begin + p.tiles_per_slice);
     const int iters = tile_end - tile_begin;
     const uint32_t n_cols = (uint32_t)nb_here * 64;
-    const uint32_t tmem_cols = n_cols <= 64 ? 64 : (n_cols <= 128 ? 128 : 256);
+    const uint32_t tmem_cols = SHORT ? 512 : n_cols <= 64 ? 64 : (n_cols <= 128 ? 128 : 256);
 
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (kMaxStages + s); };
-    const uint32_t accum_bar = bars + 8u * (2 * kMaxStages);
+    const uint32_t accum_bar = bars + 8u * (2 * kMaxStages);      // SHORT: full[2], empty[2]
+    const uint32_t accum_empty = accum_bar + 16u;
 
     if (threadIdx.x == 0) {
         failed_flag = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         mbar_init(accum_bar, 1);
+        if (SHORT) { mbar_init(accum_bar + 8u, 1); mbar_init(accum_empty, 256); mbar_init(accum_empty + 8u, 256); }
         fence_barrier_init();
         tma_prefetch_desc(&map_dz);
         tma_prefetch_desc(&map_x);
@@ -1498,6 +1510,7 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     } else if (warp == 1 && lane == 0) {
         const uint32_t idesc = instr_desc(128, (int)n_cols, 1, 1);
         bool ok = true;
+        int chain = 0;
         for (int it = 0; it < iters && ok; ++it) {
             const int s = it % p.stages;
             const uint32_t phase = (uint32_t)(it / p.stages) & 1u;
@@ -1505,79 +1518,126 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             tc_fence_after();
             const uint32_t a_addr = base + (uint32_t)s * stage_bytes;
             const uint32_t a_lo = desc_lo(a_addr, box_bytes), b_lo = desc_lo(a_addr + 2 * box_bytes, box_bytes), hi = desc_hi(1024u);
-            const int k_steps = p.px / 16;
+            const int k_steps = p.px / 16;          // K = 16 pixels = 2 groups of 8 rows = 2048 bytes per step
+            if constexpr (SHORT) {
+                for (int k0 = 0; k0 < k_steps; k0 += kChain, ++chain) {
+                    const uint32_t buf = (uint32_t)chain & 1u;
+                    if (!mbar_wait(accum_empty + 8u * buf, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 204)) { ok = false; break; }
+                    tc_fence_after();
+#pragma unroll
+                    for (int kk = k0; kk < k0 + kChain; ++kk)
+                        umma_bf16(tmem_base + buf * 256u, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, kk > k0 ? 1u : 0u);
+                    umma_commit(accum_bar + 8u * buf);
+                }
+                if (!ok) break;
+            } else {
 #pragma unroll 4
-            for (int kk = 0; kk < k_steps; ++kk) {  // K = 16 pixels = 2 groups of 8 rows = 2048 bytes per step
-                umma_bf16(tmem_base, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, (it > 0 || kk > 0) ? 1u : 0u);
+                for (int kk = 0; kk < k_steps; ++kk)
+                    umma_bf16(tmem_base, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, (it > 0 || kk > 0) ? 1u : 0u);
             }
             umma_commit(empty_bar(s));
         }
-        if (ok) umma_commit(accum_bar);
+        if (!SHORT && ok) umma_commit(accum_bar);
     } else if (warp >= 2) {
         // Thread l of a warp holds row l of each 32 x 32 block; the block goes to shared memory (swizzled rows of 128
         // bytes, over operand stages that the tensor core has read) and leaves as one tile store, clipped at the last
         // input channel of the tap and the last output channel.  (Turned blocks stored by the lanes, 128 bytes per
         // instruction, kept the last 10 us of short reductions: 256 -> 1024 at 13 x 11, 21 images 22.6 -> 15.3 us with the slice sum.)
-        const int quarter = warp % 4;
+        const int quarter = warp % 4, half = SHORT ? (warp - 2) / 4 : 0;      // SHORT: half of every 64 columns
         const int co_first = co_tile * 128 + quarter * 32;
         const int co = co_first + lane;
         const bool valid = co < p.c_out;
         const size_t row_elems = (size_t)p.k * p.k * p.c_in;
         float* dst_row = partial + ((size_t)slice * p.c_out + (valid ? co : 0)) * row_elems;
-        if (iters > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 203)) {
-            tc_fence_after();
-            const int slabs = min(8, (int)((uint32_t)p.stages * stage_bytes / (4u * 4096u)));
-            int count = 0;
-            for (int j = 0; j < nb_here; ++j) {
-                const int tap = (blk_begin + j) / cin_blocks, ch0 = (blk_begin + j) % cin_blocks * 64;
-                for (int c0 = 0; c0 < 64; c0 += 32, ++count) {
-                    if (ch0 + c0 >= p.c_in) break;
-                    // a gradient that is complete here updates its filter at once: 64 bytes of a row per lane (the update in a
-                    // pass of its own reads the gradient again: 64 us more for a 25088 x 4096 matrix)
-                    __nv_bfloat16* const w_row = upd.w && valid ? (__nv_bfloat16*)upd.w + (size_t)co * row_elems + (size_t)tap * p.c_in + ch0 + c0 : nullptr;
-                    uint4 w_old[4];
-                    if (w_row) {
+        const int slabs = SHORT ? min(4, (int)((uint32_t)p.stages * stage_bytes / (8u * 4096u))) : min(8, (int)((uint32_t)p.stages * stage_bytes / (4u * 4096u)));
+        int count = 0;
+        // columns c0 .. c0 + 31 of block j, `get` filling them in
+        auto put = [&](int j, int c0, auto get) {
+            const int tap = (blk_begin + j) / cin_blocks, ch0 = (blk_begin + j) % cin_blocks * 64;
+            if (ch0 + c0 >= p.c_in) return;
+            // a gradient that is complete here updates its filter at once: 64 bytes of a row per lane (the update in a
+            // pass of its own reads the gradient again: 64 us more for a 25088 x 4096 matrix)
+            __nv_bfloat16* const w_row = upd.w && valid ? (__nv_bfloat16*)upd.w + (size_t)co * row_elems + (size_t)tap * p.c_in + ch0 + c0 : nullptr;
+            uint4 w_old[4];
+            if (w_row) {
 #pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (ch0 + c0 + 8 * q < p.c_in) w_old[q] = reinterpret_cast<const uint4*>(w_row)[q];
-                    }
-                    uint32_t v[32];
-                    tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(j * 64 + c0), v);
-                    if (w_row) {
+                for (int q = 0; q < 4; ++q)
+                    if (ch0 + c0 + 8 * q < p.c_in) w_old[q] = reinterpret_cast<const uint4*>(w_row)[q];
+            }
+            uint32_t v[32];
+            get(v);
+            if (w_row) {
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            if (ch0 + c0 + 8 * q >= p.c_in) break;
-                            __nv_bfloat162* const pr = reinterpret_cast<__nv_bfloat162*>(&w_old[q]);
+                for (int q = 0; q < 4; ++q) {
+                    if (ch0 + c0 + 8 * q >= p.c_in) break;
+                    __nv_bfloat162* const pr = reinterpret_cast<__nv_bfloat162*>(&w_old[q]);
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float2 o = __bfloat1622float2(pr[e]);
-                                pr[e] = __floats2bfloat162_rn(fmaf(-upd.lr, __uint_as_float(v[8 * q + 2 * e]), o.x), fmaf(-upd.lr, __uint_as_float(v[8 * q + 2 * e + 1]), o.y));
-                            }
-                            reinterpret_cast<uint4*>(w_row)[q] = w_old[q];
-                        }
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 o = __bfloat1622float2(pr[e]);
+                        pr[e] = __floats2bfloat162_rn(fmaf(-upd.lr, __uint_as_float(v[8 * q + 2 * e]), o.x), fmaf(-upd.lr, __uint_as_float(v[8 * q + 2 * e + 1]), o.y));
                     }
-                    if (!p.tile_store) {
-                        if (valid) {
-#pragma unroll
-                            for (int e = 0; e < 32; ++e)
-                                if (ch0 + c0 + e < p.c_in) dst_row[(size_t)tap * p.c_in + ch0 + c0 + e] = __uint_as_float(v[e]);
-                        }
-                        continue;
-                    }
-                    const uint32_t slab = base + (uint32_t)(quarter * slabs + count % slabs) * 4096u;
-                    if (count >= slabs) {
-                        if (lane == 0) tma_store_wait_read<0>();
-                        __syncwarp();
-                    }
-                    block_to_slab(v, slab, lane);
-                    if (lane == 0 && co_first < p.c_out) {
-                        tma_store_4d(&map_out, slab, ch0 + c0, tap, co_first, slice);
-                        tma_store_commit();
-                    }
+                    reinterpret_cast<uint4*>(w_row)[q] = w_old[q];
                 }
             }
+            if (!p.tile_store) {
+                if (valid) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        if (ch0 + c0 + e < p.c_in) dst_row[(size_t)tap * p.c_in + ch0 + c0 + e] = __uint_as_float(v[e]);
+                }
+                return;
+            }
+            const uint32_t slab = base + (uint32_t)((SHORT ? warp - 2 : quarter) * slabs + count % slabs) * 4096u;
+            if (count++ >= slabs) {
+                if (lane == 0) tma_store_wait_read<0>();
+                __syncwarp();
+            }
+            block_to_slab(v, slab, lane);
+            if (lane == 0 && co_first < p.c_out) {
+                tma_store_4d(&map_out, slab, ch0 + c0, tap, co_first, slice);
+                tma_store_commit();
+            }
+        };
+        if (SHORT && iters > 0) {
+            float acc[4][32];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int e = 0; e < 32; ++e) acc[j][e] = 0.f;
+            const int chains = iters * (p.px / (16 * kChain));
+            bool ok = true;
+            for (int chain = 0; chain < chains; ++chain) {
+                const uint32_t buf = (uint32_t)chain & 1u;
+                if (!mbar_wait_warp(accum_bar + 8u * buf, (uint32_t)(chain >> 1) & 1u, failed, status, 205)) { ok = false; break; }
+                tc_fence_after();
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (j >= nb_here || (blk_begin + j) % cin_blocks * 64 + half * 32 >= p.c_in) continue;
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * 256u + (uint32_t)(j * 64 + half * 32), v);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) acc[j][e] += __uint_as_float(v[e]);
+                }
+                tc_fence_before();
+                mbar_arrive(accum_empty + 8u * buf);
+            }
+            if (ok) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (j < nb_here)
+                        put(j, half * 32, [&](uint32_t (&v)[32]) {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(acc[j][e]);
+                        });
+            }
             if (lane == 0) tma_store_wait_all();
-        } else if (iters == 0 && valid) {
+        } else if (!SHORT && iters > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 203)) {
+            tc_fence_after();
+            for (int j = 0; j < nb_here; ++j)
+                for (int c0 = 0; c0 < 64; c0 += 32)
+                    put(j, c0, [&](uint32_t (&v)[32]) { tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(j * 64 + c0), v); });
+            if (lane == 0) tma_store_wait_all();
+        } else if (iters == 0 && valid && half == 0) {
             for (int j = 0; j < nb_here; ++j) {
                 const int tap = (blk_begin + j) / cin_blocks, ch0 = (blk_begin + j) % cin_blocks * 64;
                 for (int c = ch0; c < min(ch0 + 64, p.c_in); ++c) dst_row[(size_t)tap * p.c_in + c] = 0.f;
@@ -1749,7 +1809,9 @@ struct WRowsParams {
     int total_cols;              // 3 horizontal offsets x 64-channel blocks (4 in the pair view); the last CTA may have one column only
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
+// SHORT: as in tc_conv_wgrad_kernel, one column per CTA.
+template <bool SHORT>
+__global__ void __launch_bounds__(SHORT ? kThreadsShort : kThreads, 1)
 tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
                      const __grid_constant__ CUtensorMap map_out, float* __restrict__ partial, WRowsParams p, int* status) {
     extern __shared__ uint8_t smem_raw[];
@@ -1760,7 +1822,8 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     volatile int* failed = &failed_flag;
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (kMaxStages + s); };
-    const uint32_t accum_bar = bars + 8u * (2 * kMaxStages);
+    const uint32_t accum_bar = bars + 8u * (2 * kMaxStages);      // SHORT: full[2], empty[2]
+    const uint32_t accum_empty = accum_bar + 16u;
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int slice = blockIdx.x, pair = blockIdx.y, co_tile = blockIdx.z;
@@ -1771,6 +1834,7 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         failed_flag = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         mbar_init(accum_bar, 1);
+        if (SHORT) { mbar_init(accum_bar + 8u, 1); mbar_init(accum_empty, 256); mbar_init(accum_empty + 8u, 256); }
         fence_barrier_init();
         tma_prefetch_desc(&map_dz);
         tma_prefetch_desc(&map_x);
@@ -1810,58 +1874,104 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         const uint32_t idesc = instr_desc(128, 192, 1, 1);
         const int ksteps = p.th / 2;                 // 16 pixels (two 8-pixel rows) per MMA
         bool ok = true;
+        int chain = 0;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int s = j % p.stages;
             if (!mbar_wait(full_bar(s), (uint32_t)(j / p.stages) & 1u, failed, status, 702)) { ok = false; break; }
             tc_fence_after();
             const uint32_t dz_addr = base + (uint32_t)s * p.stage_bytes;
+            if constexpr (SHORT) {
+                const uint32_t a_lo = desc_lo(dz_addr, p.dz_box), b_lo = desc_lo(dz_addr + 2 * p.dz_box, 1024u), hi = desc_hi(1024u);
+                for (int k0 = 0; k0 < ksteps; k0 += kChain, ++chain) {
+                    const uint32_t buf = (uint32_t)chain & 1u;
+                    if (!mbar_wait(accum_empty + 8u * buf, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 704)) { ok = false; break; }
+                    tc_fence_after();
+                    for (int kk = k0; kk < min(k0 + kChain, ksteps); ++kk)
+                        umma_bf16(tmem_base + buf * 256u, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, kk > k0 ? 1u : 0u);
+                    umma_commit(accum_bar + 8u * buf);
+                }
+                if (!ok) break;
+            } else {
 #pragma unroll 1
-            for (int c = 0; c < ncols; ++c) {
-                const uint32_t x_addr = dz_addr + 2 * p.dz_box + (uint32_t)c * p.patch_bytes;
-                const uint32_t a_lo = desc_lo(dz_addr, p.dz_box), b_lo = desc_lo(x_addr, 1024u), hi = desc_hi(1024u);
+                for (int c = 0; c < ncols; ++c) {
+                    const uint32_t x_addr = dz_addr + 2 * p.dz_box + (uint32_t)c * p.patch_bytes;
+                    const uint32_t a_lo = desc_lo(dz_addr, p.dz_box), b_lo = desc_lo(x_addr, 1024u), hi = desc_hi(1024u);
 #pragma unroll 2
-                for (int kk = 0; kk < ksteps; ++kk)
-                    umma_bf16(tmem_base + (uint32_t)c * 192, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, (j > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < ksteps; ++kk)
+                        umma_bf16(tmem_base + (uint32_t)c * 192, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, (j > 0 || kk > 0) ? 1u : 0u);
+                }
             }
             umma_commit(empty_bar(s));
         }
-        if (ok) umma_commit(accum_bar);
+        if (!SHORT && ok) umma_commit(accum_bar);
     } else if (warp >= 2) {
         // Blocks of 32 output channels x 32 input channels of a tap leave as tile stores through the operand stages, as in
         // tc_conv_wgrad_kernel (rows stored by the lanes in 16-byte pieces: 21.9 us with the fold at 64 -> 64, 56 x 56, 32
         // images, against 17.5; 128 -> 128 at 16 x 16, 128 images 26.9 against 17.6).
-        const int quarter = warp % 4;
+        const int quarter = warp % 4, half = SHORT ? (warp - 2) / 4 : 0;
         const int co_first = co_tile * 128 + quarter * 32, co = co_first + lane;
         const bool valid = co < p.c_out;
         const size_t row_elems = (size_t)p.row_elems;
         float* dst_row = partial + ((size_t)slice * p.c_out + (valid ? co : 0)) * row_elems;
-        if (my_tiles > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 703)) {
-            tc_fence_after();
-            const int slabs = min(12, (int)((uint32_t)p.stages * p.stage_bytes / (4u * 4096u)));
-            int count = 0;
-            for (int c = 0; c < ncols; ++c) {
-                const int col = p.cols * pair + c, cib = col / 3, dx = col % 3;
+        const int slabs = SHORT ? min(4, (int)((uint32_t)p.stages * p.stage_bytes / (8u * 4096u))) : min(12, (int)((uint32_t)p.stages * p.stage_bytes / (4u * 4096u)));
+        int count = 0;
+        // columns c0 .. c0 + 31 of filter row dy of column c, `get` filling them in
+        auto put = [&](int c, int dy, int c0, auto get) {
+            const int col = p.cols * pair + c, cib = col / 3, dx = col % 3;
+            const int tap = p.pairview ? col * 3 + dy : dy * 3 + dx, ch0 = p.pairview ? 0 : cib * 64;
+            if (c0 >= (p.pairview ? 64 : p.c_in - ch0)) return;
+            uint32_t v[32];
+            get(v);
+            const uint32_t slab = base + (uint32_t)((SHORT ? warp - 2 : quarter) * slabs + count % slabs) * 4096u;
+            if (count++ >= slabs) {
+                if (lane == 0) tma_store_wait_read<0>();
+                __syncwarp();
+            }
+            block_to_slab(v, slab, lane);
+            if (lane == 0 && co_first < p.c_out) {
+                tma_store_4d(&map_out, slab, ch0 + c0, tap, co_first, slice);
+                tma_store_commit();
+            }
+        };
+        if (SHORT && my_tiles > 0) {
+            float acc[3][32];
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                for (int e = 0; e < 32; ++e) acc[dy][e] = 0.f;
+            const int chains = my_tiles * ((p.th / 2 + kChain - 1) / kChain);
+            bool ok = true;
+            for (int chain = 0; chain < chains; ++chain) {
+                const uint32_t buf = (uint32_t)chain & 1u;
+                if (!mbar_wait_warp(accum_bar + 8u * buf, (uint32_t)(chain >> 1) & 1u, failed, status, 705)) { ok = false; break; }
+                tc_fence_after();
+#pragma unroll
                 for (int dy = 0; dy < 3; ++dy) {
-                    const int tap = p.pairview ? col * 3 + dy : dy * 3 + dx, ch0 = p.pairview ? 0 : cib * 64;
-                    const int here = p.pairview ? 64 : p.c_in - ch0;
-                    for (int c0 = 0; c0 < 64 && c0 < here; c0 += 32, ++count) {
-                        uint32_t v[32];
-                        tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * 192 + dy * 64 + c0), v);
-                        const uint32_t slab = base + (uint32_t)(quarter * slabs + count % slabs) * 4096u;
-                        if (count >= slabs) {
-                            if (lane == 0) tma_store_wait_read<0>();
-                            __syncwarp();
-                        }
-                        block_to_slab(v, slab, lane);
-                        if (lane == 0 && co_first < p.c_out) {
-                            tma_store_4d(&map_out, slab, ch0 + c0, tap, co_first, slice);
-                            tma_store_commit();
-                        }
-                    }
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * 256u + (uint32_t)(dy * 64 + half * 32), v);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) acc[dy][e] += __uint_as_float(v[e]);
                 }
+                tc_fence_before();
+                mbar_arrive(accum_empty + 8u * buf);
+            }
+            if (ok) {
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy)
+                    put(0, dy, half * 32, [&](uint32_t (&v)[32]) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(acc[dy][e]);
+                    });
             }
             if (lane == 0) tma_store_wait_all();
-        } else if (my_tiles == 0 && valid) {
+        } else if (!SHORT && my_tiles > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 703)) {
+            tc_fence_after();
+            for (int c = 0; c < ncols; ++c)
+                for (int dy = 0; dy < 3; ++dy)
+                    for (int c0 = 0; c0 < 64; c0 += 32)
+                        put(c, dy, c0, [&](uint32_t (&v)[32]) { tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * 192 + dy * 64 + c0), v); });
+            if (lane == 0) tma_store_wait_all();
+        } else if (my_tiles == 0 && valid && half == 0) {
             for (int c = 0; c < ncols; ++c) {
                 const int col = p.cols * pair + c, cib = col / 3, dx = col % 3;
                 for (int dy = 0; dy < 3; ++dy) {
@@ -2459,7 +2569,10 @@ tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
 // past the end of the row are zero-filled, and the gathered rows there are zeros too).  Each CTA keeps its two
 // accumulators over all its tiles and leaves partial[slice][c_out][147]; the slices are added in a fixed order.
 // Warps 0-7 gather, warp 8 issues the MMAs, warp 9 copies segments and dz tiles, warps 10-13 write the partial sums at the end.
-__global__ void __launch_bounds__(kStemWgradThreads, 1)
+// SHORT (output channels that are no multiple of 64): accumulation chains of 64 pixels, as in tc_conv_wgrad_kernel; warps
+// 10-13 add up the first accumulator, 14-17 the second (3 -> 32 at 224 x 224, 16 images 1.3e-6 -> 1.5e-7, CUDA cores 3.6e-7).
+template <bool SHORT>
+__global__ void __launch_bounds__(kStemWgradThreads + (SHORT ? 128 : 0), 1)
 tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant__ CUtensorMap map_dz, float* __restrict__ partial,
                      StemParams p, int* status) {
     extern __shared__ uint8_t smem_raw[];
@@ -2467,13 +2580,13 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
     uint8_t* const a_tiles = smem_al;                       // [2][atoms 2, 0, 1][128 pixels][128 bytes]
     uint8_t* const dz_tiles = smem_al + 2 * kStemATile;     // [kStemStages][128 pixels][64 channels]
     uint8_t* const stage = dz_tiles + kStemStages * 16384;  // [kStemStages][7][kStemSegBytes]
-    __shared__ __align__(8) uint64_t bar_mem[5 + 4 * kStemStages];
+    __shared__ __align__(8) uint64_t bar_mem[8 + 4 * kStemStages];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int failed_flag;
     volatile int* failed = &failed_flag;
     const uint32_t bars = smem_u32(bar_mem);
-    const uint32_t a_full0 = bars, a_empty0 = bars + 16, accum_bar = bars + 32;
-    const uint32_t seg_full0 = bars + 40, seg_empty0 = seg_full0 + 8 * kStemStages;
+    const uint32_t a_full0 = bars, a_empty0 = bars + 16, accum_bar = bars + 32, accum_empty = accum_bar + 16;     // SHORT: full[2], empty[2]
+    const uint32_t seg_full0 = bars + 64, seg_empty0 = seg_full0 + 8 * kStemStages;
     const uint32_t dz_full0 = seg_empty0 + 8 * kStemStages, dz_empty0 = dz_full0 + 8 * kStemStages;
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -2488,6 +2601,7 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
             mbar_init(dz_full0 + 8 * b, 1); mbar_init(dz_empty0 + 8 * b, 1);
         }
         mbar_init(accum_bar, 1);
+        if (SHORT) { mbar_init(accum_bar + 8u, 1); mbar_init(accum_empty, 256); mbar_init(accum_empty + 8u, 256); }
         fence_barrier_init();
         tma_prefetch_desc(&map_dz);
     }
@@ -2497,7 +2611,7 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
         if (threadIdx.x == 0) atomicCAS(status, 0, 620);
         return;
     }
-    if (warp == 8) tmem_alloc(smem_u32(&tmem_base_slot), 128);
+    if (warp == 8) tmem_alloc(smem_u32(&tmem_base_slot), SHORT ? 256 : 128);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -2530,6 +2644,7 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
         if (lane == 0) {
             const uint32_t idesc = instr_desc(128, 64, 1, 1);
             bool ok = true;
+            int chain = 0;
             for (int j = 0; j < my_tiles && ok; ++j) {
                 const int buf = j & 1, st = j % kStemStages;
                 if (!mbar_wait(a_full0 + 8 * buf, (uint32_t)(j >> 1) & 1u, failed, status, 623)) { ok = false; break; }
@@ -2539,40 +2654,80 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
                 const uint32_t dz_addr = smem_u32(dz_tiles + st * 16384);
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {            // 16 pixels per MMA
+                    const bool starts = SHORT ? kk % kChain == 0 : j == 0 && kk == 0;
+                    if (SHORT && starts) {
+                        const uint32_t b = (uint32_t)chain & 1u;
+                        if (!mbar_wait(accum_empty + 8u * b, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 628)) { ok = false; break; }
+                        tc_fence_after();
+                    }
+                    const uint32_t acc = tmem_base + (SHORT ? ((uint32_t)chain & 1u) * 128u : 0u);
                     const uint64_t bd = smem_desc(dz_addr + kk * 2048, 8192, 1024);
-                    umma_bf16(tmem_base, smem_desc(a_addr + stem_atom_offset(0) + kk * 2048, 16384, 1024), bd, idesc, (j > 0 || kk > 0) ? 1u : 0u);
-                    umma_bf16(tmem_base + 64u, smem_desc(a_addr + stem_atom_offset(2) + kk * 2048, 16384, 1024), bd, idesc, (j > 0 || kk > 0) ? 1u : 0u);
+                    umma_bf16(acc, smem_desc(a_addr + stem_atom_offset(0) + kk * 2048, 16384, 1024), bd, idesc, starts ? 0u : 1u);
+                    umma_bf16(acc + 64u, smem_desc(a_addr + stem_atom_offset(2) + kk * 2048, 16384, 1024), bd, idesc, starts ? 0u : 1u);
+                    if (SHORT && kk % kChain == kChain - 1) { umma_commit(accum_bar + 8u * ((uint32_t)chain & 1u)); ++chain; }
                 }
+                if (!ok) break;
                 umma_commit(a_empty0 + 8 * buf);
                 umma_commit(dz_empty0 + 8 * st);
             }
-            if (ok) umma_commit(accum_bar);
+            if (!SHORT && ok) umma_commit(accum_bar);
         }
     } else {
         const int quarter = warp % 4;
         const int row = quarter * 32 + lane;
         float* const base = partial + ((size_t)slice * p.c_out + (size_t)co_tile * 64) * 147;
         const int here = min(64, p.c_out - co_tile * 64);
-        if (my_tiles > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 625)) {
+        // columns c0 .. c0 + 31 of accumulator `half`, one row of it per lane
+        auto put = [&](int half, int c0, const uint32_t (&v)[32]) {
+            const int k = half * 128 + row, r = k / 24, tt = k % 24;
+            const bool valid = (half == 0 || row < 64) && r < 7 && tt < 21;
+            float* dst = base + r * 21 + tt;
+            if (valid) {
+#pragma unroll
+                for (int e = 0; e < 32; ++e)
+                    if (c0 + e < here) dst[(size_t)(c0 + e) * 147] = __uint_as_float(v[e]);
+            }
+        };
+        const uint32_t lanes = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        if (SHORT && my_tiles > 0) {
+            const int half = (warp - 10) / 4;
+            float acc[2][32];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) { acc[0][e] = 0.f; acc[1][e] = 0.f; }
+            bool ok = true;
+            for (int chain = 0; chain < my_tiles * (8 / kChain); ++chain) {
+                const uint32_t b = (uint32_t)chain & 1u;
+                if (!mbar_wait_warp(accum_bar + 8u * b, (uint32_t)(chain >> 1) & 1u, failed, status, 629)) { ok = false; break; }
+                tc_fence_after();
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    uint32_t v[32];
+                    tmem_ld32(lanes + b * 128u + (uint32_t)(half * 64 + q * 32), v);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) acc[q][e] += __uint_as_float(v[e]);
+                }
+                tc_fence_before();
+                mbar_arrive(accum_empty + 8u * b);
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t v[32];
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(acc[q][e]);
+                if (ok) put(half, q * 32, v);
+            }
+        } else if (!SHORT && my_tiles > 0 && mbar_wait_warp(accum_bar, 0, failed, status, 625)) {
             tc_fence_after();
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int k = half * 128 + row, r = k / 24, tt = k % 24;
-                const bool valid = (half == 0 || row < 64) && r < 7 && tt < 21;
-                float* dst = base + r * 21 + tt;
+            for (int half = 0; half < 2; ++half)
 #pragma unroll
                 for (int c0 = 0; c0 < 64; c0 += 32) {
                     uint32_t v[32];
-                    tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 64 + c0), v);
-                    if (valid) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (c0 + e < here) dst[(size_t)(c0 + e) * 147] = __uint_as_float(v[e]);
-                    }
+                    tmem_ld32(lanes + (uint32_t)(half * 64 + c0), v);
+                    put(half, c0, v);
                 }
-            }
         } else if (my_tiles == 0) {
-            for (int i = threadIdx.x - (kStemGather + 64); i < here * 147; i += 128) base[i] = 0.f;
+            for (int i = threadIdx.x - (kStemGather + 64); i < here * 147; i += SHORT ? 256 : 128) base[i] = 0.f;
         }
     }
     tc_fence_before();
@@ -2580,7 +2735,7 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
     if (warp == 8) {
         __syncwarp();
         tc_fence_after();
-        tmem_dealloc(tmem_base, 128);
+        tmem_dealloc(tmem_base, SHORT ? 256 : 128);
     }
 }
 
@@ -3439,6 +3594,9 @@ constexpr int WROWS_MIN_W = 14;
 bool wgrad_rows_applies(const ConvGeom& g) {
     return g.k == 3 && g.pad == 1 && g.stride == 1 && (g.cin % 128 == 0 || g.cin % 64) && g.cin % 8 == 0 && g.cout % 8 == 0 && g.w >= WROWS_MIN_W && g.h >= 8;
 }
+// Shapes that leave part of a 64-channel block to zero fill, whose weight gradients used to be float32 sums of the CUDA cores
+// (a 1x1 filter of stride 1 with whole blocks of input channels never was): accumulation chains of 64 pixels.
+bool wgrad_short_chains(const ConvGeom& g) { return (g.cin % 64 || g.cout % 64) && !(g.k == 1 && g.stride == 1 && g.cin % 64 == 0); }
 void wgrad_rows_plan(const ConvGeom& g, WRowsParams* p, int* pairs, int* co_tiles) {
     p->H = g.h; p->W = g.w; p->N = g.n; p->c_out = g.cout; p->c_in = g.cin;
     const int nt = (g.h + 15) / 16;
@@ -3447,7 +3605,8 @@ void wgrad_rows_plan(const ConvGeom& g, WRowsParams* p, int* pairs, int* co_tile
     p->tiles_w = (g.w + 7) / 8;
     p->m_tiles = p->tiles_w * p->tiles_h * g.n;
     p->total_cols = 3 * ((g.cin + 63) / 64);
-    *pairs = (p->total_cols + 1) / 2;
+    p->cols = wgrad_short_chains(g) ? 1 : 2;
+    *pairs = (p->total_cols + p->cols - 1) / p->cols;
     *co_tiles = (g.cout + 127) / 128;
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
@@ -3456,11 +3615,10 @@ void wgrad_rows_plan(const ConvGeom& g, WRowsParams* p, int* pairs, int* co_tile
     p->slices = std::max(1, std::min(sms / base_ctas, p->m_tiles));
     p->dz_box = (uint32_t)(8 * p->th) * 128;
     p->patch_bytes = (uint32_t)(8 * (p->th + 2)) * 128;
-    p->stage_bytes = 2 * p->dz_box + 2 * p->patch_bytes;
+    p->stage_bytes = 2 * p->dz_box + (uint32_t)p->cols * p->patch_bytes;
     p->stages = std::max(2, std::min<int>(kMaxStages, (int)((208 * 1024) / p->stage_bytes)));
     p->pairview = 0;
     p->row_elems = 9 * g.cin;
-    p->cols = 2;
 }
 
 // 64 input channels through the same kernel.  Two horizontally adjacent pixels are read as one pixel of twice the
@@ -3676,12 +3834,14 @@ int stem_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw,
     if (rc) return rc;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_wgrad_stem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemWgradSmem);
+        cudaError_t e = cudaFuncSetAttribute(tc_wgrad_stem_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemWgradSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_wgrad_stem_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemWgradSmem);
         if (e != cudaSuccess) return cuda_fail(e, "shared-memory opt-in of the stem wgrad kernel");
         attr_set = true;
     }
     dim3 grid((unsigned)p.slices, (unsigned)((g.cout + 63) / 64));
-    tc_wgrad_stem_kernel<<<grid, kStemWgradThreads, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
+    if (g.cout % 64) tc_wgrad_stem_kernel<true><<<grid, kStemWgradThreads + 128, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
+    else tc_wgrad_stem_kernel<false><<<grid, kStemWgradThreads, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_stem_kernel", "stem conv wgrad (tensor cores)");
     return slice_sum((const float*)scratch, dw, (int64_t)g.cout * 147, p.slices, st, upd);
 }
@@ -3880,7 +4040,8 @@ int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, vo
 static int wgrad_rows_attr() {
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_wgrad_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(tc_wgrad_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_wgrad_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024);
         if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
         attr_set = true;
     }
@@ -3888,7 +4049,7 @@ static int wgrad_rows_attr() {
 }
 
 int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes,
-                  int* device_status, void* stream, const SgdUpdate& upd) {
+                  int* device_status, void* stream, const SgdUpdate& upd, bool short_chains) {
     if (!device_status) { set_error("no status word"); return CKPT_E_NULL; }
     if (wgrad_pairview_applies(g) && (uintptr_t)dw % 16 == 0 && (uintptr_t)upd.w % 16 == 0) {      // the fold stores float4; otherwise the 64-channel kernel below
         WRowsParams p;
@@ -3907,7 +4068,7 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         dim3 grid(p.slices, 4 / p.cols, co_tiles);
         CUtensorMap mo;
         if ((rc = make_partial_map(&mo, (float*)scratch, 64, 12, 2 * g.cout, p.slices))) return rc;
-        tc_wgrad_rows_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
+        tc_wgrad_rows_kernel<false><<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_rows_kernel (pixel pairs)", "conv wgrad, 64 input channels as pixel pairs (tensor cores)");
         pairview_fold_kernel<8><<<(unsigned)((g.cout * 144 + 31) / 32), dim3(32, 8), 0, st>>>((const float*)scratch, dw, g.cout, p.slices, upd);
         CKPT_LAUNCH_CHECK_NAMED("pairview_fold_kernel", "wgrad pair fold");
@@ -3954,7 +4115,8 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         dim3 grid(p.slices, pairs, co_tiles);
         CUtensorMap mo;
         if ((rc = make_partial_map(&mo, (float*)scratch, g.cin, 9, g.cout, p.slices))) return rc;
-        tc_wgrad_rows_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
+        if (wgrad_short_chains(g)) tc_wgrad_rows_kernel<true><<<grid, kThreadsShort, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
+        else tc_wgrad_rows_kernel<false><<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_rows_kernel", "conv wgrad, shared vertical taps (tensor cores)");
         return slice_sum((const float*)scratch, dw, elems, p.slices, st, upd);
     }
@@ -3971,10 +4133,13 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
     cudaStream_t st = (cudaStream_t)stream;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
+        cudaError_t e = cudaFuncSetAttribute(tc_conv_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_conv_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
         if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
         attr_set = true;
     }
+    const bool chains = (short_chains || wgrad_short_chains(g)) && p.tiles_per_slice * p.px > 16 * kChain;       // (one chain is short as it is)
+    if (chains) p.stages = std::max(p.stages, (8 * 4096 + (2 + p.nb) * p.px * 128 - 1) / ((2 + p.nb) * p.px * 128));     // a slab per epilogue warp
     const size_t smem = (size_t)p.stages * (2 + p.nb) * p.px * 128 + 1024 + 256;
     float* target = slices > 1 ? (float*)scratch : dw;
     CUtensorMap mo;
@@ -3983,7 +4148,8 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
     if (p.tile_store && (rc = make_partial_map(&mo, target, g.cin, g.k * g.k, g.cout, slices))) return rc;
     dim3 grid(slices, groups, co_tiles);
     const bool update = slices == 1 && upd.w && upd.dtype == CKPT_DTYPE_BF16 && (uintptr_t)upd.w % 16 == 0;
-    tc_conv_wgrad_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, mo, target, p, update ? upd : SgdUpdate(), device_status);
+    if (chains) tc_conv_wgrad_kernel<true><<<grid, kThreadsShort, smem, st>>>(mdz, mx, mo, target, p, update ? upd : SgdUpdate(), device_status);
+    else tc_conv_wgrad_kernel<false><<<grid, kThreads, smem, st>>>(mdz, mx, mo, target, p, update ? upd : SgdUpdate(), device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_wgrad_kernel", "conv wgrad (tensor cores)");
     if (slices > 1) return slice_sum((const float*)scratch, dw, elems, slices, st, upd);
     if (upd.w && !update) return sgd_update(upd, dw, elems, st);

@@ -146,8 +146,9 @@ int tc_conv_fwd_known_stats(const ConvGeom& g, const void* x, const void* w, voi
 int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, void* scratch,
                   int64_t scratch_bytes, int* device_status, void* stream, const GradientJoin& join = GradientJoin());
 // upd: optional parameter update applied together with the gradient (the filter must no longer be needed by this step)
+// short_chains: the sums of a shape that the CUDA cores used to sum, as accurate as theirs (see the kernel)
 int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch,
-                  int64_t scratch_bytes, int* device_status, void* stream, const SgdUpdate& upd = SgdUpdate());
+                  int64_t scratch_bytes, int* device_status, void* stream, const SgdUpdate& upd = SgdUpdate(), bool short_chains = false);
 
 // One tiny kernel whose only wait has no producer and gives up after `limit_cycles` (1 .. 2e9), writing its code
 // into the status word: the bounded-wait path, run to its limit on purpose.

@@ -599,3 +599,31 @@ def test_bn_backward_sums_keep_their_accuracy(dtype, rows, c):
     bound = 9e-8 if dtype == ck.DTYPE_F32 else 6e-8
     errors = [float((got.double() - want).norm() / want.norm()) for got, want in ((dg, dgamma), (db, dbeta))]
     assert max(errors) <= bound, errors
+
+
+@pytest.mark.parametrize("n,h,w,cin,cout,k,stride", [(16, 96, 96, 48, 48, 3, 1), (11, 36, 61, 96, 512, 3, 1), (2, 16, 14, 72, 40, 3, 1), (4, 101, 19, 96, 512, 3, 2),
+                                                     (40, 9, 9, 200, 200, 3, 1), (1, 8, 5, 24, 40, 3, 2), (20, 40, 40, 104, 96, 1, 1), (1, 10, 10, 40, 72, 1, 1),
+                                                     (4, 9, 9, 40, 40, 1, 1), (16, 96, 96, 3, 48, 3, 1), (7, 33, 31, 3, 32, 3, 1), (16, 224, 224, 3, 32, 7, 2),
+                                                     (3, 40, 37, 3, 72, 7, 2)])
+def test_ragged_weight_gradients_keep_their_accuracy(n, h, w, cin, cout, k, stride):
+    """Weight gradients with channel counts that are no multiple of 64 against float64: chains of four MMAs, each cutting off
+    at most 2^-24 of the sum, and float32 additions of the chains (1e-7 to 2e-7 seen; one chain over the whole reduction
+    came to 5e-7 ... 2e-6 on the large shapes).  bfloat16 products are exact in float32."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(cin + cout)
+    pad = k // 2
+    ho, wo = (h + 2 * pad - k) // stride + 1, (w + 2 * pad - k) // stride + 1
+    x = torch.randn((n, h, w, cin), generator=gen, device="cuda").bfloat16()
+    dz = torch.randn((n, ho, wo, cout), generator=gen, device="cuda").bfloat16()
+    want = torch.empty((cout, k, k, cin), dtype=torch.float64, device="cuda")
+    xp = torch.nn.functional.pad(x.double(), (0, 0, pad, pad + stride, pad, pad + stride))
+    g = dz.double().reshape(-1, cout).T
+    for r in range(k):
+        for c in range(k):
+            want[:, r, c] = g @ xp[:, r:r + (ho - 1) * stride + 1:stride, c:c + (wo - 1) * stride + 1:stride].reshape(-1, cin)
+    shape = ck.ConvShape(n, h, w, cin, cout, k, stride, pad)
+    dw = torch.full((cout, k, k, cin), float("nan"), device="cuda")
+    scratch = torch.full((max(256, ck.conv2d_scratch_bytes(shape, ck.DTYPE_BF16)),), 0xFF, dtype=torch.uint8, device="cuda")
+    ck.conv2d_wgrad(shape, ck.DTYPE_BF16, 0, dz, x, dw, scratch)
+    assert ck.op_status() == 0
+    assert float((dw.double() - want).norm() / want.norm()) <= 4 * 2.0 ** -24
