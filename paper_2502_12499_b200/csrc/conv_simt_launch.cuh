@@ -11,8 +11,8 @@ static int go(const ConvGeom& g, const void* a, const void* b, void* out, const 
     using L = Tile<T, MODE, BM, BN, TM, TN>;
     auto kernel = conv_gemm_kernel<T, MODE, BM, BN, TM, TN, VA, VB>;
     if (L::smem > 48 * 1024) {
-        static const cudaError_t attr = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::smem);
-        if (attr != cudaSuccess) return cuda_fail(attr, "shared-memory opt-in of the CUDA-core convolution");
+        static DeviceFlags ready;
+        if (int bad = allow_shared_memory(ready, {(const void*)kernel}, L::smem)) return bad;
     }
     cudaLaunchConfig_t cfg = {};
     unsigned m_tiles = (unsigned)((M + BM - 1) / BM);

@@ -3077,12 +3077,8 @@ int launch_c64(const void* x, const void* w_mat, void* out, float* stat_partial,
     rc = b_mn ? make_mat_map(&mw, w_mat, 64, (int64_t)9 * c_out, 64) : make_mat_map(&mw, w_mat, c_out, 9 * 64, 64);
     if (rc) return rc;
     const size_t smem = 9 * 64 * 128 + 2 * 3 * (size_t)p.box_stride + 1024 + 256;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_conv_c64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_c64_kernel}, 220 * 1024)) return bad;
     tc_conv_c64_kernel<<<p.ctas_per_n * p.n_tiles, kThreads, smem, st>>>(mx, mw, (__nv_bfloat16*)out, stat_partial, p, status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_c64_kernel", what);
     if (stat_blocks) *stat_blocks = 4 * p.ctas_per_n;
@@ -3121,13 +3117,8 @@ int launch_generic(FwdParams p, const void* a, int a_n, int a_h, int a_w, const 
     rc = b_mn ? make_mat_map(&mw, w_mat, c_red, (int64_t)taps_total * c_out, 64) : make_mat_map(&mw, w_mat, c_out, (int64_t)taps_total * c_red, p.bn);
     if (rc) return rc;
     const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 256;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_conv_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_conv_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-        if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_fwd_kernel<false>, (const void*)tc_conv_fwd_kernel<true>}, kSmemBudget + 2048)) return bad;
     p.m_tiles = p.tiles_w * p.tiles_h * p.tiles_n;
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
@@ -3315,29 +3306,14 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     if (act_out && (rc = make_chunk_map(&madd, act_out, N, H, W, c_out, bw, bh, bnn))) return rc;
     if (p.join_mask && (rc = make_chunk_map(&mmask, p.join_mask, N, H, W, c_out, bw, bh, bnn))) return rc;
     const size_t smem = (size_t)p.stages * t_stage_bytes(p.tile_cols) + 1024 + kTBars + t_slab_bytes(p, p.split);
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaSuccess;
-        for (auto kernel : {tc_conv_t_kernel<false, false, EPI_PLAIN>, tc_conv_t_kernel<true, false, EPI_PLAIN>, tc_conv_t_kernel<false, true, EPI_PLAIN>,
-                            tc_conv_t_kernel<true, true, EPI_PLAIN>, tc_conv_t_kernel<true, false, EPI_JOIN>, tc_conv_t_kernel<true, true, EPI_JOIN>,
-                            tc_conv_t_kernel<false, false, EPI_ACT>, tc_conv_t_kernel<false, true, EPI_ACT>, tc_conv_t_kernel<false, false, EPI_RESIDUAL>,
-                            tc_conv_t_kernel<false, true, EPI_RESIDUAL>})
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTSmem);
-        if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_t_kernel<false, false, EPI_PLAIN>, (const void*)tc_conv_t_kernel<true, false, EPI_PLAIN>, (const void*)tc_conv_t_kernel<false, true, EPI_PLAIN>, (const void*)tc_conv_t_kernel<true, true, EPI_PLAIN>, (const void*)tc_conv_t_kernel<true, false, EPI_JOIN>, (const void*)tc_conv_t_kernel<true, true, EPI_JOIN>, (const void*)tc_conv_t_kernel<false, false, EPI_ACT>, (const void*)tc_conv_t_kernel<false, true, EPI_ACT>, (const void*)tc_conv_t_kernel<false, false, EPI_RESIDUAL>, (const void*)tc_conv_t_kernel<false, true, EPI_RESIDUAL>}, (int)kTSmem)) return bad;
     // partial row pairs per CTA: one per epilogue warp of a channel's quarter (the plain kernel has two), twice that
     // in the pixel-pair form; one per chunk of 32 pixels where a cluster shares a tile
     if (stat_blocks) *stat_blocks = !stat_partial ? 0 : p.split > 1 ? p.p_tiles * (p.tile_cols / 32) : (p.fold ? 2 : 1) * (patch ? kTpEpi : kTEpi) * p.ctas_per_co;
     if (patch) {
-        static bool tp_attr_set = false;
-        if (!tp_attr_set) {
-            cudaError_t e = cudaSuccess;
-            for (auto kernel : {tc_conv_tp_kernel<false, false>, tc_conv_tp_kernel<true, false>, tc_conv_tp_kernel<false, true>})
-                if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTpSmem);
-            if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-            tp_attr_set = true;
-        }
+        static DeviceFlags ready;
+        if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_tp_kernel<false, false>, (const void*)tc_conv_tp_kernel<true, false>, (const void*)tc_conv_tp_kernel<false, true>}, (int)kTpSmem)) return bad;
         const auto kernel = act_out ? tc_conv_tp_kernel<false, true> : a_mn ? tc_conv_tp_kernel<true, false> : tc_conv_tp_kernel<false, false>;
         kernel<<<p.ctas_per_co * p.co_tiles, kTpThreads, kTpSmem, st>>>(mx, mw, mo, madd, stat_blocks ? stat_partial : nullptr, p, status);
         CKPT_LAUNCH_CHECK_NAMED("tc_conv_tp_kernel", what);
@@ -3504,12 +3480,8 @@ int launch_fc(const ConvGeom& g, const void* x, const void* w, void* z, const fl
     if (rc) return rc;
     const uint32_t stage_bytes = 128 * 128 + (((uint32_t)p.bnb * 128 + 1023u) & ~1023u);
     const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 256;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_fc_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-        if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_fc_fwd_kernel}, kSmemBudget + 2048)) return bad;
     dim3 grid(m_tiles, slices);
     tc_fc_fwd_kernel<<<grid, kThreads, smem, st>>>(mw, mx, (float*)scratch, p, status);
     CKPT_LAUNCH_CHECK_NAMED("tc_fc_fwd_kernel", "fully connected forward (tensor cores)");
@@ -3742,12 +3714,8 @@ int tc_first_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, 
     CUtensorMap map_out;
     int rc = make_mat_map(&map_out, z, p.pixels, g.cout, 32);
     if (rc) return rc;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_conv_first_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFirstSmem);
-        if (e != cudaSuccess) return cuda_fail(e, "shared-memory opt-in of the first-layer kernel");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_first_kernel}, (int)kFirstSmem)) return bad;
     dim3 grid((unsigned)std::min(p.m_tiles, kFirstCtasPerSm * sms), (unsigned)((g.cout + 63) / 64));
     if (blocks) *blocks = partial ? (int)grid.x : 0;
     tc_conv_first_kernel<<<grid, kFirstThreads, kFirstSmem, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)w,
@@ -3802,12 +3770,8 @@ int stem_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, int*
     CUtensorMap map_out;
     int rc = make_act_map(&map_out, z, g.n, g.ho, g.wo, g.cout, 32, 1, 1);
     if (rc) return rc;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_conv_stem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemFwdSmem);
-        if (e != cudaSuccess) return cuda_fail(e, "shared-memory opt-in of the stem kernel");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_stem_kernel}, (int)kStemFwdSmem)) return bad;
     const int co_tiles = (g.cout + 63) / 64;
     dim3 grid((unsigned)std::min(p.m_tiles, std::max(1, sm_count() / co_tiles)), (unsigned)co_tiles);
     if (blocks) *blocks = partial ? (int)grid.x : 0;
@@ -3832,13 +3796,8 @@ int stem_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw,
     CUtensorMap map_dz;
     int rc = make_act_map(&map_dz, dz, g.n, g.ho, g.wo, g.cout, 128, 1, 1);
     if (rc) return rc;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_wgrad_stem_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemWgradSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_wgrad_stem_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemWgradSmem);
-        if (e != cudaSuccess) return cuda_fail(e, "shared-memory opt-in of the stem wgrad kernel");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_wgrad_stem_kernel<false>, (const void*)tc_wgrad_stem_kernel<true>}, (int)kStemWgradSmem)) return bad;
     dim3 grid((unsigned)p.slices, (unsigned)((g.cout + 63) / 64));
     if (g.cout % 64) tc_wgrad_stem_kernel<true><<<grid, kStemWgradThreads + 128, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
     else tc_wgrad_stem_kernel<false><<<grid, kStemWgradThreads, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
@@ -4038,13 +3997,8 @@ int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, vo
 }
 
 static int wgrad_rows_attr() {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_wgrad_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_wgrad_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024);
-        if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_wgrad_rows_kernel<false>, (const void*)tc_wgrad_rows_kernel<true>}, 222 * 1024)) return bad;
     return CKPT_OK;
 }
 
@@ -4085,12 +4039,8 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         rc = make_act_map(&mx, x, g.n, g.h, g.w, 64, 8, p.th + 2, 1);
         if (rc) return rc;
         cudaStream_t st = (cudaStream_t)stream;
-        static bool attr_set = false;
-        if (!attr_set) {
-            cudaError_t e = cudaFuncSetAttribute(tc_wgrad_c64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024);
-            if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-            attr_set = true;
-        }
+        static DeviceFlags ready;
+        if (int bad = allow_shared_memory(ready, {(const void*)tc_wgrad_c64_kernel}, 222 * 1024)) return bad;
         const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
         dim3 grid(p.slices, g.cout / 64);
         tc_wgrad_c64_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, (float*)scratch, p, device_status);
@@ -4131,13 +4081,8 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
     rc = make_act_map(&mx, x, g.n, g.h, g.w, g.cin, p.tw, p.th, p.tn, g.stride);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_conv_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_conv_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-        if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-        attr_set = true;
-    }
+    static DeviceFlags ready;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_wgrad_kernel<false>, (const void*)tc_conv_wgrad_kernel<true>}, kSmemBudget + 2048)) return bad;
     const bool chains = (short_chains || wgrad_short_chains(g)) && p.tiles_per_slice * p.px > 16 * kChain;       // (one chain is short as it is)
     if (chains) p.stages = std::max(p.stages, (8 * 4096 + (2 + p.nb) * p.px * 128 - 1) / ((2 + p.nb) * p.px * 128));     // a slab per epilogue warp
     const size_t smem = (size_t)p.stages * (2 + p.nb) * p.px * 128 + 1024 + 256;

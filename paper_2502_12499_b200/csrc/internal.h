@@ -2,10 +2,13 @@
 #pragma once
 #include <cstdint>
 #include <cstddef>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
 #include "../../include/ckpt_b200.h"
+#include "device_flags.h"
+#include "device_flags.h"
 
 namespace ckpt {
 
@@ -77,6 +80,9 @@ struct SgdUpdate {
 int sgd_update(const SgdUpdate& u, const float* g, int64_t elems, void* stream);
 // Sum of the `slices` partial results of a split weight gradient into the caller's gradient, with the update.
 int slice_sum(const float* partial, float* out, int64_t elems, int slices, void* stream, const SgdUpdate& upd = SgdUpdate());
+
+// Opts kernels in to `bytes` of dynamic shared memory on the current device, once (a function attribute belongs to a device).
+int allow_shared_memory(DeviceFlags& flags, std::initializer_list<const void*> kernels, int bytes);
 
 // ------------------------------------------------------------------ kernel launchers (kernels_simt.cu)
 struct ConvGeom {

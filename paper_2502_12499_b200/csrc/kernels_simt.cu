@@ -23,6 +23,17 @@ int cuda_fail(int err, const char* what) {
     return CKPT_E_CUDA;
 }
 
+int allow_shared_memory(DeviceFlags& flags, std::initializer_list<const void*> kernels, int bytes) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e, "asking for the device");
+    return flags.once(dev, [&] {
+        for (const void* kernel : kernels)
+            if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
+        return (int)CKPT_OK;
+    });
+}
+
 ConvGeom make_geom(const ckpt_conv_shape& s) {
     ConvGeom g;
     g.n = s.n; g.h = s.h; g.w = s.w; g.cin = s.c_in; g.cout = s.c_out; g.k = s.k; g.stride = s.stride; g.pad = s.pad;
