@@ -377,6 +377,10 @@ CKPT_API int ckpt_selftest_bounded_wait(int64_t limit_cycles, void* stream);
  * pixels per tile, CTAs that share a reduction, operand stages, bytes of the stages, bytes of the accumulators that are
  * exchanged in place of the stages (0 without sharing), shared memory in all.  CKPT_E_UNSUPPORTED: another kernel runs. */
 CKPT_API int ckpt_selftest_conv_plan(const ckpt_conv_shape* s, int epilogue, int32_t* plan);
+/* How the batch-norm backward divides a rows x c tensor on a device that holds held[0], held[1], held[2] clusters of 16, 8
+ * and 4 of its CTAs and held[3] CTAs at once (host only, no device needed).  split (host, 3 values): form (0 separate
+ * kernels, 1 one cluster per channel group, 2 one co-operative grid), channel groups, CTAs per group. */
+CKPT_API int ckpt_selftest_bn_split(int dtype, int64_t rows, int32_t c, int masked, const int32_t* held, int32_t* split);
 
 CKPT_API int ckpt_conv2d_scratch_bytes(const ckpt_conv_shape* s, int dtype, int64_t* bytes);
 CKPT_API int ckpt_conv2d_forward(const ckpt_conv_shape* s, int dtype, int impl, const void* x, const void* w,

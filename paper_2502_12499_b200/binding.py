@@ -403,6 +403,13 @@ def selftest_conv_plan(shape, epilogue):
     return dict(zip(("pixels", "split", "stages", "stage_bytes", "exchange_bytes", "smem"), out))
 
 
+def selftest_bn_split(dtype, rows, c, masked, held):
+    """(form, groups, parts) of the batch-norm backward on a device that holds `held` clusters of 16, 8, 4 and CTAs."""
+    out = (C.c_int32 * 3)()
+    _check(lib().ckpt_selftest_bn_split(C.c_int(dtype), C.c_int64(rows), C.c_int32(c), C.c_int(masked), (C.c_int32 * 4)(*held), out))
+    return tuple(out)
+
+
 # ------------------------------------------------------------------------------------------------
 # single operations
 # ------------------------------------------------------------------------------------------------

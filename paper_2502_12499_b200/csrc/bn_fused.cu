@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "device_flags.h"
 #include "internal.h"
 #include "vec.cuh"
 
@@ -336,20 +337,47 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
     if (CLUSTER) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");           // no CTA leaves while a peer reads its sums
 }
 
+// What the device holds at once, every CTA with its whole ring: clusters of 16, 8 and 4 CTAs, and CTAs.  Asked once per device
+// and instantiation (a cluster lies within a GPC; B200: 7, 15, 33 and 148).
+struct Resident { int clusters[3], ctas; };
+constexpr int kClusterSizes[3] = {16, 8, 4};
+template <typename T, int VEC, bool MASK>
+int ask(Resident* r) {
+    static Resident known[kMaxDevices];
+    static DeviceFlags asked;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e, "asking for the device");
+    return asked.once(dev, known, r, [&](Resident* out) {
+        constexpr int smem = Ring<MASK>::slots * Ring<MASK>::step_bytes;
+        const auto in_clusters = bn_bwd_fused_kernel<T, VEC, MASK, true>;
+        const auto cooperative = bn_bwd_fused_kernel<T, VEC, MASK, false>;
+        e = cudaFuncSetAttribute(in_clusters, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(cooperative, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(in_clusters, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)kClusterSizes[i]); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = (unsigned)kClusterSizes[i]; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr; cfg.numAttrs = 1;
+            // (a size that the device does not have is no error: none of it is held)
+            if (cudaOccupancyMaxActiveClusters(&out->clusters[i], in_clusters, &cfg) != cudaSuccess) { out->clusters[i] = 0; cudaGetLastError(); }
+        }
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&out->ctas, cooperative, kThreads, smem);
+        out->ctas *= sms;
+        return e == cudaSuccess ? CKPT_OK : cuda_fail(e, "preparing the fused batch-norm backward");
+    });
+}
+int resident(int dtype, bool mask, Resident* r) {
+    if (dtype == CKPT_DTYPE_BF16) return mask ? ask<__nv_bfloat16, 8, true>(r) : ask<__nv_bfloat16, 8, false>(r);
+    return mask ? ask<float, 4, true>(r) : ask<float, 4, false>(r);
+}
+
 template <typename T, int VEC>
 int launch(Params& p, bool cluster, cudaStream_t st) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        constexpr int plain = Ring<false>::slots * Ring<false>::step_bytes, masked = Ring<true>::slots * Ring<true>::step_bytes;
-        cudaError_t e = cudaFuncSetAttribute(bn_bwd_fused_kernel<T, VEC, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, plain);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(bn_bwd_fused_kernel<T, VEC, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, masked);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(bn_bwd_fused_kernel<T, VEC, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, plain);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(bn_bwd_fused_kernel<T, VEC, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, masked);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(bn_bwd_fused_kernel<T, VEC, false, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(bn_bwd_fused_kernel<T, VEC, true, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return cuda_fail(e, "raising the shared-memory limit");
-        attr_set = true;
-    }
     const int64_t steps = (p.rows_per_part + p.rows_per_step - 1) / p.rows_per_step;
     const size_t smem = p.mask ? (size_t)std::min<int64_t>(steps, Ring<true>::slots) * Ring<true>::step_bytes
                                : (size_t)std::min<int64_t>(steps, Ring<false>::slots) * Ring<false>::step_bytes;
@@ -383,6 +411,36 @@ int pick_width(int c, int vec) {
     return 0;
 }
 
+// How the rows of a tensor are divided.
+struct Split { BnForm form; int width, groups, parts; int64_t rows_per_part, rows_per_step; };
+Split divide(int dtype, int64_t rows, int c, bool mask, const Resident& r) {
+    Split s = {};
+    const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
+    s.width = c % vec ? 0 : pick_width(c, vec);
+    if (s.width == 0 || c / s.width > kBnSyncGroups) return s;
+    s.groups = c / s.width;
+    const int64_t R = (32 / (s.width / vec)) * kWarps;               // rows per step of a CTA
+    s.rows_per_step = R;
+    // One cluster per group where its CTAs get no more than 0.6 of their rings and all clusters find their SMs at once.
+    // Fewer CTAs then cost less than the meeting over global memory (with a 2 us memset: 3003 x 256 12.4 -> 10.4 us,
+    // 882 x 2048 14.4 -> 12.4, 6272 x 256 14.3 -> 12.5; above the line 8192 x 256 14.3 either way, 11025 x 128 14.4 -> 16.0).
+    for (int i = 0; i < 3; ++i) {
+        if (r.clusters[i] < s.groups) continue;
+        if (rows * 10 > (mask ? Ring<true>::slots : Ring<false>::slots) * R * kClusterSizes[i] * 6) break;
+        s.form = BnForm::clusters;
+        // no more CTAs than have a step each
+        for (s.parts = kClusterSizes[i]; s.parts > 1 && (int64_t)(s.parts / 2) * R >= rows; s.parts /= 2) {}
+        s.rows_per_part = (rows + s.parts - 1) / s.parts;
+        return s;
+    }
+    if (r.ctas < s.groups) return s;                                 // the CTAs of the grid wait for one another
+    s.form = BnForm::cooperative;
+    s.parts = (int)std::max<int64_t>(1, std::min<int64_t>(r.ctas / s.groups, (2 * rows + R - 1) / R));
+    s.rows_per_part = (rows + s.parts - 1) / s.parts;
+    s.parts = (int)((rows + s.rows_per_part - 1) / s.rows_per_part);
+    return s;
+}
+
 }  // namespace
 
 // On larger tensors the separate passes stream as fast and their blocks are balanced by the hardware (bf16 with its own
@@ -390,42 +448,31 @@ int pick_width(int c, int vec) {
 // 401408 x 256 (206 MB) 178 -> 181, 3211264 x 64 (411 MB) 317 -> 354).  With a mask the pass it saves decides.
 constexpr int64_t kLargest = 128 << 20;
 
-bool bn_backward_fused_applies(int dtype, int64_t rows, int c, const void* dy, const void* z, const void* mask, const void* dz) {
-    const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
-    if (c % vec || (((uintptr_t)dy | (uintptr_t)z | (uintptr_t)mask | (uintptr_t)dz) & 15u)) return false;
-    if (!mask && rows * c * dtype_size(dtype) > kLargest) return false;
-    const int width = pick_width(c, vec);
-    return width > 0 && c / width <= kBnSyncGroups;
+BnForm bn_backward_form(int dtype, int64_t rows, int c, const void* dy, const void* z, const void* mask, const void* dz) {
+    if (((uintptr_t)dy | (uintptr_t)z | (uintptr_t)mask | (uintptr_t)dz) & 15u) return BnForm::separate;
+    if (!mask && rows * c * dtype_size(dtype) > kLargest) return BnForm::separate;
+    Resident r;
+    return resident(dtype, mask != nullptr, &r) == CKPT_OK ? divide(dtype, rows, c, mask != nullptr, r).form : BnForm::separate;
+}
+
+void bn_selftest_split(int dtype, int64_t rows, int c, bool mask, const int* held, int* split) {
+    const Split s = divide(dtype, rows, c, mask, Resident{{held[0], held[1], held[2]}, held[3]});
+    split[0] = (int)s.form; split[1] = s.groups; split[2] = s.parts;
 }
 
 int bn_backward_fused(int dtype, int64_t rows, int c, void* dy, const void* z, const float* stats, int relu, void* dz, float* dgamma,
                       float* dbeta, float* partial, const BnBackwardExtra& ex, void* stream) {
+    Resident r;
+    int rc = resident(dtype, ex.mask != nullptr, &r);
+    if (rc) return rc;
+    const Split s = divide(dtype, rows, c, ex.mask != nullptr, r);
+    if (s.form == BnForm::separate) { set_error("the fused batch-norm backward does not take this tensor"); return CKPT_E_UNSUPPORTED; }
     Params p;
-    const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
-    int sms = 148, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     p.z = z; p.mask = ex.mask; p.dy = dy; p.dz = dz; p.stats = stats; p.partial = partial; p.dgamma = dgamma; p.dbeta = dbeta;
     p.counters = ex.counters; p.status = ex.status; p.rows = rows; p.inv_rows = 1.0 / (double)rows; p.c = c; p.relu = relu;
     p.gamma = ex.gamma; p.beta = ex.beta;
-    p.width = pick_width(c, vec);
-    p.groups = c / p.width;
-    const int64_t R = (32 / (p.width / vec)) * kWarps;               // rows per step of a CTA
-    p.parts = (int)std::max<int64_t>(1, std::min<int64_t>(sms / p.groups, (2 * rows + R - 1) / R));
-    // One cluster per group where its CTAs get no more than 0.6 of their rings; all clusters have to find their SMs at once
-    // (7 of 16, 15 of 8 or 33 of 4 do: a cluster lies within a GPC).  Fewer CTAs then cost less than the meeting over global
-    // memory (with a 2 us memset: 3003 x 256 12.4 -> 10.4 us, 882 x 2048 14.4 -> 12.4, 6272 x 256 14.3 -> 12.5; above the
-    // line 8192 x 256 14.3 either way, 11025 x 128 14.4 -> 16.0).
-    const int size = p.groups <= 7 ? 16 : p.groups <= 15 ? 8 : 4;
-    const int64_t ring = (ex.mask ? Ring<true>::slots : Ring<false>::slots) * R;
-    const bool cluster = p.groups <= 33 && rows * 10 <= ring * size * 6;
-    if (cluster) {
-        // no more CTAs than have a step each
-        for (p.parts = size; p.parts > 1 && (int64_t)(p.parts / 2) * R >= rows; p.parts /= 2) {}
-    }
-    p.rows_per_part = (rows + p.parts - 1) / p.parts;
-    if (!cluster) p.parts = (int)((rows + p.rows_per_part - 1) / p.rows_per_part);
-    p.rows_per_step = R;
+    p.width = s.width; p.groups = s.groups; p.parts = s.parts; p.rows_per_part = s.rows_per_part; p.rows_per_step = s.rows_per_step;
+    const bool cluster = s.form == BnForm::clusters;
     return dtype == CKPT_DTYPE_BF16 ? launch<__nv_bfloat16, 8>(p, cluster, (cudaStream_t)stream) : launch<float, 4>(p, cluster, (cudaStream_t)stream);
 }
 

@@ -154,6 +154,13 @@ int ckpt_selftest_conv_plan(const ckpt_conv_shape* s, int epilogue, int32_t* pla
     return tc_selftest_t_plan(make_geom(*s), epilogue, plan);
 }
 
+int ckpt_selftest_bn_split(int dtype, int64_t rows, int32_t c, int masked, const int32_t* held, int32_t* split) {
+    if (!held || !split) { set_error("null pointer"); return CKPT_E_NULL; }
+    if (rows < 1 || c < 1 || (dtype != CKPT_DTYPE_F32 && dtype != CKPT_DTYPE_BF16)) { set_error("bad shape"); return CKPT_E_BAD_ARG; }
+    bn_selftest_split(dtype, rows, c, masked != 0, held, split);
+    return CKPT_OK;
+}
+
 int ckpt_bn_scratch_bytes(int64_t rows, int32_t c, int64_t* bytes) {
     if (!bytes) { set_error("bytes is null"); return CKPT_E_NULL; }
     if (rows < 1 || c < 1) { set_error("bad shape"); return CKPT_E_BAD_ARG; }
@@ -174,7 +181,7 @@ int ckpt_bn_relu_backward(int dtype, int64_t rows, int32_t c, const void* dy, co
     if (rows < 1 || c < 1) { set_error("bad shape"); return CKPT_E_BAD_ARG; }
     // the counters of the cooperative kernel sit at the end of the caller's scratch, behind the rows it uses of it
     BnBackwardExtra ex;
-    if (bn_backward_fused_applies(dtype, rows, c, dy, z, nullptr, dz) && (uintptr_t)scratch % 16 == 0) {
+    if (bn_backward_form(dtype, rows, c, dy, z, nullptr, dz) != BnForm::separate && (uintptr_t)scratch % 16 == 0) {
         ex.counters = (unsigned*)((char*)scratch + (bn_scratch_bytes(rows, c) & ~(int64_t)15)) - 2 * kBnSyncGroups;
         ex.status = op_status_word();
         cudaError_t e = cudaMemsetAsync(ex.counters, 0, 2 * kBnSyncGroups * sizeof(unsigned), (cudaStream_t)stream);

@@ -3307,13 +3307,18 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     if (p.join_mask && (rc = make_chunk_map(&mmask, p.join_mask, N, H, W, c_out, bw, bh, bnn))) return rc;
     const size_t smem = (size_t)p.stages * t_stage_bytes(p.tile_cols) + 1024 + kTBars + t_slab_bytes(p, p.split);
     static DeviceFlags ready;
-    if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_t_kernel<false, false, EPI_PLAIN>, (const void*)tc_conv_t_kernel<true, false, EPI_PLAIN>, (const void*)tc_conv_t_kernel<false, true, EPI_PLAIN>, (const void*)tc_conv_t_kernel<true, true, EPI_PLAIN>, (const void*)tc_conv_t_kernel<true, false, EPI_JOIN>, (const void*)tc_conv_t_kernel<true, true, EPI_JOIN>, (const void*)tc_conv_t_kernel<false, false, EPI_ACT>, (const void*)tc_conv_t_kernel<false, true, EPI_ACT>, (const void*)tc_conv_t_kernel<false, false, EPI_RESIDUAL>, (const void*)tc_conv_t_kernel<false, true, EPI_RESIDUAL>}, (int)kTSmem)) return bad;
+    if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_t_kernel<false, false, EPI_PLAIN>, (const void*)tc_conv_t_kernel<true, false, EPI_PLAIN>,
+                                               (const void*)tc_conv_t_kernel<false, true, EPI_PLAIN>, (const void*)tc_conv_t_kernel<true, true, EPI_PLAIN>,
+                                               (const void*)tc_conv_t_kernel<true, false, EPI_JOIN>, (const void*)tc_conv_t_kernel<true, true, EPI_JOIN>,
+                                               (const void*)tc_conv_t_kernel<false, false, EPI_ACT>, (const void*)tc_conv_t_kernel<false, true, EPI_ACT>,
+                                               (const void*)tc_conv_t_kernel<false, false, EPI_RESIDUAL>, (const void*)tc_conv_t_kernel<false, true, EPI_RESIDUAL>}, (int)kTSmem)) return bad;
     // partial row pairs per CTA: one per epilogue warp of a channel's quarter (the plain kernel has two), twice that
     // in the pixel-pair form; one per chunk of 32 pixels where a cluster shares a tile
     if (stat_blocks) *stat_blocks = !stat_partial ? 0 : p.split > 1 ? p.p_tiles * (p.tile_cols / 32) : (p.fold ? 2 : 1) * (patch ? kTpEpi : kTEpi) * p.ctas_per_co;
     if (patch) {
         static DeviceFlags ready;
-        if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_tp_kernel<false, false>, (const void*)tc_conv_tp_kernel<true, false>, (const void*)tc_conv_tp_kernel<false, true>}, (int)kTpSmem)) return bad;
+        if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_tp_kernel<false, false>, (const void*)tc_conv_tp_kernel<true, false>,
+                                                   (const void*)tc_conv_tp_kernel<false, true>}, (int)kTpSmem)) return bad;
         const auto kernel = act_out ? tc_conv_tp_kernel<false, true> : a_mn ? tc_conv_tp_kernel<true, false> : tc_conv_tp_kernel<false, false>;
         kernel<<<p.ctas_per_co * p.co_tiles, kTpThreads, kTpSmem, st>>>(mx, mw, mo, madd, stat_blocks ? stat_partial : nullptr, p, status);
         CKPT_LAUNCH_CHECK_NAMED("tc_conv_tp_kernel", what);

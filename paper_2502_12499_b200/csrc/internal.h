@@ -178,8 +178,12 @@ struct BnBackwardExtra {
 };
 int bn_relu_backward(int dtype, int64_t rows, int c, void* dy, const void* z, const float* stats, int relu, void* dz, float* dgamma,
                      float* dbeta, void* scratch, void* stream, const BnBackwardExtra& extra);
-// The cooperative kernel (bn_fused.cu) and the tensors it takes.
-bool bn_backward_fused_applies(int dtype, int64_t rows, int c, const void* dy, const void* z, const void* mask, const void* dz);
+// The kernel that does it all (bn_fused.cu): one cluster per channel group, or one co-operative grid that meets over
+// zeroed counters; `separate` where it does not take the tensors or the device does not hold its CTAs at once.
+enum class BnForm { separate = 0, clusters = 1, cooperative = 2 };
+BnForm bn_backward_form(int dtype, int64_t rows, int c, const void* dy, const void* z, const void* mask, const void* dz);
+// {form, channel groups, CTAs per group} on a device that holds held[0..2] clusters of 16, 8, 4 CTAs and held[3] CTAs
+void bn_selftest_split(int dtype, int64_t rows, int c, bool mask, const int* held, int* split);
 int bn_backward_fused(int dtype, int64_t rows, int c, void* dy, const void* z, const float* stats, int relu, void* dz, float* dgamma,
                       float* dbeta, float* partial, const BnBackwardExtra& extra, void* stream);
 

@@ -761,7 +761,7 @@ int add_tensors(int dtype, int64_t elems, const void* a, const void* b, void* ou
 int bn_relu_backward(int dtype, int64_t rows, int c, void* dy, const void* z, const float* stats, int relu, void* dz, float* dgamma,
                      float* dbeta, void* scratch, void* stream, const BnBackwardExtra& ex) {
     cudaStream_t st = (cudaStream_t)stream;
-    if (ex.counters && ex.status && bn_backward_fused_applies(dtype, rows, c, dy, z, ex.mask, dz))
+    if (ex.counters && ex.status && bn_backward_form(dtype, rows, c, dy, z, ex.mask, dz) != BnForm::separate)
         return bn_backward_fused(dtype, rows, c, dy, z, stats, relu, dz, dgamma, dbeta, (float*)scratch, ex, stream);
     if (ex.mask) {
         int rc = relu_mask_inplace(dtype, rows * c, dy, ex.mask, stream);
