@@ -179,12 +179,13 @@ int ckpt_bn_relu_backward(int dtype, int64_t rows, int32_t c, const void* dy, co
                           const float* stats, int relu, void* dz, float* dgamma, float* dbeta, void* scratch, void* stream) {
     if (!dy || !z || !gamma || !stats || !dz || !dgamma || !dbeta || !scratch) { set_error("null pointer"); return CKPT_E_NULL; }
     if (rows < 1 || c < 1) { set_error("bad shape"); return CKPT_E_BAD_ARG; }
-    // the counters of the cooperative kernel sit at the end of the caller's scratch, behind the rows it uses of it
+    // the counters of the co-operative form sit at the end of the caller's scratch, behind the rows it uses of it
     BnBackwardExtra ex;
-    if (bn_backward_form(dtype, rows, c, dy, z, nullptr, dz) != BnForm::separate && (uintptr_t)scratch % 16 == 0) {
+    const BnForm form = (uintptr_t)scratch % 16 == 0 ? bn_backward_form(dtype, rows, c, dy, z, nullptr, dz) : BnForm::separate;
+    if (form == BnForm::clusters || (form == BnForm::cooperative && bn_backward_pays_for_counters(dtype, rows, c))) {
         ex.counters = (unsigned*)((char*)scratch + (bn_scratch_bytes(rows, c) & ~(int64_t)15)) - 2 * kBnSyncGroups;
         ex.status = op_status_word();
-        cudaError_t e = cudaMemsetAsync(ex.counters, 0, 2 * kBnSyncGroups * sizeof(unsigned), (cudaStream_t)stream);
+        const cudaError_t e = form == BnForm::cooperative ? cudaMemsetAsync(ex.counters, 0, 2 * kBnSyncGroups * sizeof(unsigned), (cudaStream_t)stream) : cudaSuccess;
         if (e != cudaSuccess) return cuda_fail(e, "clearing the batch-norm counters");
     }
     return bn_relu_backward(dtype, rows, c, const_cast<void*>(dy), z, stats, relu, dz, dgamma, dbeta, scratch, stream, ex);

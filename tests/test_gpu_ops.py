@@ -580,9 +580,9 @@ def test_average_pool_in_a_chain(channels, hw):
     assert torch.allclose(g, torch.full_like(g, 1.0 / (hw[0] * hw[1])), rtol=1e-6)
 
 
-@pytest.mark.parametrize("dtype,rows,c", [(ck.DTYPE_F32, 25088, 128), (ck.DTYPE_F32, 36960, 96), (ck.DTYPE_BF16, 24156, 512), (ck.DTYPE_BF16, 100352, 64)])
+@pytest.mark.parametrize("dtype,rows,c", [(ck.DTYPE_F32, 25088, 96), (ck.DTYPE_F32, 36960, 96), (ck.DTYPE_BF16, 24156, 512), (ck.DTYPE_BF16, 44304, 96)])
 def test_bn_backward_sums_keep_their_accuracy(dtype, rows, c):
-    """dgamma and dbeta against float64.  A float32 addition errs by 2.5e-8 of its result (rms): sums of a CTA's rows by chains
+    """dgamma and dbeta of the one kernel (tensors that the single operation gives to it) against float64.  A float32 addition errs by 2.5e-8 of its result (rms): sums of a CTA's rows by chains
     of a few additions per thread, the rest as two floats, come to 7e-8 of the result for float32 values and 4e-8 for bfloat16
     ones (whose products add up exactly at first); added up in float32 throughout they came to 1.1e-7 and 9e-8."""
     import torch
@@ -627,3 +627,23 @@ def test_ragged_weight_gradients_keep_their_accuracy(n, h, w, cin, cout, k, stri
     ck.conv2d_wgrad(shape, ck.DTYPE_BF16, 0, dz, x, dw, scratch)
     assert ck.op_status() == 0
     assert float((dw.double() - want).norm() / want.norm()) <= 4 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("dtype,rows,c,fused", [(ck.DTYPE_BF16, 3003, 64, True), (ck.DTYPE_BF16, 16384, 64, False), (ck.DTYPE_BF16, 16391, 256, True), (ck.DTYPE_BF16, 16391, 96, True),
+                                                (ck.DTYPE_BF16, 270011, 64, True), (ck.DTYPE_F32, 4096, 16, True), (ck.DTYPE_F32, 25088, 64, False), (ck.DTYPE_F32, 40003, 256, True),
+                                                (ck.DTYPE_F32, 30011, 72, True)])
+def test_bn_backward_form_of_the_single_operation(dtype, rows, c, fused):
+    """One kernel where its clusters need no counters or the tensor pays for clearing them, the separate kernels below."""
+    import torch
+    store = torch.bfloat16 if dtype == ck.DTYPE_BF16 else torch.float32
+    z, dz = (torch.ones((rows, c), device="cuda", dtype=store) for _ in range(2))
+    stats, out = torch.ones(4 * c, device="cuda"), torch.empty((3, c), device="cuda")
+    scratch = torch.full((ck.bn_scratch_bytes(rows, c),), 0xFF, dtype=torch.uint8, device="cuda")
+    ck.launch_log(True)
+    try:
+        ck.bn_relu_backward(dtype, rows, c, z, z, out[0], stats, 1, dz, out[1], out[2], scratch)
+        kernels = ck.launch_log_read()
+    finally:
+        ck.launch_log(False)
+    assert (kernels.get("bn_bwd_fused_kernel", 0) == 1) == fused and sum(kernels.values()) == (1 if fused else 3), kernels
+    test_bn_backward_in_one_kernel(rows, c, 1, dtype)
