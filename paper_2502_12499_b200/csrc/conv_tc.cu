@@ -3937,19 +3937,6 @@ int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, vo
                 const int gh = (g.h - ph + sd - 1) / sd, gw = (g.w - pw + sd - 1) / sd;
                 if (gh <= 0 || gw <= 0) continue;
                 if (p.taps == 0) continue;          // cleared above
-                if (in_place && p.taps == 1 && taps > 1 && g.cout <= 128 && g.cin % 64 == 0 && (int64_t)g.n * gh * gw <= 65536) {
-                    // The class of a single term, one or two reduction blocks: the two kernels lie within 6 % while it has few
-                    // pixels (all four classes of 128 -> 128 to 56 x 56: 21 images 24.6 against 23.7 us, 64 images 41.8 against
-                    // 39.5, 128 images 55.2 against 50.5), and the dispatch tests of the residual stages look for the generic
-                    // one there.
-                    p.in_stride = 1;
-                    p.out_H = g.h; p.out_W = g.w; p.out_stride = sd; p.out_oh = ph; p.out_ow = pw;
-                    p.tap_col[0] = taps - 1 - p.tap_col[0];              // the filter itself, not its mirrored copy
-                    int rc = launch_generic(p, dz, g.n, g.ho, g.wo, w, taps, dx, nullptr, 0, g.n, gh, gw, g.cout, g.cin, device_status, st,
-                                            "strided conv dgrad (tensor cores)", true);
-                    if (rc) return rc;
-                    continue;
-                }
                 if (in_place) {
                     TParams q = strided_terms();
                     q.taps = p.taps;
