@@ -3510,11 +3510,18 @@ void wgrad_plan(const ConvGeom& g, WgradParams* p, int* slices, int* groups, int
     choose_tile(p->px, g.wo, g.ho, g.n, &p->tw, &p->th, &p->tn);
     p->tiles_w = (g.wo + p->tw - 1) / p->tw; p->tiles_h = (g.ho + p->th - 1) / p->th; p->tiles_n = (g.n + p->tn - 1) / p->tn;
     p->total_tiles = p->tiles_w * p->tiles_h * p->tiles_n;
-    // Short reductions of few columns do not fill the SMs with 256-column CTAs: half as wide for 1x1 filters and for fewer
-    // than 800 pixels, and slices down to 256 pixels below (us with the slice sum, four blocks and 512 pixels -> chosen:
-    // 256 -> 1024 at 13 x 11, 21 images 15.4 -> 12.3, at 14 x 14, 32 images 14.4 -> 12.2; 3x3 512 -> 512 at 2 x 2, 128 images
-    // 12.5 -> 10.8; 3x3 256 -> 256 at 13 x 11 keeps four blocks, 16.6 against 19.9).
-    if (p->nb > 2 && ((g.k == 1 && pixels <= 65536) || pixels <= 800)) p->nb = 2;
+    // 256-column CTAs read dz half as often as 128-column ones, which decides where the operands' way from the L2 bounds; on
+    // small products the number of CTAs and their accumulators' way out do.  The line lies at 40000 pixels x CTAs of a slice
+    // (us with the slice sum, four blocks / two): 512 -> 2048 at 7 x 7, 21 images (33 thousand) 16.7 / 15.8, 32 images (50)
+    // 17.4 / 18.4, 128 images 24.8 / 26.4; 512 -> 1024 at 28 x 28 with stride 2, 8 images (25) 13.5 / 13.3, 21 images (66)
+    // 17.9 / 23.2, 128 images 46.6 / 79.2; 3x3 256 -> 256 at 7 x 7, 21 images (19) 14.1 / 12.7; 3x3 512 -> 512, 21 images (74)
+    // 19.7 / 21.0.  A few CTAs of a 1x1 filter without stride stay ahead further on: 256 -> 64 at 56 x 56, 64 images
+    // 32.4 / 29.3, 1024 -> 256 at 14 x 14, 128 images 26.3 / 25.1, 512 -> 256 at 28 x 28, 64 images 27.7 / 25.8, 256 images
+    // 72.5 / 77.8.  Slices down to 256 pixels, below (1024 -> 256 at 14 x 14, 8 images: 14.0 us with 512, 10.2).
+    if (p->nb > 2) {
+        const int64_t ctas = (int64_t)((p->total_blocks + p->nb - 1) / p->nb) * ((g.cout + 127) / 128);
+        if (pixels * ctas <= 40000 || (g.k == 1 && g.stride == 1 && ctas <= 8 && pixels * ctas * ctas <= 1 << 21)) p->nb = 2;
+    }
     // a reduction of one or two pixel tiles is all stores: narrower CTAs (128 accumulator columns) fit four to an SM
     if (p->total_tiles <= 2 && p->total_blocks >= 2) p->nb = 2;
     *groups = (p->total_blocks + p->nb - 1) / p->nb;
