@@ -60,6 +60,9 @@ __device__ __forceinline__ void lds(const T* p, float* v) {
 __device__ __forceinline__ void copy16(void* dst, const void* src, bool in) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
+__device__ __forceinline__ void copy4(void* dst, const void* src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
 
 template <typename T, int MODE, int BM, int BN, int TM, int TN>
 struct Tile {
@@ -95,7 +98,9 @@ struct Pixel {
 };
 
 // VA / VB: the operand is fetched in 16-byte chunks (its contiguous dimension is a multiple of a chunk and 16-byte
-// aligned); otherwise value by value, through registers: loaded before the FMAs of a step, stored after them.
+// aligned); otherwise value by value: float32 by asynchronous copies too, bfloat16 through registers, loaded before the FMAs
+// of a step and stored after them.  A forward layer of that kind often has a short reduction (27 values for three input
+// channels), whose last step stops where it ends (3 -> 256, 1x1, 49 images of 78 x 18, bfloat16: 81 us with whole steps, 46).
 // gridDim.z = slices * cluster; slice z of the reduction starts at z * k_per_slice (a multiple of BK).
 // Mode 1 with a stride: the input pixels fall into stride x stride parity classes, each reached by every stride-th filter
 // row and column only; a block works on one class (classes follow one another in blockIdx.x) and its K covers just those.
@@ -185,7 +190,10 @@ conv_gemm_kernel(ConvGeom g, const T* __restrict__ A, const T* __restrict__ B, v
         if ((unsigned)ih >= (unsigned)g.h || (unsigned)iw >= (unsigned)g.w) return nullptr;
         return B + (((int64_t)p.n * g.h + ih) * g.w + iw) * g.cin + b_ci;
     };
-    T a_reg[VA ? 1 : CA], b_reg[VB ? 1 : CB];
+    // values fetched through registers (also the filter of an input gradient to a few channels, whose rows of three values are
+    // copied no faster: 256 -> 3, 28 images of 13 x 49, float32 85.6 us, 90.6 by copies)
+    constexpr bool a_regs = !VA && sizeof(T) == 2, b_regs = !VB && (sizeof(T) == 2 || (MODE == 1 && VA));
+    T a_reg[a_regs ? CA : 1], b_reg[b_regs ? CB : 1];
 
     auto fetch = [&](int step) {
         T* const as_ = stages + (size_t)(step % kStages) * (L::a_elems + L::b_elems);
@@ -207,6 +215,7 @@ conv_gemm_kernel(ConvGeom g, const T* __restrict__ A, const T* __restrict__ B, v
                 row_px.advance(a_dr, W, H);
             }
             if constexpr (VA) copy16(as_ + row * L::a_row + a_c, src ? src : A, src != nullptr);
+            else if constexpr (!a_regs) copy4(as_ + row * L::a_row + a_c, src ? src : A, src != nullptr);
             else a_reg[i] = src ? *src : from_f<T>(0.f);
         }
         if (MODE != 2) a_pos.advance(BK, kc, cols);
@@ -231,20 +240,21 @@ conv_gemm_kernel(ConvGeom g, const T* __restrict__ A, const T* __restrict__ B, v
                 }
             }
             if constexpr (VB) copy16(bs_ + row * L::b_row + b_c, src ? src : B, src != nullptr);
+            else if constexpr (!b_regs) copy4(bs_ + row * L::b_row + b_c, src ? src : B, src != nullptr);
             else b_reg[i] = src ? *src : from_f<T>(0.f);
         }
     };
     auto settle = [&](int step) {                             // values fetched through registers
         T* const as_ = stages + (size_t)(step % kStages) * (L::a_elems + L::b_elems);
         T* const bs_ = as_ + L::a_elems;
-        if constexpr (!VA) {
+        if constexpr (a_regs) {
 #pragma unroll
             for (int i = 0; i < CA; ++i) {
                 const int row = a_r + i * a_dr;
                 if (a_items % NT == 0 || row < L::a_rows) as_[row * L::a_row + a_c] = a_reg[i];
             }
         }
-        if constexpr (!VB) {
+        if constexpr (b_regs) {
 #pragma unroll
             for (int i = 0; i < CB; ++i) {
                 const int row = b_r + i * b_dr;
@@ -281,6 +291,7 @@ conv_gemm_kernel(ConvGeom g, const T* __restrict__ A, const T* __restrict__ B, v
         const T* const bs_ = as_ + L::a_elems;
 #pragma unroll
         for (int k4 = 0; k4 < BK; k4 += 4) {
+            if (MODE == 0 && !VA && k_begin + step * BK + k4 >= k_end) break;
             float a[TM][4];
             if constexpr (L::a_k) {
 #pragma unroll

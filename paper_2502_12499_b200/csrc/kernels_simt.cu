@@ -50,7 +50,11 @@ namespace simt {
 // The tile shape, the CTAs of a cluster that share a tile's reduction and (wgrad) the slices whose partial sums a second
 // kernel adds: the cheapest by a model of clocks per SM.  FMA time is the tile volume over 128 lanes and the share of the
 // peak a tile shape reaches (narrower blocks per thread read more operand bytes per FMA); a cluster costs its exchange,
-// further slices a launch and a pass over the partial sums.
+// further slices a launch and a pass over the partial sums.  A weight gradient fetched value by value takes a CTA some 2200
+// clocks per step of 16 whatever its tile - four warps do not hide their addresses and reads - so that its long reduction
+// wants more CTAs, also such a number of slices as rounds to fewer (us, 3 -> 256, 28 images of 13 x 49 float32 87 -> 34,
+// 5 -> 20 at 28 x 28 69 -> 16, 3 -> 64 1x1 at 40 x 40, 20 images 67 -> 18, bfloat16 65 -> 21).  148 SMs are written in: the scratch
+// size of a chain comes from here and must not depend on the device at hand.
 Plan plan(int mode, int M, int N, int K, bool vectors) {
     static const int tile_m[7] = {128, 128, 64, 128, 64, 128, 64}, tile_n[7] = {128, 64, 64, 32, 32, 16, 16};
     static const double share[7] = {0.85, 0.8, 0.7, 0.6, 0.5, 0.4, 0.35};
@@ -62,15 +66,21 @@ Plan plan(int mode, int M, int N, int K, bool vectors) {
         const int64_t tiles = (int64_t)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
         for (int cluster = 1; cluster <= 8; cluster *= 2) {
             // 1, 2, 3, 4, 6, 8, 12, ... slices: a finer search costs the host 17 us per layer and gains nothing
-            for (int slices = 1; slices <= (mode == 2 ? 128 : 1); slices = slices < 3 ? slices + 1 : (slices & (slices - 1)) ? slices / 3 * 4 : slices / 2 * 3) {
+            for (int step = 1; step <= (mode == 2 ? 128 : 1); step = step < 3 ? step + 1 : (step & (step - 1)) ? step / 3 * 4 : step / 2 * 3) {
+                const int per = ((K + cluster * step - 1) / (cluster * step) + 31) / 32 * 32;
+                if (cluster * step > 1 && per < 64) break;
+                int slices = step;
+                if (cluster * step > 1 && (int64_t)per * (cluster * step - 1) >= K) {
+                    if (vectors || mode != 2) continue;
+                    slices = (int)((K + (int64_t)per * cluster - 1) / ((int64_t)per * cluster));      // rounding up leaves fewer
+                }
                 const int parts = cluster * slices;
-                const int per = ((K + parts - 1) / parts + 31) / 32 * 32;
-                if (parts > 1 && per < 64) break;
-                if (parts > 1 && (int64_t)per * (parts - 1) >= K) continue;
                 // CTAs per SM; one or two of 128 threads do not hide the latency of their shared-memory reads
                 const double load = std::ceil((double)(tiles * parts) / 148.0);
                 const double hidden = t == 0 ? (load < 2 ? 0.8 : 1.0) : (load < 2 ? 0.6 : load < 3 ? 0.8 : 1.0);
-                double clk = load * ((double)bm * bn * per / (128.0 * share[t] * hidden) + 300.0) + 2000.0;
+                double clk = load * ((double)bm * bn * per / (128.0 * share[t] * hidden) + 300.0);
+                if (!vectors && mode == 2) clk = std::max(clk, 140.0 * per);
+                clk += 2000.0;
                 if (cluster > 1) clk += 1000.0 + load * bm * bn / 32.0;
                 if (slices > 1) clk += 4000.0 + (double)slices * M * N * 8.0 / 2500.0;
                 if (clk < best_t) { best_t = clk; best = Plan{t, cluster, slices, per}; }
