@@ -43,13 +43,6 @@ __device__ __forceinline__ void copy_16(uint32_t dst, const void* src) {
 __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// sum (x + y) += v without losing what the addition rounds off (Knuth's two-sum)
-__device__ __forceinline__ void add_to(float2& sum, float v) {
-    const float t = sum.x + v, b = t - sum.x;
-    sum.y += (sum.x - (t - b)) + (v - b);
-    sum.x = t;
-}
-
 template <bool MASK> struct Ring {
     static constexpr int tensors = MASK ? 3 : 2;                // g, z (, mask)
     static constexpr int step_bytes = tensors * kThreads * 16;
@@ -206,10 +199,10 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
 #pragma unroll 1
         for (int w = 0; w < kWarps; w += 4) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) add_to(part4[q], red[(w + q) * columns + tid]);
+            for (int q = 0; q < 4; ++q) two_sum(part4[q], red[(w + q) * columns + tid]);
         }
 #pragma unroll
-        for (int q = 1; q < 4; ++q) { add_to(part4[0], part4[q].x); part4[0].y += part4[q].y; }
+        for (int q = 1; q < 4; ++q) { two_sum(part4[0], part4[q].x); part4[0].y += part4[q].y; }
         const float a = part4[0].x + part4[0].y;
         if (CLUSTER) sums[tid] = a;
         else __stcg(p.partial + ((size_t)part * 2 + tid / p.width) * c + group * p.width + tid % p.width, a);
@@ -257,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
             float2 a = {};
 #pragma unroll
             for (int r = 0; r < 16; ++r)
-                if (r < p.parts) add_to(a, x[r]);
+                if (r < p.parts) two_sum(a, x[r]);
             pair[tid] = a;
         }
         const int quads = columns / 4, split = CLUSTER ? 1 : min(min(kThreads / quads, kMaxSplit), p.parts), quad = tid % quads, q = tid / quads;
@@ -273,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
                     if (b0 + b * split < p.parts) x[b] = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(b0 + b * split) * 2 * c));
 #pragma unroll
                 for (int b = 0; b < B; ++b)
-                    if (b0 + b * split < p.parts) { add_to(a[0], x[b].x); add_to(a[1], x[b].y); add_to(a[2], x[b].z); add_to(a[3], x[b].w); }
+                    if (b0 + b * split < p.parts) { two_sum(a[0], x[b].x); two_sum(a[1], x[b].y); two_sum(a[2], x[b].z); two_sum(a[3], x[b].w); }
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) pair[q * columns + col + k] = a[k];
@@ -288,8 +281,8 @@ __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
             float2 s2 = {}, gz2 = {};
             for (int k = 0; k < split; ++k) {
                 const float2 a = pair[k * columns + tid], b = pair[k * columns + p.width + tid];
-                add_to(s2, a.x); s2.y += a.y;
-                add_to(gz2, b.x); gz2.y += b.y;
+                two_sum(s2, a.x); s2.y += a.y;
+                two_sum(gz2, b.x); gz2.y += b.y;
             }
             const double s = (double)s2.x + s2.y, gz = (double)gz2.x + gz2.y;
             const int chn = group * p.width + tid;

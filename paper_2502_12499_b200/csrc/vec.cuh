@@ -82,4 +82,11 @@ template <typename T> __device__ __forceinline__ float element(const uint4& u, i
     return __uint_as_float(sizeof(T) == 4 ? x : k % 2 ? x & 0xffff0000u : x << 16);
 }
 
+// sum (x + y) += v without losing what the addition rounds off (Knuth's two-sum)
+__device__ __forceinline__ void two_sum(float2& sum, float v) {
+    const float t = sum.x + v, b = t - sum.x;
+    sum.y += (sum.x - (t - b)) + (v - b);
+    sum.x = t;
+}
+
 }  // namespace ckpt
