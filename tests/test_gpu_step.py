@@ -437,9 +437,9 @@ def test_store_all_that_keeps_block_interiors(dtype):
 
 
 @pytest.mark.parametrize("graph", [False, True])
-def test_joined_gradients_equal_separate_ones(graph):
+def test_joined_relu_equals_a_separate_one(graph):
     """The input gradient of a residual block takes the shortcut's gradient and the previous block's ReLU on its way out.
-    With the gradient tap on, that ReLU is applied by the block it ends instead: the same bits."""
+    With the gradient tap on, that ReLU follows in a pass of its own: the same bits."""
     import torch
     spec = wl.resnet_chain([2, 2, 1, 1], 5, hw=(70, 90), classes=24)
     params = wl.make_params(spec, seed=5, bn_affine="random")
@@ -494,3 +494,20 @@ def test_gradient_tap_changes_no_bits(channels, hw, batch):
     runner.chain.set_gradient_tap(None)
     for a, b in zip(plain, tapped):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("channels,mid,hw,batch", [(256, 64, (13, 11), 5), (1024, 256, (14, 14), 3), (512, 1024, (9, 7), 6), (2048, 2048, (7, 7), 6), (2048, 2048, (7, 7), 13)])
+def test_joined_gradients_take_the_shortcut(channels, mid, hw, batch):
+    """The input gradient of a residual block takes the shortcut's gradient in its epilogue.  With a first filter of zeros that
+    is all there is to it: the gradient leaving the block equals the one entering it, where the block's ReLU passed, bit for
+    bit.  Whole tiles and a ragged last one, one CTA per tile and reductions shared by a cluster."""
+    from tests import parity_util as pu
+    block = {"kind": "bottleneck", "cin": channels, "mid": mid, "cout": channels, "stride": 1, "project": False}
+    spec = dict(units=[dict(block) for _ in range(3)], input_hwc=(hw[0], hw[1], channels), batch=batch, dtype="bf16", loss="sum", name="joined")
+    params = wl.make_params(spec, seed=11, bn_affine="random")
+    params[1]["w1"][:] = 0.0
+    x, _ = wl.make_batch(spec, seed=12)
+    step = pu.StoredStep(StepRunner(spec, params), x, None)
+    assert step.report["device_status"] == 0 and not [k for k in step.kernels if "CUDA cores" in k or k == "gradient join"], step.kernels
+    entering = np.where(step.stored(2) > 0, step.gradient(2), 0.0)
+    assert np.abs(entering).max() > 0 and np.array_equal(step.gradient(1), entering)
