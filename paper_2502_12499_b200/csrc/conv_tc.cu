@@ -3575,6 +3575,8 @@ void wgrad_c64_plan(const ConvGeom& g, W64Params* p) {
 
 namespace {
 constexpr int WROWS_MIN_W = 14;
+// (192, 320, .. input channels, an odd number of whole blocks, stay with the generic kernel: the last CTA could own a single
+// column there as it does for ragged counts, but that has not been measured.)
 bool wgrad_rows_applies(const ConvGeom& g) {
     return g.k == 3 && g.pad == 1 && g.stride == 1 && (g.cin % 128 == 0 || g.cin % 64) && g.cin % 8 == 0 && g.cout % 8 == 0 && g.w >= WROWS_MIN_W && g.h >= 8;
 }
@@ -3897,6 +3899,8 @@ int tc_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, const 
                            "conv forward (tensor cores)");
 }
 
+// (A whole tile of pixels at least: the tensors of fewer are under a megabyte for up to 1024 channels, and the addition by
+// itself a launch of 3 us; not measured below.)
 bool tc_dgrad_joins(const ConvGeom& g) {
     return tc_conv_supported(CKPT_DTYPE_BF16, g) && g.k == 1 && g.stride == 1 && t_applies(g.cout, g.cin, 1, 0) && (int64_t)g.n * g.h * g.w >= 256;
 }
