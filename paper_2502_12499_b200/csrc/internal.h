@@ -182,7 +182,6 @@ int bn_relu_backward(int dtype, int64_t rows, int c, void* dy, const void* z, co
 // zeroed counters; `separate` where it does not take the tensors or the device does not hold its CTAs at once.
 enum class BnForm { separate = 0, clusters = 1, cooperative = 2 };
 BnForm bn_backward_form(int dtype, int64_t rows, int c, const void* dy, const void* z, const void* mask, const void* dz);
-bool bn_backward_pays_for_counters(int dtype, int64_t rows, int c);      // (with a memset before the co-operative form)
 // {form, channel groups, CTAs per group} on a device that holds held[0..2] clusters of 16, 8, 4 CTAs and held[3] CTAs
 void bn_selftest_split(int dtype, int64_t rows, int c, bool mask, const int* held, int* split);
 int bn_backward_fused(int dtype, int64_t rows, int c, void* dy, const void* z, const float* stats, int relu, void* dz, float* dgamma,

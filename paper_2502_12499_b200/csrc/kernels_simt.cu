@@ -551,14 +551,6 @@ __global__ void __launch_bounds__(BNF_THREADS, 2) bn_partial_stream_kernel(const
 // The streaming kernel needs: lanes a power of two between 8 and 128 (so that 128 and the block
 // size are multiples of it).
 static bool bn_stream_ok(int lanes) { return lanes >= 8 && lanes <= 128 && (lanes & (lanes - 1)) == 0; }
-// A single operation clears the counters of the co-operative kernel with a launch of its own (3.5 us in a graph).  Where the
-// separate kernels stream their sums that costs more than the one kernel saves, up to about 32 MB (bf16 up to 128 channels,
-// us, one kernel with its memset / separate: 16384 x 64 14.4 / 11.5, 50176 x 128 20.6 / 19.7, 100352 x 128 28.7 / 29.2,
-// 401408 x 64 49 / 53, 16384 x 256 16.5 / 21.5; float32 25088 x 64 14.5 / 10.1, 16384 x 256 18.6 / 15.0, 50176 x 256 43 / 47).
-bool bn_backward_pays_for_counters(int dtype, int64_t rows, int c) {
-    const bool f32 = dtype == CKPT_DTYPE_F32;
-    return !bn_stream_ok(c / (f32 ? 4 : 8)) || (!f32 && c > 128) || rows * c * dtype_size(dtype) > 32 << 20;
-}
 static int bn_stream_blocks(int64_t vecs) {
     int64_t b = (vecs + (int64_t)BNF_THREADS * 8 - 1) / ((int64_t)BNF_THREADS * 8);
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, 148 * 2));
