@@ -156,6 +156,18 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32
         "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
         ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
 }
+// Warp index in a form that is the same register for all lanes.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x / 32), 0); }
+// One lane of a converged warp, the same one every time.  The warp that issues the MMAs walks its loop as a whole and elects
+// that lane around them: descriptors and barriers are then uniform values, as the instructions want them.  (In a branch
+// of lane 0 alone every operand was moved over for each MMA, and narrow instructions waited for that: 256 -> 256 3x3 at
+// 8 x 8, 128 images 15.8 -> 12.2 us, 1x1 1024 -> 256 at 13 x 11, 21 images 8.3 -> 6.7.  The halo-patch kernel's instructions of
+// 192 to 256 pixels hide it, and its more frequent waits are cheaper in one lane: 256 -> 256 at 56 x 56 158 -> 169-178 us.)
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+    return ok != 0;
+}
 // The mbarrier is signalled once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -307,7 +319,7 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     __shared__ int failed_flag;
     volatile int* failed = &failed_flag;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int n_tile = blockIdx.x % p.n_tiles;
     const int first = blockIdx.x / p.n_tiles;
     const int my_tiles = first < p.m_tiles ? (p.m_tiles - first + p.ctas_per_n - 1) / p.ctas_per_n : 0;
@@ -372,7 +384,7 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             for (int q = max(0, g - p.stages); q < g; ++q)
                 mbar_drain(full_bar(q % p.stages), (uint32_t)(q / p.stages) & 1u);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ---------------- MMA issuer
         const uint32_t idesc = instr_desc(128, p.bn, 0, B_MN ? 1 : 0);
         constexpr uint32_t b_step = B_MN ? 2048u : 32u, b_lbo = B_MN ? 8192u : 0u;
@@ -380,23 +392,27 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         int g = 0;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int buf = j & 1;
-            if (!mbar_wait(acc_empty0 + 8 * buf, ((uint32_t)(j >> 1) & 1u) ^ 1u, failed, status, 104)) { ok = false; break; }
+            if (!mbar_wait_warp(acc_empty0 + 8 * buf, ((uint32_t)(j >> 1) & 1u) ^ 1u, failed, status, 104)) { ok = false; break; }
             const uint32_t acc = tmem_base + (uint32_t)(buf * p.bn);
             for (int it = 0; it < iters; ++it, ++g) {
                 const int s = g % p.stages;
                 const uint32_t phase = (uint32_t)(g / p.stages) & 1u;
-                if (!mbar_wait(full_bar(s), phase, failed, status, 102)) { ok = false; break; }
+                if (!mbar_wait_warp(full_bar(s), phase, failed, status, 102)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t a_addr = base + (uint32_t)s * stage_bytes;
                 const uint32_t b_addr = a_addr + a_bytes;
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {        // 4 x (K = 16 bf16): 32 bytes along a row, or 16 rows when B_MN
-                    umma_bf16(acc, smem_desc(a_addr + kk * 32, 0, 1024), smem_desc(b_addr + kk * b_step, b_lbo, 1024), idesc,
-                              (it > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < 4; ++kk) {        // 4 x (K = 16 bf16): 32 bytes along a row, or 16 rows when B_MN
+                        umma_bf16(acc, smem_desc(a_addr + kk * 32, 0, 1024), smem_desc(b_addr + kk * b_step, b_lbo, 1024), idesc,
+                                  (it > 0 || kk > 0) ? 1u : 0u);
+                    }
+                    umma_commit(empty_bar(s));              // frees the stage when these MMAs have read it
                 }
-                umma_commit(empty_bar(s));              // frees the stage when these MMAs have read it
+                __syncwarp();
             }
-            if (ok) umma_commit(acc_full0 + 8 * buf);   // accumulator complete
+            if (ok && elect_one()) umma_commit(acc_full0 + 8 * buf);   // accumulator complete
+            __syncwarp();
         }
     } else if (warp >= 2) {
         // ---------------- epilogue: TMEM -> registers -> bf16 -> global
@@ -685,7 +701,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     __shared__ int failed_flag;
     volatile int* failed = &failed_flag;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int rank = SPLIT ? (int)cluster_rank() : 0;
     const int work = SPLIT ? blockIdx.x / p.split : blockIdx.x;
     const int co_tile = work % p.co_tiles;
@@ -760,7 +776,7 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         if (*failed && lane == 0) {
             for (int q = max(0, g - p.stages); q < g; ++q) mbar_drain(full_bar(q % p.stages), (uint32_t)(q / p.stages) & 1u);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ---------------- MMA issuer
         const uint32_t idesc = instr_desc(128, p.tile_cols, A_MN ? 1 : 0, 0);
         constexpr uint32_t a_step = (A_MN ? 2048u : 32u) / 16, b_step = 32u / 16;
@@ -770,21 +786,25 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         uint32_t phase = 0u, a_lo = a_lo0, b_lo = b_lo0;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int buf = j & 1;
-            if (!mbar_wait(acc_empty0 + 8 * buf, ((uint32_t)(j >> 1) & 1u) ^ 1u, failed, status, 904)) { ok = false; break; }
+            if (!mbar_wait_warp(acc_empty0 + 8 * buf, ((uint32_t)(j >> 1) & 1u) ^ 1u, failed, status, 904)) { ok = false; break; }
             const uint32_t acc = tmem_base + (uint32_t)(buf * 256);
             uint32_t more = 0u;
             for (int it = it0; it < it1; ++it) {
-                if (!mbar_wait(full_bar(s), phase, failed, status, 902)) { ok = false; break; }
+                if (!mbar_wait_warp(full_bar(s), phase, failed, status, 902)) { ok = false; break; }
                 tc_fence_after();
-                umma_bf16(acc, a_lo, hi, b_lo, hi, idesc, more);
-                more = 1u;
+                if (elect_one()) {
+                    umma_bf16(acc, a_lo, hi, b_lo, hi, idesc, more);
 #pragma unroll
-                for (int kk = 1; kk < 4; ++kk) umma_bf16(acc, a_lo + kk * a_step, hi, b_lo + kk * b_step, hi, idesc, 1u);
-                umma_commit(empty_bar(s));
+                    for (int kk = 1; kk < 4; ++kk) umma_bf16(acc, a_lo + kk * a_step, hi, b_lo + kk * b_step, hi, idesc, 1u);
+                    umma_commit(empty_bar(s));
+                }
+                __syncwarp();
+                more = 1u;
                 a_lo += lo_step; b_lo += lo_step;
                 if (++s == p.stages) { s = 0; phase ^= 1u; a_lo = a_lo0; b_lo = b_lo0; }
             }
-            if (ok) umma_commit(acc_full0 + 8 * buf);
+            if (ok && elect_one()) umma_commit(acc_full0 + 8 * buf);
+            __syncwarp();
         }
     } else if (SPLIT && warp >= 2) {
         // ---------------- accumulator to shared memory, [pixel][channel] floats over the operand stages (all of them read)
@@ -1267,7 +1287,7 @@ tc_conv_c64_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     volatile int* failed = &failed_flag;
     const uint32_t w_full = bars, a_full0 = bars + 8, a_empty0 = bars + 24, acc_full0 = bars + 40, acc_empty0 = bars + 56;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int n_tile = blockIdx.x % p.n_tiles;
     const int first = blockIdx.x / p.n_tiles;
     const int my_tiles = first < p.m_tiles ? (p.m_tiles - first + p.ctas_per_n - 1) / p.ctas_per_n : 0;
@@ -1324,29 +1344,32 @@ tc_conv_c64_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             mbar_drain(w_full, 0);
             for (int j = max(0, issued - 2); j < issued; ++j) mbar_drain(a_full0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ---------------- MMA issuer
         const uint32_t idesc = instr_desc(128, 64, 0, p.b_mn);
         const uint32_t b_step = p.b_mn ? 2048u : 32u, b_lbo = p.b_mn ? 8192u : 0u;      // 16 reduction rows, or 32 bytes along a row
-        bool ok = mbar_wait(w_full, 0, failed, status, 302);
+        bool ok = mbar_wait_warp(w_full, 0, failed, status, 302);
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int b = j & 1;
             const uint32_t ph = (uint32_t)(j >> 1) & 1u;
-            if (!mbar_wait(acc_empty0 + 8 * b, ph ^ 1u, failed, status, 303)) { ok = false; break; }
-            if (!mbar_wait(a_full0 + 8 * b, ph, failed, status, 304)) { ok = false; break; }
+            if (!mbar_wait_warp(acc_empty0 + 8 * b, ph ^ 1u, failed, status, 303)) { ok = false; break; }
+            if (!mbar_wait_warp(a_full0 + 8 * b, ph, failed, status, 304)) { ok = false; break; }
             tc_fence_after();
             const uint32_t acc = tmem_base + (uint32_t)b * 64;
+            if (elect_one()) {
 #pragma unroll 1
-            for (int tap = 0; tap < 9; ++tap) {
-                const uint32_t a_addr = a_base + b * stage_bytes + (tap % 3) * p.box_stride + (tap / 3) * 1024;
-                const uint32_t b_addr = base + tap * 8192;
+                for (int tap = 0; tap < 9; ++tap) {
+                    const uint32_t a_addr = a_base + b * stage_bytes + (tap % 3) * p.box_stride + (tap / 3) * 1024;
+                    const uint32_t b_addr = base + tap * 8192;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma_bf16(acc, smem_desc(a_addr + kk * 32, 0, 1024), smem_desc(b_addr + kk * b_step, b_lbo, 1024), idesc,
-                              (tap > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma_bf16(acc, smem_desc(a_addr + kk * 32, 0, 1024), smem_desc(b_addr + kk * b_step, b_lbo, 1024), idesc,
+                                  (tap > 0 || kk > 0) ? 1u : 0u);
+                }
+                umma_commit(a_empty0 + 8 * b);
+                umma_commit(acc_full0 + 8 * b);
             }
-            umma_commit(a_empty0 + 8 * b);
-            umma_commit(acc_full0 + 8 * b);
+            __syncwarp();
         }
     } else if (warp >= 2) {
         // ---------------- epilogue
@@ -1444,7 +1467,7 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     __shared__ int failed_flag;
     volatile int* failed = &failed_flag;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int slice = blockIdx.x, group = blockIdx.y, co_tile = blockIdx.z;
     const int blk_begin = group * p.nb;
     const int nb_here = min(p.nb, p.total_blocks - blk_begin);
@@ -1507,14 +1530,14 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             for (int it = max(0, issued - p.stages); it < issued; ++it)
                 mbar_drain(full_bar(it % p.stages), (uint32_t)(it / p.stages) & 1u);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         const uint32_t idesc = instr_desc(128, (int)n_cols, 1, 1);
         bool ok = true;
         int chain = 0;
         for (int it = 0; it < iters && ok; ++it) {
             const int s = it % p.stages;
             const uint32_t phase = (uint32_t)(it / p.stages) & 1u;
-            if (!mbar_wait(full_bar(s), phase, failed, status, 202)) { ok = false; break; }
+            if (!mbar_wait_warp(full_bar(s), phase, failed, status, 202)) { ok = false; break; }
             tc_fence_after();
             const uint32_t a_addr = base + (uint32_t)s * stage_bytes;
             const uint32_t a_lo = desc_lo(a_addr, box_bytes), b_lo = desc_lo(a_addr + 2 * box_bytes, box_bytes), hi = desc_hi(1024u);
@@ -1522,22 +1545,28 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             if constexpr (SHORT) {
                 for (int k0 = 0; k0 < k_steps; k0 += kChain, ++chain) {
                     const uint32_t buf = (uint32_t)chain & 1u;
-                    if (!mbar_wait(accum_empty + 8u * buf, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 204)) { ok = false; break; }
+                    if (!mbar_wait_warp(accum_empty + 8u * buf, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 204)) { ok = false; break; }
                     tc_fence_after();
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = k0; kk < k0 + kChain; ++kk)
-                        umma_bf16(tmem_base + buf * 256u, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, kk > k0 ? 1u : 0u);
-                    umma_commit(accum_bar + 8u * buf);
+                        for (int kk = k0; kk < k0 + kChain; ++kk)
+                            umma_bf16(tmem_base + buf * 256u, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, kk > k0 ? 1u : 0u);
+                        umma_commit(accum_bar + 8u * buf);
+                    }
+                    __syncwarp();
                 }
                 if (!ok) break;
-            } else {
+            } else if (elect_one()) {
 #pragma unroll 4
                 for (int kk = 0; kk < k_steps; ++kk)
                     umma_bf16(tmem_base, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, (it > 0 || kk > 0) ? 1u : 0u);
             }
-            umma_commit(empty_bar(s));
+            __syncwarp();
+            if (elect_one()) umma_commit(empty_bar(s));
+            __syncwarp();
         }
-        if (!SHORT && ok) umma_commit(accum_bar);
+        if (!SHORT && ok && elect_one()) umma_commit(accum_bar);
+        __syncwarp();
     } else if (warp >= 2) {
         // Thread l of a warp holds row l of each 32 x 32 block; the block goes to shared memory (swizzled rows of 128
         // bytes, over operand stages that the tensor core has read) and leaves as one tile store, clipped at the last
@@ -1686,7 +1715,7 @@ tc_wgrad_c64_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_con
     auto empty_bar = [&](int s) { return bars + 8u * (kMaxStages + s); };
     const uint32_t accum_bar = bars + 8u * (2 * kMaxStages);
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int slice = blockIdx.x, co_tile = blockIdx.y;
     const int my_tiles = slice < p.m_tiles ? (p.m_tiles - slice + p.slices - 1) / p.slices : 0;
     const uint32_t patch_bytes = (uint32_t)(8 * (p.th + 2)) * 128;
@@ -1724,31 +1753,35 @@ tc_wgrad_c64_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_con
         }
         if (*failed && lane == 0)
             for (int j = max(0, issued - p.stages); j < issued; ++j) mbar_drain(full_bar(j % p.stages), (uint32_t)(j / p.stages) & 1u);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         const uint32_t idesc = instr_desc(128, 64, 1, 1);
         const int ksteps = p.th / 2;                 // 16 pixels (two 8-pixel rows) per MMA
         bool ok = true;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int s = j % p.stages;
             const uint32_t phase = (uint32_t)(j / p.stages) & 1u;
-            if (!mbar_wait(full_bar(s), phase, failed, status, 402)) { ok = false; break; }
+            if (!mbar_wait_warp(full_bar(s), phase, failed, status, 402)) { ok = false; break; }
             tc_fence_after();
             const uint32_t dz_addr = base + (uint32_t)s * p.stage_bytes;
             const uint32_t x_addr = dz_addr + p.dz_bytes;
+            if (elect_one()) {
 #pragma unroll 1
-            for (int pair = 0; pair < 5; ++pair) {
-                // first tap of the pair and the distance to the second one
-                const uint32_t a0 = pair < 3 ? x_addr + (uint32_t)pair * 1024                       // (r = pair, s = 0) + (r, 1)
-                                  : pair == 3 ? x_addr + 2 * p.box_stride                           // (0, 2) + (1, 2)
-                                              : x_addr + 2 * p.box_stride + 2 * 1024;               // (2, 2) + unused rows
-                const uint32_t lbo = pair < 3 ? p.box_stride : 1024u;
-                for (int kk = 0; kk < ksteps; ++kk)
-                    umma_bf16(tmem_base + (uint32_t)pair * 64, smem_desc(a0 + kk * 2048, lbo, 1024), smem_desc(dz_addr + kk * 2048, 8192, 1024),
-                              idesc, (j > 0 || kk > 0) ? 1u : 0u);
+                for (int pair = 0; pair < 5; ++pair) {
+                    // first tap of the pair and the distance to the second one
+                    const uint32_t a0 = pair < 3 ? x_addr + (uint32_t)pair * 1024                       // (r = pair, s = 0) + (r, 1)
+                                      : pair == 3 ? x_addr + 2 * p.box_stride                           // (0, 2) + (1, 2)
+                                                  : x_addr + 2 * p.box_stride + 2 * 1024;               // (2, 2) + unused rows
+                    const uint32_t lbo = pair < 3 ? p.box_stride : 1024u;
+                    for (int kk = 0; kk < ksteps; ++kk)
+                        umma_bf16(tmem_base + (uint32_t)pair * 64, smem_desc(a0 + kk * 2048, lbo, 1024), smem_desc(dz_addr + kk * 2048, 8192, 1024),
+                                  idesc, (j > 0 || kk > 0) ? 1u : 0u);
+                }
+                umma_commit(empty_bar(s));
             }
-            umma_commit(empty_bar(s));
+            __syncwarp();
         }
-        if (ok) umma_commit(accum_bar);
+        if (ok && elect_one()) umma_commit(accum_bar);
+        __syncwarp();
     } else if (warp >= 2) {
         const int quarter = warp % 4;
         const int row = quarter * 32 + lane;         // (tap of the pair) * 64 + c_in
@@ -1825,7 +1858,7 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     const uint32_t accum_bar = bars + 8u * (2 * kMaxStages);      // SHORT: full[2], empty[2]
     const uint32_t accum_empty = accum_bar + 16u;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int slice = blockIdx.x, pair = blockIdx.y, co_tile = blockIdx.z;
     const int ncols = min(p.cols, p.total_cols - p.cols * pair);
     const int my_tiles = slice < p.m_tiles ? (p.m_tiles - slice + p.slices - 1) / p.slices : 0;
@@ -1870,28 +1903,31 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
         }
         if (*failed && lane == 0)
             for (int j = max(0, issued - p.stages); j < issued; ++j) mbar_drain(full_bar(j % p.stages), (uint32_t)(j / p.stages) & 1u);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         const uint32_t idesc = instr_desc(128, 192, 1, 1);
         const int ksteps = p.th / 2;                 // 16 pixels (two 8-pixel rows) per MMA
         bool ok = true;
         int chain = 0;
         for (int j = 0; j < my_tiles && ok; ++j) {
             const int s = j % p.stages;
-            if (!mbar_wait(full_bar(s), (uint32_t)(j / p.stages) & 1u, failed, status, 702)) { ok = false; break; }
+            if (!mbar_wait_warp(full_bar(s), (uint32_t)(j / p.stages) & 1u, failed, status, 702)) { ok = false; break; }
             tc_fence_after();
             const uint32_t dz_addr = base + (uint32_t)s * p.stage_bytes;
             if constexpr (SHORT) {
                 const uint32_t a_lo = desc_lo(dz_addr, p.dz_box), b_lo = desc_lo(dz_addr + 2 * p.dz_box, 1024u), hi = desc_hi(1024u);
                 for (int k0 = 0; k0 < ksteps; k0 += kChain, ++chain) {
                     const uint32_t buf = (uint32_t)chain & 1u;
-                    if (!mbar_wait(accum_empty + 8u * buf, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 704)) { ok = false; break; }
+                    if (!mbar_wait_warp(accum_empty + 8u * buf, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 704)) { ok = false; break; }
                     tc_fence_after();
-                    for (int kk = k0; kk < min(k0 + kChain, ksteps); ++kk)
-                        umma_bf16(tmem_base + buf * 256u, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, kk > k0 ? 1u : 0u);
-                    umma_commit(accum_bar + 8u * buf);
+                    if (elect_one()) {
+                        for (int kk = k0; kk < min(k0 + kChain, ksteps); ++kk)
+                            umma_bf16(tmem_base + buf * 256u, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, kk > k0 ? 1u : 0u);
+                        umma_commit(accum_bar + 8u * buf);
+                    }
+                    __syncwarp();
                 }
                 if (!ok) break;
-            } else {
+            } else if (elect_one()) {
 #pragma unroll 1
                 for (int c = 0; c < ncols; ++c) {
                     const uint32_t x_addr = dz_addr + 2 * p.dz_box + (uint32_t)c * p.patch_bytes;
@@ -1901,9 +1937,12 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
                         umma_bf16(tmem_base + (uint32_t)c * 192, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, (j > 0 || kk > 0) ? 1u : 0u);
                 }
             }
-            umma_commit(empty_bar(s));
+            __syncwarp();
+            if (elect_one()) umma_commit(empty_bar(s));
+            __syncwarp();
         }
-        if (!SHORT && ok) umma_commit(accum_bar);
+        if (!SHORT && ok && elect_one()) umma_commit(accum_bar);
+        __syncwarp();
     } else if (warp >= 2) {
         // Blocks of 32 output channels x 32 input channels of a tap leave as tile stores through the operand stages, as in
         // tc_conv_wgrad_kernel (rows stored by the lanes in 16-byte pieces: 21.9 us with the fold at 64 -> 64, 56 x 56, 32
@@ -2036,7 +2075,7 @@ tc_conv_first_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* _
     const uint32_t bars = smem_u32(bar_mem);
     const uint32_t a_full0 = bars, a_empty0 = bars + 16, acc_full0 = bars + 32, acc_empty0 = bars + 48;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int co0 = blockIdx.y * 64;
     const int my_tiles = (int)blockIdx.x < p.m_tiles ? (p.m_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
 
@@ -2413,7 +2452,7 @@ tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
     const uint32_t a_full0 = bars, a_empty0 = bars + 16, acc_full0 = bars + 32, acc_empty0 = bars + 48;
     const uint32_t seg_full0 = bars + 64, seg_empty0 = seg_full0 + 8 * kStemStages;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int co0 = blockIdx.y * 64;
     const int my_tiles = (int)blockIdx.x < p.m_tiles ? (p.m_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
 
@@ -2589,7 +2628,7 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant_
     const uint32_t seg_full0 = bars + 64, seg_empty0 = seg_full0 + 8 * kStemStages;
     const uint32_t dz_full0 = seg_empty0 + 8 * kStemStages, dz_empty0 = dz_full0 + 8 * kStemStages;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int slice = blockIdx.x, co_tile = blockIdx.y;
     const int my_tiles = slice < p.m_tiles ? (p.m_tiles - slice + p.slices - 1) / p.slices : 0;
 
@@ -2763,7 +2802,7 @@ tc_fc_fwd_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     __shared__ uint32_t tmem_base_slot;
     __shared__ int failed_flag;
     volatile int* failed = &failed_flag;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const int m_tile = blockIdx.x, slice = blockIdx.y;
     const int kb_begin = slice * p.blocks_per_slice;
     const int iters = max(0, min(p.k_blocks, kb_begin + p.blocks_per_slice) - kb_begin);
@@ -2801,22 +2840,26 @@ tc_fc_fwd_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
             for (int it = max(0, issued - p.stages); it < issued; ++it)
                 mbar_drain(full_bar(it % p.stages), (uint32_t)(it / p.stages) & 1u);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         const uint32_t idesc = instr_desc(128, p.bnb, 0, 0);
         bool ok = true;
         for (int it = 0; it < iters && ok; ++it) {
             const int s = it % p.stages;
-            if (!mbar_wait(full_bar(s), (uint32_t)(it / p.stages) & 1u, failed, status, 702)) { ok = false; break; }
+            if (!mbar_wait_warp(full_bar(s), (uint32_t)(it / p.stages) & 1u, failed, status, 702)) { ok = false; break; }
             tc_fence_after();
             const uint32_t a_addr = base + (uint32_t)s * stage_bytes;
             const uint32_t b_addr = a_addr + a_bytes;
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                umma_bf16(tmem_base, smem_desc(a_addr + kk * 32, 0, 1024), smem_desc(b_addr + kk * 32, 0, 1024), idesc,
-                          (it > 0 || kk > 0) ? 1u : 0u);
-            umma_commit(empty_bar(s));
+                for (int kk = 0; kk < 4; ++kk)
+                    umma_bf16(tmem_base, smem_desc(a_addr + kk * 32, 0, 1024), smem_desc(b_addr + kk * 32, 0, 1024), idesc,
+                              (it > 0 || kk > 0) ? 1u : 0u);
+                umma_commit(empty_bar(s));
+            }
+            __syncwarp();
         }
-        if (ok) umma_commit(accum_bar);
+        if (ok && elect_one()) umma_commit(accum_bar);
+        __syncwarp();
     } else if (warp >= 2) {
         // thread = accumulator lane = output feature: consecutive lanes write consecutive floats of a row of [b][co]
         const int quarter = warp % 4;
