@@ -7,6 +7,7 @@
 
 #include "device_flags.h"
 #include "internal.h"
+#include "overlap.cuh"
 #include "vec.cuh"
 
 namespace ckpt {
@@ -65,6 +66,8 @@ template <bool MASK> struct Ring {
 template <typename T, int VEC, bool MASK, bool CLUSTER>
 __global__ void __launch_bounds__(kThreads, 1) bn_bwd_fused_kernel(Params p) {
     using Rg = Ring<MASK>;
+    previous_grid_done();
+    next_grid_may_start();
     extern __shared__ uint4 ring[];                                  // [slot][g | z | mask][thread]
     __shared__ __align__(16) float red[kWarps * 2 * kMaxWidth];      // sums per warp; then the group's sums
     __shared__ float coef[2][kMaxWidth];
@@ -378,10 +381,11 @@ int launch(Params& p, bool cluster, cudaStream_t st) {
     if (cluster) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(p.groups * p.parts)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = (unsigned)p.parts; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr; cfg.numAttrs = 1;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)p.parts; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        start_early(&cfg, attr, Start::ON_STREAMS);
         e = p.mask ? cudaLaunchKernelEx(&cfg, bn_bwd_fused_kernel<T, VEC, true, true>, p) : cudaLaunchKernelEx(&cfg, bn_bwd_fused_kernel<T, VEC, false, true>, p);
     } else {
         void* args[] = {&p};

@@ -24,6 +24,7 @@
 #include <cstdint>
 
 #include "internal.h"
+#include "overlap.cuh"
 
 namespace ckpt {
 namespace simt {
@@ -106,8 +107,10 @@ struct Pixel {
 // row and column only; a block works on one class (classes follow one another in blockIdx.x) and its K covers just those.
 template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
-conv_gemm_kernel(ConvGeom g, const T* __restrict__ A, const T* __restrict__ B, void* __restrict__ out, const float* __restrict__ bias,
+conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bias,
                  int relu, int M, int N, int K, int k_per_slice, int cluster, SgdUpdate upd) {
+    previous_grid_done();
+    next_grid_may_start();
     using L = Tile<T, MODE, BM, BN, TM, TN>;
     constexpr int NT = L::threads, V = L::V, BK = L::BK;
     extern __shared__ __align__(16) uint8_t smem[];

@@ -24,11 +24,12 @@ static int go(const ConvGeom& g, const void* a, const void* b, void* out, const 
     cfg.blockDim = dim3(L::threads);
     cfg.dynamicSmemBytes = L::smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)p.cluster;
     cfg.attrs = attr;
     cfg.numAttrs = p.cluster > 1 ? 1 : 0;
+    start_early(&cfg, attr, Start::ON_STREAMS);
     cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, g, (const T*)a, (const T*)b, out, bias, relu, M, N, K, p.k_per_slice, p.cluster, upd);
     if (e != cudaSuccess) return cuda_fail(e, "launching the CUDA-core convolution");
     static const char* const names[3] = {"conv forward (CUDA cores)", "conv dgrad (CUDA cores)", "conv wgrad (CUDA cores)"};

@@ -14,14 +14,17 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "overlap.cuh"
 
 namespace ckpt {
 
 namespace {
 
 template <int CIN>
-__global__ void __launch_bounds__(128) small_fwd_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w,
-                                                        __nv_bfloat16* __restrict__ z, int n, int h, int wd, int cout) {
+__global__ void __launch_bounds__(128) small_fwd_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
+                                                        __nv_bfloat16* z, int n, int h, int wd, int cout) {
+    previous_grid_done();
+    next_grid_may_start();
     constexpr int K = 9 * CIN;
     __shared__ __align__(16) float ws[K][64];              // ws[k][co] for this block's 64 output channels
     const int co0 = blockIdx.y * 64;
@@ -79,8 +82,10 @@ __global__ void __launch_bounds__(128) small_fwd_kernel(const __nv_bfloat16* __r
 // from the word below them and five funnel shifts; the rest of the row is zero.  Pixels at the left border and the
 // last two of a row (whose words would reach past the row) go value by value.
 template <int WIDTH>
-__global__ void __launch_bounds__(256) unfold3x3_rows_kernel(const __nv_bfloat16* __restrict__ x, uint4* __restrict__ xcol, int n, int h,
+__global__ void __launch_bounds__(256) unfold3x3_rows_kernel(const __nv_bfloat16* x, uint4* xcol, int n, int h,
                                                              int wd, int word_aligned) {
+    previous_grid_done();
+    next_grid_may_start();
     const uint32_t* x32 = reinterpret_cast<const uint32_t*>(x);
     const uint16_t* x16 = reinterpret_cast<const uint16_t*>(x);
     const int64_t pixels = (int64_t)n * h * wd;
@@ -101,7 +106,7 @@ __global__ void __launch_bounds__(256) unfold3x3_rows_kernel(const __nv_bfloat16
                 const uint32_t sh = (uint32_t)(e0 & 1) * 16u;
                 uint32_t w[6];
 #pragma unroll
-                for (int q = 0; q < 6; ++q) w[q] = __ldg(src + q);
+                for (int q = 0; q < 6; ++q) w[q] = src[q];
 #pragma unroll
                 for (int q = 0; q < 5; ++q) o[5 * r + q] = __funnelshift_r(w[q], w[q + 1], sh);
                 o[5 * r + 4] &= 0xffffu;
@@ -129,12 +134,16 @@ __device__ __forceinline__ void take(float v, float* dw, int i, const SgdUpdate&
     if (upd.w) { __nv_bfloat16* w = (__nv_bfloat16*)upd.w + i; *w = __float2bfloat16_rn(fmaf(-upd.lr, v, __bfloat162float(*w))); }
 }
 // dw[co][0..K) out of the padded [c_out][64] result
-__global__ void take_columns_kernel(const float* __restrict__ dwp, float* __restrict__ dw, int cout, int k, SgdUpdate upd) {
+__global__ void take_columns_kernel(const float* dwp, float* dw, int cout, int k, SgdUpdate upd) {
+    previous_grid_done();
+    next_grid_may_start();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < cout * k) take(dwp[(i / k) * 64 + unfolded_column(i % k)], dw, i, upd);
 }
 // Paired pixels: dwp is [(parity, co)][(parity, column)]; the gradient is the sum of its two diagonal blocks.
-__global__ void take_paired_columns_kernel(const float* __restrict__ dwp, float* __restrict__ dw, int cout, int k, SgdUpdate upd) {
+__global__ void take_paired_columns_kernel(const float* dwp, float* dw, int cout, int k, SgdUpdate upd) {
+    previous_grid_done();
+    next_grid_may_start();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < cout * k) {
         const int co = i / k, col = unfolded_column(i % k);
@@ -165,7 +174,7 @@ int64_t small_conv_scratch_bytes(const ConvGeom& g) {
 int small_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, void* stream) {
     const int64_t pixels = (int64_t)g.n * g.h * g.w;
     dim3 grid((unsigned)std::min<int64_t>((pixels + 127) / 128, 148 * 16), g.cout / 64);
-    small_fwd_kernel<3><<<grid, 128, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)w, (__nv_bfloat16*)z,
+    launch(Start::ON_STREAMS, small_fwd_kernel<3>, grid, 128, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)w, (__nv_bfloat16*)z,
                                                                 g.n, g.h, g.w, g.cout);
     CKPT_LAUNCH_CHECK("first-layer conv forward");
     return CKPT_OK;
@@ -185,14 +194,14 @@ int small_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw
     const int64_t pixels = (int64_t)g.n * g.h * g.w;
     const unsigned ugrid = (unsigned)std::min<int64_t>((pixels + 255) / 256, 148 * 16);
     const int word_aligned = (uintptr_t)x % 4 == 0 ? 1 : 0;
-    if (paired(g)) unfold3x3_rows_kernel<32><<<ugrid, 256, 0, st>>>((const __nv_bfloat16*)x, (uint4*)xcol, g.n, g.h, g.w, word_aligned);
-    else unfold3x3_rows_kernel<64><<<ugrid, 256, 0, st>>>((const __nv_bfloat16*)x, (uint4*)xcol, g.n, g.h, g.w, word_aligned);
+    if (paired(g)) launch(Start::ON_STREAMS, unfold3x3_rows_kernel<32>, ugrid, 256, 0, st, (const __nv_bfloat16*)x, (uint4*)xcol, g.n, g.h, g.w, word_aligned);
+    else launch(Start::ON_STREAMS, unfold3x3_rows_kernel<64>, ugrid, 256, 0, st, (const __nv_bfloat16*)x, (uint4*)xcol, g.n, g.h, g.w, word_aligned);
     CKPT_LAUNCH_CHECK("first-layer unfold");
     const ConvGeom u = unfolded_geom(g);
     int rc = tc_conv_wgrad(u, dz, xcol, dwp, tc_scratch, scratch_bytes - xcol_bytes(g) - dwp_bytes(g), device_status, stream, SgdUpdate(), g.cout % 64 != 0);
     if (rc) return rc;
-    if (paired(g)) take_paired_columns_kernel<<<(g.cout * 27 + 255) / 256, 256, 0, st>>>(dwp, dw, g.cout, 27, upd);
-    else take_columns_kernel<<<(g.cout * 27 + 255) / 256, 256, 0, st>>>(dwp, dw, g.cout, 27, upd);
+    if (paired(g)) launch(Start::ON_STREAMS, take_paired_columns_kernel, (g.cout * 27 + 255) / 256, 256, 0, st, dwp, dw, g.cout, 27, upd);
+    else launch(Start::ON_STREAMS, take_columns_kernel, (g.cout * 27 + 255) / 256, 256, 0, st, dwp, dw, g.cout, 27, upd);
     CKPT_LAUNCH_CHECK("first-layer wgrad column pick");
     return CKPT_OK;
 }

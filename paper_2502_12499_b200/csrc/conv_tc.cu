@@ -26,6 +26,7 @@
 #include <cstring>
 
 #include "internal.h"
+#include "overlap.cuh"
 
 namespace ckpt {
 
@@ -306,7 +307,7 @@ struct FwdParams {
 template <bool B_MN>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                   __nv_bfloat16* __restrict__ out, const float* __restrict__ bias, int relu, float* __restrict__ stat_partial,
+                   __nv_bfloat16* out, const float* bias, int relu, float* stat_partial,
                    FwdParams p, int* status) {
     // Persistent: CTA (first, n_tile) walks the pixel tiles first, first + ctas_per_n, ... of its output-channel
     // tile.  The operand ring runs on across tile boundaries and the accumulator is double-buffered in tensor
@@ -350,6 +351,8 @@ tc_conv_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     if (warp == 0 && (lane == 0 || B_MN)) {
         // ---------------- TMA producer.  Filter as a [c_out][k*k*c_red] matrix: two copies per stage, measured
@@ -653,7 +656,7 @@ __device__ __forceinline__ void residual_chunk(const TParams& p, size_t pixel, i
 #pragma unroll
     for (int e = 0; e < 32; ++e) {
         if (!((in_mask >> e) & 1u) || co >= p.c_out) continue;
-        v[e] = __float_as_uint(residual(p, a, __uint_as_float(v[e]), __ldg(add + (size_t)e * p.c_out)));
+        v[e] = __float_as_uint(residual(p, a, __uint_as_float(v[e]), add[(size_t)e * p.c_out]));
     }
 }
 // The join by plain loads: channel `co` of 32 consecutive pixels from `pixel` on.
@@ -663,8 +666,8 @@ __device__ __forceinline__ void join_chunk(const TParams& p, size_t pixel, int c
 #pragma unroll
     for (int e = 0; e < 32; ++e) {
         if (!((in_mask >> e) & 1u) || co >= p.c_out) continue;
-        const float sum = __uint_as_float(v[e]) + __uint_as_float((uint32_t)__ldg(add + (size_t)e * p.c_out) << 16);
-        v[e] = !p.join_mask || __uint_as_float((uint32_t)__ldg(mask + (size_t)e * p.c_out) << 16) > 0.f ? __float_as_uint(sum) : 0u;
+        const float sum = __uint_as_float(v[e]) + __uint_as_float((uint32_t)add[(size_t)e * p.c_out] << 16);
+        v[e] = !p.join_mask || __uint_as_float((uint32_t)mask[(size_t)e * p.c_out] << 16) > 0.f ? __float_as_uint(sum) : 0u;
     }
 }
 
@@ -688,7 +691,7 @@ template <bool A_MN, bool SPLIT, int EPI>
 __global__ void __launch_bounds__(kThreadsT, 1)
 tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_add,
-                 const __grid_constant__ CUtensorMap map_mask, float* __restrict__ stat_partial, TParams p, int* status) {
+                 const __grid_constant__ CUtensorMap map_mask, float* stat_partial, TParams p, int* status) {
     constexpr bool LOADS = EPI == EPI_JOIN || EPI == EPI_RESIDUAL;         // the epilogue reads tensors of its own
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -736,6 +739,8 @@ tc_conv_t_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     if (warp == 0) {
         // ---------------- TMA producer: pixel box (N operand, lane 0) and filter box or boxes (M operand, lanes 1 and 2)
@@ -1061,7 +1066,7 @@ constexpr uint32_t kTpSmem = kTpBoxes * 16384 + kTpPatches * kTpPatchSlot + 256 
 template <bool A_MN, bool ACT>
 __global__ void __launch_bounds__(kTpThreads, 1)
 tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_act, float* __restrict__ stat_partial, TParams p,
+                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_act, float* stat_partial, TParams p,
                   int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -1107,6 +1112,8 @@ tc_conv_tp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer: per column one patch, then the filter boxes of its three vertical taps
@@ -1275,7 +1282,7 @@ struct C64Params {
 
 __global__ void __launch_bounds__(kThreads, 1)
 tc_conv_c64_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                   __nv_bfloat16* __restrict__ out, float* __restrict__ stat_partial, C64Params p, int* status) {
+                   __nv_bfloat16* out, float* stat_partial, C64Params p, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     constexpr uint32_t w_bytes = 9 * 64 * 128;                       // resident filter
@@ -1309,6 +1316,8 @@ tc_conv_c64_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     auto tile_origin = [&](int j, int& w0, int& h0, int& img) {
         int t = first + j * p.ctas_per_n;
@@ -1452,7 +1461,7 @@ struct WgradParams {
 template <bool SHORT>
 __global__ void __launch_bounds__(SHORT ? kThreadsShort : kThreads, 1)
 tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
-                     const __grid_constant__ CUtensorMap map_out, float* __restrict__ partial, WgradParams p, SgdUpdate upd, int* status) {
+                     const __grid_constant__ CUtensorMap map_out, float* partial, WgradParams p, SgdUpdate upd, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     // One copy brings px pixels x 64 channels (px = 64, 128 or 256: as many as leave two stages in shared memory, so
@@ -1497,6 +1506,8 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     if (warp == 0) {
         // six copies per stage: one lane each (issuing a bulk-tensor copy occupies a thread for a few hundred cycles)
@@ -1704,7 +1715,7 @@ struct W64Params {
 
 __global__ void __launch_bounds__(kThreads, 1)
 tc_wgrad_c64_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
-                    float* __restrict__ partial, W64Params p, int* status) {
+                    float* partial, W64Params p, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t bars = base + (uint32_t)p.stages * p.stage_bytes;
@@ -1733,6 +1744,8 @@ tc_wgrad_c64_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     if (warp == 0) {
         int issued = 0;
@@ -1846,7 +1859,7 @@ struct WRowsParams {
 template <bool SHORT>
 __global__ void __launch_bounds__(SHORT ? kThreadsShort : kThreads, 1)
 tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
-                     const __grid_constant__ CUtensorMap map_out, float* __restrict__ partial, WRowsParams p, int* status) {
+                     const __grid_constant__ CUtensorMap map_out, float* partial, WRowsParams p, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t bars = base + (uint32_t)p.stages * p.stage_bytes;
@@ -1877,6 +1890,8 @@ tc_wgrad_rows_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     if (warp == 0) {
         // four copies per stage, one lane each; every lane watches the barrier itself
@@ -2059,8 +2074,10 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __global__ void __launch_bounds__(kFirstThreads, kFirstCtasPerSm)
-tc_conv_first_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w,
-                     const __grid_constant__ CUtensorMap map_out, float* __restrict__ stat_partial, FirstParams p, int* status) {
+tc_conv_first_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
+                     const __grid_constant__ CUtensorMap map_out, float* stat_partial, FirstParams p, int* status) {
+    previous_grid_done();
+    next_grid_may_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* const smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t (*a_tiles)[128 * 128] = reinterpret_cast<uint8_t (*)[128 * 128]>(smem_al);
@@ -2095,7 +2112,7 @@ tc_conv_first_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* _
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int k = chunk * 8 + e, r = k / 10, tt = k % 10;      // filter row r in columns 10 r .. 10 r + 8
-            v[e] = (r < 3 && tt < 9 && co0 + co < p.c_out) ? __ldg(reinterpret_cast<const uint16_t*>(w) + (size_t)(co0 + co) * 27 + r * 9 + tt) : (uint16_t)0;
+            v[e] = (r < 3 && tt < 9 && co0 + co < p.c_out) ? reinterpret_cast<const uint16_t*>(w)[(size_t)(co0 + co) * 27 + r * 9 + tt] : (uint16_t)0;
         }
         *reinterpret_cast<uint4*>(b_tile + co * 128 + ((chunk ^ (co & 7)) * 16)) = *reinterpret_cast<const uint4*>(v);
     }
@@ -2435,8 +2452,10 @@ __device__ __forceinline__ void stem_gather_role(const StemParams& p, const uint
 // role runs at instruction latency, hence the many warps: four epilogue warps needed 1600 clocks per tile against
 // 1000 of MMAs.
 __global__ void __launch_bounds__(kStemFwdThreads, 1)
-tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w,
-                    const __grid_constant__ CUtensorMap map_out, float* __restrict__ stat_partial, StemParams p, int* status) {
+tc_conv_stem_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
+                    const __grid_constant__ CUtensorMap map_out, float* stat_partial, StemParams p, int* status) {
+    previous_grid_done();
+    next_grid_may_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* const smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* const a_tiles = smem_al;                       // [2][atoms 2, 0, 1][128 rows][128 bytes]
@@ -2473,7 +2492,7 @@ tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int k = chunk * 8 + e, r = k / 24, tt = k % 24;
-            v[e] = (r < 7 && tt < 21 && co0 + co < p.c_out) ? __ldg(reinterpret_cast<const uint16_t*>(w) + (size_t)(co0 + co) * 147 + r * 21 + tt) : (uint16_t)0;
+            v[e] = (r < 7 && tt < 21 && co0 + co < p.c_out) ? reinterpret_cast<const uint16_t*>(w)[(size_t)(co0 + co) * 147 + r * 21 + tt] : (uint16_t)0;
         }
         *reinterpret_cast<uint4*>(b_tile + (chunk >> 3) * 8192 + co * 128 + (((chunk & 7) ^ (co & 7)) * 16)) = *reinterpret_cast<const uint4*>(v);
     }
@@ -2612,8 +2631,10 @@ tc_conv_stem_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
 // 10-13 add up the first accumulator, 14-17 the second (3 -> 32 at 224 x 224, 16 images 1.3e-6 -> 1.5e-7, CUDA cores 3.6e-7).
 template <bool SHORT>
 __global__ void __launch_bounds__(kStemWgradThreads + (SHORT ? 128 : 0), 1)
-tc_wgrad_stem_kernel(const __nv_bfloat16* __restrict__ x, const __grid_constant__ CUtensorMap map_dz, float* __restrict__ partial,
+tc_wgrad_stem_kernel(const __nv_bfloat16* x, const __grid_constant__ CUtensorMap map_dz, float* partial,
                      StemParams p, int* status) {
+    previous_grid_done();
+    next_grid_may_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* const smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* const a_tiles = smem_al;                       // [2][atoms 2, 0, 1][128 pixels][128 bytes]
@@ -2793,7 +2814,7 @@ struct FcParams {
 };
 
 __global__ void __launch_bounds__(kThreads, 1)
-tc_fc_fwd_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, float* __restrict__ partial,
+tc_fc_fwd_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, float* partial,
                  FcParams p, int* status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -2824,6 +2845,8 @@ tc_fc_fwd_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     if (warp == 0 && lane == 0) {
         int issued = 0;
@@ -2892,8 +2915,10 @@ tc_fc_fwd_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
 }
 
 // out[b][co] = round(act(bias[co] + sum over slices, in slice order))
-__global__ void fc_reduce_kernel(const float* __restrict__ partial, int slices, int64_t elems, int c_out, const float* __restrict__ bias,
-                                 int relu, __nv_bfloat16* __restrict__ out) {
+__global__ void fc_reduce_kernel(const float* partial, int slices, int64_t elems, int c_out, const float* bias,
+                                 int relu, __nv_bfloat16* out) {
+    previous_grid_done();
+    next_grid_may_start();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= elems) return;
     float sum = 0.f;
@@ -2904,7 +2929,9 @@ __global__ void fc_reduce_kernel(const float* __restrict__ partial, int slices, 
 }
 
 // wt[ci][tap'][co] = w[co][taps-1-tap'][ci]: the matrix of the transposed convolution (stride 1).
-__global__ void transpose_flip_kernel(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wt, int c_out, int taps, int c_in) {
+__global__ void transpose_flip_kernel(const __nv_bfloat16* w, __nv_bfloat16* wt, int c_out, int taps, int c_in) {
+    previous_grid_done();
+    next_grid_may_start();
     const int64_t total = (int64_t)c_out * taps * c_in;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int co = (int)(i % c_out);
@@ -2953,7 +2980,9 @@ __device__ __forceinline__ void store_group_sum(float4 acc, float4* out, bool ok
 // Pair-view wgrad partials [slice][(q, c_out)][column 4][dy 3][c_in 64] -> dW[c_out][dy][dx][c_in]: pixel q of a pair
 // sees filter column dx in accumulator column dx + q.
 template <int Y>
-__global__ void __launch_bounds__(32 * Y) pairview_fold_kernel(const float* __restrict__ partial, float* __restrict__ out, int c_out, int slices, SgdUpdate upd) {
+__global__ void __launch_bounds__(32 * Y) pairview_fold_kernel(const float* partial, float* out, int c_out, int slices, SgdUpdate upd) {
+    previous_grid_done();
+    next_grid_may_start();
     const int idx = blockIdx.x * 32 + threadIdx.x;            // one float4 of the output
     const bool ok = idx < c_out * 144;
     const int ci = (idx % 16) * 4, dx = (idx / 16) % 3, dy = (idx / 48) % 3, co = ok ? idx / 144 : 0;
@@ -2972,7 +3001,9 @@ __global__ void __launch_bounds__(32 * Y) pairview_fold_kernel(const float* __re
 }
 
 template <int X, int Y>
-__global__ void __launch_bounds__(X * Y) slice_sum4_kernel(const float4* __restrict__ partial, float4* __restrict__ out, int64_t elems4, int slices, SgdUpdate upd) {
+__global__ void __launch_bounds__(X * Y) slice_sum4_kernel(const float4* partial, float4* out, int64_t elems4, int slices, SgdUpdate upd) {
+    previous_grid_done();
+    next_grid_may_start();
     const int64_t e = (int64_t)blockIdx.x * X + threadIdx.x;
     const bool ok = e < elems4;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -2983,7 +3014,9 @@ __global__ void __launch_bounds__(X * Y) slice_sum4_kernel(const float4* __restr
     store_group_sum<X, Y>(acc, out + e, ok, upd, e);
 }
 
-__global__ void slice_sum_tc_kernel(const float* __restrict__ partial, float* __restrict__ out, int64_t elems, int slices) {
+__global__ void slice_sum_tc_kernel(const float* partial, float* out, int64_t elems, int slices) {
+    previous_grid_done();
+    next_grid_may_start();
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= elems) return;
     float s = 0.f;
@@ -2997,15 +3030,15 @@ __global__ void slice_sum_tc_kernel(const float* __restrict__ partial, float* __
 int slice_sum(const float* partial, float* out, int64_t elems, int slices, void* stream, const SgdUpdate& upd) {
     cudaStream_t st = (cudaStream_t)stream;
     if (elems % 4 || ((uintptr_t)partial | (uintptr_t)out) % 16 || (upd.w && (uintptr_t)upd.w % 16)) {
-        slice_sum_tc_kernel<<<(unsigned)((elems + 255) / 256), 256, 0, st>>>(partial, out, elems, slices);
+        launch(Start::ON_STREAMS, slice_sum_tc_kernel, (unsigned)((elems + 255) / 256), 256, 0, st, partial, out, elems, slices);
         CKPT_LAUNCH_CHECK_NAMED("slice_sum_kernel", "wgrad slice sum");
         return sgd_update(upd, out, elems, st);
     }
     const int64_t elems4 = elems / 4;
     const unsigned blocks = (unsigned)((elems4 + 31) / 32);
-    if (slices >= 16) slice_sum4_kernel<32, 8><<<blocks, dim3(32, 8), 0, st>>>((const float4*)partial, (float4*)out, elems4, slices, upd);
-    else if (slices >= 4) slice_sum4_kernel<32, 4><<<blocks, dim3(32, 4), 0, st>>>((const float4*)partial, (float4*)out, elems4, slices, upd);
-    else slice_sum4_kernel<256, 1><<<(unsigned)((elems4 + 255) / 256), dim3(256, 1), 0, st>>>((const float4*)partial, (float4*)out, elems4, slices, upd);
+    if (slices >= 16) launch(Start::ON_STREAMS, slice_sum4_kernel<32, 8>, blocks, dim3(32, 8), 0, st, (const float4*)partial, (float4*)out, elems4, slices, upd);
+    else if (slices >= 4) launch(Start::ON_STREAMS, slice_sum4_kernel<32, 4>, blocks, dim3(32, 4), 0, st, (const float4*)partial, (float4*)out, elems4, slices, upd);
+    else launch(Start::ON_STREAMS, slice_sum4_kernel<256, 1>, (unsigned)((elems4 + 255) / 256), dim3(256, 1), 0, st, (const float4*)partial, (float4*)out, elems4, slices, upd);
     CKPT_LAUNCH_CHECK_NAMED("slice_sum_kernel", "wgrad slice sum");
     return CKPT_OK;
 }
@@ -3122,7 +3155,7 @@ int launch_c64(const void* x, const void* w_mat, void* out, float* stat_partial,
     const size_t smem = 9 * 64 * 128 + 2 * 3 * (size_t)p.box_stride + 1024 + 256;
     static DeviceFlags ready;
     if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_c64_kernel}, 220 * 1024)) return bad;
-    tc_conv_c64_kernel<<<p.ctas_per_n * p.n_tiles, kThreads, smem, st>>>(mx, mw, (__nv_bfloat16*)out, stat_partial, p, status);
+    launch(Start::EARLY, tc_conv_c64_kernel, p.ctas_per_n * p.n_tiles, kThreads, smem, st, mx, mw, (__nv_bfloat16*)out, stat_partial, p, status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_c64_kernel", what);
     if (stat_blocks) *stat_blocks = 4 * p.ctas_per_n;
     return CKPT_OK;
@@ -3174,8 +3207,8 @@ int launch_generic(FwdParams p, const void* a, int a_n, int a_h, int a_w, const 
     const bool gather = stat_partial && stat_blocks && !bias && !relu && !b_mn && p.bn >= 32 && p.out_stride == 1 &&
                         p.taps * ((c_red + 63) / 64) >= 16;
     if (gather) *stat_blocks = 4 * p.ctas_per_n;
-    if (b_mn) tc_conv_fwd_kernel<true><<<(unsigned)ctas, kThreads, smem, st>>>(mx, mw, (__nv_bfloat16*)out, bias, relu, nullptr, p, status);
-    else tc_conv_fwd_kernel<false><<<(unsigned)ctas, kThreads, smem, st>>>(mx, mw, (__nv_bfloat16*)out, bias, relu, gather ? stat_partial : nullptr, p, status);
+    if (b_mn) launch(Start::EARLY, tc_conv_fwd_kernel<true>, (unsigned)ctas, kThreads, smem, st, mx, mw, (__nv_bfloat16*)out, bias, relu, nullptr, p, status);
+    else launch(Start::EARLY, tc_conv_fwd_kernel<false>, (unsigned)ctas, kThreads, smem, st, mx, mw, (__nv_bfloat16*)out, bias, relu, gather ? stat_partial : nullptr, p, status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_fwd_kernel", what);
     return CKPT_OK;
 }
@@ -3363,7 +3396,7 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
         if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_tp_kernel<false, false>, (const void*)tc_conv_tp_kernel<true, false>,
                                                    (const void*)tc_conv_tp_kernel<false, true>}, (int)kTpSmem)) return bad;
         const auto kernel = act_out ? tc_conv_tp_kernel<false, true> : a_mn ? tc_conv_tp_kernel<true, false> : tc_conv_tp_kernel<false, false>;
-        kernel<<<p.ctas_per_co * p.co_tiles, kTpThreads, kTpSmem, st>>>(mx, mw, mo, madd, stat_blocks ? stat_partial : nullptr, p, status);
+        launch(Start::EARLY, kernel, p.ctas_per_co * p.co_tiles, kTpThreads, kTpSmem, st, mx, mw, mo, madd, stat_blocks ? stat_partial : nullptr, p, status);
         CKPT_LAUNCH_CHECK_NAMED("tc_conv_tp_kernel", what);
         return CKPT_OK;
     }
@@ -3372,10 +3405,11 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
     if (p.split > 1) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreadsT); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = (unsigned)p.split; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr; cfg.numAttrs = 1;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)p.split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        start_early(&cfg, attr, Start::EARLY);
         const auto kernel = p.join_add ? (a_mn ? tc_conv_t_kernel<true, true, EPI_JOIN> : tc_conv_t_kernel<false, true, EPI_RESIDUAL>)
                             : act_out ? tc_conv_t_kernel<false, true, EPI_ACT>
                             : a_mn ? tc_conv_t_kernel<true, true, EPI_PLAIN> : tc_conv_t_kernel<false, true, EPI_PLAIN>;
@@ -3385,7 +3419,7 @@ int launch_t_core(TParams p, const void* x, int x_channels, const CUtensorMap& m
         const auto kernel = p.join_add ? (a_mn ? tc_conv_t_kernel<true, false, EPI_JOIN> : tc_conv_t_kernel<false, false, EPI_RESIDUAL>)
                             : act_out ? tc_conv_t_kernel<false, false, EPI_ACT>
                             : a_mn ? tc_conv_t_kernel<true, false, EPI_PLAIN> : tc_conv_t_kernel<false, false, EPI_PLAIN>;
-        kernel<<<grid, kThreadsT, smem, st>>>(mx, mw, mo, madd, mmask, stats, p, status);
+        launch(Start::EARLY, kernel, grid, kThreadsT, smem, st, mx, mw, mo, madd, mmask, stats, p, status);
     }
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_t_kernel", what);
     return CKPT_OK;
@@ -3531,10 +3565,10 @@ int launch_fc(const ConvGeom& g, const void* x, const void* w, void* z, const fl
     static DeviceFlags ready;
     if (int bad = allow_shared_memory(ready, {(const void*)tc_fc_fwd_kernel}, kSmemBudget + 2048)) return bad;
     dim3 grid(m_tiles, slices);
-    tc_fc_fwd_kernel<<<grid, kThreads, smem, st>>>(mw, mx, (float*)scratch, p, status);
+    launch(Start::EARLY, tc_fc_fwd_kernel, grid, kThreads, smem, st, mw, mx, (float*)scratch, p, status);
     CKPT_LAUNCH_CHECK_NAMED("tc_fc_fwd_kernel", "fully connected forward (tensor cores)");
     const int64_t elems = (int64_t)g.n * g.cout;
-    fc_reduce_kernel<<<(unsigned)((elems + 255) / 256), 256, 0, st>>>((const float*)scratch, slices, elems, g.cout, bias, relu,
+    launch(Start::ON_STREAMS, fc_reduce_kernel, (unsigned)((elems + 255) / 256), 256, 0, st, (const float*)scratch, slices, elems, g.cout, bias, relu,
                                                                       (__nv_bfloat16*)z);
     CKPT_LAUNCH_CHECK_NAMED("fc_reduce_kernel", "fully connected slice sum");
     return CKPT_OK;
@@ -3775,7 +3809,7 @@ int tc_first_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, 
     if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_first_kernel}, (int)kFirstSmem)) return bad;
     dim3 grid((unsigned)std::min(p.m_tiles, kFirstCtasPerSm * sms), (unsigned)((g.cout + 63) / 64));
     if (blocks) *blocks = partial ? (int)grid.x : 0;
-    tc_conv_first_kernel<<<grid, kFirstThreads, kFirstSmem, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)w,
+    launch(Start::ON_STREAMS, tc_conv_first_kernel, grid, kFirstThreads, kFirstSmem, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)w,
                                                                                    map_out, partial, p, device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_first_kernel", "first-layer conv forward (tensor cores)");
     return CKPT_OK;
@@ -3832,7 +3866,7 @@ int stem_conv_fwd(const ConvGeom& g, const void* x, const void* w, void* z, int*
     const int co_tiles = (g.cout + 63) / 64;
     dim3 grid((unsigned)std::min(p.m_tiles, std::max(1, sm_count() / co_tiles)), (unsigned)co_tiles);
     if (blocks) *blocks = partial ? (int)grid.x : 0;
-    tc_conv_stem_kernel<<<grid, kStemFwdThreads, kStemFwdSmem, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)w,
+    launch(Start::EARLY, tc_conv_stem_kernel, grid, kStemFwdThreads, kStemFwdSmem, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)w,
                                                                                   map_out, partial, p, device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_stem_kernel", "stem conv forward (tensor cores)");
     return CKPT_OK;
@@ -3856,8 +3890,8 @@ int stem_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw,
     static DeviceFlags ready;
     if (int bad = allow_shared_memory(ready, {(const void*)tc_wgrad_stem_kernel<false>, (const void*)tc_wgrad_stem_kernel<true>}, (int)kStemWgradSmem)) return bad;
     dim3 grid((unsigned)p.slices, (unsigned)((g.cout + 63) / 64));
-    if (g.cout % 64) tc_wgrad_stem_kernel<true><<<grid, kStemWgradThreads + 128, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
-    else tc_wgrad_stem_kernel<false><<<grid, kStemWgradThreads, kStemWgradSmem, st>>>((const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
+    if (g.cout % 64) launch(Start::EARLY, tc_wgrad_stem_kernel<true>, grid, kStemWgradThreads + 128, kStemWgradSmem, st, (const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
+    else launch(Start::EARLY, tc_wgrad_stem_kernel<false>, grid, kStemWgradThreads, kStemWgradSmem, st, (const __nv_bfloat16*)x, map_dz, (float*)scratch, p, device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_stem_kernel", "stem conv wgrad (tensor cores)");
     return slice_sum((const float*)scratch, dw, (int64_t)g.cout * 147, p.slices, st, upd);
 }
@@ -3964,7 +3998,7 @@ int tc_conv_dgrad(const ConvGeom& g, const void* dz, const void* w, void* dx, vo
             const int64_t elems = (int64_t)g.cout * taps * g.cin;
             if (!scratch || scratch_bytes < elems * 2) { set_error("dgrad scratch too small"); return CKPT_E_WORKSPACE; }
             const unsigned grid = (unsigned)std::min<int64_t>((elems + 255) / 256, 148 * 8);
-            transpose_flip_kernel<<<grid, 256, 0, st>>>((const __nv_bfloat16*)w, (__nv_bfloat16*)scratch, g.cout, taps, g.cin);
+            launch(Start::ON_STREAMS, transpose_flip_kernel, grid, 256, 0, st, (const __nv_bfloat16*)w, (__nv_bfloat16*)scratch, g.cout, taps, g.cin);
             CKPT_LAUNCH_CHECK_NAMED("transpose_flip_kernel", "dgrad matrix transpose");
             w_mat = scratch;
         }
@@ -4068,9 +4102,9 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         dim3 grid(p.slices, 4 / p.cols, co_tiles);
         CUtensorMap mo;
         if ((rc = make_partial_map(&mo, (float*)scratch, 64, 12, 2 * g.cout, p.slices))) return rc;
-        tc_wgrad_rows_kernel<false><<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
+        launch(Start::EARLY, tc_wgrad_rows_kernel<false>, grid, kThreads, smem, st, mdz, mx, mo, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_rows_kernel (pixel pairs)", "conv wgrad, 64 input channels as pixel pairs (tensor cores)");
-        pairview_fold_kernel<8><<<(unsigned)((g.cout * 144 + 31) / 32), dim3(32, 8), 0, st>>>((const float*)scratch, dw, g.cout, p.slices, upd);
+        launch(Start::ON_STREAMS, pairview_fold_kernel<8>, (unsigned)((g.cout * 144 + 31) / 32), dim3(32, 8), 0, st, (const float*)scratch, dw, g.cout, p.slices, upd);
         CKPT_LAUNCH_CHECK_NAMED("pairview_fold_kernel", "wgrad pair fold");
         return CKPT_OK;
     }
@@ -4089,7 +4123,7 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         if (int bad = allow_shared_memory(ready, {(const void*)tc_wgrad_c64_kernel}, 222 * 1024)) return bad;
         const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
         dim3 grid(p.slices, g.cout / 64);
-        tc_wgrad_c64_kernel<<<grid, kThreads, smem, st>>>(mdz, mx, (float*)scratch, p, device_status);
+        launch(Start::EARLY, tc_wgrad_c64_kernel, grid, kThreads, smem, st, mdz, mx, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_c64_kernel", "conv wgrad, 64 input channels (tensor cores)");
         return slice_sum((const float*)scratch, dw, elems, p.slices, st, upd);
     }
@@ -4111,8 +4145,8 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
         dim3 grid(p.slices, pairs, co_tiles);
         CUtensorMap mo;
         if ((rc = make_partial_map(&mo, (float*)scratch, g.cin, 9, g.cout, p.slices))) return rc;
-        if (wgrad_short_chains(g)) tc_wgrad_rows_kernel<true><<<grid, kThreadsShort, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
-        else tc_wgrad_rows_kernel<false><<<grid, kThreads, smem, st>>>(mdz, mx, mo, (float*)scratch, p, device_status);
+        if (wgrad_short_chains(g)) launch(Start::EARLY, tc_wgrad_rows_kernel<true>, grid, kThreadsShort, smem, st, mdz, mx, mo, (float*)scratch, p, device_status);
+        else launch(Start::EARLY, tc_wgrad_rows_kernel<false>, grid, kThreads, smem, st, mdz, mx, mo, (float*)scratch, p, device_status);
         CKPT_LAUNCH_CHECK_NAMED("tc_wgrad_rows_kernel", "conv wgrad, shared vertical taps (tensor cores)");
         return slice_sum((const float*)scratch, dw, elems, p.slices, st, upd);
     }
@@ -4139,8 +4173,8 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
     if (p.tile_store && (rc = make_partial_map(&mo, target, g.cin, g.k * g.k, g.cout, slices))) return rc;
     dim3 grid(slices, groups, co_tiles);
     const bool update = slices == 1 && upd.w && upd.dtype == CKPT_DTYPE_BF16 && (uintptr_t)upd.w % 16 == 0;
-    if (chains) tc_conv_wgrad_kernel<true><<<grid, kThreadsShort, smem, st>>>(mdz, mx, mo, target, p, update ? upd : SgdUpdate(), device_status);
-    else tc_conv_wgrad_kernel<false><<<grid, kThreads, smem, st>>>(mdz, mx, mo, target, p, update ? upd : SgdUpdate(), device_status);
+    if (chains) launch(Start::EARLY, tc_conv_wgrad_kernel<true>, grid, kThreadsShort, smem, st, mdz, mx, mo, target, p, update ? upd : SgdUpdate(), device_status);
+    else launch(Start::EARLY, tc_conv_wgrad_kernel<false>, grid, kThreads, smem, st, mdz, mx, mo, target, p, update ? upd : SgdUpdate(), device_status);
     CKPT_LAUNCH_CHECK_NAMED("tc_conv_wgrad_kernel", "conv wgrad (tensor cores)");
     if (slices > 1) return slice_sum((const float*)scratch, dw, elems, slices, st, upd);
     if (upd.w && !update) return sgd_update(upd, dw, elems, st);

@@ -14,6 +14,7 @@
 
 #include "conv_simt.cuh"
 #include "internal.h"
+#include "overlap.cuh"
 #include "vec.cuh"
 
 namespace ckpt {
@@ -188,10 +189,12 @@ int64_t bn_scratch_bytes(int64_t rows, int c) {
 // g = dy masked by the ReLU of the forward output (the normalised form g*xhat follows in the
 // finalize step: sum g*xhat = inv_std * (sum g*z - mean * sum g)).
 template <typename T, int VEC, int WHAT>
-__global__ void __launch_bounds__(BN_THREADS, 3) bn_partial_kernel(const T* __restrict__ z, const T* __restrict__ dy,
-                                                                   const float* __restrict__ stats, int relu, int64_t rows,
+__global__ void __launch_bounds__(BN_THREADS, 3) bn_partial_kernel(const T* z, const T* dy,
+                                                                   const float* stats, int relu, int64_t rows,
                                                                    int c, int lanes, int rows_per_iter, int64_t rows_per_block,
-                                                                   float* __restrict__ partial) {
+                                                                   float* partial) {
+    previous_grid_done();
+    next_grid_may_start();
     extern __shared__ float red[];          // [BN_THREADS][2*VEC]
     constexpr int U = WHAT == 0 ? 4 : 2;    // rows in flight per thread
     const int lanes_here = min(lanes, BN_THREADS);
@@ -269,7 +272,7 @@ __global__ void __launch_bounds__(BN_THREADS, 3) bn_partial_kernel(const T* __re
 // of the warps' sums (batch norm forward of 25088 x 64, us: one channel per warp in doubles 8.8, eight lanes adding up sixteen
 // warps in turn 9.6, this 9.2; backward by separate kernels 13.0 -> 12.3).
 constexpr int FIN_CH = 8, FIN_ROWS = 64, FIN_THREADS = FIN_CH * FIN_ROWS;
-__device__ __forceinline__ bool block_channel_sums(const float* __restrict__ partial, int blocks, int c, int ch, double& s, double& q) {
+__device__ __forceinline__ bool block_channel_sums(const float* partial, int blocks, int c, int ch, double& s, double& q) {
     __shared__ float4 red[FIN_THREADS / 32][FIN_CH];
     const int row = threadIdx.x / FIN_CH, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
@@ -316,8 +319,10 @@ __device__ __forceinline__ bool block_channel_sums(const float* __restrict__ par
 }
 
 // mean, 1/sqrt(var+eps), scale = gamma*inv, shift = beta - mean*scale.
-__global__ void __launch_bounds__(FIN_THREADS) bn_finalize_fwd_kernel(const float* __restrict__ partial, int blocks, int c, double inv_rows,
-                                       const float* __restrict__ gamma, const float* __restrict__ beta, float* __restrict__ stats) {
+__global__ void __launch_bounds__(FIN_THREADS) bn_finalize_fwd_kernel(const float* partial, int blocks, int c, double inv_rows,
+                                       const float* gamma, const float* beta, float* stats) {
+    previous_grid_done();
+    next_grid_may_start();
     const int ch = blockIdx.x * FIN_CH + threadIdx.x % FIN_CH;
     const float g = ch < c ? gamma[ch] : 0.f, b = ch < c ? beta[ch] : 0.f;
     double s, q;
@@ -335,9 +340,11 @@ __global__ void __launch_bounds__(FIN_THREADS) bn_finalize_fwd_kernel(const floa
 
 // dbeta, dgamma and the two per-channel coefficients of the input gradient:
 //   dz = scale*g - k1 - xhat*k2,  k1 = scale*dbeta/rows, k2 = scale*dgamma/rows
-__global__ void __launch_bounds__(FIN_THREADS) bn_finalize_bwd_kernel(const float* __restrict__ partial, int blocks, int c, double inv_rows,
-                                       const float* __restrict__ stats, float* __restrict__ dgamma, float* __restrict__ dbeta,
-                                       float* __restrict__ coef, SgdUpdate gamma, SgdUpdate beta) {
+__global__ void __launch_bounds__(FIN_THREADS) bn_finalize_bwd_kernel(const float* partial, int blocks, int c, double inv_rows,
+                                       const float* stats, float* dgamma, float* dbeta,
+                                       float* coef, SgdUpdate gamma, SgdUpdate beta) {
+    previous_grid_done();
+    next_grid_may_start();
     const int ch = blockIdx.x * FIN_CH + threadIdx.x % FIN_CH;
     double s, q;
     if (!block_channel_sums(partial, blocks, c, ch, s, q)) return;
@@ -361,8 +368,10 @@ __global__ void __launch_bounds__(FIN_THREADS) bn_finalize_bwd_kernel(const floa
 // coefficients in registers and has U packed 16-byte loads in flight.
 constexpr int BN_APPLY_U = 8;
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256, 4) bn_apply_kernel(const T* __restrict__ z, const float* __restrict__ stats, int relu,
-                                                          int64_t vecs, int lanes, int c, int per_block, T* __restrict__ y) {
+__global__ void __launch_bounds__(256, 4) bn_apply_kernel(const T* z, const float* stats, int relu,
+                                                          int64_t vecs, int lanes, int c, int per_block, T* y) {
+    previous_grid_done();
+    next_grid_may_start();
     constexpr int U = BN_APPLY_U;
     const int64_t chunk = 256 * U;
     const int64_t begin = (int64_t)blockIdx.x * per_block * chunk;
@@ -422,10 +431,12 @@ __device__ __forceinline__ void bn_bwd_point(const float (&v)[VEC], const float 
 
 constexpr int BN_BWD_U = 4;
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256, 3) bn_bwd_apply_kernel(const T* __restrict__ dy, const T* __restrict__ z,
-                                                              const float* __restrict__ stats, const float* __restrict__ coef,
+__global__ void __launch_bounds__(256, 3) bn_bwd_apply_kernel(const T* dy, const T* z,
+                                                              const float* stats, const float* coef,
                                                               int relu, int64_t vecs, int lanes, int c, int per_block,
-                                                              T* __restrict__ dz) {
+                                                              T* dz) {
+    previous_grid_done();
+    next_grid_may_start();
     constexpr int U = BN_BWD_U;
     const int64_t chunk = 256 * U;
     const int64_t begin = (int64_t)blockIdx.x * per_block * chunk;
@@ -475,10 +486,12 @@ __global__ void __launch_bounds__(256, 3) bn_bwd_apply_kernel(const T* __restric
 // its threads by a fixed tree.  Same two sums as bn_partial_kernel.
 constexpr int BNF_THREADS = 384;
 template <typename T, int VEC, int WHAT>
-__global__ void __launch_bounds__(BNF_THREADS, 2) bn_partial_stream_kernel(const T* __restrict__ z, const T* __restrict__ dy,
-                                                                           const float* __restrict__ stats, int relu,
+__global__ void __launch_bounds__(BNF_THREADS, 2) bn_partial_stream_kernel(const T* z, const T* dy,
+                                                                           const float* stats, int relu,
                                                                            int64_t vecs, int lanes, int c,
-                                                                           float* __restrict__ partial) {
+                                                                           float* partial) {
+    previous_grid_done();
+    next_grid_may_start();
     __shared__ float red[BNF_THREADS][2 * VEC + 1];
     constexpr int U = WHAT == 0 ? 8 : 4;
     const int64_t stride = (int64_t)gridDim.x * BNF_THREADS;
@@ -565,14 +578,14 @@ static int bn_stats_t(int64_t rows, int c, const void* z, const float* gamma, co
     if (VEC > 1 && bn_stream_ok(L.lanes)) {
         const int64_t vecs = rows * c / VEC;
         blocks = bn_stream_blocks(vecs);
-        bn_partial_stream_kernel<T, VEC, 0><<<blocks, BNF_THREADS, 0, st>>>((const T*)z, nullptr, nullptr, 0, vecs, L.lanes, c, partial);
+        launch(Start::ON_STREAMS, bn_partial_stream_kernel<T, VEC, 0>, blocks, BNF_THREADS, 0, st, (const T*)z, nullptr, nullptr, 0, vecs, L.lanes, c, partial);
     } else {
         size_t smem = (size_t)BN_THREADS * 2 * VEC * sizeof(float);
-        bn_partial_kernel<T, VEC, 0><<<L.blocks, BN_THREADS, smem, st>>>((const T*)z, nullptr, nullptr, 0, rows, c, L.lanes,
+        launch(Start::ON_STREAMS, bn_partial_kernel<T, VEC, 0>, L.blocks, BN_THREADS, smem, st, (const T*)z, nullptr, nullptr, 0, rows, c, L.lanes,
                                                                           L.rows_per_iter, L.rows_per_block, partial);
     }
     CKPT_LAUNCH_CHECK("batch-norm statistics");
-    bn_finalize_fwd_kernel<<<(c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st>>>(partial, blocks, c, 1.0 / (double)rows, gamma, beta, stats);
+    launch(Start::ON_STREAMS, bn_finalize_fwd_kernel, (c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st, partial, blocks, c, 1.0 / (double)rows, gamma, beta, stats);
     CKPT_LAUNCH_CHECK("batch-norm finalize");
     return CKPT_OK;
 }
@@ -581,7 +594,7 @@ template <typename T, int VEC>
 static int bn_apply_t(int64_t rows, int c, const void* z, const float* stats, int relu, void* y, cudaStream_t st) {
     int64_t vecs = rows * c / VEC;
     const StreamGrid sg = stream_grid(vecs, 256, BN_APPLY_U);
-    bn_apply_kernel<T, VEC><<<sg.blocks, 256, 0, st>>>((const T*)z, stats, relu, vecs, c / VEC, c, sg.per_block, (T*)y);
+    launch(Start::ON_STREAMS, bn_apply_kernel<T, VEC>, sg.blocks, 256, 0, st, (const T*)z, stats, relu, vecs, c / VEC, c, sg.per_block, (T*)y);
     CKPT_LAUNCH_CHECK("batch-norm apply");
     return CKPT_OK;
 }
@@ -596,18 +609,18 @@ static int bn_backward_t(int64_t rows, int c, const void* dy, const void* z, con
     if (VEC > 1 && bn_stream_ok(L.lanes)) {
         const int64_t nvecs = rows * c / VEC;
         blocks = bn_stream_blocks(nvecs);
-        bn_partial_stream_kernel<T, VEC, 1><<<blocks, BNF_THREADS, 0, st>>>((const T*)z, (const T*)dy, stats, relu, nvecs, L.lanes, c, partial);
+        launch(Start::ON_STREAMS, bn_partial_stream_kernel<T, VEC, 1>, blocks, BNF_THREADS, 0, st, (const T*)z, (const T*)dy, stats, relu, nvecs, L.lanes, c, partial);
     } else {
         size_t smem = (size_t)BN_THREADS * 2 * VEC * sizeof(float);
-        bn_partial_kernel<T, VEC, 1><<<L.blocks, BN_THREADS, smem, st>>>((const T*)z, (const T*)dy, stats, relu, rows, c, L.lanes,
+        launch(Start::ON_STREAMS, bn_partial_kernel<T, VEC, 1>, L.blocks, BN_THREADS, smem, st, (const T*)z, (const T*)dy, stats, relu, rows, c, L.lanes,
                                                                           L.rows_per_iter, L.rows_per_block, partial);
     }
     CKPT_LAUNCH_CHECK("batch-norm backward sums");
-    bn_finalize_bwd_kernel<<<(c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st>>>(partial, blocks, c, 1.0 / (double)rows, stats, dgamma, dbeta, coef, ex.gamma, ex.beta);
+    launch(Start::ON_STREAMS, bn_finalize_bwd_kernel, (c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st, partial, blocks, c, 1.0 / (double)rows, stats, dgamma, dbeta, coef, ex.gamma, ex.beta);
     CKPT_LAUNCH_CHECK("batch-norm backward finalize");
     int64_t vecs = rows * c / VEC;
     const StreamGrid sg = stream_grid(vecs, 256, BN_BWD_U);
-    bn_bwd_apply_kernel<T, VEC><<<sg.blocks, 256, 0, st>>>((const T*)dy, (const T*)z, stats, coef, relu, vecs, L.lanes, c,
+    launch(Start::ON_STREAMS, bn_bwd_apply_kernel<T, VEC>, sg.blocks, 256, 0, st, (const T*)dy, (const T*)z, stats, coef, relu, vecs, L.lanes, c,
                                                            sg.per_block, (T*)dz);
     CKPT_LAUNCH_CHECK("batch-norm backward apply");
     return CKPT_OK;
@@ -617,7 +630,7 @@ static int bn_backward_t(int64_t rows, int c, const void* dy, const void* z, con
 // partial = [blocks][sum | sum of squares][c] floats.
 int bn_statistics_from_partials(const float* partial, int blocks, int64_t rows, int c, const float* gamma, const float* beta,
                                 float* stats, void* stream) {
-    bn_finalize_fwd_kernel<<<(c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, (cudaStream_t)stream>>>(partial, blocks, c, 1.0 / (double)rows, gamma, beta, stats);
+    launch(Start::ON_STREAMS, bn_finalize_fwd_kernel, (c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, (cudaStream_t)stream, partial, blocks, c, 1.0 / (double)rows, gamma, beta, stats);
     CKPT_LAUNCH_CHECK("batch-norm finalize");
     return CKPT_OK;
 }
@@ -652,9 +665,11 @@ int bn_relu_forward(int dtype, int64_t rows, int c, const void* z, const float* 
 // either an already activated tensor (stats_sc == nullptr) or a second pre-normalisation tensor with
 // its own scale/shift (projection branch).
 template <typename T>
-__global__ void __launch_bounds__(256) bn_add_relu_kernel(const T* __restrict__ z, const float* __restrict__ stats,
-                                                          const T* __restrict__ sc, const float* __restrict__ stats_sc,
-                                                          int64_t elems, int c, T* __restrict__ y) {
+__global__ void __launch_bounds__(256) bn_add_relu_kernel(const T* z, const float* stats,
+                                                          const T* sc, const float* stats_sc,
+                                                          int64_t elems, int c, T* y) {
+    previous_grid_done();
+    next_grid_may_start();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < elems; i += (int64_t)gridDim.x * blockDim.x) {
         const int ch = (int)(i % c);
         float v = fmaf(ld(z + i), stats[2 * c + ch], stats[3 * c + ch]);
@@ -667,9 +682,11 @@ __global__ void __launch_bounds__(256) bn_add_relu_kernel(const T* __restrict__ 
 // (the block size is a multiple of the number of groups) and keeps its coefficients in registers.
 constexpr int BN_JOIN_U = 4;
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256, 3) bn_add_relu_vec_kernel(const T* __restrict__ z, const float* __restrict__ stats,
-                                                                 const T* __restrict__ sc, const float* __restrict__ stats_sc,
-                                                                 int64_t vecs, int lanes, int c, int per_block, T* __restrict__ y) {
+__global__ void __launch_bounds__(256, 3) bn_add_relu_vec_kernel(const T* z, const float* stats,
+                                                                 const T* sc, const float* stats_sc,
+                                                                 int64_t vecs, int lanes, int c, int per_block, T* y) {
+    previous_grid_done();
+    next_grid_may_start();
     constexpr int U = BN_JOIN_U;
     const int64_t chunk = 256 * U;
     const int64_t begin = (int64_t)blockIdx.x * per_block * chunk;
@@ -710,7 +727,7 @@ static bool bn_add_relu_vec(int64_t rows, int c, const void* z, const float* sta
     if (c % VEC || 256 % (c / VEC)) return false;
     const int64_t vecs = rows * c / VEC;
     const StreamGrid sg = stream_grid(vecs, 256, BN_JOIN_U);
-    bn_add_relu_vec_kernel<T, VEC><<<sg.blocks, 256, 0, st>>>((const T*)z, stats, (const T*)shortcut, stats_shortcut, vecs, c / VEC, c,
+    launch(Start::ON_STREAMS, bn_add_relu_vec_kernel<T, VEC>, sg.blocks, 256, 0, st, (const T*)z, stats, (const T*)shortcut, stats_shortcut, vecs, c / VEC, c,
                                                               sg.per_block, (T*)y);
     return true;
 }
@@ -720,10 +737,10 @@ int bn_add_relu(int dtype, int64_t rows, int c, const void* z, const float* stat
     cudaStream_t st = (cudaStream_t)stream;
     if (dtype == CKPT_DTYPE_BF16) {
         if (!bn_add_relu_vec<__nv_bfloat16, 8>(rows, c, z, stats, shortcut, stats_shortcut, y, st))
-            bn_add_relu_kernel<__nv_bfloat16><<<elementwise_grid(elems), 256, 0, st>>>(
+            launch(Start::ON_STREAMS, bn_add_relu_kernel<__nv_bfloat16>, elementwise_grid(elems), 256, 0, st, 
                 (const __nv_bfloat16*)z, stats, (const __nv_bfloat16*)shortcut, stats_shortcut, elems, c, (__nv_bfloat16*)y);
     } else if (!bn_add_relu_vec<float, 4>(rows, c, z, stats, shortcut, stats_shortcut, y, st)) {
-        bn_add_relu_kernel<float><<<elementwise_grid(elems), 256, 0, st>>>(
+        launch(Start::ON_STREAMS, bn_add_relu_kernel<float>, elementwise_grid(elems), 256, 0, st, 
             (const float*)z, stats, (const float*)shortcut, stats_shortcut, elems, c, (float*)y);
     }
     CKPT_LAUNCH_CHECK("residual join");
@@ -731,13 +748,17 @@ int bn_add_relu(int dtype, int64_t rows, int c, const void* z, const float* stat
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) add_kernel(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out, int64_t elems) {
+__global__ void __launch_bounds__(256) add_kernel(const T* a, const T* b, T* out, int64_t elems) {
+    previous_grid_done();
+    next_grid_may_start();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < elems; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = cvt<T>(ld(a + i) + ld(b + i));
 }
 // 16-byte form of the sum (out may alias an input); four packed loads per operand in flight.
 template <typename T, int VEC>
 __global__ void __launch_bounds__(256) add_vec_kernel(const T* a, const T* b, T* out, int64_t vecs) {
+    previous_grid_done();
+    next_grid_may_start();
     constexpr int U = 4;
     for (int64_t i0 = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; i0 < vecs; i0 += (int64_t)gridDim.x * (256 * U)) {
         RawVec<T, VEC> ra[U], rb[U];
@@ -763,12 +784,12 @@ int add_tensors(int dtype, int64_t elems, const void* a, const void* b, void* ou
     if (elems % vec == 0 && aligned16(a) && aligned16(b) && aligned16(out)) {
         const int64_t vecs = elems / vec;
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((vecs + 1023) / 1024, 148 * 32));
-        if (dtype == CKPT_DTYPE_BF16) add_vec_kernel<__nv_bfloat16, 8><<<grid, 256, 0, st>>>((const __nv_bfloat16*)a, (const __nv_bfloat16*)b, (__nv_bfloat16*)out, vecs);
-        else add_vec_kernel<float, 4><<<grid, 256, 0, st>>>((const float*)a, (const float*)b, (float*)out, vecs);
+        if (dtype == CKPT_DTYPE_BF16) launch(Start::ON_STREAMS, add_vec_kernel<__nv_bfloat16, 8>, grid, 256, 0, st, (const __nv_bfloat16*)a, (const __nv_bfloat16*)b, (__nv_bfloat16*)out, vecs);
+        else launch(Start::ON_STREAMS, add_vec_kernel<float, 4>, grid, 256, 0, st, (const float*)a, (const float*)b, (float*)out, vecs);
     } else if (dtype == CKPT_DTYPE_BF16) {
-        add_kernel<__nv_bfloat16><<<elementwise_grid(elems), 256, 0, st>>>((const __nv_bfloat16*)a, (const __nv_bfloat16*)b, (__nv_bfloat16*)out, elems);
+        launch(Start::ON_STREAMS, add_kernel<__nv_bfloat16>, elementwise_grid(elems), 256, 0, st, (const __nv_bfloat16*)a, (const __nv_bfloat16*)b, (__nv_bfloat16*)out, elems);
     } else {
-        add_kernel<float><<<elementwise_grid(elems), 256, 0, st>>>((const float*)a, (const float*)b, (float*)out, elems);
+        launch(Start::ON_STREAMS, add_kernel<float>, elementwise_grid(elems), 256, 0, st, (const float*)a, (const float*)b, (float*)out, elems);
     }
     CKPT_LAUNCH_CHECK("gradient join");
     return CKPT_OK;
@@ -798,11 +819,11 @@ static int bn_backward_tail_t(int64_t rows, int c, const void* dy, const void* z
                               float* dgamma, float* dbeta, void* scratch, int blocks, const BnBackwardExtra& ex, cudaStream_t st) {
     float* partial = (float*)scratch;
     float* coef = partial + (size_t)BN_MAX_BLOCKS * c * 2;
-    bn_finalize_bwd_kernel<<<(c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st>>>(partial, blocks, c, 1.0 / (double)rows, stats, dgamma, dbeta, coef, ex.gamma, ex.beta);
+    launch(Start::ON_STREAMS, bn_finalize_bwd_kernel, (c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st, partial, blocks, c, 1.0 / (double)rows, stats, dgamma, dbeta, coef, ex.gamma, ex.beta);
     CKPT_LAUNCH_CHECK("batch-norm backward finalize");
     const int64_t vecs = rows * c / VEC;
     const StreamGrid sg = stream_grid(vecs, 256, BN_BWD_U);
-    bn_bwd_apply_kernel<T, VEC><<<sg.blocks, 256, 0, st>>>((const T*)dy, (const T*)z, stats, coef, relu, vecs, c / VEC, c,
+    launch(Start::ON_STREAMS, bn_bwd_apply_kernel<T, VEC>, sg.blocks, 256, 0, st, (const T*)dy, (const T*)z, stats, coef, relu, vecs, c / VEC, c,
                                                            sg.per_block, (T*)dz);
     CKPT_LAUNCH_CHECK("batch-norm backward apply");
     return CKPT_OK;
@@ -824,8 +845,10 @@ int bn_relu_backward_from_partials(int dtype, int64_t rows, int c, const void* d
 // Pooling
 // ================================================================================================
 template <typename T>
-__global__ void maxpool_fwd_kernel(const T* __restrict__ x, T* __restrict__ y, int n, int h, int w, int c, int ho, int wo,
+__global__ void maxpool_fwd_kernel(const T* x, T* y, int n, int h, int w, int c, int ho, int wo,
                                    int k, int stride, int pad) {
+    previous_grid_done();
+    next_grid_may_start();
     int64_t total = (int64_t)n * ho * wo * c;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         int ch = (int)(i % c);
@@ -850,8 +873,10 @@ __global__ void maxpool_fwd_kernel(const T* __restrict__ x, T* __restrict__ y, i
 // Gather form: every input element looks at the windows that contain it and takes the gradient of
 // those in which it is the first maximum (row-major window order).
 template <typename T>
-__global__ void maxpool_bwd_kernel(const T* __restrict__ x, const T* __restrict__ dy, T* __restrict__ dx, int n, int h, int w,
+__global__ void maxpool_bwd_kernel(const T* x, const T* dy, T* dx, int n, int h, int w,
                                    int c, int ho, int wo, int k, int stride, int pad) {
+    previous_grid_done();
+    next_grid_may_start();
     int64_t total = (int64_t)n * h * w * c;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         int ch = (int)(i % c);
@@ -890,15 +915,17 @@ __global__ void maxpool_bwd_kernel(const T* __restrict__ x, const T* __restrict_
 // Optional pending activation of the producer: value = round_T(max(v*scale + shift, 0)), exactly what a
 // materialised copy of the activated tensor would hold.
 template <typename T, int VEC>
-__device__ __forceinline__ void pending_act(float (&v)[VEC], const float* __restrict__ act, int c, int ch) {
+__device__ __forceinline__ void pending_act(float (&v)[VEC], const float* act, int c, int ch) {
     if (!act) return;
 #pragma unroll
     for (int k = 0; k < VEC; ++k) v[k] = (float)cvt<T>(fmaxf(fmaf(v[k], act[2 * c + ch + k], act[3 * c + ch + k]), 0.f));
 }
 
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) maxpool2x2_fwd_kernel(const T* __restrict__ x, T* __restrict__ y, int64_t items, int wo, int ho, int cv, int c,
-                                                             const float* __restrict__ act) {
+__global__ void __launch_bounds__(256) maxpool2x2_fwd_kernel(const T* x, T* y, int64_t items, int wo, int ho, int cv, int c,
+                                                             const float* act) {
+    previous_grid_done();
+    next_grid_may_start();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
         const int cg = (int)(i % cv);
         int64_t t = i / cv;
@@ -921,8 +948,10 @@ __global__ void __launch_bounds__(256) maxpool2x2_fwd_kernel(const T* __restrict
 
 // Backward of the same: the first maximum of the window in row-major order takes the gradient.
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) maxpool2x2_bwd_kernel(const T* __restrict__ x, const T* __restrict__ dy, T* __restrict__ dx,
-                                                             int64_t items, int wo, int ho, int cv, int c, const float* __restrict__ act) {
+__global__ void __launch_bounds__(256) maxpool2x2_bwd_kernel(const T* x, const T* dy, T* dx,
+                                                             int64_t items, int wo, int ho, int cv, int c, const float* act) {
+    previous_grid_done();
+    next_grid_may_start();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
         const int cg = (int)(i % cv);
         int64_t t = i / cv;
@@ -958,9 +987,11 @@ __global__ void __launch_bounds__(256) maxpool2x2_bwd_kernel(const T* __restrict
 // for free.  Every thread keeps one channel group (grid stride a multiple of the group count); partial
 // rows [block][sum | sum g*z][c] in a fixed order.
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) maxpool2x2_bwd_sums_kernel(const T* __restrict__ x, const T* __restrict__ dy, T* __restrict__ dx,
+__global__ void __launch_bounds__(256) maxpool2x2_bwd_sums_kernel(const T* x, const T* dy, T* dx,
                                                                   int64_t items, int wo, int ho, int cv, int c,
-                                                                  const float* __restrict__ act, float* __restrict__ partial) {
+                                                                  const float* act, float* partial) {
+    previous_grid_done();
+    next_grid_may_start();
     __shared__ float red[256][2 * VEC + 1];
     const int cg = (int)(((int64_t)blockIdx.x * 256 + threadIdx.x) % cv);
     float sc[VEC], sh[VEC], s0[VEC], s1[VEC];
@@ -1036,7 +1067,7 @@ bool maxpool_fuses_activation(int dtype, int h, int w, int c, int k, int stride,
 // grows with z where the scale is positive and falls where it is negative, so the forward takes the maximum of z (its sign
 // flipped for negative scales) in packed pairs and normalises nine times less.  A thread owns eight channels of a window,
 // its nine loads in flight at once.
-__device__ __forceinline__ void pool3_load(const __nv_bfloat16* __restrict__ z, int64_t img, int oh, int ow, int h, int w, int c, int ch, uint4 (&r)[9], uint32_t& valid) {
+__device__ __forceinline__ void pool3_load(const __nv_bfloat16* z, int64_t img, int oh, int ow, int h, int w, int c, int ch, uint4 (&r)[9], uint32_t& valid) {
     valid = 0u;
 #pragma unroll
     for (int t = 0; t < 9; ++t) {
@@ -1048,8 +1079,10 @@ __device__ __forceinline__ void pool3_load(const __nv_bfloat16* __restrict__ z, 
     }
 }
 __device__ __forceinline__ uint32_t& word(uint4& v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
-__global__ void __launch_bounds__(256) maxpool3_fwd_act_kernel(const __nv_bfloat16* __restrict__ z, __nv_bfloat16* __restrict__ y, int64_t items, int h, int w,
-                                                               int c, int ho, int wo, const float* __restrict__ act) {
+__global__ void __launch_bounds__(256) maxpool3_fwd_act_kernel(const __nv_bfloat16* z, __nv_bfloat16* y, int64_t items, int h, int w,
+                                                               int c, int ho, int wo, const float* act) {
+    previous_grid_done();
+    next_grid_may_start();
     const int lanes = c / 8;
     const int ch = (int)(threadIdx.x % lanes) * 8;              // 256 and the grid stride are multiples of `lanes`
     float sc[8], sh[8];
@@ -1087,8 +1120,10 @@ __global__ void __launch_bounds__(256) maxpool3_fwd_act_kernel(const __nv_bfloat
     }
 }
 // Position (0..8) of the first maximum of the normalised values, one byte per channel.
-__global__ void __launch_bounds__(256) maxpool3_arg_act_kernel(const __nv_bfloat16* __restrict__ z, uint8_t* __restrict__ arg, int64_t items, int h, int w,
-                                                               int c, int ho, int wo, const float* __restrict__ act) {
+__global__ void __launch_bounds__(256) maxpool3_arg_act_kernel(const __nv_bfloat16* z, uint8_t* arg, int64_t items, int h, int w,
+                                                               int c, int ho, int wo, const float* act) {
+    previous_grid_done();
+    next_grid_may_start();
     const int lanes = c / 8;
     const int ch = (int)(threadIdx.x % lanes) * 8;
     float sc[8], sh[8];
@@ -1125,9 +1160,11 @@ __global__ void __launch_bounds__(256) maxpool3_arg_act_kernel(const __nv_bfloat
 // to window a only (its middle row), an odd one to windows a (last row) and a + 1 (first row).  With `act` the producer's
 // batch-norm backward sums (sum g, sum g*z over the values its ReLU passes) go to `partial` as in the 2x2 kernel.
 template <bool SUMS>
-__global__ void __launch_bounds__(256) maxpool3_bwd_kernel(const uint8_t* __restrict__ arg, const __nv_bfloat16* __restrict__ dy, __nv_bfloat16* __restrict__ dx,
-                                                           int64_t items, int h, int w, int c, int ho, int wo, const __nv_bfloat16* __restrict__ z,
-                                                           const float* __restrict__ act, float* __restrict__ partial) {
+__global__ void __launch_bounds__(256) maxpool3_bwd_kernel(const uint8_t* arg, const __nv_bfloat16* dy, __nv_bfloat16* dx,
+                                                           int64_t items, int h, int w, int c, int ho, int wo, const __nv_bfloat16* z,
+                                                           const float* act, float* partial) {
+    previous_grid_done();
+    next_grid_may_start();
     __shared__ float red[SUMS ? 256 : 1][17];
     const int lanes = c / 8;
     const int ch = (int)(threadIdx.x % lanes) * 8;
@@ -1203,8 +1240,10 @@ __global__ void __launch_bounds__(256) maxpool3_bwd_kernel(const uint8_t* __rest
 // Vector forms of the two general pooling kernels: one thread handles VEC consecutive channels of a
 // pixel with 16-byte accesses; same window order and tie rule as the scalar kernels.
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) maxpool_fwd_vec_kernel(const T* __restrict__ x, T* __restrict__ y, int64_t items, int h, int w,
+__global__ void __launch_bounds__(256) maxpool_fwd_vec_kernel(const T* x, T* y, int64_t items, int h, int w,
                                                               int c, int ho, int wo, int k, int stride, int pad) {
+    previous_grid_done();
+    next_grid_may_start();
     const int lanes = c / VEC;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
         const int ch = (int)(i % lanes) * VEC;
@@ -1232,9 +1271,11 @@ __global__ void __launch_bounds__(256) maxpool_fwd_vec_kernel(const T* __restric
 }
 
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) maxpool_bwd_vec_kernel(const T* __restrict__ x, const T* __restrict__ dy, T* __restrict__ dx,
+__global__ void __launch_bounds__(256) maxpool_bwd_vec_kernel(const T* x, const T* dy, T* dx,
                                                               int64_t items, int h, int w, int c, int ho, int wo, int k, int stride,
                                                               int pad) {
+    previous_grid_done();
+    next_grid_may_start();
     const int lanes = c / VEC;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
         const int ch = (int)(i % lanes) * VEC;
@@ -1284,8 +1325,10 @@ __global__ void __launch_bounds__(256) maxpool_bwd_vec_kernel(const T* __restric
 // window's gradient where the recorded position is this pixel's.  Pass 2 never reads x: eight small loads per
 // thread instead of re-scanning up to four whole windows.
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) maxpool_argmax_kernel(const T* __restrict__ x, uint8_t* __restrict__ arg, int64_t items, int h,
+__global__ void __launch_bounds__(256) maxpool_argmax_kernel(const T* x, uint8_t* arg, int64_t items, int h,
                                                              int w, int c, int ho, int wo, int k, int stride, int pad) {
+    previous_grid_done();
+    next_grid_may_start();
     const int lanes = c / VEC;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
         const int ch = (int)(i % lanes) * VEC;
@@ -1316,9 +1359,11 @@ __global__ void __launch_bounds__(256) maxpool_argmax_kernel(const T* __restrict
 }
 
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) maxpool_bwd_arg_kernel(const uint8_t* __restrict__ arg, const T* __restrict__ dy, T* __restrict__ dx,
+__global__ void __launch_bounds__(256) maxpool_bwd_arg_kernel(const uint8_t* arg, const T* dy, T* dx,
                                                               int64_t items, int h, int w, int c, int ho, int wo, int k, int stride,
                                                               int pad) {
+    previous_grid_done();
+    next_grid_may_start();
     const int lanes = c / VEC;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
         const int ch = (int)(i % lanes) * VEC;
@@ -1363,15 +1408,15 @@ int maxpool_forward(int dtype, int n, int h, int w, int c, int k, int stride, in
         const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
         const int64_t items = (int64_t)n * ho * wo * (c / vec);
         if (dtype == CKPT_DTYPE_BF16)
-            maxpool2x2_fwd_kernel<__nv_bfloat16, 8><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)y, items, wo, ho, c / vec, c, act);
+            launch(Start::ON_STREAMS, maxpool2x2_fwd_kernel<__nv_bfloat16, 8>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (__nv_bfloat16*)y, items, wo, ho, c / vec, c, act);
         else
-            maxpool2x2_fwd_kernel<float, 4><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const float*)x, (float*)y, items, wo, ho, c / vec, c, act);
+            launch(Start::ON_STREAMS, maxpool2x2_fwd_kernel<float, 4>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const float*)x, (float*)y, items, wo, ho, c / vec, c, act);
         CKPT_LAUNCH_CHECK("max-pool 2x2 forward");
         return CKPT_OK;
     }
     if (act && pool_3x3(dtype, c, k, stride, pad)) {
         const int64_t items = (int64_t)n * ho * wo * (c / 8);
-        maxpool3_fwd_act_kernel<<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)y, items, h, w, c, ho, wo, act);
+        launch(Start::ON_STREAMS, maxpool3_fwd_act_kernel, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (__nv_bfloat16*)y, items, h, w, c, ho, wo, act);
         CKPT_LAUNCH_CHECK("max-pool 3x3 forward");
         return CKPT_OK;
     }
@@ -1379,17 +1424,17 @@ int maxpool_forward(int dtype, int n, int h, int w, int c, int k, int stride, in
     if (c % bn_vec(dtype, c) == 0 && bn_vec(dtype, c) > 1) {
         const int64_t items = (int64_t)n * ho * wo * (c / bn_vec(dtype, c));
         if (dtype == CKPT_DTYPE_BF16)
-            maxpool_fwd_vec_kernel<__nv_bfloat16, 8><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)y, items, h, w, c, ho, wo, k, stride, pad);
+            launch(Start::ON_STREAMS, maxpool_fwd_vec_kernel<__nv_bfloat16, 8>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (__nv_bfloat16*)y, items, h, w, c, ho, wo, k, stride, pad);
         else
-            maxpool_fwd_vec_kernel<float, 4><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const float*)x, (float*)y, items, h, w, c, ho, wo, k, stride, pad);
+            launch(Start::ON_STREAMS, maxpool_fwd_vec_kernel<float, 4>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const float*)x, (float*)y, items, h, w, c, ho, wo, k, stride, pad);
         CKPT_LAUNCH_CHECK("max-pool forward");
         return CKPT_OK;
     }
     unsigned grid = elementwise_grid((int64_t)n * ho * wo * c);
     if (dtype == CKPT_DTYPE_BF16)
-        maxpool_fwd_kernel<__nv_bfloat16><<<grid, 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)y, n, h, w, c, ho, wo, k, stride, pad);
+        launch(Start::ON_STREAMS, maxpool_fwd_kernel<__nv_bfloat16>, grid, 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (__nv_bfloat16*)y, n, h, w, c, ho, wo, k, stride, pad);
     else
-        maxpool_fwd_kernel<float><<<grid, 256, 0, (cudaStream_t)stream>>>((const float*)x, (float*)y, n, h, w, c, ho, wo, k, stride, pad);
+        launch(Start::ON_STREAMS, maxpool_fwd_kernel<float>, grid, 256, 0, (cudaStream_t)stream, (const float*)x, (float*)y, n, h, w, c, ho, wo, k, stride, pad);
     CKPT_LAUNCH_CHECK("max-pool forward");
     return CKPT_OK;
 }
@@ -1406,17 +1451,17 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
             // the producer's batch-norm backward sums come out of this pass (one partial row pair per block)
             const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + 255) / 256, BN_MAX_BLOCKS));
             if (dtype == CKPT_DTYPE_BF16)
-                maxpool2x2_bwd_sums_kernel<__nv_bfloat16, 8><<<grid, 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, items, wo, ho, cv, c, act, bn_partial);
+                launch(Start::ON_STREAMS, maxpool2x2_bwd_sums_kernel<__nv_bfloat16, 8>, grid, 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, items, wo, ho, cv, c, act, bn_partial);
             else
-                maxpool2x2_bwd_sums_kernel<float, 4><<<grid, 256, 0, (cudaStream_t)stream>>>((const float*)x, (const float*)dy, (float*)dx, items, wo, ho, cv, c, act, bn_partial);
+                launch(Start::ON_STREAMS, maxpool2x2_bwd_sums_kernel<float, 4>, grid, 256, 0, (cudaStream_t)stream, (const float*)x, (const float*)dy, (float*)dx, items, wo, ho, cv, c, act, bn_partial);
             CKPT_LAUNCH_CHECK("max-pool 2x2 backward with batch-norm sums");
             *bn_blocks = (int)grid;
             return CKPT_OK;
         }
         if (dtype == CKPT_DTYPE_BF16)
-            maxpool2x2_bwd_kernel<__nv_bfloat16, 8><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, items, wo, ho, c / vec, c, act);
+            launch(Start::ON_STREAMS, maxpool2x2_bwd_kernel<__nv_bfloat16, 8>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, items, wo, ho, c / vec, c, act);
         else
-            maxpool2x2_bwd_kernel<float, 4><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const float*)x, (const float*)dy, (float*)dx, items, wo, ho, c / vec, c, act);
+            launch(Start::ON_STREAMS, maxpool2x2_bwd_kernel<float, 4>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const float*)x, (const float*)dy, (float*)dx, items, wo, ho, c / vec, c, act);
         CKPT_LAUNCH_CHECK("max-pool 2x2 backward");
         return CKPT_OK;
     }
@@ -1426,14 +1471,14 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
         if (!scratch || scratch_bytes < sums + windows * 8 || (uintptr_t)scratch % 16) { set_error("pooling scratch too small"); return CKPT_E_WORKSPACE; }
         uint8_t* const arg = (uint8_t*)scratch + sums;
         cudaStream_t st = (cudaStream_t)stream;
-        maxpool3_arg_act_kernel<<<elementwise_grid(windows), 256, 0, st>>>((const __nv_bfloat16*)x, arg, windows, h, w, c, ho, wo, act);
+        launch(Start::ON_STREAMS, maxpool3_arg_act_kernel, elementwise_grid(windows), 256, 0, st, (const __nv_bfloat16*)x, arg, windows, h, w, c, ho, wo, act);
         CKPT_LAUNCH_CHECK("max-pool 3x3 arg-max");
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((windows + 255) / 256, BN_MAX_BLOCKS));
         if (bn_partial && bn_blocks) {
-            maxpool3_bwd_kernel<true><<<grid, 256, 0, st>>>(arg, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, (const __nv_bfloat16*)x, act, bn_partial);
+            launch(Start::ON_STREAMS, maxpool3_bwd_kernel<true>, grid, 256, 0, st, arg, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, (const __nv_bfloat16*)x, act, bn_partial);
             *bn_blocks = (int)grid;
         } else {
-            maxpool3_bwd_kernel<false><<<grid, 256, 0, st>>>(arg, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, nullptr, nullptr, nullptr);
+            launch(Start::ON_STREAMS, maxpool3_bwd_kernel<false>, grid, 256, 0, st, arg, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, nullptr, nullptr, nullptr);
         }
         CKPT_LAUNCH_CHECK("max-pool backward from arg-max");
         return CKPT_OK;
@@ -1445,14 +1490,14 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
         const int64_t windows = (int64_t)n * ho * wo * (c / vec), pixels = (int64_t)n * h * w * (c / vec);
         cudaStream_t st = (cudaStream_t)stream;
         if (dtype == CKPT_DTYPE_BF16) {
-            maxpool_argmax_kernel<__nv_bfloat16, 8><<<elementwise_grid(windows), 256, 0, st>>>((const __nv_bfloat16*)x, (uint8_t*)scratch, windows, h, w, c, ho, wo, k, stride, pad);
+            launch(Start::ON_STREAMS, maxpool_argmax_kernel<__nv_bfloat16, 8>, elementwise_grid(windows), 256, 0, st, (const __nv_bfloat16*)x, (uint8_t*)scratch, windows, h, w, c, ho, wo, k, stride, pad);
             CKPT_LAUNCH_CHECK("max-pool arg-max");
-            if (pool_3x3(dtype, c, k, stride, pad)) maxpool3_bwd_kernel<false><<<elementwise_grid(windows), 256, 0, st>>>((const uint8_t*)scratch, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, nullptr, nullptr, nullptr);
-            else maxpool_bwd_arg_kernel<__nv_bfloat16, 8><<<elementwise_grid(pixels), 256, 0, st>>>((const uint8_t*)scratch, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, pixels, h, w, c, ho, wo, k, stride, pad);
+            if (pool_3x3(dtype, c, k, stride, pad)) launch(Start::ON_STREAMS, maxpool3_bwd_kernel<false>, elementwise_grid(windows), 256, 0, st, (const uint8_t*)scratch, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, windows, h, w, c, ho, wo, nullptr, nullptr, nullptr);
+            else launch(Start::ON_STREAMS, maxpool_bwd_arg_kernel<__nv_bfloat16, 8>, elementwise_grid(pixels), 256, 0, st, (const uint8_t*)scratch, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, pixels, h, w, c, ho, wo, k, stride, pad);
         } else {
-            maxpool_argmax_kernel<float, 4><<<elementwise_grid(windows), 256, 0, st>>>((const float*)x, (uint8_t*)scratch, windows, h, w, c, ho, wo, k, stride, pad);
+            launch(Start::ON_STREAMS, maxpool_argmax_kernel<float, 4>, elementwise_grid(windows), 256, 0, st, (const float*)x, (uint8_t*)scratch, windows, h, w, c, ho, wo, k, stride, pad);
             CKPT_LAUNCH_CHECK("max-pool arg-max");
-            maxpool_bwd_arg_kernel<float, 4><<<elementwise_grid(pixels), 256, 0, st>>>((const uint8_t*)scratch, (const float*)dy, (float*)dx, pixels, h, w, c, ho, wo, k, stride, pad);
+            launch(Start::ON_STREAMS, maxpool_bwd_arg_kernel<float, 4>, elementwise_grid(pixels), 256, 0, st, (const uint8_t*)scratch, (const float*)dy, (float*)dx, pixels, h, w, c, ho, wo, k, stride, pad);
         }
         CKPT_LAUNCH_CHECK("max-pool backward from arg-max");
         return CKPT_OK;
@@ -1460,17 +1505,17 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
     if (c % bn_vec(dtype, c) == 0 && bn_vec(dtype, c) > 1) {
         const int64_t items = (int64_t)n * h * w * (c / bn_vec(dtype, c));
         if (dtype == CKPT_DTYPE_BF16)
-            maxpool_bwd_vec_kernel<__nv_bfloat16, 8><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, items, h, w, c, ho, wo, k, stride, pad);
+            launch(Start::ON_STREAMS, maxpool_bwd_vec_kernel<__nv_bfloat16, 8>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, items, h, w, c, ho, wo, k, stride, pad);
         else
-            maxpool_bwd_vec_kernel<float, 4><<<elementwise_grid(items), 256, 0, (cudaStream_t)stream>>>((const float*)x, (const float*)dy, (float*)dx, items, h, w, c, ho, wo, k, stride, pad);
+            launch(Start::ON_STREAMS, maxpool_bwd_vec_kernel<float, 4>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const float*)x, (const float*)dy, (float*)dx, items, h, w, c, ho, wo, k, stride, pad);
         CKPT_LAUNCH_CHECK("max-pool backward");
         return CKPT_OK;
     }
     unsigned grid = elementwise_grid((int64_t)n * h * w * c);
     if (dtype == CKPT_DTYPE_BF16)
-        maxpool_bwd_kernel<__nv_bfloat16><<<grid, 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, n, h, w, c, ho, wo, k, stride, pad);
+        launch(Start::ON_STREAMS, maxpool_bwd_kernel<__nv_bfloat16>, grid, 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, n, h, w, c, ho, wo, k, stride, pad);
     else
-        maxpool_bwd_kernel<float><<<grid, 256, 0, (cudaStream_t)stream>>>((const float*)x, (const float*)dy, (float*)dx, n, h, w, c, ho, wo, k, stride, pad);
+        launch(Start::ON_STREAMS, maxpool_bwd_kernel<float>, grid, 256, 0, (cudaStream_t)stream, (const float*)x, (const float*)dy, (float*)dx, n, h, w, c, ho, wo, k, stride, pad);
     CKPT_LAUNCH_CHECK("max-pool backward");
     return CKPT_OK;
 }
@@ -1478,7 +1523,9 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
 // One block per (image, 32 vectors of channels): eight warps share the positions, four loads in flight each, and their sums
 // are added in order.  (A thread per channel walking all positions: 111 us for 32 images of 56 x 56 x 64, 18 now.)
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) avgpool_fwd_kernel(const T* __restrict__ x, T* __restrict__ y, int hw, int c) {
+__global__ void __launch_bounds__(256) avgpool_fwd_kernel(const T* x, T* y, int hw, int c) {
+    previous_grid_done();
+    next_grid_may_start();
     __shared__ float red[8][32][VEC + 1];
     const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, vecs = c / VEC;
     // narrow tensors: the lanes of a warp cover several positions
@@ -1522,7 +1569,9 @@ __global__ void __launch_bounds__(256) avgpool_fwd_kernel(const T* __restrict__ 
     }
 }
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) avgpool_bwd_kernel(const T* __restrict__ dy, T* __restrict__ dx, int64_t vecs, int hw, int lanes) {
+__global__ void __launch_bounds__(256) avgpool_bwd_kernel(const T* dy, T* dx, int64_t vecs, int hw, int lanes) {
+    previous_grid_done();
+    next_grid_may_start();
     const float area = (float)hw;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vecs; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t pix = i / lanes;
@@ -1535,12 +1584,12 @@ __global__ void __launch_bounds__(256) avgpool_bwd_kernel(const T* __restrict__ 
 }
 template <typename T, int VEC>
 static void launch_avgpool_fwd(int n, int hw, int c, const void* x, void* y, cudaStream_t st) {
-    avgpool_fwd_kernel<T, VEC><<<(unsigned)n * (unsigned)((c / VEC + 31) / 32), 256, 0, st>>>((const T*)x, (T*)y, hw, c);
+    launch(Start::ON_STREAMS, avgpool_fwd_kernel<T, VEC>, (unsigned)n * (unsigned)((c / VEC + 31) / 32), 256, 0, st, (const T*)x, (T*)y, hw, c);
 }
 template <typename T, int VEC>
 static void launch_avgpool_bwd(int n, int hw, int c, const void* dy, void* dx, cudaStream_t st) {
     const int64_t vecs = (int64_t)n * hw * c / VEC;
-    avgpool_bwd_kernel<T, VEC><<<elementwise_grid(vecs), 256, 0, st>>>((const T*)dy, (T*)dx, vecs, hw, c / VEC);
+    launch(Start::ON_STREAMS, avgpool_bwd_kernel<T, VEC>, elementwise_grid(vecs), 256, 0, st, (const T*)dy, (T*)dx, vecs, hw, c / VEC);
 }
 int avgpool_forward(int dtype, int n, int h, int w, int c, const void* x, void* y, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
@@ -1565,13 +1614,17 @@ int avgpool_backward(int dtype, int n, int h, int w, int c, const void* dy, void
 // Small helpers for the fully connected units and the losses
 // ================================================================================================
 template <typename T>
-__global__ void relu_mask_kernel(T* __restrict__ g, const T* __restrict__ y, int64_t elems) {
+__global__ void relu_mask_kernel(T* g, const T* y, int64_t elems) {
+    previous_grid_done();
+    next_grid_may_start();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < elems; i += (int64_t)gridDim.x * blockDim.x)
         if (!(ld(y + i) > 0.f)) g[i] = cvt<T>(0.f);
 }
 // 16-byte form: g is rewritten whole (the kept elements unchanged), four packed loads per operand in flight.
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) relu_mask_vec_kernel(T* __restrict__ g, const T* __restrict__ y, int64_t vecs) {
+__global__ void __launch_bounds__(256) relu_mask_vec_kernel(T* g, const T* y, int64_t vecs) {
+    previous_grid_done();
+    next_grid_may_start();
     constexpr int U = 4;
     for (int64_t i0 = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; i0 < vecs; i0 += (int64_t)gridDim.x * (256 * U)) {
         RawVec<T, VEC> rg[U], ry[U];
@@ -1596,12 +1649,12 @@ int relu_mask_inplace(int dtype, int64_t elems, void* g, const void* y, void* st
     if (elems % vec == 0 && aligned16(g) && aligned16(y)) {
         const int64_t vecs = elems / vec;
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((vecs + 1023) / 1024, 148 * 32));
-        if (dtype == CKPT_DTYPE_BF16) relu_mask_vec_kernel<__nv_bfloat16, 8><<<grid, 256, 0, st>>>((__nv_bfloat16*)g, (const __nv_bfloat16*)y, vecs);
-        else relu_mask_vec_kernel<float, 4><<<grid, 256, 0, st>>>((float*)g, (const float*)y, vecs);
+        if (dtype == CKPT_DTYPE_BF16) launch(Start::ON_STREAMS, relu_mask_vec_kernel<__nv_bfloat16, 8>, grid, 256, 0, st, (__nv_bfloat16*)g, (const __nv_bfloat16*)y, vecs);
+        else launch(Start::ON_STREAMS, relu_mask_vec_kernel<float, 4>, grid, 256, 0, st, (float*)g, (const float*)y, vecs);
     } else if (dtype == CKPT_DTYPE_BF16) {
-        relu_mask_kernel<__nv_bfloat16><<<elementwise_grid(elems), 256, 0, st>>>((__nv_bfloat16*)g, (const __nv_bfloat16*)y, elems);
+        launch(Start::ON_STREAMS, relu_mask_kernel<__nv_bfloat16>, elementwise_grid(elems), 256, 0, st, (__nv_bfloat16*)g, (const __nv_bfloat16*)y, elems);
     } else {
-        relu_mask_kernel<float><<<elementwise_grid(elems), 256, 0, st>>>((float*)g, (const float*)y, elems);
+        launch(Start::ON_STREAMS, relu_mask_kernel<float>, elementwise_grid(elems), 256, 0, st, (float*)g, (const float*)y, elems);
     }
     CKPT_LAUNCH_CHECK("ReLU mask");
     return CKPT_OK;
@@ -1609,11 +1662,13 @@ int relu_mask_inplace(int dtype, int64_t elems, void* g, const void* y, void* st
 
 // ReLU as a chain unit of its own: 16-byte accesses, scalar tail.  y may alias x, dx may alias dy.
 template <typename T>
-__global__ void __launch_bounds__(256) relu_fwd_kernel(const T* __restrict__ x, T* __restrict__ y, int64_t elems) {
+__global__ void __launch_bounds__(256) relu_fwd_kernel(const T* x, T* y, int64_t elems) {
+    previous_grid_done();
+    next_grid_may_start();
     constexpr int V = 16 / sizeof(T);
     const int64_t vecs = elems / V;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vecs; i += (int64_t)gridDim.x * blockDim.x) {
-        uint4 raw = __ldg(reinterpret_cast<const uint4*>(x) + i);
+        uint4 raw = reinterpret_cast<const uint4*>(x)[i];
         T* e = reinterpret_cast<T*>(&raw);
 #pragma unroll
         for (int k = 0; k < V; ++k) e[k] = cvt<T>(fmaxf(ld(e + k), 0.f));
@@ -1623,13 +1678,15 @@ __global__ void __launch_bounds__(256) relu_fwd_kernel(const T* __restrict__ x, 
         for (int64_t i = vecs * V + threadIdx.x; i < elems; i += blockDim.x) y[i] = cvt<T>(fmaxf(ld(x + i), 0.f));
 }
 template <typename T>
-__global__ void __launch_bounds__(256) relu_bwd_kernel(const T* __restrict__ dy, const T* __restrict__ y, T* __restrict__ dx,
+__global__ void __launch_bounds__(256) relu_bwd_kernel(const T* dy, const T* y, T* dx,
                                                        int64_t elems) {
+    previous_grid_done();
+    next_grid_may_start();
     constexpr int V = 16 / sizeof(T);
     const int64_t vecs = elems / V;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vecs; i += (int64_t)gridDim.x * blockDim.x) {
-        uint4 g = __ldg(reinterpret_cast<const uint4*>(dy) + i);
-        uint4 o = __ldg(reinterpret_cast<const uint4*>(y) + i);
+        uint4 g = reinterpret_cast<const uint4*>(dy)[i];
+        uint4 o = reinterpret_cast<const uint4*>(y)[i];
         T* ge = reinterpret_cast<T*>(&g);
         const T* oe = reinterpret_cast<const T*>(&o);
 #pragma unroll
@@ -1641,22 +1698,24 @@ __global__ void __launch_bounds__(256) relu_bwd_kernel(const T* __restrict__ dy,
 }
 int relu_forward(int dtype, int64_t elems, const void* x, void* y, void* stream) {
     const int64_t vecs = elems / (dtype == CKPT_DTYPE_BF16 ? 8 : 4);
-    if (dtype == CKPT_DTYPE_BF16) relu_fwd_kernel<__nv_bfloat16><<<elementwise_grid(vecs), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)y, elems);
-    else relu_fwd_kernel<float><<<elementwise_grid(vecs), 256, 0, (cudaStream_t)stream>>>((const float*)x, (float*)y, elems);
+    if (dtype == CKPT_DTYPE_BF16) launch(Start::ON_STREAMS, relu_fwd_kernel<__nv_bfloat16>, elementwise_grid(vecs), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (__nv_bfloat16*)y, elems);
+    else launch(Start::ON_STREAMS, relu_fwd_kernel<float>, elementwise_grid(vecs), 256, 0, (cudaStream_t)stream, (const float*)x, (float*)y, elems);
     CKPT_LAUNCH_CHECK("ReLU forward");
     return CKPT_OK;
 }
 int relu_backward(int dtype, int64_t elems, const void* dy, const void* y, void* dx, void* stream) {
     const int64_t vecs = elems / (dtype == CKPT_DTYPE_BF16 ? 8 : 4);
-    if (dtype == CKPT_DTYPE_BF16) relu_bwd_kernel<__nv_bfloat16><<<elementwise_grid(vecs), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)dy, (const __nv_bfloat16*)y, (__nv_bfloat16*)dx, elems);
-    else relu_bwd_kernel<float><<<elementwise_grid(vecs), 256, 0, (cudaStream_t)stream>>>((const float*)dy, (const float*)y, (float*)dx, elems);
+    if (dtype == CKPT_DTYPE_BF16) launch(Start::ON_STREAMS, relu_bwd_kernel<__nv_bfloat16>, elementwise_grid(vecs), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)dy, (const __nv_bfloat16*)y, (__nv_bfloat16*)dx, elems);
+    else launch(Start::ON_STREAMS, relu_bwd_kernel<float>, elementwise_grid(vecs), 256, 0, (cudaStream_t)stream, (const float*)dy, (const float*)y, (float*)dx, elems);
     CKPT_LAUNCH_CHECK("ReLU backward");
     return CKPT_OK;
 }
 
 // A block sums 32 columns, eight threads each.
 template <typename T>
-__global__ void __launch_bounds__(256) column_sum_kernel(const T* __restrict__ g, float* __restrict__ out, int64_t rows, int c, SgdUpdate upd) {
+__global__ void __launch_bounds__(256) column_sum_kernel(const T* g, float* out, int64_t rows, int c, SgdUpdate upd) {
+    previous_grid_done();
+    next_grid_may_start();
     __shared__ float red[8][32];
     const int lane = threadIdx.x % 32, part = threadIdx.x / 32, ch = blockIdx.x * 32 + lane;
     float s = 0.f;
@@ -1672,17 +1731,19 @@ __global__ void __launch_bounds__(256) column_sum_kernel(const T* __restrict__ g
     if (upd.w) { float* w = (float*)upd.w + ch; *w = fmaf(-upd.lr, s, *w); }
 }
 int column_sums(int dtype, int64_t rows, int c, const void* g, float* out, void* stream, const SgdUpdate& upd) {
-    if (dtype == CKPT_DTYPE_BF16) column_sum_kernel<__nv_bfloat16><<<(c + 31) / 32, 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)g, out, rows, c, upd);
-    else column_sum_kernel<float><<<(c + 31) / 32, 256, 0, (cudaStream_t)stream>>>((const float*)g, out, rows, c, upd);
+    if (dtype == CKPT_DTYPE_BF16) launch(Start::ON_STREAMS, column_sum_kernel<__nv_bfloat16>, (c + 31) / 32, 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)g, out, rows, c, upd);
+    else launch(Start::ON_STREAMS, column_sum_kernel<float>, (c + 31) / 32, 256, 0, (cudaStream_t)stream, (const float*)g, out, rows, c, upd);
     CKPT_LAUNCH_CHECK("column sums");
     return CKPT_OK;
 }
 
 // One block per sample: max, sum of exponentials, loss term, gradient (softmax - onehot)/batch.
 template <typename T>
-__global__ void __launch_bounds__(256) softmax_ce_kernel(const T* __restrict__ logits, const int32_t* __restrict__ labels,
-                                                         int classes, float inv_batch, float* __restrict__ row_loss,
-                                                         T* __restrict__ dlogits) {
+__global__ void __launch_bounds__(256) softmax_ce_kernel(const T* logits, const int32_t* labels,
+                                                         int classes, float inv_batch, float* row_loss,
+                                                         T* dlogits) {
+    previous_grid_done();
+    next_grid_may_start();
     __shared__ float red[256];
     const T* row = logits + (size_t)blockIdx.x * classes;
     float m = -INFINITY;
@@ -1706,7 +1767,9 @@ __global__ void __launch_bounds__(256) softmax_ce_kernel(const T* __restrict__ l
     }
     if (threadIdx.x == 0) row_loss[blockIdx.x] = logf(sum) + m - ld(row + label);
 }
-__global__ void mean_rows_kernel(const float* __restrict__ row_loss, int batch, float* __restrict__ loss) {
+__global__ void mean_rows_kernel(const float* row_loss, int batch, float* loss) {
+    previous_grid_done();
+    next_grid_may_start();
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         double s = 0.0;
         for (int i = 0; i < batch; ++i) s += row_loss[i];
@@ -1717,19 +1780,21 @@ int softmax_ce(int dtype, int batch, int classes, const void* logits, const int3
                float* row_scratch, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     if (dtype == CKPT_DTYPE_BF16)
-        softmax_ce_kernel<__nv_bfloat16><<<batch, 256, 0, st>>>((const __nv_bfloat16*)logits, labels, classes, 1.f / batch, row_scratch, (__nv_bfloat16*)dlogits);
+        launch(Start::ON_STREAMS, softmax_ce_kernel<__nv_bfloat16>, batch, 256, 0, st, (const __nv_bfloat16*)logits, labels, classes, 1.f / batch, row_scratch, (__nv_bfloat16*)dlogits);
     else
-        softmax_ce_kernel<float><<<batch, 256, 0, st>>>((const float*)logits, labels, classes, 1.f / batch, row_scratch, (float*)dlogits);
+        launch(Start::ON_STREAMS, softmax_ce_kernel<float>, batch, 256, 0, st, (const float*)logits, labels, classes, 1.f / batch, row_scratch, (float*)dlogits);
     CKPT_LAUNCH_CHECK("softmax cross-entropy");
-    mean_rows_kernel<<<1, 32, 0, st>>>(row_scratch, batch, loss);
+    launch(Start::ON_STREAMS, mean_rows_kernel, 1, 32, 0, st, row_scratch, batch, loss);
     CKPT_LAUNCH_CHECK("loss mean");
     return CKPT_OK;
 }
 
 constexpr int SUM_BLOCKS = 256;
 template <typename T>
-__global__ void __launch_bounds__(256) sum_partial_kernel(const T* __restrict__ y, int64_t elems, double* __restrict__ partial,
-                                                          T* __restrict__ grad) {
+__global__ void __launch_bounds__(256) sum_partial_kernel(const T* y, int64_t elems, double* partial,
+                                                          T* grad) {
+    previous_grid_done();
+    next_grid_may_start();
     __shared__ double red[256];
     double s = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < elems; i += (int64_t)gridDim.x * blockDim.x) {
@@ -1741,7 +1806,9 @@ __global__ void __launch_bounds__(256) sum_partial_kernel(const T* __restrict__ 
     for (int k = 128; k > 0; k >>= 1) { if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k]; __syncthreads(); }
     if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
-__global__ void sum_final_kernel(const double* __restrict__ partial, int blocks, double* __restrict__ loss) {
+__global__ void sum_final_kernel(const double* partial, int blocks, double* loss) {
+    previous_grid_done();
+    next_grid_may_start();
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         double s = 0.0;
         for (int i = 0; i < blocks; ++i) s += partial[i];
@@ -1751,28 +1818,32 @@ __global__ void sum_final_kernel(const double* __restrict__ partial, int blocks,
 int64_t sum_loss_scratch_bytes() { return SUM_BLOCKS * (int64_t)sizeof(double); }
 int sum_loss(int dtype, int64_t elems, const void* y, double* loss, void* grad, double* scratch, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    if (dtype == CKPT_DTYPE_BF16) sum_partial_kernel<__nv_bfloat16><<<SUM_BLOCKS, 256, 0, st>>>((const __nv_bfloat16*)y, elems, scratch, (__nv_bfloat16*)grad);
-    else sum_partial_kernel<float><<<SUM_BLOCKS, 256, 0, st>>>((const float*)y, elems, scratch, (float*)grad);
+    if (dtype == CKPT_DTYPE_BF16) launch(Start::ON_STREAMS, sum_partial_kernel<__nv_bfloat16>, SUM_BLOCKS, 256, 0, st, (const __nv_bfloat16*)y, elems, scratch, (__nv_bfloat16*)grad);
+    else launch(Start::ON_STREAMS, sum_partial_kernel<float>, SUM_BLOCKS, 256, 0, st, (const float*)y, elems, scratch, (float*)grad);
     CKPT_LAUNCH_CHECK("sum loss");
-    sum_final_kernel<<<1, 32, 0, st>>>(scratch, SUM_BLOCKS, loss);
+    launch(Start::ON_STREAMS, sum_final_kernel, 1, 32, 0, st, scratch, SUM_BLOCKS, loss);
     CKPT_LAUNCH_CHECK("sum loss final");
     return CKPT_OK;
 }
 
-__global__ void copy_kernel(uint4* __restrict__ dst, const uint4* __restrict__ src, int64_t vecs) {
+__global__ void copy_kernel(uint4* dst, const uint4* src, int64_t vecs) {
+    previous_grid_done();
+    next_grid_may_start();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vecs; i += (int64_t)gridDim.x * blockDim.x) dst[i] = src[i];
 }
 int device_copy(void* dst, const void* src, int64_t bytes, void* stream) {
     // sizes and offsets inside the arena and the workspace are multiples of 256 bytes
     int64_t vecs = bytes / 16;
-    copy_kernel<<<elementwise_grid(vecs), 256, 0, (cudaStream_t)stream>>>((uint4*)dst, (const uint4*)src, vecs);
+    launch(Start::ON_STREAMS, copy_kernel, elementwise_grid(vecs), 256, 0, (cudaStream_t)stream, (uint4*)dst, (const uint4*)src, vecs);
     CKPT_LAUNCH_CHECK("gradient carry copy");
     return CKPT_OK;
 }
 
 // w <- w - lr * g, element by element (float32 arithmetic; bf16 parameters rounded to nearest even).
 template <typename T>
-__global__ void sgd_update_kernel(T* __restrict__ w, const float* __restrict__ g, int64_t elems, float lr) {
+__global__ void sgd_update_kernel(T* w, const float* g, int64_t elems, float lr) {
+    previous_grid_done();
+    next_grid_may_start();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < elems; i += (int64_t)gridDim.x * blockDim.x) {
         if constexpr (sizeof(T) == 2) w[i] = __float2bfloat16_rn(fmaf(-lr, g[i], __bfloat162float(w[i])));
         else w[i] = fmaf(-lr, g[i], w[i]);
@@ -1780,8 +1851,8 @@ __global__ void sgd_update_kernel(T* __restrict__ w, const float* __restrict__ g
 }
 int sgd_update(const SgdUpdate& u, const float* g, int64_t elems, void* stream) {
     if (!u.w || elems <= 0) return CKPT_OK;
-    if (u.dtype == CKPT_DTYPE_BF16) sgd_update_kernel<__nv_bfloat16><<<elementwise_grid(elems), 256, 0, (cudaStream_t)stream>>>((__nv_bfloat16*)u.w, g, elems, u.lr);
-    else sgd_update_kernel<float><<<elementwise_grid(elems), 256, 0, (cudaStream_t)stream>>>((float*)u.w, g, elems, u.lr);
+    if (u.dtype == CKPT_DTYPE_BF16) launch(Start::ON_STREAMS, sgd_update_kernel<__nv_bfloat16>, elementwise_grid(elems), 256, 0, (cudaStream_t)stream, (__nv_bfloat16*)u.w, g, elems, u.lr);
+    else launch(Start::ON_STREAMS, sgd_update_kernel<float>, elementwise_grid(elems), 256, 0, (cudaStream_t)stream, (float*)u.w, g, elems, u.lr);
     CKPT_LAUNCH_CHECK("parameter update");
     return CKPT_OK;
 }
