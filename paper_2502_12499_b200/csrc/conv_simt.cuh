@@ -11,10 +11,11 @@
 // reduction of a tile can be split over the CTAs of a cluster, whose partial tiles are added over distributed shared
 // memory in rank order (one launch, no scratch), and a weight gradient's over further slices whose partial sums another
 // kernel adds in slice order.  Every summation order is fixed by the shape.
-// Measured (float32, forward / dgrad / wgrad in us) against 64 x 64 tiles of 4 x 4 blocks fetched value by value into one
-// buffer: 32 x 16 x 16 x 64 -> 64 3x3 102/146/61 -> 27/28/26; 32 x 4 x 4 x 256 -> 256 401/592/62 -> 27/29/35;
-// 16 x 112 x 112 x 64 -> 64 1140/1494/1410 -> 431/418/524 (35 of the 72 TFLOP/s of the FMA units);
-// 16 x 28 x 28 x 256 -> 256 3x3 stride 2 516/1628/311 -> 164/319/165; 4 x 32 x 32 x 16 -> 16 24/38/48 -> 8/8/9.
+// A sum is taken in chains of kChain products, whose totals are added: a chain of 1152 has two to three times the error.
+// Measured (float32, forward / dgrad / wgrad in us): 32 x 16 x 16 x 64 -> 64 3x3 32/34/22; 32 x 8 x 8 x 128 -> 128 30/31/22;
+// 16 x 112 x 112 x 64 -> 64 412/511/400 (36 of the 72 TFLOP/s of the FMA units); 16 x 28 x 28 x 256 -> 256 3x3 stride 2
+// 124/207/109; 4 x 32 x 32 x 16 -> 16 7/7/7.  What stands between is the issue of everything but FMAs - shared-memory reads, addresses
+// and bounds of the copies - and their latency at 16 warps per SM.
 #pragma once
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
@@ -30,6 +31,7 @@ namespace ckpt {
 namespace simt {
 
 constexpr int kStages = 4;
+constexpr int kChain = 64;         // additions in a row (see the kernel)
 
 template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
@@ -68,6 +70,8 @@ __device__ __forceinline__ void copy4(void* dst, const void* src, bool in) {
 template <typename T, int MODE, int BM, int BN, int TM, int TN>
 struct Tile {
     static constexpr int threads = (BM / TM) * (BN / TN);
+    // CTAs that an SM shall hold: registers for the chain and the total of a block, operands and addresses
+    static constexpr int held = TM * TN >= 64 ? 256 / threads : TM * TN >= 32 ? (sizeof(T) == 4 ? 4 : 3) : TM * TN >= 16 ? 5 : 7;
     static constexpr int V = 16 / (int)sizeof(T);            // values of a 16-byte chunk
     static constexpr int BK = 4 * V;                         // reduction depth of a stage
     static constexpr bool a_k = MODE != 2, b_k = MODE == 0;  // K contiguous in shared memory (and in memory)
@@ -106,7 +110,7 @@ struct Pixel {
 // Mode 1 with a stride: the input pixels fall into stride x stride parity classes, each reached by every stride-th filter
 // row and column only; a block works on one class (classes follow one another in blockIdx.x) and its K covers just those.
 template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), (Tile<T, MODE, BM, BN, TM, TN>::held))
 conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bias,
                  int relu, int M, int N, int K, int k_per_slice, int cluster, SgdUpdate upd) {
     previous_grid_done();
@@ -140,17 +144,17 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
         if (MODE == 0) {
             const int ih = bh + t.r, iw = bw + t.s;
             if ((unsigned)ih >= (unsigned)g.h || (unsigned)iw >= (unsigned)g.w) return nullptr;
-            return A + (((int64_t)n * g.h + ih) * g.w + iw) * g.cin + t.c;
+            return A + (int64_t)(((uint32_t)n * g.h + ih) * g.w + iw) * g.cin + t.c;
         }
         const int th = bh - t.r, tw = bw - t.s;
         if ((unsigned)th >= (unsigned)g.ho || (unsigned)tw >= (unsigned)g.wo) return nullptr;
-        return A + (((int64_t)n * g.ho + th) * g.wo + tw) * g.cout + t.c;
+        return A + (int64_t)(((uint32_t)n * g.ho + th) * g.wo + tw) * g.cout + t.c;
     };
     // corner of a pixel's window in the gathered tensor.  Mode 1: output row of filter row r0 + stride * t is base - t
     auto a_base_h = [&](int h) { return MODE == 0 ? h * g.stride - g.pad : (h * g.stride + ph + g.pad - r0) / g.stride; };
     auto a_base_w = [&](int w) { return MODE == 0 ? w * g.stride - g.pad : (w * g.stride + pw + g.pad - s0) / g.stride; };
     // value (tap position, n) of the filter in mode 1
-    auto b_off = [&](const TapPos& t) { return ((int64_t)t.c * g.k * g.k + (r0 + t.r * g.stride) * g.k + s0 + t.s * g.stride) * g.cin; };
+    auto b_off = [&](const TapPos& t) { return (int64_t)(((uint32_t)t.c * g.k + r0 + t.r * g.stride) * g.k + s0 + t.s * g.stride) * g.cin; };
 
     // ---- what a thread fetches in every stage: chunk c = tid + i * NT of each tile, or value e = tid + i * NT
     constexpr int a_len = (VA ? 1 : V) * (L::a_k ? 4 : BM / V), b_len = (VB ? 1 : V) * (L::b_k ? 4 : BN / V);      // items of a row
@@ -160,7 +164,10 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
     constexpr int a_dr = NT / a_len, b_dr = NT / b_len, a_w = VA ? V : 1, b_w = VB ? V : 1;                          // rows apart, values
     const int a_c = tid % a_len * a_w, a_r = tid / a_len, b_c = tid % b_len * b_w, b_r = tid / b_len;
     TapPos a_pos = {0, 0, 0};                                 // modes 0, 1: this thread's place along K
-    int a_n[VA ? CA : 1], a_h[VA ? CA : 1], a_wd[VA ? CA : 1];   // chunks: the rows' pixels
+    // chunks: the corner of a row's window, and which filter rows (low half) and columns (high half) of it lie inside the
+    // tensor (chunks are taken for up to 16 of each): an address is one addition per step, and no multiplication
+    const T* a_corner[VA ? CA : 1];
+    uint32_t a_inside[VA ? CA : 1];
     if (MODE != 2) {
         a_pos.set(k_begin + a_c, kc, cols);
         if (VA) {
@@ -169,8 +176,14 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
                 const int m = m0 + a_r + i * a_dr;
                 Pixel p;
                 p.set(min(m, M - 1), W, H);
-                a_n[VA ? i : 0] = p.n; a_wd[VA ? i : 0] = a_base_w(p.w);
-                a_h[VA ? i : 0] = m < M ? a_base_h(p.h) : -(1 << 28);             // outside for every filter position
+                const int bh = a_base_h(p.h), bw = a_base_w(p.w), th = MODE == 0 ? g.h : g.ho, tw = MODE == 0 ? g.w : g.wo;
+                a_corner[VA ? i : 0] = A + (((int64_t)p.n * th + bh) * tw + bw) * kc;
+                uint32_t inside = 0u;
+                for (int t = 0; t < g.k && m < M; ++t) {
+                    const int ih = MODE == 0 ? bh + t : bh - t, iw = MODE == 0 ? bw + t : bw - t;
+                    inside |= ((unsigned)ih < (unsigned)th ? 1u : 0u) << t | ((unsigned)iw < (unsigned)tw ? 0x10000u : 0u) << t;
+                }
+                a_inside[VA ? i : 0] = inside;
             }
         }
     }
@@ -191,7 +204,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
     auto x_ptr = [&](const Pixel& p) -> const T* {            // mode 2: x at this thread's column for an output pixel
         const int ih = p.h * g.stride + b_tap_h, iw = p.w * g.stride + b_tap_w;
         if ((unsigned)ih >= (unsigned)g.h || (unsigned)iw >= (unsigned)g.w) return nullptr;
-        return B + (((int64_t)p.n * g.h + ih) * g.w + iw) * g.cin + b_ci;
+        return B + (int64_t)(((uint32_t)p.n * g.h + ih) * g.w + iw) * g.cin + b_ci;
     };
     // values fetched through registers (also the filter of an input gradient to a few channels, whose rows of three values are
     // copied no faster: 256 -> 3, 28 images of 13 x 49, float32 85.6 us, 90.6 by copies)
@@ -204,6 +217,13 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
         const int k0 = k_begin + step * BK;
         Pixel row_px;
         if (!VA && MODE != 2) row_px.set(min(m0 + a_r, M - 1), W, H);
+        int64_t a_off = 0;
+        uint32_t a_bits = 0u;
+        if (VA && MODE != 2 && k0 + a_c < k_end) {
+            const int at = a_pos.r * (MODE == 0 ? g.w : g.wo) + a_pos.s;
+            a_off = (int64_t)(MODE == 0 ? at : -at) * kc + a_pos.c;
+            a_bits = 1u << a_pos.r | 0x10000u << a_pos.s;
+        }
 #pragma unroll
         for (int i = 0; i < CA; ++i) {
             const int row = a_r + i * a_dr;
@@ -212,7 +232,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
             if (MODE == 2) {
                 if (k0 + row < k_end && m0 + a_c < M) src = A + (int64_t)(k0 + row) * g.cout + m0 + a_c;
             } else if (VA) {
-                if (k0 + a_c < k_end) src = a_ptr(a_n[VA ? i : 0], a_h[VA ? i : 0], a_wd[VA ? i : 0], a_pos);
+                if (a_bits != 0u && (a_inside[VA ? i : 0] & a_bits) == a_bits) src = a_corner[VA ? i : 0] + a_off;
             } else {
                 if (k0 + a_c < k_end && m0 + row < M) src = a_ptr(row_px.n, a_base_h(row_px.h), a_base_w(row_px.w), a_pos);
                 row_px.advance(a_dr, W, H);
@@ -272,11 +292,19 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
     constexpr int GM = TM < 4 ? TM : 4, GN = TN < 4 ? TN : 4;         // values per read of an MN-contiguous operand
     auto m_of = [&](int i) { return L::a_k ? ty + i * TY : (i / GM) * (TY * GM) + ty * GM + i % GM; };
     auto n_of = [&](int j) { return L::b_k ? tx + j * TX : (j / GN) * (TX * GN) + tx * GN + j % GN; };
-    float acc[TM][TN];
+    // chains of kChain products, added up: the error of one float32 chain grows with the square root of its length (in 1e-7 of
+    // the result's norm, a chain for the whole reduction -> this: 128 -> 128 3x3 at 28 x 28 6.0 -> 1.6, 512 -> 512 4.3 -> 1.7)
+    float acc[TM][TN], total[TM][TN];
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < TN; ++j) acc[i][j] = total[i][j] = 0.f;
+    auto close_chain = [&] {
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j) { total[i][j] += acc[i][j]; acc[i][j] = 0.f; }
+    };
 
 #pragma unroll 1
     for (int p = 0; p < kStages - 1; ++p) {
@@ -292,7 +320,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
         asm volatile("cp.async.commit_group;" ::: "memory");
         const T* const as_ = stages + (size_t)(step % kStages) * (L::a_elems + L::b_elems);
         const T* const bs_ = as_ + L::a_elems;
-#pragma unroll
+#pragma unroll (MODE == 2 ? 4 : TM * TN >= 32 ? 1 : 2)     // (registers: four CTAs of 64 x 64 per SM)
         for (int k4 = 0; k4 < BK; k4 += 4) {
             if (MODE == 0 && !VA && k_begin + step * BK + k4 >= k_end) break;
             float a[TM][4];
@@ -334,7 +362,9 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
             }
         }
         if (more) settle(step + kStages - 1);
+        if (step % (kChain / BK) == kChain / BK - 1) close_chain();
     }
+    close_chain();
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 
     auto store = [&](int m, int n, float v, int z) {
@@ -361,7 +391,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < TN; ++j) store(m0 + m_of(i), n0 + n_of(j), acc[i][j], blockIdx.z);
+            for (int j = 0; j < TN; ++j) store(m0 + m_of(i), n0 + n_of(j), total[i][j], blockIdx.z);
         return;
     }
     // ---- partial tiles of the cluster, added in rank order by the CTA that stores that share of the tile
@@ -372,7 +402,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) tile[m_of(i) * BN + n_of(j)] = acc[i][j];
+        for (int j = 0; j < TN; ++j) tile[m_of(i) * BN + n_of(j)] = total[i][j];
     cl.sync();
     const int rank = (int)cl.block_rank(), share = BM * BN / cluster;
     for (int e = rank * share + tid; e < (rank + 1) * share; e += NT) {

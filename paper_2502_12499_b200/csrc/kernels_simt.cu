@@ -49,16 +49,49 @@ ConvGeom make_geom(const ckpt_conv_shape& s) {
 // ================================================================================================
 namespace simt {
 // The tile shape, the CTAs of a cluster that share a tile's reduction and (wgrad) the slices whose partial sums a second
-// kernel adds: the cheapest by a model of clocks per SM.  FMA time is the tile volume over 128 lanes and the share of the
-// peak a tile shape reaches (narrower blocks per thread read more operand bytes per FMA); a cluster costs its exchange,
-// further slices a launch and a pass over the partial sums.  A weight gradient fetched value by value takes a CTA some 2200
-// clocks per step of 16 whatever its tile - four warps do not hide their addresses and reads - so that its long reduction
+// kernel adds: the cheapest by a model of clocks per SM.  148 SMs are written in: the scratch size of a chain comes from
+// here and must not depend on the device at hand.
+//
+// Operands in 16-byte chunks: an SM holds `held` CTAs of a tile shape at once and works them off in rounds.  n of them need, per
+// step along K, n times the tile's FMAs at the share of the peak that the shape reaches, and a wait that they spend once
+// together.  (Share and wait fitted to 2,700 measured plans of 93 layers, each within 7 % on average; the chosen plan
+// is 2-3 % behind the best of the layer's in the mean.  Before, with one share per shape and no view of how many CTAs an SM
+// holds, 128 x 128 tiles alone on their SMs were taken for fast: us, float32, forward / dgrad / wgrad of 128 -> 128 at 8 x 8, 32
+// images 51/52/35 -> 30/31/22, 256 -> 256 3x3 stride 2 at 28 x 28, 16 images 164/319/149 -> 124/207/109, 1x1 64 -> 256 at 56 x 56,
+// 8 images 32/39/63 -> 33/34/42.)
+struct TileCost { double share, wait; int held; };
+static const TileCost kTileCost[3][7] = {
+    {{0.47, 40, 1}, {0.66, 70, 2}, {0.67, 55, 4}, {0.62, 65, 4}, {0.54, 44, 5}, {0.43, 39, 4}, {0.41, 32, 7}},
+    {{0.45, 40, 1}, {0.65, 86, 2}, {0.66, 67, 4}, {0.62, 69, 4}, {0.63, 44, 5}, {0.52, 59, 4}, {0.44, 33, 7}},
+    {{0.59, 10, 1}, {0.74, 84, 2}, {0.71, 51, 4}, {0.69, 75, 4}, {0.63, 46, 5}, {0.56, 74, 5}, {0.47, 51, 7}}};
+static const double kRound[3] = {2150, 2390, 1340}, kExchange[3] = {2000, 1730, 1310}, kExchangeTile[3] = {21.7, 21.8, 23.6};
+static double clocks_of_chunks(int mode, int t, int bm, int bn, double load, int per, int cluster, int slices, double outputs) {
+    const TileCost& c = kTileCost[mode][t];
+    const double fma = (double)bm * bn / 128.0 / c.share, rounds = std::floor(load / c.held), rest = load - rounds * c.held;
+    double clk = 3000.0 + rounds * (per * (fma * c.held + c.wait) + kRound[mode]);
+    if (rest > 0) clk += per * (fma * rest + c.wait) + kRound[mode];
+    if (cluster > 1) clk += kExchange[mode] + load * kExchangeTile[mode] * bm * bn / 32.0;
+    if (slices > 1) clk += 3950.0 + 0.76 * slices * outputs * 8.0 / 2500.0;
+    return clk;
+}
+// Operands fetched value by value: FMA time is the tile volume over 128 lanes and the share of the peak a tile shape reaches; a
+// cluster costs its exchange, further slices a launch and a pass over the partial sums.  Such a weight gradient takes a CTA some
+// 2200 clocks per step of 16 whatever its tile - four warps do not hide their addresses and reads - so that its long reduction
 // wants more CTAs, also such a number of slices as rounds to fewer (us, 3 -> 256, 28 images of 13 x 49 float32 87 -> 34,
-// 5 -> 20 at 28 x 28 69 -> 16, 3 -> 64 1x1 at 40 x 40, 20 images 67 -> 18, bfloat16 65 -> 21).  148 SMs are written in: the scratch
-// size of a chain comes from here and must not depend on the device at hand.
+// 5 -> 20 at 28 x 28 69 -> 16, 3 -> 64 1x1 at 40 x 40, 20 images 67 -> 18, bfloat16 65 -> 21).
+static double clocks_of_values(int mode, int t, int bm, int bn, double load, int per, int cluster, int slices, double outputs) {
+    static const double share[7] = {0.85, 0.8, 0.7, 0.6, 0.5, 0.4, 0.35};
+    // CTAs per SM; one or two of 128 threads do not hide the latency of their shared-memory reads
+    const double hidden = load < 2 ? 0.6 : load < 3 ? 0.8 : 1.0;
+    double clk = load * ((double)bm * bn * per / (128.0 * share[t] * hidden) + 300.0);
+    if (mode == 2) clk = std::max(clk, 140.0 * per);
+    clk += 2000.0;
+    if (cluster > 1) clk += 1000.0 + load * bm * bn / 32.0;
+    if (slices > 1) clk += 4000.0 + (double)slices * outputs * 8.0 / 2500.0;
+    return clk;
+}
 Plan plan(int mode, int M, int N, int K, bool vectors) {
     static const int tile_m[7] = {128, 128, 64, 128, 64, 128, 64}, tile_n[7] = {128, 64, 64, 32, 32, 16, 16};
-    static const double share[7] = {0.85, 0.8, 0.7, 0.6, 0.5, 0.4, 0.35};
     Plan best{2, 1, 1, K};
     double best_t = 1e300;
     for (int t = 0; t < 7; ++t) {
@@ -75,15 +108,9 @@ Plan plan(int mode, int M, int N, int K, bool vectors) {
                     if (vectors || mode != 2) continue;
                     slices = (int)((K + (int64_t)per * cluster - 1) / ((int64_t)per * cluster));      // rounding up leaves fewer
                 }
-                const int parts = cluster * slices;
-                // CTAs per SM; one or two of 128 threads do not hide the latency of their shared-memory reads
-                const double load = std::ceil((double)(tiles * parts) / 148.0);
-                const double hidden = t == 0 ? (load < 2 ? 0.8 : 1.0) : (load < 2 ? 0.6 : load < 3 ? 0.8 : 1.0);
-                double clk = load * ((double)bm * bn * per / (128.0 * share[t] * hidden) + 300.0);
-                if (!vectors && mode == 2) clk = std::max(clk, 140.0 * per);
-                clk += 2000.0;
-                if (cluster > 1) clk += 1000.0 + load * bm * bn / 32.0;
-                if (slices > 1) clk += 4000.0 + (double)slices * M * N * 8.0 / 2500.0;
+                const double load = std::ceil((double)(tiles * cluster * slices) / 148.0), outputs = (double)M * N;
+                const double clk = vectors ? clocks_of_chunks(mode, t, bm, bn, load, per, cluster, slices, outputs)
+                                           : clocks_of_values(mode, t, bm, bn, load, per, cluster, slices, outputs);
                 if (clk < best_t) { best_t = clk; best = Plan{t, cluster, slices, per}; }
             }
         }
@@ -103,14 +130,14 @@ static int simt_conv(int mode, int dtype, const ConvGeom& g, const void* a, cons
 int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, void* stream) {
     if (!bias && !relu && small_conv_supported(dtype, g) && g.cout % 64 == 0) return small_conv_fwd(g, x, w, z, stream);
     const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
-    const bool v = whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
+    const bool v = g.k <= 16 && whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
     return simt_conv(0, dtype, g, x, w, z, bias, relu, M, N, K, v, v, simt::plan(0, M, N, K, v), (cudaStream_t)stream);
 }
 int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w, void* dx, void* stream) {
     // (a strided layer's K splits over the parity classes of the input: the longest class has ceil(k / stride)^2 positions)
     const int taps = (g.k + g.stride - 1) / g.stride;
     const int M = g.n * g.h * g.w, N = g.cin, K = taps * taps * g.cout;
-    const bool va = whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, w);
+    const bool va = g.k <= 16 && whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, w);
     return simt_conv(1, dtype, g, dz, w, dx, nullptr, 0, M, N, K, va, vb, simt::plan(1, M, N, K, va && vb), (cudaStream_t)stream);
 }
 
