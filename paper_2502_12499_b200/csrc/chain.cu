@@ -458,6 +458,12 @@ static int unit_backward(StepCtx& c, int64_t i, const void* x_raw, const void* y
         case CKPT_UNIT_MAXPOOL: {
             if (!g_out) break;
             const float* act = nullptr;
+            if (pending_act(c.ch, i - 1) &&
+                maxpool_joins_bn_backward(dt, (int)c.ch->batch, u.in.h, u.in.w, u.in.c, u.desc.k, u.desc.stride, u.desc.pad, x, g_in, g_out)) {
+                const int pf = c.ch->units[i - 2].param_first;
+                return maxpool_bn_backward(dt, (int)c.ch->batch, u.in.h, u.in.w, u.in.c, x, g_in, stats_of(c, i - 1), g_out, (float*)c.grads[pf + 1],
+                                           (float*)c.grads[pf + 2], c.ws + c.ch->off_scr, c.stream, bn_extra(c, pf + 1));
+            }
             if (pending_act(c.ch, i - 1)) {
                 if (maxpool_fuses_activation(dt, u.in.h, u.in.w, u.in.c, u.desc.k, u.desc.stride, u.desc.pad)) act = stats_of(c, i - 1);
                 else if ((rc = activated(c, i - 1, x_raw, &x))) return rc;

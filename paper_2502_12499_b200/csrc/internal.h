@@ -205,7 +205,12 @@ int add_tensors(int dtype, int64_t elems, const void* a, const void* b, void* ou
 bool maxpool_fuses_activation(int dtype, int h, int w, int c, int k, int stride, int pad);
 int maxpool_forward(int dtype, int n, int h, int w, int c, int k, int stride, int pad, const void* x,
                     void* y, const float* act, void* stream);
-// bn_partial / bn_blocks (optional, with act): the 2x2 kernel also leaves the producer's batch-norm backward
+// The 2x2 backward and the batch-norm backward (with ReLU) of the convolution in front of it as one: dz from z, the pooling's dy
+// and the saved statistics; scratch as for the batch-norm backward.  dz must not overlap dy.
+bool maxpool_joins_bn_backward(int dtype, int n, int h, int w, int c, int k, int stride, int pad, const void* z, const void* dy, const void* dz);
+int maxpool_bn_backward(int dtype, int n, int h, int w, int c, const void* z, const void* dy, const float* stats, void* dz, float* dgamma, float* dbeta,
+                        void* scratch, void* stream, const BnBackwardExtra& extra);
+// bn_partial / bn_blocks (optional, with act): the 3x3 kernel also leaves the producer's batch-norm backward
 // sums there ([*bn_blocks][sum g | sum g*z][c] floats; *bn_blocks = 0 when it did not)
 int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, int pad, const void* x,
                      const void* dy, void* dx, const float* act, void* stream, float* bn_partial = nullptr,

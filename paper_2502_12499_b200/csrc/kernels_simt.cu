@@ -171,6 +171,7 @@ static unsigned elementwise_grid(int64_t items) {
 
 constexpr int BN_THREADS = 256;
 constexpr int BN_MAX_BLOCKS = 148 * 8;
+constexpr int POOL_BN_BLOCKS = 148 * 2;      // what the device holds of the pooling's sums at once
 constexpr float BN_EPS = 1e-5f;
 
 // Launch shape of the streaming element-wise kernels: a block works through `per_block` consecutive
@@ -1008,73 +1009,231 @@ __global__ void __launch_bounds__(256) maxpool2x2_bwd_kernel(const T* x, const T
     }
 }
 
-// The same backward with the batch-norm backward sums of the producer gathered on the way: the window's
-// four raw values z and their gradients g = dx masked by the producer's ReLU are all in registers, so
-// sum g and sum g*z per channel (what bn_partial_stream_kernel<.., 1> would re-read both tensors for) come
-// for free.  Every thread keeps one channel group (grid stride a multiple of the group count); partial
-// rows [block][sum | sum g*z][c] in a fixed order.
+// Backward of a 2x2 pooling together with the batch-norm backward of the convolution whose output it reads through the
+// pending normalisation.  The gradient between the two is a quarter of values of dy and three quarters of zeros: both passes
+// route dy again from the window's four raw values instead of writing and reading that tensor (3.5 passes over z instead of
+// 5.25; first the sums of g and g*z, then dz = scale*g - A - z*B).  HBM bound: 64 images of 224 x 224 x 64 390 -> 257 us with
+// the finalisation between them (the second pass at 6.1 TB/s), 128 of 32 x 32 x 64 29.6 -> 19.8, 128 of 2 x 2 x 512 11.0 -> 10.5.
+// Every thread keeps one channel group; a block has as many windows side by side as groups fit into 256 threads, and U windows in
+// flight per thread (five 16-byte loads each).
+//
+// One channel (float) or two (bf16, packed) of a window: the activated values as the pooling saw them, the first maximum in row-major
+// order takes dy, and the producer's ReLU lets it pass where that maximum is positive.  Packed, every step after the
+// normalisation is one instruction for two channels (value by value the sums of VGG-16's five poolings
+// took 365 us together where they take 217: issue slots).
+template <typename T> struct Word;                 // 32 bits of a tensor
+template <> struct Word<float> {
+    static constexpr int channels = 1;
+    static __device__ __forceinline__ float value(uint32_t w, int) { return __uint_as_float(w); }
+    static __device__ __forceinline__ uint32_t pack(const float (&v)[1]) { return __float_as_uint(v[0]); }
+    static __device__ __forceinline__ uint32_t max(uint32_t a, uint32_t b) { return __float_as_uint(fmaxf(__uint_as_float(a), __uint_as_float(b))); }
+    static __device__ __forceinline__ uint32_t equal(uint32_t a, uint32_t b) { return __uint_as_float(a) == __uint_as_float(b) ? ~0u : 0u; }
+    static __device__ __forceinline__ uint32_t above(uint32_t a, uint32_t b) { return __uint_as_float(a) > __uint_as_float(b) ? ~0u : 0u; }
+};
+template <> struct Word<__nv_bfloat16> {
+    static constexpr int channels = 2;
+    static __device__ __forceinline__ float value(uint32_t w, int i) { return __uint_as_float(i ? w & 0xffff0000u : w << 16); }
+    static __device__ __forceinline__ __nv_bfloat162 pair(uint32_t w) { return *reinterpret_cast<__nv_bfloat162*>(&w); }
+    static __device__ __forceinline__ uint32_t bits(__nv_bfloat162 p) { return *reinterpret_cast<uint32_t*>(&p); }
+    static __device__ __forceinline__ uint32_t pack(const float (&v)[2]) { return bits(__floats2bfloat162_rn(v[0], v[1])); }
+    static __device__ __forceinline__ uint32_t max(uint32_t a, uint32_t b) { return bits(__hmax2(pair(a), pair(b))); }
+    static __device__ __forceinline__ uint32_t equal(uint32_t a, uint32_t b) { return __heq2_mask(pair(a), pair(b)); }
+    static __device__ __forceinline__ uint32_t above(uint32_t a, uint32_t b) { return __hgt2_mask(pair(a), pair(b)); }
+};
+// z: a word of each of the window's pixels, as values and as bits; returns dy's word where it passes, take[q]: where pixel q gets it
+template <typename T>
+__device__ __forceinline__ uint32_t route_2x2(const float (&z)[4][Word<T>::channels], uint32_t g, const float* sc, const float* sh, uint32_t (&take)[4]) {
+    using W = Word<T>;
+    uint32_t a[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float v[W::channels];
+#pragma unroll
+        for (int i = 0; i < W::channels; ++i) v[i] = fmaf(z[q][i], sc[i], sh[i]);
+        a[q] = W::max(W::pack(v), 0u);
+    }
+    const uint32_t m = W::max(W::max(a[0], a[1]), W::max(a[2], a[3]));
+    take[0] = W::equal(a[0], m);
+    take[1] = W::equal(a[1], m) & ~take[0];
+    take[2] = W::equal(a[2], m) & ~(take[0] | take[1]);
+    take[3] = ~(take[0] | take[1] | take[2]);
+    return g & W::above(m, 0u);
+}
+struct PoolBn {
+    int64_t windows;
+    int wo, c, groups, across;         // groups = c / VEC; across = windows side by side in a block
+};
+constexpr int kPoolBnU = 2;
+// five vectors of a window: its four pixels and dy
 template <typename T, int VEC>
-__global__ void __launch_bounds__(256) maxpool2x2_bwd_sums_kernel(const T* x, const T* dy, T* dx,
-                                                                  int64_t items, int wo, int ho, int cv, int c,
-                                                                  const float* act, float* partial) {
+struct PoolWindow {
+    uint32_t z[4][4], g[4];
+    int64_t off;
+    static __device__ __forceinline__ void fetch(uint32_t (&d)[4], const T* p) {
+        const uint4 q = *reinterpret_cast<const uint4*>(p);
+        d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
+    }
+    // window w = (image and row) * wo + column: its first pixel is 4 w - 2 column
+    __device__ __forceinline__ void load(const PoolBn& p, const T* zp, const T* dy, uint32_t w, int ch) {
+        off = ((int64_t)4 * w - 2 * (int64_t)(w % (uint32_t)p.wo)) * p.c + ch;
+        const int64_t down = (int64_t)2 * p.wo * p.c;
+        fetch(z[0], zp + off); fetch(z[1], zp + off + p.c); fetch(z[2], zp + off + down); fetch(z[3], zp + off + down + p.c);
+        fetch(g, dy + (int64_t)w * p.c + ch);
+    }
+};
+template <typename T, int VEC>
+__global__ void __launch_bounds__(256, 2) maxpool2x2_bn_sums_kernel(const T* z, const T* dy, const float* stats, PoolBn p, float* partial) {
     previous_grid_done();
     next_grid_may_start();
+    using W = Word<T>;
+    constexpr int U = kPoolBnU, C = W::channels;
     __shared__ float red[256][2 * VEC + 1];
-    const int cg = (int)(((int64_t)blockIdx.x * 256 + threadIdx.x) % cv);
-    float sc[VEC], sh[VEC], s0[VEC], s1[VEC];
+    const int group = threadIdx.x % p.groups, row = threadIdx.x / p.groups, ch = group * VEC;
+    float s0[VEC], s1[VEC], sc[VEC], sh[VEC];
 #pragma unroll
-    for (int k = 0; k < VEC; ++k) { sc[k] = act[2 * c + cg * VEC + k]; sh[k] = act[3 * c + cg * VEC + k]; s0[k] = 0.f; s1[k] = 0.f; }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t t = i / cv;
-        const int ow = (int)(t % wo); t /= wo;
-        const int oh = (int)(t % ho);
-        const int64_t img = t / ho;
-        const int64_t off = ((img * (2 * ho) + 2 * oh) * (int64_t)(2 * wo) + 2 * ow) * c + cg * VEC;
-        const int64_t down = (int64_t)2 * wo * c;
-        float z[4][VEC], g[VEC], o[4][VEC];
-        load_vec<T, VEC>(x + off, z[0]);
-        load_vec<T, VEC>(x + off + c, z[1]);
-        load_vec<T, VEC>(x + off + down, z[2]);
-        load_vec<T, VEC>(x + off + down + c, z[3]);
-        load_vec<T, VEC>(dy + i * VEC, g);
+    for (int k = 0; k < VEC; ++k) { sc[k] = stats[2 * p.c + ch + k]; sh[k] = stats[3 * p.c + ch + k]; s0[k] = 0.f; s1[k] = 0.f; }
+    const int64_t hop = (int64_t)gridDim.x * p.across;
+    if (row < p.across) {
+        for (int64_t w0 = (int64_t)blockIdx.x * p.across + row; w0 < p.windows; w0 += U * hop) {
+            PoolWindow<T, VEC> win[U];
 #pragma unroll
-        for (int k = 0; k < VEC; ++k) {
-            float a[4];
+            for (int u = 0; u < U; ++u)
+                if (w0 + u * hop < p.windows) win[u].load(p, z, dy, (uint32_t)(w0 + u * hop), ch);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) a[q] = (float)cvt<T>(fmaxf(fmaf(z[q][k], sc[k], sh[k]), 0.f));
-            const float m = fmaxf(fmaxf(a[0], a[1]), fmaxf(a[2], a[3]));
-            const bool ta = a[0] == m, tb = !ta && a[1] == m, td = !ta && !tb && a[2] == m, te = !ta && !tb && !td;
-            o[0][k] = ta ? g[k] : 0.f; o[1][k] = tb ? g[k] : 0.f; o[2][k] = td ? g[k] : 0.f; o[3][k] = te ? g[k] : 0.f;
+            for (int j = 0; j < 4; ++j) {
+                // (the windows of a step are added up before they join the running sums: shorter chains)
+                float t0[C], t1[C];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float gi = a[q] > 0.f ? o[q][k] : 0.f;
-                s0[k] += gi;
-                s1[k] = fmaf(gi, z[q][k], s1[k]);
+                for (int i = 0; i < C; ++i) t0[i] = t1[i] = 0.f;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (w0 + u * hop >= p.windows) break;
+                    float v[4][C];
+                    uint32_t take[4], at = 0u;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int i = 0; i < C; ++i) v[q][i] = W::value(win[u].z[q][j], i);
+                    const uint32_t g = route_2x2<T>(v, win[u].g[j], sc + j * C, sh + j * C, take);
+                    // one of the four has the gradient: its z is the only one that counts
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) at |= win[u].z[q][j] & take[q];
+#pragma unroll
+                    for (int i = 0; i < C; ++i) { t0[i] += W::value(g, i); t1[i] = fmaf(W::value(g, i), W::value(at, i), t1[i]); }
+                }
+#pragma unroll
+                for (int i = 0; i < C; ++i) { s0[j * C + i] += t0[i]; s1[j * C + i] += t1[i]; }
             }
         }
-        store_vec<T, VEC>(dx + off, o[0]);
-        store_vec<T, VEC>(dx + off + c, o[1]);
-        store_vec<T, VEC>(dx + off + down, o[2]);
-        store_vec<T, VEC>(dx + off + down + c, o[3]);
     }
 #pragma unroll
     for (int k = 0; k < VEC; ++k) { red[threadIdx.x][k] = s0[k]; red[threadIdx.x][VEC + k] = s1[k]; }
     __syncthreads();
-    // halving down to one row per channel group: threads t and t + off hold the same group (off a multiple of cv)
-    for (int off = 128; off >= cv; off >>= 1) {
-        if ((int)threadIdx.x < off) {
+    for (int n = p.across; n > 1;) {
+        const int half = (n + 1) / 2;
+        if (row < n - half) {
 #pragma unroll
-            for (int k = 0; k < 2 * VEC; ++k) red[threadIdx.x][k] += red[threadIdx.x + off][k];
+            for (int k = 0; k < 2 * VEC; ++k) red[threadIdx.x][k] += red[threadIdx.x + half * p.groups][k];
         }
         __syncthreads();
+        n = half;
     }
-    if ((int)threadIdx.x < cv) {
-        const int chn = (int)(((int64_t)blockIdx.x * 256 + threadIdx.x) % cv) * VEC;
+    if (row == 0) {
 #pragma unroll
         for (int k = 0; k < VEC; ++k) {
-            partial[((size_t)blockIdx.x * 2 + 0) * c + chn + k] = red[threadIdx.x][k];
-            partial[((size_t)blockIdx.x * 2 + 1) * c + chn + k] = red[threadIdx.x][VEC + k];
+            partial[((size_t)blockIdx.x * 2 + 0) * p.c + ch + k] = red[threadIdx.x][k];
+            partial[((size_t)blockIdx.x * 2 + 1) * p.c + ch + k] = red[threadIdx.x][VEC + k];
         }
+    }
+}
+template <typename T, int VEC>
+__global__ void __launch_bounds__(256, 2) maxpool2x2_bn_apply_kernel(const T* z, const T* dy, const float* stats, const float* coef, PoolBn p, T* dz) {
+    previous_grid_done();
+    next_grid_may_start();
+    using W = Word<T>;
+    constexpr int U = kPoolBnU, C = W::channels;
+    const int group = threadIdx.x % p.groups, row = threadIdx.x / p.groups, ch = group * VEC;
+    if (row >= p.across) return;
+    const int64_t w0 = (int64_t)blockIdx.x * p.across * U + row;
+    PoolWindow<T, VEC> win[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (w0 + u * p.across < p.windows) win[u].load(p, z, dy, (uint32_t)(w0 + u * p.across), ch);
+    float sc[VEC], sh[VEC], ca[VEC], cb[VEC];
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) { sc[k] = stats[2 * p.c + ch + k]; sh[k] = stats[3 * p.c + ch + k]; ca[k] = coef[ch + k]; cb[k] = coef[p.c + ch + k]; }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        if (w0 + u * p.across >= p.windows) break;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float v[4][C];
+            uint32_t take[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < C; ++i) v[q][i] = W::value(win[u].z[q][j], i);
+            const uint32_t g = route_2x2<T>(v, win[u].g[j], sc + j * C, sh + j * C, take);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float o[C];
+#pragma unroll
+                for (int i = 0; i < C; ++i) o[i] = fmaf(-v[q][i], cb[j * C + i], fmaf(sc[j * C + i], W::value(g & take[q], i), -ca[j * C + i]));
+                win[u].z[q][j] = W::pack(o);
+            }
+        }
+        const int64_t down = (int64_t)2 * p.wo * p.c;
+        auto leave = [&](T* to, const uint32_t (&d)[4]) { *reinterpret_cast<uint4*>(to) = make_uint4(d[0], d[1], d[2], d[3]); };
+        leave(dz + win[u].off, win[u].z[0]);
+        leave(dz + win[u].off + p.c, win[u].z[1]);
+        leave(dz + win[u].off + down, win[u].z[2]);
+        leave(dz + win[u].off + down + p.c, win[u].z[3]);
+    }
+}
+
+// Forward, optionally through the pending normalisation, in the same shape (value by value, with the coefficients read again for
+// every window: 107 us for 64 images of 224 x 224 x 64, this 80).
+template <typename T, int VEC, bool ACT>
+__global__ void __launch_bounds__(256, 3) maxpool2x2_windows_kernel(const T* z, const float* stats, PoolBn p, T* y) {
+    previous_grid_done();
+    next_grid_may_start();
+    using W = Word<T>;
+    constexpr int U = kPoolBnU, C = W::channels;
+    const int group = threadIdx.x % p.groups, row = threadIdx.x / p.groups, ch = group * VEC;
+    if (row >= p.across) return;
+    const int64_t w0 = (int64_t)blockIdx.x * p.across * U + row, down = (int64_t)2 * p.wo * p.c;
+    uint4 q[U][4];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int64_t w = w0 + u * p.across;
+        if (w >= p.windows) break;
+        const T* const at = z + (4 * w - 2 * (int64_t)((uint32_t)w % (uint32_t)p.wo)) * p.c + ch;
+        q[u][0] = *reinterpret_cast<const uint4*>(at); q[u][1] = *reinterpret_cast<const uint4*>(at + p.c);
+        q[u][2] = *reinterpret_cast<const uint4*>(at + down); q[u][3] = *reinterpret_cast<const uint4*>(at + down + p.c);
+    }
+    float sc[VEC], sh[VEC];
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) { sc[k] = ACT ? stats[2 * p.c + ch + k] : 1.f; sh[k] = ACT ? stats[3 * p.c + ch + k] : 0.f; }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int64_t w = w0 + u * p.across;
+        if (w >= p.windows) break;
+        uint32_t out[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t word = j == 0 ? q[u][e].x : j == 1 ? q[u][e].y : j == 2 ? q[u][e].z : q[u][e].w;
+                if (ACT) {
+                    float v[C];
+#pragma unroll
+                    for (int i = 0; i < C; ++i) v[i] = fmaf(W::value(word, i), sc[j * C + i], sh[j * C + i]);
+                    word = W::pack(v);
+                }
+                out[j] = e > 0 ? W::max(out[j], word) : ACT ? W::max(word, 0u) : word;         // (0: the ReLU)
+            }
+        }
+        *reinterpret_cast<uint4*>(y + w * p.c + ch) = make_uint4(out[0], out[1], out[2], out[3]);
     }
 }
 
@@ -1429,10 +1588,32 @@ int64_t maxpool_backward_scratch_bytes(int dtype, int n, int h, int w, int c, in
     return align_up((int64_t)n * ho * wo * c, 256) + (pool_3x3(dtype, c, k, stride, pad) ? bn_scratch_bytes(0, c) : 0);
 }
 
+// (the kernels that walk windows by a 32-bit number and keep a channel group per thread)
+static bool pool_2x2_windows(int dtype, int n, int h, int w, int c, const void* a, const void* b) {
+    return c / (dtype == CKPT_DTYPE_BF16 ? 8 : 4) <= 256 && (int64_t)n * (h / 2) * (w / 2) < ((int64_t)1 << 31) && !(((uintptr_t)a | (uintptr_t)b) & 15u);
+}
+static PoolBn pool_windows(int n, int h, int w, int c, int vec) {
+    PoolBn p;
+    p.wo = w / 2; p.windows = (int64_t)n * (h / 2) * p.wo; p.c = c; p.groups = c / vec; p.across = 256 / p.groups;
+    return p;
+}
+static unsigned pool_blocks(const PoolBn& p) { return (unsigned)std::max<int64_t>(1, (p.windows + p.across * kPoolBnU - 1) / (p.across * kPoolBnU)); }
 int maxpool_forward(int dtype, int n, int h, int w, int c, int k, int stride, int pad, const void* x, void* y, const float* act, void* stream) {
     int ho = (h + 2 * pad - k) / stride + 1, wo = (w + 2 * pad - k) / stride + 1;
     if (pool_2x2(dtype, h, w, c, k, stride, pad)) {
         const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
+        if (pool_2x2_windows(dtype, n, h, w, c, x, y)) {
+            const PoolBn p = pool_windows(n, h, w, c, vec);
+            const unsigned blocks = pool_blocks(p);
+            cudaStream_t st = (cudaStream_t)stream;
+            if (dtype == CKPT_DTYPE_BF16)
+                launch(Start::ON_STREAMS, act ? maxpool2x2_windows_kernel<__nv_bfloat16, 8, true> : maxpool2x2_windows_kernel<__nv_bfloat16, 8, false>, blocks, 256, 0, st,
+                       (const __nv_bfloat16*)x, act, p, (__nv_bfloat16*)y);
+            else
+                launch(Start::ON_STREAMS, act ? maxpool2x2_windows_kernel<float, 4, true> : maxpool2x2_windows_kernel<float, 4, false>, blocks, 256, 0, st, (const float*)x, act, p, (float*)y);
+            CKPT_LAUNCH_CHECK("max-pool 2x2 forward");
+            return CKPT_OK;
+        }
         const int64_t items = (int64_t)n * ho * wo * (c / vec);
         if (dtype == CKPT_DTYPE_BF16)
             launch(Start::ON_STREAMS, maxpool2x2_fwd_kernel<__nv_bfloat16, 8>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (__nv_bfloat16*)y, items, wo, ho, c / vec, c, act);
@@ -1466,6 +1647,31 @@ int maxpool_forward(int dtype, int n, int h, int w, int c, int k, int stride, in
     return CKPT_OK;
 }
 
+bool maxpool_joins_bn_backward(int dtype, int n, int h, int w, int c, int k, int stride, int pad, const void* z, const void* dy, const void* dz) {
+    return pool_2x2(dtype, h, w, c, k, stride, pad) && pool_2x2_windows(dtype, n, h, w, c, z, dy) && (uintptr_t)dz % 16 == 0;
+}
+template <typename T, int VEC>
+static int maxpool_bn_backward_t(int n, int h, int w, int c, const void* z, const void* dy, const float* stats, void* dz, float* dgamma, float* dbeta,
+                                 void* scratch, const BnBackwardExtra& ex, cudaStream_t st) {
+    const PoolBn p = pool_windows(n, h, w, c, VEC);
+    float* const partial = (float*)scratch;
+    float* const coef = partial + (size_t)BN_MAX_BLOCKS * c * 2;
+    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(pool_blocks(p), POOL_BN_BLOCKS));
+    launch(Start::ON_STREAMS, maxpool2x2_bn_sums_kernel<T, VEC>, blocks, 256, 0, st, (const T*)z, (const T*)dy, stats, p, partial);
+    CKPT_LAUNCH_CHECK("max-pool 2x2 backward with batch-norm sums");
+    launch(Start::ON_STREAMS, bn_finalize_bwd_kernel, (c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st, partial, (int)blocks, c, 1.0 / (double)(4 * p.windows), stats, dgamma,
+           dbeta, coef, ex.gamma, ex.beta);
+    CKPT_LAUNCH_CHECK("batch-norm backward finalize");
+    launch(Start::ON_STREAMS, maxpool2x2_bn_apply_kernel<T, VEC>, pool_blocks(p), 256, 0, st, (const T*)z,
+           (const T*)dy, stats, coef, p, (T*)dz);
+    CKPT_LAUNCH_CHECK("max-pool 2x2 backward through batch norm");
+    return CKPT_OK;
+}
+int maxpool_bn_backward(int dtype, int n, int h, int w, int c, const void* z, const void* dy, const float* stats, void* dz, float* dgamma, float* dbeta,
+                        void* scratch, void* stream, const BnBackwardExtra& ex) {
+    return dtype == CKPT_DTYPE_BF16 ? maxpool_bn_backward_t<__nv_bfloat16, 8>(n, h, w, c, z, dy, stats, dz, dgamma, dbeta, scratch, ex, (cudaStream_t)stream)
+                                    : maxpool_bn_backward_t<float, 4>(n, h, w, c, z, dy, stats, dz, dgamma, dbeta, scratch, ex, (cudaStream_t)stream);
+}
 int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, int pad, const void* x, const void* dy, void* dx, const float* act, void* stream,
                      float* bn_partial, int* bn_blocks, void* scratch, int64_t scratch_bytes) {
     int ho = (h + 2 * pad - k) / stride + 1, wo = (w + 2 * pad - k) / stride + 1;
@@ -1473,18 +1679,6 @@ int maxpool_backward(int dtype, int n, int h, int w, int c, int k, int stride, i
     if (pool_2x2(dtype, h, w, c, k, stride, pad)) {
         const int vec = dtype == CKPT_DTYPE_BF16 ? 8 : 4;
         const int64_t items = (int64_t)n * ho * wo * (c / vec);
-        const int cv = c / vec;
-        if (act && bn_partial && bn_blocks && cv <= 128 && 256 % cv == 0) {
-            // the producer's batch-norm backward sums come out of this pass (one partial row pair per block)
-            const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + 255) / 256, BN_MAX_BLOCKS));
-            if (dtype == CKPT_DTYPE_BF16)
-                launch(Start::ON_STREAMS, maxpool2x2_bwd_sums_kernel<__nv_bfloat16, 8>, grid, 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, items, wo, ho, cv, c, act, bn_partial);
-            else
-                launch(Start::ON_STREAMS, maxpool2x2_bwd_sums_kernel<float, 4>, grid, 256, 0, (cudaStream_t)stream, (const float*)x, (const float*)dy, (float*)dx, items, wo, ho, cv, c, act, bn_partial);
-            CKPT_LAUNCH_CHECK("max-pool 2x2 backward with batch-norm sums");
-            *bn_blocks = (int)grid;
-            return CKPT_OK;
-        }
         if (dtype == CKPT_DTYPE_BF16)
             launch(Start::ON_STREAMS, maxpool2x2_bwd_kernel<__nv_bfloat16, 8>, elementwise_grid(items), 256, 0, (cudaStream_t)stream, (const __nv_bfloat16*)x, (const __nv_bfloat16*)dy, (__nv_bfloat16*)dx, items, wo, ho, c / vec, c, act);
         else
