@@ -1450,6 +1450,7 @@ struct WgradParams {
     int tiles_per_slice;         // pixel tiles per CTA along the reduction
     int total_tiles;
     int stages;
+    int chain;                   // kChain MMAs each that a chain of the form with short ones has
 };
 
 // SHORT: the tensor core cuts its running sum off at every MMA, toward zero, so that the error of a sum grows with the
@@ -1544,7 +1545,7 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
     } else if (warp == 1) {
         const uint32_t idesc = instr_desc(128, (int)n_cols, 1, 1);
         bool ok = true;
-        int chain = 0;
+        int chain = 0, quads = 0;                    // quads: of kChain MMAs in the open chain
         for (int it = 0; it < iters && ok; ++it) {
             const int s = it % p.stages;
             const uint32_t phase = (uint32_t)(it / p.stages) & 1u;
@@ -1554,17 +1555,21 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             const uint32_t a_lo = desc_lo(a_addr, box_bytes), b_lo = desc_lo(a_addr + 2 * box_bytes, box_bytes), hi = desc_hi(1024u);
             const int k_steps = p.px / 16;          // K = 16 pixels = 2 groups of 8 rows = 2048 bytes per step
             if constexpr (SHORT) {
-                for (int k0 = 0; k0 < k_steps; k0 += kChain, ++chain) {
+                for (int k0 = 0; k0 < k_steps; k0 += kChain) {
                     const uint32_t buf = (uint32_t)chain & 1u;
-                    if (!mbar_wait_warp(accum_empty + 8u * buf, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 204)) { ok = false; break; }
-                    tc_fence_after();
+                    if (quads == 0) {
+                        if (!mbar_wait_warp(accum_empty + 8u * buf, ((uint32_t)(chain >> 1) & 1u) ^ 1u, failed, status, 204)) { ok = false; break; }
+                        tc_fence_after();
+                    }
+                    const bool closes = ++quads == p.chain || (it == iters - 1 && k0 + kChain == k_steps);
                     if (elect_one()) {
 #pragma unroll
                         for (int kk = k0; kk < k0 + kChain; ++kk)
-                            umma_bf16(tmem_base + buf * 256u, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, kk > k0 ? 1u : 0u);
-                        umma_commit(accum_bar + 8u * buf);
+                            umma_bf16(tmem_base + buf * 256u, a_lo + kk * 128u, hi, b_lo + kk * 128u, hi, idesc, kk > k0 || quads > 1 ? 1u : 0u);
+                        if (closes) umma_commit(accum_bar + 8u * buf);
                     }
                     __syncwarp();
+                    if (closes) { quads = 0; ++chain; }
                 }
                 if (!ok) break;
             } else if (elect_one()) {
@@ -1644,7 +1649,7 @@ tc_conv_wgrad_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_co
             for (int j = 0; j < 4; ++j)
 #pragma unroll
                 for (int e = 0; e < 32; ++e) acc[j][e] = 0.f;
-            const int chains = iters * (p.px / (16 * kChain));
+            const int chains = (iters * (p.px / (16 * kChain)) + p.chain - 1) / p.chain;
             bool ok = true;
             for (int chain = 0; chain < chains; ++chain) {
                 const uint32_t buf = (uint32_t)chain & 1u;
@@ -3574,9 +3579,55 @@ int launch_fc(const ConvGeom& g, const void* x, const void* w, void* z, const fl
     return CKPT_OK;
 }
 
+// Shapes that leave part of a 64-channel block to zero fill, whose weight gradients used to be float32 sums of the CUDA cores
+// (a 1x1 filter of stride 1 with whole blocks of input channels never was): accumulation chains of 64 pixels.
+bool wgrad_short_chains(const ConvGeom& g) { return (g.cin % 64 || g.cout % 64) && !(g.k == 1 && g.stride == 1 && g.cin % 64 == 0); }
+// Reductions below 4096 pixels: column blocks per CTA and slices by a model of clocks, over CTAs with accumulation chains of 256
+// pixels at most (see the kernel), which a longer slice does not make less accurate.  A CTA pays a start, its stages - MMAs and
+// waits, or operand bytes from the L2 - and its accumulator's way out; more than one slice pays their sum.  Few slices of narrow
+// CTAs win: fitted to 900 plans of 31 layers within 5 %, the choice 2.3 % behind the best in the mean (us with the slice sum, the
+// rules for long reductions -> this: 3x3 512 -> 512 at 7 x 6, 21 images 16.7 -> 11.8, 256 -> 512 at 4 x 4, 128 images 22.2 -> 11.7,
+// 1x1 2048 -> 512 at 7 x 7, 32 images 20.5 -> 10.9, 1024 -> 256 at 13 x 11, 21 images 12.2 -> 10.5; error against float64 in 1e-7
+// of the norm 3.9 -> 1.8, 3.9 -> 2.0, 3.8 -> 2.2, 3.3 -> 1.9).  From 4096 pixels on the plain chains are ahead by 1-10 %.
+bool wgrad_short_plan(const ConvGeom& g, WgradParams* p, int* slices, int sms) {
+    const int64_t pixels = (int64_t)g.n * g.ho * g.wo;
+    if (pixels <= 256 || pixels >= 4096) return false;
+    const int co_tiles = (g.cout + 127) / 128;
+    const double elems = (double)g.cout * g.k * g.k * g.cin;
+    double best = 1e30;
+    for (int nb = 1; nb <= std::min(4, p->total_blocks); ++nb) {
+        const int px = nb == 1 ? 256 : 128, groups = (p->total_blocks + nb - 1) / nb;
+        int tw, th, tn;
+        choose_tile(px, g.wo, g.ho, g.n, &tw, &th, &tn);
+        if (tw * g.stride > 256 || th * g.stride > 256) continue;             // the box of a strided tensor map
+        const int tiles_w = (g.wo + tw - 1) / tw, tiles_h = (g.ho + th - 1) / th, tiles_n = (g.n + tn - 1) / tn, total = tiles_w * tiles_h * tiles_n;
+        for (int want = 1; want <= total && (want == 1 || groups * co_tiles * want <= sms); ++want) {
+            const int per = (total + want - 1) / want, s = (total + per - 1) / per;
+            const double ctas = (double)groups * co_tiles * s, rounds = std::ceil(ctas / sms), bytes = (2.0 + nb) * px * 128.0;
+            const double stage = std::max(113.0 + px / 16 * 4.4 * std::max(1.0, nb / 2.0), bytes / std::min(43.0, 5870.0 / std::min<double>(ctas, sms)));
+            const double t = 3160.0 + rounds * (per * stage + 760.0 * nb) + 9.5 * ctas * nb + (s > 1 ? 4300.0 + 8.9e-4 * s * elems : 0.0);
+            if (t >= best) continue;
+            best = t;
+            p->nb = nb; p->px = px; p->tw = tw; p->th = th; p->tn = tn; p->tiles_w = tiles_w; p->tiles_h = tiles_h; p->tiles_n = tiles_n;
+            p->total_tiles = total; p->tiles_per_slice = per; *slices = s;
+        }
+    }
+    return best < 1e30;
+}
 void wgrad_plan(const ConvGeom& g, WgradParams* p, int* slices, int* groups, int* co_tiles) {
     p->H = g.ho; p->W = g.wo; p->N = g.n; p->c_out = g.cout; p->c_in = g.cin; p->k = g.k; p->pad = g.pad; p->stride = g.stride;
     p->total_blocks = g.k * g.k * ((g.cin + 63) / 64);
+    int sms = 148, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    p->chain = 1;
+    if (wgrad_short_plan(g, p, slices, sms)) {
+        *groups = (p->total_blocks + p->nb - 1) / p->nb;
+        *co_tiles = (g.cout + 127) / 128;
+        p->chain = wgrad_short_chains(g) ? 1 : 4;
+        p->stages = std::max(1, std::min<int>(std::min<int>(kMaxStages, kSmemBudget / ((2 + p->nb) * (uint32_t)p->px * 128)), p->tiles_per_slice));
+        return;
+    }
     // column blocks per CTA: 4 when that divides evenly or the remainder is small, else 3
     p->nb = p->total_blocks % 4 == 0 ? 4 : (p->total_blocks % 3 == 0 ? 3 : (p->total_blocks >= 4 ? 4 : p->total_blocks));
     // pixels per stage: as many as leave two stages in shared memory (96 KB per stage at most), for reductions long
@@ -3607,9 +3658,6 @@ void wgrad_plan(const ConvGeom& g, WgradParams* p, int* slices, int* groups, int
     // for its accumulator's way out - 128 KB of partial sums - once, so fewer and longer CTAs win: 256 -> 1024 at
     // 14 x 14, batch 128: 35 us in one wave of 144 against 49 us in two waves of 288), at least 256 pixels per slice
     const int64_t base_ctas = (int64_t)*groups * *co_tiles;
-    int sms = 148, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int64_t by_k = std::max<int64_t>(1, (int64_t)p->total_tiles * p->px / 256);
     int64_t s = 1;
     double best_eff = -1.0;
@@ -3657,9 +3705,6 @@ constexpr int WROWS_MIN_W = 14;
 bool wgrad_rows_applies(const ConvGeom& g) {
     return g.k == 3 && g.pad == 1 && g.stride == 1 && (g.cin % 128 == 0 || g.cin % 64) && g.cin % 8 == 0 && g.cout % 8 == 0 && g.w >= WROWS_MIN_W && g.h >= 8;
 }
-// Shapes that leave part of a 64-channel block to zero fill, whose weight gradients used to be float32 sums of the CUDA cores
-// (a 1x1 filter of stride 1 with whole blocks of input channels never was): accumulation chains of 64 pixels.
-bool wgrad_short_chains(const ConvGeom& g) { return (g.cin % 64 || g.cout % 64) && !(g.k == 1 && g.stride == 1 && g.cin % 64 == 0); }
 void wgrad_rows_plan(const ConvGeom& g, WRowsParams* p, int* pairs, int* co_tiles) {
     p->H = g.h; p->W = g.w; p->N = g.n; p->c_out = g.cout; p->c_in = g.cin;
     const int nt = (g.h + 15) / 16;
@@ -4163,7 +4208,8 @@ int tc_conv_wgrad(const ConvGeom& g, const void* dz, const void* x, float* dw, v
     cudaStream_t st = (cudaStream_t)stream;
     static DeviceFlags ready;
     if (int bad = allow_shared_memory(ready, {(const void*)tc_conv_wgrad_kernel<false>, (const void*)tc_conv_wgrad_kernel<true>}, kSmemBudget + 2048)) return bad;
-    const bool chains = (short_chains || wgrad_short_chains(g)) && p.tiles_per_slice * p.px > 16 * kChain;       // (one chain is short as it is)
+    if (short_chains) p.chain = 1;
+    const bool chains = (short_chains || p.chain > 1 || wgrad_short_chains(g)) && p.tiles_per_slice * p.px > 16 * kChain * p.chain;       // (one chain is short as it is)
     if (chains) p.stages = std::max(p.stages, (8 * 4096 + (2 + p.nb) * p.px * 128 - 1) / ((2 + p.nb) * p.px * 128));     // a slab per epilogue warp
     const size_t smem = (size_t)p.stages * (2 + p.nb) * p.px * 128 + 1024 + 256;
     float* target = slices > 1 ? (float*)scratch : dw;
