@@ -186,8 +186,8 @@ static BnBackwardExtra bn_extra(StepCtx& c, int first, const void* mask = nullpt
     return ex;
 }
 
-// Convolution followed by the batch statistics of its stored output.  The tensor-core kernels gather the
-// partial sums in their epilogue; every other shape takes a separate pass over z.
+// Convolution followed by the batch statistics of its stored output.  Most kernels gather the partial sums in their epilogue;
+// what does not (blocks == 0) takes a separate pass over z.
 static int conv_with_statistics(StepCtx& c, const ConvGeom& g, const void* x, const void* w, void* z, const float* gamma,
                                 const float* beta, float* stats) {
     const int dt = c.ch->dtype;
@@ -202,8 +202,10 @@ static int conv_with_statistics(StepCtx& c, const ConvGeom& g, const void* x, co
         else rc = tc_first_conv_fwd(g, x, w, z, c.status(), c.stream, (float*)scr, &blocks);
         if (rc) return rc;
         if (blocks > 0) return bn_statistics_from_partials((const float*)scr, blocks, rows, g.cout, gamma, beta, stats, c.stream);
-    } else if ((rc = conv_forward_any(c, g, x, w, z, nullptr, 0))) {
-        return rc;
+    } else {
+        int blocks = 0;
+        if ((rc = simt_conv_fwd_stats(dt, g, x, w, z, (float*)scr, &blocks, c.stream))) return rc;
+        if (blocks > 0) return bn_statistics_from_partials((const float*)scr, blocks, rows, g.cout, gamma, beta, stats, c.stream);
     }
     return bn_statistics(dt, rows, g.cout, z, gamma, beta, stats, scr, c.stream);
 }

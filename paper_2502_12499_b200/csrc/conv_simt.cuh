@@ -106,13 +106,16 @@ struct Pixel {
 // aligned); otherwise value by value: float32 by asynchronous copies too, bfloat16 through registers, loaded before the FMAs
 // of a step and stored after them.  A forward layer of that kind often has a short reduction (27 values for three input
 // channels), whose last step stops where it ends (3 -> 256, 1x1, 49 images of 78 x 18, bfloat16: 81 us with whole steps, 46).
+// sums (mode 0, or null): batch-norm sums of the stored values, a row pair [sum | sum of squares][N] per CTA that stores a share of
+// a tile (a pass of its own costs its launch and 2.4-4.6 us: eight units of 16 channels, 4 images of 32 x 32, launched one by one 400 -> 379 us,
+// a float32 VGG-16 on 32 images 1154 -> 1131).
 // gridDim.z = slices * cluster; slice z of the reduction starts at z * k_per_slice (a multiple of BK).
 // Mode 1 with a stride: the input pixels fall into stride x stride parity classes, each reached by every stride-th filter
 // row and column only; a block works on one class (classes follow one another in blockIdx.x) and its K covers just those.
 template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), (Tile<T, MODE, BM, BN, TM, TN>::held))
 conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bias,
-                 int relu, int M, int N, int K, int k_per_slice, int cluster, SgdUpdate upd) {
+                 int relu, int M, int N, int K, int k_per_slice, int cluster, SgdUpdate upd, float* sums) {
     previous_grid_done();
     next_grid_may_start();
     using L = Tile<T, MODE, BM, BN, TM, TN>;
@@ -387,11 +390,36 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
             ((T*)out)[row * N + n] = from_f<T>(v);
         }
     };
+    // what a thread adds up of one column, or of its TN columns, meets the other threads' in shared memory, in a fixed order
+    float* const red = reinterpret_cast<float*>(smem);
+    auto leave_sums = [&](int row, int per_column) {          // red: [per_column][BN][sum | sum of squares]
+        __syncthreads();
+        if (tid < BN && n0 + tid < N) {
+            float s = 0.f, q = 0.f;
+            for (int r = 0; r < per_column; ++r) { s += red[(r * BN + tid) * 2]; q += red[(r * BN + tid) * 2 + 1]; }
+            sums[(size_t)row * 2 * N + n0 + tid] = s;
+            sums[((size_t)row * 2 + 1) * N + n0 + tid] = q;
+        }
+    };
+    auto add = [&](float v, float& s, float& q) { const float r = to_f(from_f<T>(v)); s += r; q = fmaf(r, r, q); };
     if (cluster == 1) {
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
             for (int j = 0; j < TN; ++j) store(m0 + m_of(i), n0 + n_of(j), total[i][j], blockIdx.z);
+        if (MODE == 0 && sums) {
+            __syncthreads();                                  // every stage has been read
+#pragma unroll
+            for (int j = 0; j < TN; ++j) {
+                float s = 0.f, q = 0.f;
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+                    if (m0 + m_of(i) < M) add(total[i][j], s, q);
+                red[(ty * BN + n_of(j)) * 2] = s;
+                red[(ty * BN + n_of(j)) * 2 + 1] = q;
+            }
+            leave_sums(blockIdx.x, TY);
+        }
         return;
     }
     // ---- partial tiles of the cluster, added in rank order by the CTA that stores that share of the tile
@@ -405,12 +433,20 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
         for (int j = 0; j < TN; ++j) tile[m_of(i) * BN + n_of(j)] = total[i][j];
     cl.sync();
     const int rank = (int)cl.block_rank(), share = BM * BN / cluster;
+    static_assert(NT % BN == 0, "a thread keeps its column of the tile");
+    float sum = 0.f, sumsq = 0.f;
     for (int e = rank * share + tid; e < (rank + 1) * share; e += NT) {
         float v = 0.f;
         for (int s = 0; s < cluster; ++s) v += cl.map_shared_rank(tile, s)[e];
         store(m0 + e / BN, n0 + e % BN, v, blockIdx.z / cluster);
+        if (MODE == 0 && sums && m0 + e / BN < M) add(v, sum, sumsq);
     }
-    cl.sync();                                                // no CTA may leave while its tile is being read
+    cl.sync();                                                // no CTA may leave, or use its tile's room, while it is being read
+    if (MODE == 0 && sums) {
+        red[tid * 2] = sum;                                   // thread tid: part tid / BN of column tid % BN
+        red[tid * 2 + 1] = sumsq;
+        leave_sums(blockIdx.x * cluster + rank, NT / BN);
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -429,7 +465,7 @@ Plan plan(int mode, int M, int N, int K, bool vectors);
 
 template <typename T>
 int launch(int mode, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K,
-           bool va, bool vb, const Plan& p, const SgdUpdate& upd, cudaStream_t st);
+           bool va, bool vb, const Plan& p, const SgdUpdate& upd, cudaStream_t st, float* sums = nullptr);
 
 }  // namespace simt
 }  // namespace ckpt

@@ -7,7 +7,7 @@ namespace simt {
 
 template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB>
 static int go(const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K, const Plan& p,
-              const SgdUpdate& upd, cudaStream_t st) {
+              const SgdUpdate& upd, cudaStream_t st, float* sums) {
     using L = Tile<T, MODE, BM, BN, TM, TN>;
     auto kernel = conv_gemm_kernel<T, MODE, BM, BN, TM, TN, VA, VB>;
     if (L::smem > 48 * 1024) {
@@ -30,7 +30,7 @@ static int go(const ConvGeom& g, const void* a, const void* b, void* out, const 
     cfg.attrs = attr;
     cfg.numAttrs = p.cluster > 1 ? 1 : 0;
     start_early(&cfg, attr, Start::ON_STREAMS);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, g, (const T*)a, (const T*)b, out, bias, relu, M, N, K, p.k_per_slice, p.cluster, upd);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, g, (const T*)a, (const T*)b, out, bias, relu, M, N, K, p.k_per_slice, p.cluster, upd, sums);
     if (e != cudaSuccess) return cuda_fail(e, "launching the CUDA-core convolution");
     static const char* const names[3] = {"conv forward (CUDA cores)", "conv dgrad (CUDA cores)", "conv wgrad (CUDA cores)"};
     CKPT_LAUNCH_CHECK_NAMED(names[MODE], names[MODE]);
@@ -40,10 +40,10 @@ static int go(const ConvGeom& g, const void* a, const void* b, void* out, const 
 // 16-byte chunks: every tile shape; value by value: the smaller shapes only (see plan)
 template <typename T, int MODE, bool VA, bool VB>
 static int pick(const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K, const Plan& p,
-                const SgdUpdate& upd, cudaStream_t st) {
+                const SgdUpdate& upd, cudaStream_t st, float* sums) {
 #define CKPT_CASE(I, BM, BN, TM, TN)                                                                                   \
     if constexpr ((VA && VB) || I == 2 || I == 4 || I == 6)                                                            \
-        if (p.tile == I) return go<T, MODE, BM, BN, TM, TN, VA, VB>(g, a, b, out, bias, relu, M, N, K, p, upd, st);
+        if (p.tile == I) return go<T, MODE, BM, BN, TM, TN, VA, VB>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);
     if constexpr (MODE == 2) { CKPT_SIMT_TILES_W(CKPT_CASE) } else { CKPT_SIMT_TILES(CKPT_CASE) }
 #undef CKPT_CASE
     set_error("CUDA-core convolution: no such tile");
@@ -52,14 +52,14 @@ static int pick(const ConvGeom& g, const void* a, const void* b, void* out, cons
 
 template <typename T>
 int launch(int mode, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K,
-           bool va, bool vb, const Plan& p, const SgdUpdate& upd, cudaStream_t st) {
+           bool va, bool vb, const Plan& p, const SgdUpdate& upd, cudaStream_t st, float* sums) {
     if (mode == 0)      // both operands run along the input channels
-        return va && vb ? pick<T, 0, true, true>(g, a, b, out, bias, relu, M, N, K, p, upd, st) : pick<T, 0, false, false>(g, a, b, out, bias, relu, M, N, K, p, upd, st);
+        return va && vb ? pick<T, 0, true, true>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums) : pick<T, 0, false, false>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);
 #define CKPT_MODE(MODE)                                                                                                \
-    if (va && vb) return pick<T, MODE, true, true>(g, a, b, out, bias, relu, M, N, K, p, upd, st);                          \
-    if (va) return pick<T, MODE, true, false>(g, a, b, out, bias, relu, M, N, K, p, upd, st);                               \
-    if (vb) return pick<T, MODE, false, true>(g, a, b, out, bias, relu, M, N, K, p, upd, st);                               \
-    return pick<T, MODE, false, false>(g, a, b, out, bias, relu, M, N, K, p, upd, st);
+    if (va && vb) return pick<T, MODE, true, true>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);                          \
+    if (va) return pick<T, MODE, true, false>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);                               \
+    if (vb) return pick<T, MODE, false, true>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);                               \
+    return pick<T, MODE, false, false>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);
     if (mode == 1) { CKPT_MODE(1) }
     CKPT_MODE(2)
 #undef CKPT_MODE

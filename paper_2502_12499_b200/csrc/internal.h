@@ -93,6 +93,9 @@ ConvGeom make_geom(const ckpt_conv_shape& s);
 // CUDA-core implicit-GEMM kernels (any k / stride / pad / channel count).
 int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, void* z,
                   const float* bias, int relu, void* stream);
+// The same without bias and ReLU, also leaving the batch-norm partial sums of its output ([blocks][sum | sum of squares][c_out] floats;
+// blocks == 0: it did not).
+int simt_conv_fwd_stats(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, float* partial, int* blocks, void* stream);
 int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w, void* dx, void* stream);
 int64_t simt_wgrad_scratch_bytes(const ConvGeom& g);
 int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw,

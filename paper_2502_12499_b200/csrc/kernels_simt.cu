@@ -90,13 +90,13 @@ static double clocks_of_values(int mode, int t, int bm, int bn, double load, int
     if (slices > 1) clk += 4000.0 + (double)slices * outputs * 8.0 / 2500.0;
     return clk;
 }
+static const int kTileM[7] = {128, 128, 64, 128, 64, 128, 64}, kTileN[7] = {128, 64, 64, 32, 32, 16, 16};      // modes 0 and 1
 Plan plan(int mode, int M, int N, int K, bool vectors) {
-    static const int tile_m[7] = {128, 128, 64, 128, 64, 128, 64}, tile_n[7] = {128, 64, 64, 32, 32, 16, 16};
     Plan best{2, 1, 1, K};
     double best_t = 1e300;
     for (int t = 0; t < 7; ++t) {
         if (!vectors && t != 2 && t != 4 && t != 6) continue;
-        const int bm = mode == 2 ? tile_n[t] : tile_m[t], bn = mode == 2 ? tile_m[t] : tile_n[t];
+        const int bm = mode == 2 ? kTileN[t] : kTileM[t], bn = mode == 2 ? kTileM[t] : kTileN[t];
         const int64_t tiles = (int64_t)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
         for (int cluster = 1; cluster <= 8; cluster *= 2) {
             // 1, 2, 3, 4, 6, 8, 12, ... slices: a finer search costs the host 17 us per layer and gains nothing
@@ -119,12 +119,13 @@ Plan plan(int mode, int M, int N, int K, bool vectors) {
 }
 }  // namespace simt
 
+constexpr int BN_MAX_BLOCKS = 148 * 8;        // partial rows of batch-norm sums
 static bool whole_chunks(int dtype, int channels, const void* p) { return channels % (dtype == CKPT_DTYPE_BF16 ? 8 : 4) == 0 && (uintptr_t)p % 16 == 0; }
 
 static int simt_conv(int mode, int dtype, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N,
-                     int K, bool va, bool vb, const simt::Plan& p, cudaStream_t st, const SgdUpdate& upd = SgdUpdate()) {
-    return dtype == CKPT_DTYPE_BF16 ? simt::launch<__nv_bfloat16>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, upd, st)
-                                    : simt::launch<float>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, upd, st);
+                     int K, bool va, bool vb, const simt::Plan& p, cudaStream_t st, const SgdUpdate& upd = SgdUpdate(), float* sums = nullptr) {
+    return dtype == CKPT_DTYPE_BF16 ? simt::launch<__nv_bfloat16>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, upd, st, sums)
+                                    : simt::launch<float>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, upd, st, sums);
 }
 
 int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, void* stream) {
@@ -132,6 +133,17 @@ int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, vo
     const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
     const bool v = g.k <= 16 && whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
     return simt_conv(0, dtype, g, x, w, z, bias, relu, M, N, K, v, v, simt::plan(0, M, N, K, v), (cudaStream_t)stream);
+}
+int simt_conv_fwd_stats(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, float* partial, int* blocks, void* stream) {
+    const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
+    const bool v = g.k <= 16 && whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
+    const simt::Plan p = simt::plan(0, M, N, K, v);
+    const int64_t rows = ((int64_t)M + simt::kTileM[p.tile] - 1) / simt::kTileM[p.tile] * p.cluster;
+    *blocks = 0;
+    // (the first layer's kernel of its own gathers none; more partial rows than the scratch region is sized for neither)
+    if ((small_conv_supported(dtype, g) && g.cout % 64 == 0) || rows > BN_MAX_BLOCKS) return simt_conv_fwd(dtype, g, x, w, z, nullptr, 0, stream);
+    *blocks = (int)rows;
+    return simt_conv(0, dtype, g, x, w, z, nullptr, 0, M, N, K, v, v, p, (cudaStream_t)stream, SgdUpdate(), partial);
 }
 int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w, void* dx, void* stream) {
     // (a strided layer's K splits over the parity classes of the input: the longest class has ceil(k / stride)^2 positions)
@@ -170,7 +182,6 @@ static unsigned elementwise_grid(int64_t items) {
 }
 
 constexpr int BN_THREADS = 256;
-constexpr int BN_MAX_BLOCKS = 148 * 8;
 constexpr int POOL_BN_BLOCKS = 148 * 2;      // what the device holds of the pooling's sums at once
 constexpr float BN_EPS = 1e-5f;
 
