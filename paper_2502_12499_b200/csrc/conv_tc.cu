@@ -3301,11 +3301,11 @@ bool t_fits(const TParams& p, int cols, int split) {
 }
 
 // Pixel tile and reduction split of the plain role-swapped kernel, by a model of clocks fitted to a sweep of both over
-// 30 shapes in both directions (6 % off on average, the choice 0.4 % behind the best in the mean): a stage (64 reduction channels
-// of one term) takes its four MMAs - 395 however few pixels, 2 per pixel above 197 - or its bytes from the L2; the epilogue of a
-// tile takes about 700 and 12 per pixel and runs under the next tile's stages; a cluster that shares a reduction costs
-// its exchange and 1450 per CTA.  (With the exchange taken for cheaper, four CTAs shared what two do better: us, 512 -> 512 at 7 x 6,
-// 21 images 16.0 -> 12.5, at 4 x 4, 128 images 17.1 -> 13.9, at 10 x 6, 13 images 16.0 -> 11.7, 1x1 2048 -> 512 at 7 x 6 9.4 -> 7.9.)
+// 26 shapes: a stage (64 reduction channels of one term) takes its four MMAs - 430 however few pixels, 2 per pixel above
+// 215 - or its bytes from the L2; the epilogue of a tile takes about 1100 and 15 per pixel and runs under the next tile's stages; a
+// cluster that shares a reduction costs its launch and exchange.  us, one 256-pixel tile per CTA -> chosen: 512 -> 512 at
+// 2 x 2, 128 images 25.5 -> 11.8 (64 pixels, 4 CTAs each), 512 -> 512 at 20 x 12, 13 images 26.2 -> 20.2 (256, 2),
+// 256 -> 256 at 13 x 11, 21 images 16.0 -> 12.6 (128, 2), 1x1 1024 -> 256 at 14 x 14, 128 images 17.1 -> 15.1 (192, 1).
 // 1x1 filters see the pixels as one row (tiles of any multiple of 32, no ragged edges but the last).
 void t_plan(TParams* p, int* W, int* H, int* N, bool dense) {
     const bool flat = p->taps == 1 && !p->fold && dense;
@@ -3326,10 +3326,10 @@ void t_plan(TParams* p, int* W, int* H, int* N, bool dense) {
             if (split > 1 && (p->fold || terms < 2 * split || (int64_t)tiles * co * split > sms - 4 * split)) break;
             if (!t_fits(*p, cols, split)) continue;
             const double active = std::min<double>(sms, (double)tiles * co * split);
-            const double bytes = 16384.0 + 128.0 * cols, stage = std::max(std::max(2.0 * cols, 395.0), bytes / std::min(89.0, 8800.0 / active));
-            const double loop = std::ceil((double)terms / split) * stage, out = 680.0 + 11.8 * cols;
+            const double bytes = 16384.0 + 128.0 * cols, stage = std::max(std::max(2.0 * cols, 430.0), bytes / std::min(100.0, 9000.0 / active));
+            const double loop = std::ceil((double)terms / split) * stage, out = 1100.0 + 15.0 * cols;
             const int64_t per_co = std::max<int64_t>(1, std::min<int64_t>(tiles, sms / co)), rounds = (tiles + per_co - 1) / per_co;
-            const double t = split == 1 ? rounds * std::max(loop, out) + std::min(loop, out) + 200.0 : loop + out + 15.0 * cols + 1450.0 * split;
+            const double t = split == 1 ? rounds * std::max(loop, out) + std::min(loop, out) : loop + out + 2000.0 + 10.0 * cols + 300.0 * split;
             if (t < best) { best = t; p->tile_cols = cols; p->split = split; p->tw = tw; p->th = th; p->tn = tn; }
         }
     }
