@@ -2081,8 +2081,6 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 __global__ void __launch_bounds__(kFirstThreads, kFirstCtasPerSm)
 tc_conv_first_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
                      const __grid_constant__ CUtensorMap map_out, float* stat_partial, FirstParams p, int* status) {
-    previous_grid_done();
-    next_grid_may_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* const smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t (*a_tiles)[128 * 128] = reinterpret_cast<uint8_t (*)[128 * 128]>(smem_al);
@@ -2110,6 +2108,17 @@ tc_conv_first_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
         fence_barrier_init();
         tma_prefetch_desc(&map_out);
     }
+    if ((smem_u32(a_tiles[0]) | smem_u32(b_tile)) & 1023u) {       // the swizzle pattern assumes 1024-byte aligned tiles
+        if (threadIdx.x == 0) atomicCAS(status, 0, 600);
+        return;
+    }
+    if (warp == 4) tmem_alloc(smem_u32(&tmem_base_slot), 128);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
     // filter tile: row = output channel, K = filter row r in columns 10 r .. 10 r + 8 (its 3 x 3 values), zeros elsewhere
     for (int i = threadIdx.x; i < 64 * 8; i += blockDim.x) {
         const int co = i / 8, chunk = i % 8;
@@ -2122,15 +2131,7 @@ tc_conv_first_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
         *reinterpret_cast<uint4*>(b_tile + co * 128 + ((chunk ^ (co & 7)) * 16)) = *reinterpret_cast<const uint4*>(v);
     }
     fence_proxy_async();
-    if ((smem_u32(a_tiles[0]) | smem_u32(b_tile)) & 1023u) {       // the swizzle pattern assumes 1024-byte aligned tiles
-        if (threadIdx.x == 0) atomicCAS(status, 0, 600);
-        return;
-    }
-    if (warp == 4) tmem_alloc(smem_u32(&tmem_base_slot), 128);
-    tc_fence_before();
     __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = tmem_base_slot;
 
     if (warp < 4) {
         // ---------------- gather: thread t builds row t of the operand tile.  The 128 pixels of a tile are
@@ -2459,8 +2460,6 @@ __device__ __forceinline__ void stem_gather_role(const StemParams& p, const uint
 __global__ void __launch_bounds__(kStemFwdThreads, 1)
 tc_conv_stem_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
                     const __grid_constant__ CUtensorMap map_out, float* stat_partial, StemParams p, int* status) {
-    previous_grid_done();
-    next_grid_may_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* const smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* const a_tiles = smem_al;                       // [2][atoms 2, 0, 1][128 rows][128 bytes]
@@ -2490,6 +2489,18 @@ tc_conv_stem_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
         fence_barrier_init();
         tma_prefetch_desc(&map_out);
     }
+    stem_zero_padding(a_tiles);
+    if ((smem_u32(a_tiles) | smem_u32(b_tile)) & 1023u) {       // the swizzle pattern assumes 1024-byte aligned tiles
+        if (threadIdx.x == 0) atomicCAS(status, 0, 610);
+        return;
+    }
+    if (warp == 8) tmem_alloc(smem_u32(&tmem_base_slot), 128);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
     // filter tile: row = output channel, K = filter row r in columns 24 r .. 24 r + 20, zeros elsewhere
     for (int i = threadIdx.x; i < 64 * 24; i += blockDim.x) {
         const int co = i / 24, chunk = i % 24;
@@ -2501,17 +2512,8 @@ tc_conv_stem_kernel(const __nv_bfloat16* x, const __nv_bfloat16* w,
         }
         *reinterpret_cast<uint4*>(b_tile + (chunk >> 3) * 8192 + co * 128 + (((chunk & 7) ^ (co & 7)) * 16)) = *reinterpret_cast<const uint4*>(v);
     }
-    stem_zero_padding(a_tiles);
     fence_proxy_async();
-    if ((smem_u32(a_tiles) | smem_u32(b_tile)) & 1023u) {       // the swizzle pattern assumes 1024-byte aligned tiles
-        if (threadIdx.x == 0) atomicCAS(status, 0, 610);
-        return;
-    }
-    if (warp == 8) tmem_alloc(smem_u32(&tmem_base_slot), 128);
-    tc_fence_before();
     __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = tmem_base_slot;
 
     if (warp < 8) {
         stem_gather_role(p, stage, a_tiles, (int)blockIdx.x, (int)gridDim.x, my_tiles, seg_full0, seg_empty0, a_full0, a_empty0, failed, status, 615);
@@ -2638,8 +2640,6 @@ template <bool SHORT>
 __global__ void __launch_bounds__(kStemWgradThreads + (SHORT ? 128 : 0), 1)
 tc_wgrad_stem_kernel(const __nv_bfloat16* x, const __grid_constant__ CUtensorMap map_dz, float* partial,
                      StemParams p, int* status) {
-    previous_grid_done();
-    next_grid_may_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* const smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* const a_tiles = smem_al;                       // [2][atoms 2, 0, 1][128 pixels][128 bytes]
@@ -2681,6 +2681,8 @@ tc_wgrad_stem_kernel(const __nv_bfloat16* x, const __grid_constant__ CUtensorMap
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    previous_grid_done();
+    next_grid_may_start();
 
     if (warp < 8) {
         stem_gather_role(p, stage, a_tiles, slice, p.slices, my_tiles, seg_full0, seg_empty0, a_full0, a_empty0, failed, status, 626);

@@ -1,10 +1,15 @@
 // Kernels that start while the one before them on the stream drains (programmatic dependent launch).
 //
 // Every kernel of this library calls previous_grid_done() before its first access to global memory and next_grid_may_start()
-// right behind it, so that nothing it reads or writes can meet the previous kernel's accesses, while launch latency, barrier
+// behind it, so that nothing it reads or writes can meet the previous kernel's accesses, while launch latency, barrier
 // set-up and the allocation of tensor memory lie under the previous kernel's tail.  The completion of a kernel implies that
 // of all before it (its own wait has passed), so the order of the stream is kept as a whole.  A kernel launched without the
 // attribute passes the wait at once: it starts behind the previous one anyway.
+//
+// A kernel with tensor memory lets the next one start only when its CTA holds its columns: allocation, __syncthreads(), then
+// next_grid_may_start().  The allocation blocks while too few columns of the SM are free.  If the next kernel's CTA could
+// take them first, it would hold them in its wait for this kernel, which would wait for them.  As it is, a CTA that
+// waits with columns in its hands waits only for grids whose CTAs have theirs.
 // No kernel launched this way reads global memory through the read-only path (__restrict__ const parameters, __ldg): such
 // loads may be moved ahead of the wait.
 #pragma once

@@ -45,3 +45,57 @@ def test_queued_operations_see_one_another(dtype, n, h, w, c):
         for a, b in zip(walk(False), want):
             assert torch.equal(a, b)
     ck.op_status()
+
+
+# a layer 3 -> cin in front of weight gradients of every form (the names are those of the launch log)
+WGRADS = [(3, 16, 16, 64, 64, 3, 1, "tc_wgrad_c64_kernel"), (1, 16, 15, 64, 128, 3, 1, "tc_wgrad_c64_kernel"), (2, 16, 32, 64, 64, 3, 1, "tc_wgrad_rows_kernel (pixel pairs)"),
+          (2, 14, 14, 128, 128, 3, 1, "tc_wgrad_rows_kernel"), (2, 20, 18, 48, 48, 3, 1, "tc_wgrad_rows_kernel"), (9, 7, 7, 256, 256, 3, 1, "tc_conv_wgrad_kernel"),
+          (11, 12, 12, 96, 136, 3, 2, "tc_conv_wgrad_kernel"), (2, 12, 12, 64, 320, 1, 1, "tc_conv_wgrad_kernel")]
+
+
+@pytest.mark.parametrize("n,h,w,cin,cout,k,stride,kernel", WGRADS)
+def test_kernels_with_tensor_memory_follow_one_another(n, h, w, cin, cout, k, stride, kernel):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(6)
+    dtype = ck.DTYPE_BF16
+
+    def rand(*dims, scale=1.0):
+        return (torch.randn(dims, generator=gen, device="cuda") * scale).bfloat16()
+
+    pad = k // 2
+    ho, wo = (h + 2 * pad - k) // stride + 1, (w + 2 * pad - k) // stride + 1
+    first, stem = ck.ConvShape(n, h, w, 3, cin, 3, 1, 1), ck.ConvShape(n, 2 * h, 2 * w, 3, cin, 7, 2, 3)
+    layer = ck.ConvShape(n, h, w, cin, cout, k, stride, pad)
+    small, large, dz = rand(n, h, w, 3), rand(n, 2 * h, 2 * w, 3), rand(n, ho, wo, cout)
+    w3, w7 = rand(cin, 3, 3, 3, scale=0.2), rand(cin, 7, 7, 3, scale=0.1)
+    scratch = torch.empty(max(ck.conv2d_scratch_bytes(s, dtype) for s in (first, stem, layer)) + 256, dtype=torch.uint8, device="cuda")
+
+    def walk(idle):
+        x = torch.zeros((n, h, w, cin), dtype=torch.bfloat16, device="cuda")
+        dw, dw3, dw7 = torch.zeros(cout, k, k, cin, device="cuda"), torch.zeros(cin, 3, 3, 3, device="cuda"), torch.zeros(cin, 7, 7, 3, device="cuda")
+        out = []
+        torch.cuda.synchronize()
+        for _ in range(3):
+            # every layer's output is what the weight gradient behind it reads, and what the next one overwrites
+            for op in (lambda: ck.conv2d_forward(first, dtype, 0, small, w3, x, scratch), lambda: ck.conv2d_wgrad(layer, dtype, 0, dz, x, dw, scratch),
+                       lambda: out.append(dw.clone()),
+                       lambda: ck.conv2d_forward(stem, dtype, 0, large, w7, x, scratch), lambda: ck.conv2d_wgrad(layer, dtype, 0, dz, x, dw, scratch),
+                       lambda: ck.conv2d_wgrad(stem, dtype, 0, x, large, dw7, scratch), lambda: ck.conv2d_wgrad(layer, dtype, 0, dz, x, dw, scratch),
+                       lambda: ck.conv2d_wgrad(first, dtype, 0, x, small, dw3, scratch)):
+                op()
+                if idle:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return out + [x, dw, dw3, dw7]
+
+    ck.launch_log(True)
+    want = walk(True)
+    kernels = ck.launch_log_read()
+    ck.launch_log(False)
+    for name in (kernel, "tc_conv_first_kernel", "tc_conv_stem_kernel", "tc_wgrad_stem_kernel"):
+        assert name in kernels, (name, kernels)
+    for _ in range(3):
+        for a, b in zip(walk(False), want):
+            assert torch.equal(a, b)
+    ck.op_status()
