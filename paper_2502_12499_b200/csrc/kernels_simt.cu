@@ -182,7 +182,8 @@ static unsigned elementwise_grid(int64_t items) {
 }
 
 constexpr int BN_THREADS = 256;
-constexpr int POOL_BN_BLOCKS = 148 * 2;      // what the device holds of the pooling's sums at once
+constexpr int POOL_BN_BLOCKS = 148 * 2;      // what the device holds of the pooling's sums at once; each leaves two partial rows
+static_assert(2 * POOL_BN_BLOCKS <= BN_MAX_BLOCKS, "partial rows of the pooling's sums");
 constexpr float BN_EPS = 1e-5f;
 
 // Launch shape of the streaming element-wise kernels: a block works through `per_block` consecutive
@@ -1023,8 +1024,12 @@ __global__ void __launch_bounds__(256) maxpool2x2_bwd_kernel(const T* x, const T
 // Backward of a 2x2 pooling together with the batch-norm backward of the convolution whose output it reads through the
 // pending normalisation.  The gradient between the two is a quarter of values of dy and three quarters of zeros: both passes
 // route dy again from the window's four raw values instead of writing and reading that tensor (3.5 passes over z instead of
-// 5.25; first the sums of g and g*z, then dz = scale*g - A - z*B).  HBM bound: 64 images of 224 x 224 x 64 390 -> 257 us with
+// 5.25; first the sums of g and g*z, then dz = scale*g - A - z*B).  HBM bound: 64 images of 224 x 224 x 64 390 -> 261 us with
 // the finalisation between them (the second pass at 6.1 TB/s), 128 of 32 x 32 x 64 29.6 -> 19.8, 128 of 2 x 2 x 512 11.0 -> 10.5.
+// The few blocks of the sums add many windows each: sums are two floats from a thread's on, also where they leave the block,
+// so that only two windows are ever added in one (error of dgamma against float64, in 1e-8 of its norm, plain chains -> this: 64
+// images of 56 x 56 x 256 5.1 -> 2.6, 128 of 32 x 32 x 64 5.4 -> 2.5, of which 2.5 is the rounding of the result; us of the
+// pass, replayed: 28.7 -> 30.4 and 7.2 -> 7.1).
 // Every thread keeps one channel group; a block has as many windows side by side as groups fit into 256 threads, and U windows in
 // flight per thread (five 16-byte loads each).
 //
@@ -1098,11 +1103,12 @@ __global__ void __launch_bounds__(256, 2) maxpool2x2_bn_sums_kernel(const T* z, 
     next_grid_may_start();
     using W = Word<T>;
     constexpr int U = kPoolBnU, C = W::channels;
-    __shared__ float red[256][2 * VEC + 1];
+    __shared__ float2 red[256][2 * VEC + 1], few[256];
     const int group = threadIdx.x % p.groups, row = threadIdx.x / p.groups, ch = group * VEC;
-    float s0[VEC], s1[VEC], sc[VEC], sh[VEC];
+    float2 s0[VEC], s1[VEC];
+    float sc[VEC], sh[VEC];
 #pragma unroll
-    for (int k = 0; k < VEC; ++k) { sc[k] = stats[2 * p.c + ch + k]; sh[k] = stats[3 * p.c + ch + k]; s0[k] = 0.f; s1[k] = 0.f; }
+    for (int k = 0; k < VEC; ++k) { sc[k] = stats[2 * p.c + ch + k]; sh[k] = stats[3 * p.c + ch + k]; s0[k] = s1[k] = make_float2(0.f, 0.f); }
     const int64_t hop = (int64_t)gridDim.x * p.across;
     if (row < p.across) {
         for (int64_t w0 = (int64_t)blockIdx.x * p.across + row; w0 < p.windows; w0 += U * hop) {
@@ -1112,7 +1118,7 @@ __global__ void __launch_bounds__(256, 2) maxpool2x2_bn_sums_kernel(const T* z, 
                 if (w0 + u * hop < p.windows) win[u].load(p, z, dy, (uint32_t)(w0 + u * hop), ch);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                // (the windows of a step are added up before they join the running sums: shorter chains)
+                // (the windows of a step are added up before they join the running sums, which are two floats each)
                 float t0[C], t1[C];
 #pragma unroll
                 for (int i = 0; i < C; ++i) t0[i] = t1[i] = 0.f;
@@ -1133,28 +1139,42 @@ __global__ void __launch_bounds__(256, 2) maxpool2x2_bn_sums_kernel(const T* z, 
                     for (int i = 0; i < C; ++i) { t0[i] += W::value(g, i); t1[i] = fmaf(W::value(g, i), W::value(at, i), t1[i]); }
                 }
 #pragma unroll
-                for (int i = 0; i < C; ++i) { s0[j * C + i] += t0[i]; s1[j * C + i] += t1[i]; }
+                for (int i = 0; i < C; ++i) { carry_sum(s0[j * C + i], t0[i]); carry_sum(s1[j * C + i], t1[i]); }
             }
         }
     }
 #pragma unroll
     for (int k = 0; k < VEC; ++k) { red[threadIdx.x][k] = s0[k]; red[threadIdx.x][VEC + k] = s1[k]; }
     __syncthreads();
-    for (int n = p.across; n > 1;) {
-        const int half = (n + 1) / 2;
-        if (row < n - half) {
+    // a thread or a few per column (channel group, sum) add up its rows, and one of them the few; both floats of a sum leave, as
+    // rows of their own
+    const int columns = 2 * VEC * p.groups, share = max(1, 256 / columns);
+    auto leave = [&](int col, float2 sum) {
+        const int k = col % (2 * VEC);
+        float* const to = partial + ((size_t)blockIdx.x * 4 + k / VEC) * p.c + col / (2 * VEC) * VEC + k % VEC;
+        to[0] = sum.x;
+        to[2 * p.c] = sum.y;
+    };
+    for (int i = threadIdx.x; i < columns * share; i += 256) {
+        const int col = i % columns, part = i / columns;
+        float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        for (int r = part; r < p.across; r += 4 * share) {
+            float2 v[4];
 #pragma unroll
-            for (int k = 0; k < 2 * VEC; ++k) red[threadIdx.x][k] += red[threadIdx.x + half * p.groups][k];
+            for (int u = 0; u < 4; ++u) v[u] = r + u * share < p.across ? red[(r + u * share) * p.groups + col / (2 * VEC)][col % (2 * VEC)] : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { two_sum(sum[u & 1], v[u].x); sum[u & 1].y += v[u].y; }
         }
-        __syncthreads();
-        n = half;
+        two_sum(sum[0], sum[1].x); sum[0].y += sum[1].y;
+        if (share == 1) leave(col, sum[0]);
+        else few[i] = sum[0];
     }
-    if (row == 0) {
-#pragma unroll
-        for (int k = 0; k < VEC; ++k) {
-            partial[((size_t)blockIdx.x * 2 + 0) * p.c + ch + k] = red[threadIdx.x][k];
-            partial[((size_t)blockIdx.x * 2 + 1) * p.c + ch + k] = red[threadIdx.x][VEC + k];
-        }
+    if (share == 1) return;
+    __syncthreads();
+    if ((int)threadIdx.x < columns) {
+        float2 sum = few[threadIdx.x];
+        for (int part = 1; part < share; ++part) { const float2 v = few[part * columns + threadIdx.x]; two_sum(sum, v.x); sum.y += v.y; }
+        leave(threadIdx.x, sum);
     }
 }
 template <typename T, int VEC>
@@ -1670,7 +1690,7 @@ static int maxpool_bn_backward_t(int n, int h, int w, int c, const void* z, cons
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(pool_blocks(p), POOL_BN_BLOCKS));
     launch(Start::ON_STREAMS, maxpool2x2_bn_sums_kernel<T, VEC>, blocks, 256, 0, st, (const T*)z, (const T*)dy, stats, p, partial);
     CKPT_LAUNCH_CHECK("max-pool 2x2 backward with batch-norm sums");
-    launch(Start::ON_STREAMS, bn_finalize_bwd_kernel, (c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st, partial, (int)blocks, c, 1.0 / (double)(4 * p.windows), stats, dgamma,
+    launch(Start::ON_STREAMS, bn_finalize_bwd_kernel, (c + FIN_CH - 1) / FIN_CH, FIN_THREADS, 0, st, partial, (int)(2 * blocks), c, 1.0 / (double)(4 * p.windows), stats, dgamma,
            dbeta, coef, ex.gamma, ex.beta);
     CKPT_LAUNCH_CHECK("batch-norm backward finalize");
     launch(Start::ON_STREAMS, maxpool2x2_bn_apply_kernel<T, VEC>, pool_blocks(p), 256, 0, st, (const T*)z,

@@ -88,5 +88,12 @@ __device__ __forceinline__ void two_sum(float2& sum, float v) {
     sum.y += (sum.x - (t - b)) + (v - b);
     sum.x = t;
 }
+// The same with the carry taken along in the next addition (Kahan): four operations instead of seven.  What it loses is of the order of
+// a last bit of v.
+__device__ __forceinline__ void carry_sum(float2& sum, float v) {
+    const float y = v + sum.y, t = sum.x + y;
+    sum.y = y - (t - sum.x);
+    sum.x = t;
+}
 
 }  // namespace ckpt
