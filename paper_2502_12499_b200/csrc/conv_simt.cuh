@@ -12,10 +12,12 @@
 // memory in rank order (one launch, no scratch), and a weight gradient's over further slices whose partial sums another
 // kernel adds in slice order.  Every summation order is fixed by the shape.
 // A sum is taken in chains of kChain products, whose totals are added: a chain of 1152 has two to three times the error.
-// Measured (float32, forward / dgrad / wgrad in us): 32 x 16 x 16 x 64 -> 64 3x3 32/34/22; 32 x 8 x 8 x 128 -> 128 30/31/22;
-// 16 x 112 x 112 x 64 -> 64 412/511/400 (36 of the 72 TFLOP/s of the FMA units); 16 x 28 x 28 x 256 -> 256 3x3 stride 2
-// 124/207/109; 4 x 32 x 32 x 16 -> 16 7/7/7.  What stands between is the issue of everything but FMAs - shared-memory reads, addresses
-// and bounds of the copies - and their latency at 16 warps per SM.
+// Measured (float32, forward / dgrad / wgrad in us, replayed; in brackets one chain per sum, whose registers let an SM hold more
+// CTAs): 32 x 16 x 16 x 64 -> 64 3x3 32/30/22 (27/28/27); 32 x 8 x 8 x 128 -> 128 29/28/23 (51/52/35); 16 x 112 x 112 x 64 -> 64
+// 405/423/352 (431/438/452; 37 of the 72 TFLOP/s of the FMA units); 16 x 28 x 28 x 256 -> 256 3x3 stride 2 124/204/102 (165/320/147);
+// 4 x 32 x 32 x 16 -> 16 8/8/8 (8/8/8).  At equal plans the chains cost 2-4 %, 128-wide weight-gradient tiles 7 %.  What stands
+// between is the issue of everything but FMAs - shared-memory reads, addresses and bounds of the copies - and their latency at 16
+// warps per SM.
 #pragma once
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
@@ -323,23 +325,17 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
         asm volatile("cp.async.commit_group;" ::: "memory");
         const T* const as_ = stages + (size_t)(step % kStages) * (L::a_elems + L::b_elems);
         const T* const bs_ = as_ + L::a_elems;
-#pragma unroll (MODE == 2 ? 4 : TM * TN >= 32 ? 1 : 2)     // (registers: four CTAs of 64 x 64 per SM)
+        // Whole steps unrolled, so that shared-memory reads run ahead of the FMAs (float32, at equal plans, us: 3x3 64 -> 64 at 112 x 112,
+        // 16 images, forward / input gradient 418/438 with groups of four one at a time, 405/423 so).  Eight by eight blocks have no
+        // registers for more than four groups, 128 x 32 tiles of float32 outputs spill.  In mode 2 the fragments of one k at a time:
+        // 64 x 64 tiles 3 % faster than with four fetched in front.
+#pragma unroll (TM * TN >= 64 ? 4 : sizeof(T) == 4 && MODE == 0 && BM == 4 * BN ? 1 : BK / 4)
         for (int k4 = 0; k4 < BK; k4 += 4) {
             if (MODE == 0 && !VA && k_begin + step * BK + k4 >= k_end) break;
-            float a[TM][4];
+            float a[TM][L::a_k ? 4 : 1];
             if constexpr (L::a_k) {
 #pragma unroll
                 for (int i = 0; i < TM; ++i) lds<T, 4>(as_ + m_of(i) * L::a_row + k4, a[i]);
-            } else {
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-#pragma unroll
-                    for (int i = 0; i < TM; i += GM) {
-                        float t[GM];
-                        lds<T, GM>(as_ + (k4 + kk) * L::a_row + m_of(i), t);
-#pragma unroll
-                        for (int e = 0; e < GM; ++e) a[i + e][kk] = t[e];
-                    }
             }
             if constexpr (L::b_k) {
 #pragma unroll
@@ -357,10 +353,19 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
                     float b[TN];
 #pragma unroll
                     for (int j = 0; j < TN; j += GN) lds<T, GN>(bs_ + (k4 + kk) * L::b_row + n_of(j), b + j);
+                    if constexpr (!L::a_k) {
+#pragma unroll
+                        for (int i = 0; i < TM; i += GM) {
+                            float t[GM];
+                            lds<T, GM>(as_ + (k4 + kk) * L::a_row + m_of(i), t);
+#pragma unroll
+                            for (int e = 0; e < GM; ++e) a[i + e][0] = t[e];
+                        }
+                    }
 #pragma unroll
                     for (int i = 0; i < TM; ++i)
 #pragma unroll
-                        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i][kk], b[j], acc[i][j]);
+                        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i][L::a_k ? kk : 0], b[j], acc[i][j]);
                 }
             }
         }
