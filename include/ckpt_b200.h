@@ -377,6 +377,11 @@ CKPT_API int ckpt_selftest_bounded_wait(int64_t limit_cycles, void* stream);
  * pixels per tile, CTAs that share a reduction, operand stages, bytes of the stages, bytes of the accumulators that are
  * exchanged in place of the stages (0 without sharing), shared memory in all.  CKPT_E_UNSUPPORTED: another kernel runs. */
 CKPT_API int ckpt_selftest_conv_plan(const ckpt_conv_shape* s, int epilogue, int32_t* plan);
+/* How the CUDA-core convolution divides its work (host only, no device needed).  mode: 0 forward, 1 input gradient, 2 weight
+ * gradient; chunks: 1 for operands fetched 16 bytes at a time, 0 value by value.  plan (host, 6 values): rows and columns of a
+ * tile, CTAs of a cluster that share a reduction, slices of the reduction, its length per CTA, CTAs that an SM is counted on to
+ * hold. */
+CKPT_API int ckpt_selftest_simt_plan(const ckpt_conv_shape* s, int dtype, int mode, int chunks, int32_t* plan);
 /* How the batch-norm backward divides a rows x c tensor on a device that holds held[0], held[1], held[2] clusters of 16, 8
  * and 4 of its CTAs and held[3] CTAs at once (host only, no device needed).  split (host, 3 values): form (0 separate
  * kernels, 1 one cluster per channel group, 2 one co-operative grid), channel groups, CTAs per group. */

@@ -403,6 +403,13 @@ def selftest_conv_plan(shape, epilogue):
     return dict(zip(("pixels", "split", "stages", "stage_bytes", "exchange_bytes", "smem"), out))
 
 
+def selftest_simt_plan(shape, dtype, mode, chunks):
+    """Plan of the CUDA-core convolution: dict of rows, columns, cluster, slices, length, held (host only)."""
+    out = (C.c_int32 * 6)()
+    _check(lib().ckpt_selftest_simt_plan(C.byref(shape), C.c_int(dtype), C.c_int(mode), C.c_int(chunks), out))
+    return dict(zip(("rows", "columns", "cluster", "slices", "length", "held"), out))
+
+
 def selftest_bn_split(dtype, rows, c, masked, held):
     """(form, groups, parts) of the batch-norm backward on a device that holds `held` clusters of 16, 8, 4 and CTAs."""
     out = (C.c_int32 * 3)()

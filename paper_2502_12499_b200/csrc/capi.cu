@@ -44,7 +44,7 @@ int ckpt_conv2d_scratch_bytes(const ckpt_conv_shape* s, int dtype, int64_t* byte
     if (rc) return rc;
     if (!bytes) { set_error("bytes is null"); return CKPT_E_NULL; }
     ConvGeom g = make_geom(*s);
-    int64_t b = simt_wgrad_scratch_bytes(g);
+    int64_t b = simt_wgrad_scratch_bytes(dtype, g);
     if (tc_conv_supported(dtype, g)) b = b > tc_conv_scratch_bytes(g) ? b : tc_conv_scratch_bytes(g);
     if (small_conv_supported(dtype, g)) b = b > small_conv_scratch_bytes(g) ? b : small_conv_scratch_bytes(g);
     if (stem_conv_supported(dtype, g)) b = b > stem_conv_scratch_bytes(g) ? b : stem_conv_scratch_bytes(g);
@@ -152,6 +152,14 @@ int ckpt_selftest_conv_plan(const ckpt_conv_shape* s, int epilogue, int32_t* pla
     if (!plan) { set_error("plan is null"); return CKPT_E_NULL; }
     if (epilogue < 0 || epilogue > 2) { set_error("unknown epilogue %d", epilogue); return CKPT_E_BAD_ARG; }
     return tc_selftest_t_plan(make_geom(*s), epilogue, plan);
+}
+
+int ckpt_selftest_simt_plan(const ckpt_conv_shape* s, int dtype, int mode, int chunks, int32_t* plan) {
+    int rc = check_shape(s, dtype);
+    if (rc) return rc;
+    if (!plan) { set_error("plan is null"); return CKPT_E_NULL; }
+    if (mode < 0 || mode > 2) { set_error("unknown mode %d", mode); return CKPT_E_BAD_ARG; }
+    return simt_selftest_plan(make_geom(*s), dtype, mode, chunks != 0, plan);
 }
 
 int ckpt_selftest_bn_split(int dtype, int64_t rows, int32_t c, int masked, const int32_t* held, int32_t* split) {

@@ -876,7 +876,7 @@ int ckpt_chain_create(const ckpt_unit_desc* units, int64_t n, int64_t batch, int
         for (const ConvGeom& o : sized)
             if (std::memcmp(&o, &g, sizeof g) == 0) return;
         sized.push_back(g);
-        scr = std::max(scr, simt_wgrad_scratch_bytes(g));
+        scr = std::max(scr, simt_wgrad_scratch_bytes(dtype, g));
         if (tc_conv_supported(dtype, g)) scr = std::max(scr, tc_conv_scratch_bytes(g));
         if (small_conv_supported(dtype, g)) scr = std::max(scr, small_conv_scratch_bytes(g));
         if (stem_conv_supported(dtype, g)) scr = std::max(scr, stem_conv_scratch_bytes(g));

@@ -13,9 +13,9 @@
 // kernel adds in slice order.  Every summation order is fixed by the shape.
 // A sum is taken in chains of kChain products, whose totals are added: a chain of 1152 has two to three times the error.
 // Measured (float32, forward / dgrad / wgrad in us, replayed; in brackets one chain per sum, whose registers let an SM hold more
-// CTAs): 32 x 16 x 16 x 64 -> 64 3x3 32/30/22 (27/28/27); 32 x 8 x 8 x 128 -> 128 29/28/23 (51/52/35); 16 x 112 x 112 x 64 -> 64
-// 405/423/352 (431/438/452; 37 of the 72 TFLOP/s of the FMA units); 16 x 28 x 28 x 256 -> 256 3x3 stride 2 124/204/102 (165/320/147);
-// 4 x 32 x 32 x 16 -> 16 8/8/8 (8/8/8).  At equal plans the chains cost 2-4 %, 128-wide weight-gradient tiles 7 %.  What stands
+// CTAs): 32 x 16 x 16 x 64 -> 64 3x3 29/30/22 (27/28/27); 32 x 8 x 8 x 128 -> 128 29/28/22 (51/52/36); 16 x 112 x 112 x 64 -> 64
+// 405/424/353 (431/438/453; 37 of the 72 TFLOP/s of the FMA units); 16 x 28 x 28 x 256 -> 256 3x3 stride 2 125/206/100 (165/320/148);
+// 4 x 32 x 32 x 16 -> 16 8/8/8 (8/9/9).  At equal plans the chains cost 2-4 %, 128-wide weight-gradient tiles 7 %.  What stands
 // between is the issue of everything but FMAs - shared-memory reads, addresses and bounds of the copies - and their latency at 16
 // warps per SM.
 #pragma once
@@ -72,8 +72,6 @@ __device__ __forceinline__ void copy4(void* dst, const void* src, bool in) {
 template <typename T, int MODE, int BM, int BN, int TM, int TN>
 struct Tile {
     static constexpr int threads = (BM / TM) * (BN / TN);
-    // CTAs that an SM shall hold: registers for the chain and the total of a block, operands and addresses
-    static constexpr int held = TM * TN >= 64 ? 256 / threads : TM * TN >= 32 ? (sizeof(T) == 4 ? 4 : 3) : TM * TN >= 16 ? 5 : 7;
     static constexpr int V = 16 / (int)sizeof(T);            // values of a 16-byte chunk
     static constexpr int BK = 4 * V;                         // reduction depth of a stage
     static constexpr bool a_k = MODE != 2, b_k = MODE == 0;  // K contiguous in shared memory (and in memory)
@@ -83,6 +81,11 @@ struct Tile {
     static constexpr int a_elems = a_rows * a_row, b_elems = b_rows * b_row;
     static constexpr int stage_bytes = (a_elems + b_elems) * (int)sizeof(T);
     static constexpr int smem = kStages * stage_bytes > BM * BN * 4 ? kStages * stage_bytes : BM * BN * 4;
+    // CTAs that an SM shall hold - what the kernel is compiled for and what the plan counts on: by the registers for the chain and
+    // the total of a block, operands and addresses, and by shared memory
+    static constexpr int by_registers = TM * TN >= 64 ? 256 / threads : TM * TN >= 32 ? (sizeof(T) == 4 ? 4 : 3) : TM * TN >= 16 ? 5 : 7;
+    static constexpr int by_memory = 228 * 1024 / (smem + 1024);
+    static constexpr int held = by_registers < by_memory ? by_registers : by_memory;
 };
 
 // A position along K of modes 0 and 1: channel within a filter position, and the filter position as (row, column) indices.
@@ -466,7 +469,7 @@ struct Plan { int tile, cluster, slices, k_per_slice; };
 #define CKPT_SIMT_TILES_W(F)                                                                                           \
     F(0, 128, 128, 8, 8) F(1, 64, 128, 8, 8) F(2, 64, 64, 8, 4) F(3, 32, 128, 4, 8) F(4, 32, 64, 4, 4) F(5, 16, 128, 4, 4) F(6, 16, 64, 2, 4)
 
-Plan plan(int mode, int M, int N, int K, bool vectors);
+Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors);
 
 template <typename T>
 int launch(int mode, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K,

@@ -3894,7 +3894,7 @@ static int stem_wgrad_slices(const ConvGeom& g) {
 int64_t stem_conv_scratch_bytes(const ConvGeom& g) {
     const int64_t partial = (int64_t)stem_wgrad_slices(g) * g.cout * 147 * 4;
     const int64_t stat = (int64_t)sm_count() * 2 * g.cout * 4;
-    return align_up(std::max(std::max(partial, stat), simt_wgrad_scratch_bytes(g)), 256);
+    return align_up(std::max(std::max(partial, stat), simt_wgrad_scratch_bytes(CKPT_DTYPE_BF16, g)), 256);
 }
 
 // partial / blocks: null, or where the kernel leaves the batch-norm partial sums of its output

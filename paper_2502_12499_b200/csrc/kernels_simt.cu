@@ -52,26 +52,45 @@ namespace simt {
 // kernel adds: the cheapest by a model of clocks per SM.  148 SMs are written in: the scratch size of a chain comes from
 // here and must not depend on the device at hand.
 //
-// Operands in 16-byte chunks: an SM holds `held` CTAs of a tile shape at once and works them off in rounds.  n of them need, per
-// step along K, n times the tile's FMAs at the share of the peak that the shape reaches, and a wait that they spend once
-// together.  (Share and wait fitted to 2,700 measured plans of 93 layers, each within 7 % on average; the chosen plan
-// is 2-3 % behind the best of the layer's in the mean.  Before, with one share per shape and no view of how many CTAs an SM
-// holds, 128 x 128 tiles alone on their SMs were taken for fast: us, float32, forward / dgrad / wgrad of 128 -> 128 at 8 x 8, 32
-// images 51/52/35 -> 30/31/22, 256 -> 256 3x3 stride 2 at 28 x 28, 16 images 164/319/149 -> 124/207/109, 1x1 64 -> 256 at 56 x 56,
-// 8 images 32/39/63 -> 33/34/42.)
-struct TileCost { double share, wait; int held; };
-static const TileCost kTileCost[3][7] = {
-    {{0.47, 40, 1}, {0.66, 70, 2}, {0.67, 55, 4}, {0.62, 65, 4}, {0.54, 44, 5}, {0.43, 39, 4}, {0.41, 32, 7}},
-    {{0.45, 40, 1}, {0.65, 86, 2}, {0.66, 67, 4}, {0.62, 69, 4}, {0.63, 44, 5}, {0.52, 59, 4}, {0.44, 33, 7}},
-    {{0.59, 10, 1}, {0.74, 84, 2}, {0.71, 51, 4}, {0.69, 75, 4}, {0.63, 46, 5}, {0.56, 74, 5}, {0.47, 51, 7}}};
-static const double kRound[3] = {2150, 2390, 1340}, kExchange[3] = {2000, 1730, 1310}, kExchangeTile[3] = {21.7, 21.8, 23.6};
-static double clocks_of_chunks(int mode, int t, int bm, int bn, double load, int per, int cluster, int slices, double outputs) {
-    const TileCost& c = kTileCost[mode][t];
-    const double fma = (double)bm * bn / 128.0 / c.share, rounds = std::floor(load / c.held), rest = load - rounds * c.held;
-    double clk = 3000.0 + rounds * (per * (fma * c.held + c.wait) + kRound[mode]);
-    if (rest > 0) clk += per * (fma * rest + c.wait) + kRound[mode];
-    if (cluster > 1) clk += kExchange[mode] + load * kExchangeTile[mode] * bm * bn / 32.0;
-    if (slices > 1) clk += 3950.0 + 0.76 * slices * outputs * 8.0 / 2500.0;
+// Operands in 16-byte chunks: an SM holds `held` CTAs of a tile shape at once (the number that its kernel is compiled for) and works
+// them off in rounds.  n of them need, per step along K, n times the tile's FMAs at the share of the peak that the shape reaches, and
+// a wait that they spend once together.  The CTAs of a cluster share a GPC, which leaves some SMs short: clusters reach fewer of
+// them (without that the choice is 3.0 % behind the best of a layer's plans in the mean, float32 forward of 62 layers, so 2.1).
+// Fitted for each type to some 10,000 measured plans of 104 layers, each within 5-9 % on average; the chosen plan is 0.9-1.9 % behind
+// the best of its layer in the mean, for bfloat16 1.1-2.9 (2.4-6.2 with float32's figures for both).
+// us, float32, forward / dgrad / wgrad, one share per shape and no view of how many CTAs an SM holds -> this: 128 -> 128 at 8 x 8,
+// 32 images 51/52/36 -> 29/28/22, 256 -> 256 3x3 stride 2 at 28 x 28, 16 images 165/320/148 -> 125/206/100, 1x1 64 -> 256 at 56 x 56, 8 images
+// 33/39/63 -> 31/32/42.
+struct TileShape { int m, n, held[2]; };         // held: float32, bfloat16
+#define CKPT_SHAPE(MODE, BM, BN, TM, TN) {BM, BN, {Tile<float, MODE, BM, BN, TM, TN>::held, Tile<__nv_bfloat16, MODE, BM, BN, TM, TN>::held}},
+#define CKPT_SHAPE0(I, BM, BN, TM, TN) CKPT_SHAPE(0, BM, BN, TM, TN)
+#define CKPT_SHAPE1(I, BM, BN, TM, TN) CKPT_SHAPE(1, BM, BN, TM, TN)
+#define CKPT_SHAPE2(I, BM, BN, TM, TN) CKPT_SHAPE(2, BM, BN, TM, TN)
+static constexpr TileShape kShapes[3][7] = {{CKPT_SIMT_TILES(CKPT_SHAPE0)}, {CKPT_SIMT_TILES(CKPT_SHAPE1)}, {CKPT_SIMT_TILES_W(CKPT_SHAPE2)}};
+#undef CKPT_SHAPE
+#undef CKPT_SHAPE0
+#undef CKPT_SHAPE1
+#undef CKPT_SHAPE2
+struct TileCost { double share, wait; };
+struct ModeCost { TileCost tile[7]; double round, exchange, exchange_tile, slice_sum, slice_share; };
+static const ModeCost kCost[2][3] = {            // float32, bfloat16; modes
+    {{{{0.47, 40}, {0.66, 70}, {0.67, 55}, {0.62, 65}, {0.54, 44}, {0.43, 39}, {0.41, 32}}, 2150, 2000, 21.7, 0, 0},
+     {{{0.45, 40}, {0.65, 86}, {0.66, 67}, {0.62, 69}, {0.63, 44}, {0.52, 59}, {0.44, 33}}, 2390, 1730, 21.8, 0, 0},
+     {{{0.63, 11}, {0.91, 98}, {0.82, 51}, {0.78, 77}, {0.73, 47}, {0.69, 73}, {0.48, 46}}, 40, 2700, 17.2, 2470, 0.91}},
+    {{{{0.65, 26}, {0.92, 76}, {0.72, 49}, {0.65, 50}, {0.68, 35}, {0.68, 44}, {0.45, 19}}, 1410, 1850, 29.0, 0, 0},
+     {{{0.49, 14}, {0.63, 70}, {0.86, 64}, {0.66, 52}, {0.73, 40}, {0.61, 42}, {0.45, 20}}, 870, 2000, 28.8, 0, 0},
+     {{{0.60, 10}, {0.79, 65}, {0.72, 39}, {0.55, 42}, {0.57, 25}, {0.51, 34}, {0.41, 21}}, 40, 2550, 16.4, 2300, 0.84}}};
+static double clocks_of_chunks(int mode, int value_bytes, int t, double ctas, int per, int cluster, int slices, double outputs) {
+    const ModeCost& c = kCost[value_bytes == 2][mode];
+    const TileShape& s = kShapes[mode][t];
+    const int held = s.held[value_bytes == 2];
+    const double load = std::ceil(ctas / (148.0 - (cluster > 1 ? 1.5 * cluster : 0.0)));
+    const double fma = (double)s.m * s.n / 128.0 / c.tile[t].share, rounds = std::floor(load / held), rest = load - rounds * held;
+    double clk = rounds * (per * (fma * held + c.tile[t].wait) + c.round);
+    if (rest > 0) clk += per * (fma * rest + c.tile[t].wait) + c.round;
+    if (cluster == 2 && load <= 2) clk *= 1.1;                // (a pair may come to share an SM while others have none: 9-16 % more, measured)
+    if (cluster > 1) clk += c.exchange + load * c.exchange_tile * s.m * s.n / 32.0;
+    if (slices > 1) clk += c.slice_sum + c.slice_share * slices * outputs * 8.0 / 2500.0;
     return clk;
 }
 // Operands fetched value by value: FMA time is the tile volume over 128 lanes and the share of the peak a tile shape reaches; a
@@ -90,13 +109,12 @@ static double clocks_of_values(int mode, int t, int bm, int bn, double load, int
     if (slices > 1) clk += 4000.0 + (double)slices * outputs * 8.0 / 2500.0;
     return clk;
 }
-static const int kTileM[7] = {128, 128, 64, 128, 64, 128, 64}, kTileN[7] = {128, 64, 64, 32, 32, 16, 16};      // modes 0 and 1
-Plan plan(int mode, int M, int N, int K, bool vectors) {
+Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors) {
     Plan best{2, 1, 1, K};
     double best_t = 1e300;
     for (int t = 0; t < 7; ++t) {
         if (!vectors && t != 2 && t != 4 && t != 6) continue;
-        const int bm = mode == 2 ? kTileN[t] : kTileM[t], bn = mode == 2 ? kTileM[t] : kTileN[t];
+        const int bm = kShapes[mode][t].m, bn = kShapes[mode][t].n;
         const int64_t tiles = (int64_t)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
         for (int cluster = 1; cluster <= 8; cluster *= 2) {
             // 1, 2, 3, 4, 6, 8, 12, ... slices: a finer search costs the host 17 us per layer and gains nothing
@@ -108,9 +126,9 @@ Plan plan(int mode, int M, int N, int K, bool vectors) {
                     if (vectors || mode != 2) continue;
                     slices = (int)((K + (int64_t)per * cluster - 1) / ((int64_t)per * cluster));      // rounding up leaves fewer
                 }
-                const double load = std::ceil((double)(tiles * cluster * slices) / 148.0), outputs = (double)M * N;
-                const double clk = vectors ? clocks_of_chunks(mode, t, bm, bn, load, per, cluster, slices, outputs)
-                                           : clocks_of_values(mode, t, bm, bn, load, per, cluster, slices, outputs);
+                const double ctas = (double)(tiles * cluster * slices), outputs = (double)M * N;
+                const double clk = vectors ? clocks_of_chunks(mode, value_bytes, t, ctas, per, cluster, slices, outputs)
+                                           : clocks_of_values(mode, t, bm, bn, std::ceil(ctas / 148.0), per, cluster, slices, outputs);
                 if (clk < best_t) { best_t = clk; best = Plan{t, cluster, slices, per}; }
             }
         }
@@ -132,13 +150,13 @@ int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, vo
     if (!bias && !relu && small_conv_supported(dtype, g) && g.cout % 64 == 0) return small_conv_fwd(g, x, w, z, stream);
     const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
     const bool v = g.k <= 16 && whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
-    return simt_conv(0, dtype, g, x, w, z, bias, relu, M, N, K, v, v, simt::plan(0, M, N, K, v), (cudaStream_t)stream);
+    return simt_conv(0, dtype, g, x, w, z, bias, relu, M, N, K, v, v, simt::plan(0, dtype_size(dtype), M, N, K, v), (cudaStream_t)stream);
 }
 int simt_conv_fwd_stats(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, float* partial, int* blocks, void* stream) {
     const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
     const bool v = g.k <= 16 && whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
-    const simt::Plan p = simt::plan(0, M, N, K, v);
-    const int64_t rows = ((int64_t)M + simt::kTileM[p.tile] - 1) / simt::kTileM[p.tile] * p.cluster;
+    const simt::Plan p = simt::plan(0, dtype_size(dtype), M, N, K, v);
+    const int64_t tile = simt::kShapes[0][p.tile].m, rows = (M + tile - 1) / tile * p.cluster;
     *blocks = 0;
     // (the first layer's kernel of its own gathers none; more partial rows than the scratch region is sized for neither)
     if ((small_conv_supported(dtype, g) && g.cout % 64 == 0) || rows > BN_MAX_BLOCKS) return simt_conv_fwd(dtype, g, x, w, z, nullptr, 0, stream);
@@ -150,19 +168,29 @@ int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w,
     const int taps = (g.k + g.stride - 1) / g.stride;
     const int M = g.n * g.h * g.w, N = g.cin, K = taps * taps * g.cout;
     const bool va = g.k <= 16 && whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, w);
-    return simt_conv(1, dtype, g, dz, w, dx, nullptr, 0, M, N, K, va, vb, simt::plan(1, M, N, K, va && vb), (cudaStream_t)stream);
+    return simt_conv(1, dtype, g, dz, w, dx, nullptr, 0, M, N, K, va, vb, simt::plan(1, dtype_size(dtype), M, N, K, va && vb), (cudaStream_t)stream);
 }
 
-int64_t simt_wgrad_scratch_bytes(const ConvGeom& g) {
+int simt_selftest_plan(const ConvGeom& g, int dtype, int mode, bool chunks, int32_t* plan) {
+    const int taps = mode == 1 ? (g.k + g.stride - 1) / g.stride : g.k, in = g.n * g.h * g.w, out = g.n * g.ho * g.wo;
+    const simt::Plan p = mode == 0 ? simt::plan(0, dtype_size(dtype), out, g.cout, taps * taps * g.cin, chunks)
+                       : mode == 1 ? simt::plan(1, dtype_size(dtype), in, g.cin, taps * taps * g.cout, chunks)
+                                   : simt::plan(2, dtype_size(dtype), g.cout, taps * taps * g.cin, out, chunks);
+    const simt::TileShape& s = simt::kShapes[mode][p.tile];
+    plan[0] = s.m; plan[1] = s.n; plan[2] = p.cluster; plan[3] = p.slices; plan[4] = p.k_per_slice; plan[5] = s.held[dtype == CKPT_DTYPE_BF16];
+    return CKPT_OK;
+}
+
+int64_t simt_wgrad_scratch_bytes(int dtype, const ConvGeom& g) {
     const int M = g.cout, N = g.k * g.k * g.cin, K = g.n * g.ho * g.wo;
-    const int slices = std::max(simt::plan(2, M, N, K, true).slices, simt::plan(2, M, N, K, false).slices);
+    const int slices = std::max(simt::plan(2, dtype_size(dtype), M, N, K, true).slices, simt::plan(2, dtype_size(dtype), M, N, K, false).slices);
     return slices <= 1 ? 0 : (int64_t)slices * M * N * (int64_t)sizeof(float);
 }
 int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes, void* stream,
                     const SgdUpdate& upd) {
     const int M = g.cout, N = g.k * g.k * g.cin, K = g.n * g.ho * g.wo;
     const bool va = whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, x);
-    const simt::Plan p = simt::plan(2, M, N, K, va && vb);
+    const simt::Plan p = simt::plan(2, dtype_size(dtype), M, N, K, va && vb);
     const int64_t elems = (int64_t)M * N;
     if (p.slices > 1 && (!scratch || scratch_bytes < p.slices * elems * 4)) { set_error("wgrad scratch too small"); return CKPT_E_WORKSPACE; }
     int rc = simt_conv(2, dtype, g, dz, x, p.slices > 1 ? scratch : dw, nullptr, 0, M, N, K, va, vb, p, (cudaStream_t)stream,
