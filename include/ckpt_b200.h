@@ -378,10 +378,10 @@ CKPT_API int ckpt_selftest_bounded_wait(int64_t limit_cycles, void* stream);
  * exchanged in place of the stages (0 without sharing), shared memory in all.  CKPT_E_UNSUPPORTED: another kernel runs. */
 CKPT_API int ckpt_selftest_conv_plan(const ckpt_conv_shape* s, int epilogue, int32_t* plan);
 /* How the CUDA-core convolution divides its work (host only, no device needed).  mode: 0 forward, 1 input gradient, 2 weight
- * gradient; chunks: 1 for operands fetched 16 bytes at a time, 0 value by value.  plan (host, 6 values): rows and columns of a
- * tile, CTAs of a cluster that share a reduction, slices of the reduction, its length per CTA, CTAs that an SM is counted on to
- * hold. */
-CKPT_API int ckpt_selftest_simt_plan(const ckpt_conv_shape* s, int dtype, int mode, int chunks, int32_t* plan);
+ * gradient; aligned: 1 for operands that start on 16 bytes, else 0.  plan (host, 7 values): rows and columns of a tile, CTAs of a
+ * cluster that share a reduction, slices of the reduction, its length per CTA, CTAs that an SM is counted on to hold, and
+ * how operands are fetched (sum of 1: the first 16 bytes at a time, 2: the second, 4: through a filter of more than 16 rows). */
+CKPT_API int ckpt_selftest_simt_plan(const ckpt_conv_shape* s, int dtype, int mode, int aligned, int32_t* plan);
 /* How the batch-norm backward divides a rows x c tensor on a device that holds held[0], held[1], held[2] clusters of 16, 8
  * and 4 of its CTAs and held[3] CTAs at once (host only, no device needed).  split (host, 3 values): form (0 separate
  * kernels, 1 one cluster per channel group, 2 one co-operative grid), channel groups, CTAs per group. */

@@ -403,11 +403,11 @@ def selftest_conv_plan(shape, epilogue):
     return dict(zip(("pixels", "split", "stages", "stage_bytes", "exchange_bytes", "smem"), out))
 
 
-def selftest_simt_plan(shape, dtype, mode, chunks):
-    """Plan of the CUDA-core convolution: dict of rows, columns, cluster, slices, length, held (host only)."""
-    out = (C.c_int32 * 6)()
-    _check(lib().ckpt_selftest_simt_plan(C.byref(shape), C.c_int(dtype), C.c_int(mode), C.c_int(chunks), out))
-    return dict(zip(("rows", "columns", "cluster", "slices", "length", "held"), out))
+def selftest_simt_plan(shape, dtype, mode, aligned):
+    """Plan of the CUDA-core convolution: dict of rows, columns, cluster, slices, length, held, fetch (host only)."""
+    out = (C.c_int32 * 7)()
+    _check(lib().ckpt_selftest_simt_plan(C.byref(shape), C.c_int(dtype), C.c_int(mode), C.c_int(aligned), out))
+    return dict(zip(("rows", "columns", "cluster", "slices", "length", "held", "fetch"), out))
 
 
 def selftest_bn_split(dtype, rows, c, masked, held):

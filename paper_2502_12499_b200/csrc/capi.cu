@@ -154,12 +154,12 @@ int ckpt_selftest_conv_plan(const ckpt_conv_shape* s, int epilogue, int32_t* pla
     return tc_selftest_t_plan(make_geom(*s), epilogue, plan);
 }
 
-int ckpt_selftest_simt_plan(const ckpt_conv_shape* s, int dtype, int mode, int chunks, int32_t* plan) {
+int ckpt_selftest_simt_plan(const ckpt_conv_shape* s, int dtype, int mode, int aligned, int32_t* plan) {
     int rc = check_shape(s, dtype);
     if (rc) return rc;
     if (!plan) { set_error("plan is null"); return CKPT_E_NULL; }
     if (mode < 0 || mode > 2) { set_error("unknown mode %d", mode); return CKPT_E_BAD_ARG; }
-    return simt_selftest_plan(make_geom(*s), dtype, mode, chunks != 0, plan);
+    return simt_selftest_plan(make_geom(*s), dtype, mode, aligned != 0, plan);
 }
 
 int ckpt_selftest_bn_split(int dtype, int64_t rows, int32_t c, int masked, const int32_t* held, int32_t* split) {

@@ -117,7 +117,8 @@ struct Pixel {
 // gridDim.z = slices * cluster; slice z of the reduction starts at z * k_per_slice (a multiple of BK).
 // Mode 1 with a stride: the input pixels fall into stride x stride parity classes, each reached by every stride-th filter
 // row and column only; a block works on one class (classes follow one another in blockIdx.x) and its K covers just those.
-template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB>
+// WIDE (modes 0, 1, chunks of A): filters of more than 16 rows, whose places outside the tensor are found by coordinates instead.
+template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB, bool WIDE>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), (Tile<T, MODE, BM, BN, TM, TN>::held))
 conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bias,
                  int relu, int M, int N, int K, int k_per_slice, int cluster, SgdUpdate upd, float* sums) {
@@ -173,9 +174,10 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
     const int a_c = tid % a_len * a_w, a_r = tid / a_len, b_c = tid % b_len * b_w, b_r = tid / b_len;
     TapPos a_pos = {0, 0, 0};                                 // modes 0, 1: this thread's place along K
     // chunks: the corner of a row's window, and which filter rows (low half) and columns (high half) of it lie inside the
-    // tensor (chunks are taken for up to 16 of each): an address is one addition per step, and no multiplication
+    // tensor (up to 16 of each): an address is one addition per step, and no multiplication
     const T* a_corner[VA ? CA : 1];
     uint32_t a_inside[VA ? CA : 1];
+    int a_top[WIDE ? CA : 1], a_left[WIDE ? CA : 1];          // WIDE: the corner's place
     if (MODE != 2) {
         a_pos.set(k_begin + a_c, kc, cols);
         if (VA) {
@@ -186,6 +188,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
                 p.set(min(m, M - 1), W, H);
                 const int bh = a_base_h(p.h), bw = a_base_w(p.w), th = MODE == 0 ? g.h : g.ho, tw = MODE == 0 ? g.w : g.wo;
                 a_corner[VA ? i : 0] = A + (((int64_t)p.n * th + bh) * tw + bw) * kc;
+                if (WIDE) { a_top[WIDE ? i : 0] = m < M ? bh : -(1 << 28); a_left[WIDE ? i : 0] = bw; continue; }
                 uint32_t inside = 0u;
                 for (int t = 0; t < g.k && m < M; ++t) {
                     const int ih = MODE == 0 ? bh + t : bh - t, iw = MODE == 0 ? bw + t : bw - t;
@@ -230,7 +233,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
         if (VA && MODE != 2 && k0 + a_c < k_end) {
             const int at = a_pos.r * (MODE == 0 ? g.w : g.wo) + a_pos.s;
             a_off = (int64_t)(MODE == 0 ? at : -at) * kc + a_pos.c;
-            a_bits = 1u << a_pos.r | 0x10000u << a_pos.s;
+            a_bits = WIDE ? 1u : 1u << a_pos.r | 0x10000u << a_pos.s;
         }
 #pragma unroll
         for (int i = 0; i < CA; ++i) {
@@ -240,7 +243,14 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
             if (MODE == 2) {
                 if (k0 + row < k_end && m0 + a_c < M) src = A + (int64_t)(k0 + row) * g.cout + m0 + a_c;
             } else if (VA) {
-                if (a_bits != 0u && (a_inside[VA ? i : 0] & a_bits) == a_bits) src = a_corner[VA ? i : 0] + a_off;
+                bool in = a_bits != 0u;
+                if (WIDE) {
+                    const int h = a_top[WIDE ? i : 0], w = a_left[WIDE ? i : 0], ih = MODE == 0 ? h + a_pos.r : h - a_pos.r, iw = MODE == 0 ? w + a_pos.s : w - a_pos.s;
+                    in = in && (unsigned)ih < (unsigned)(MODE == 0 ? g.h : g.ho) && (unsigned)iw < (unsigned)(MODE == 0 ? g.w : g.wo);
+                } else {
+                    in = in && (a_inside[VA ? i : 0] & a_bits) == a_bits;
+                }
+                if (in) src = a_corner[VA ? i : 0] + a_off;
             } else {
                 if (k0 + a_c < k_end && m0 + row < M) src = a_ptr(row_px.n, a_base_h(row_px.h), a_base_w(row_px.w), a_pos);
                 row_px.advance(a_dr, W, H);
@@ -460,7 +470,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-struct Plan { int tile, cluster, slices, k_per_slice; };
+struct Plan { int tile, cluster, slices, k_per_slice; bool wide = false; };
 
 // Tile shapes, largest first.  Modes 0 and 1 keep M (pixels) long and N (channels) as narrow as the layer; a weight
 // gradient is the other way round.  (BM, BN, TM, TN)
@@ -469,7 +479,7 @@ struct Plan { int tile, cluster, slices, k_per_slice; };
 #define CKPT_SIMT_TILES_W(F)                                                                                           \
     F(0, 128, 128, 8, 8) F(1, 64, 128, 8, 8) F(2, 64, 64, 8, 4) F(3, 32, 128, 4, 8) F(4, 32, 64, 4, 4) F(5, 16, 128, 4, 4) F(6, 16, 64, 2, 4)
 
-Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors);
+Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors, bool wide = false);
 
 template <typename T>
 int launch(int mode, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K,

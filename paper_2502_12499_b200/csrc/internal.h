@@ -98,7 +98,7 @@ int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, vo
 int simt_conv_fwd_stats(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, float* partial, int* blocks, void* stream);
 int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w, void* dx, void* stream);
 int64_t simt_wgrad_scratch_bytes(int dtype, const ConvGeom& g);
-int simt_selftest_plan(const ConvGeom& g, int dtype, int mode, bool chunks, int32_t* plan);
+int simt_selftest_plan(const ConvGeom& g, int dtype, int mode, bool aligned, int32_t* plan);
 int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw,
                     void* scratch, int64_t scratch_bytes, void* stream, const SgdUpdate& upd = SgdUpdate());
 

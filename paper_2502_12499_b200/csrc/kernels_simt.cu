@@ -56,7 +56,7 @@ namespace simt {
 // them off in rounds.  n of them need, per step along K, n times the tile's FMAs at the share of the peak that the shape reaches, and
 // a wait that they spend once together.  The CTAs of a cluster share a GPC, which leaves some SMs short: clusters reach fewer of
 // them (without that the choice is 3.0 % behind the best of a layer's plans in the mean, float32 forward of 62 layers, so 2.1).
-// Fitted for each type to some 10,000 measured plans of 104 layers, each within 5-9 % on average; the chosen plan is 0.9-1.9 % behind
+// Fitted for each type to some 17,000 measured plans of 104 layers, each within 5-9 % on average; the chosen plan is 0.9-1.9 % behind
 // the best of its layer in the mean, for bfloat16 1.1-2.9 (2.4-6.2 with float32's figures for both).
 // us, float32, forward / dgrad / wgrad, one share per shape and no view of how many CTAs an SM holds -> this: 128 -> 128 at 8 x 8,
 // 32 images 51/52/36 -> 29/28/22, 256 -> 256 3x3 stride 2 at 28 x 28, 16 images 165/320/148 -> 125/206/100, 1x1 64 -> 256 at 56 x 56, 8 images
@@ -109,11 +109,11 @@ static double clocks_of_values(int mode, int t, int bm, int bn, double load, int
     if (slices > 1) clk += 4000.0 + (double)slices * outputs * 8.0 / 2500.0;
     return clk;
 }
-Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors) {
-    Plan best{2, 1, 1, K};
+Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors, bool wide) {
+    Plan best{2, 1, 1, K, wide};
     double best_t = 1e300;
     for (int t = 0; t < 7; ++t) {
-        if (!vectors && t != 2 && t != 4 && t != 6) continue;
+        if ((!vectors || wide) && t != 2 && t != 4 && t != 6 && !(vectors && t == 3)) continue;
         const int bm = kShapes[mode][t].m, bn = kShapes[mode][t].n;
         const int64_t tiles = (int64_t)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
         for (int cluster = 1; cluster <= 8; cluster *= 2) {
@@ -129,7 +129,7 @@ Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors) {
                 const double ctas = (double)(tiles * cluster * slices), outputs = (double)M * N;
                 const double clk = vectors ? clocks_of_chunks(mode, value_bytes, t, ctas, per, cluster, slices, outputs)
                                            : clocks_of_values(mode, t, bm, bn, std::ceil(ctas / 148.0), per, cluster, slices, outputs);
-                if (clk < best_t) { best_t = clk; best = Plan{t, cluster, slices, per}; }
+                if (clk < best_t) { best_t = clk; best = Plan{t, cluster, slices, per, wide}; }
             }
         }
     }
@@ -140,61 +140,78 @@ Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors) {
 constexpr int BN_MAX_BLOCKS = 148 * 8;        // partial rows of batch-norm sums
 static bool whole_chunks(int dtype, int channels, const void* p) { return channels % (dtype == CKPT_DTYPE_BF16 ? 8 : 4) == 0 && (uintptr_t)p % 16 == 0; }
 
-static int simt_conv(int mode, int dtype, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N,
-                     int K, bool va, bool vb, const simt::Plan& p, cudaStream_t st, const SgdUpdate& upd = SgdUpdate(), float* sums = nullptr) {
-    return dtype == CKPT_DTYPE_BF16 ? simt::launch<__nv_bfloat16>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, upd, st, sums)
-                                    : simt::launch<float>(mode, g, a, b, out, bias, relu, M, N, K, va, vb, p, upd, st, sums);
+// How a call's operands are fetched: each in 16-byte chunks or value by value.  wide: chunks through a filter of more than 16 rows,
+// whose mask of places inside the tensor outgrows the 32 bits that the kernel keeps (us, float32, forward / input gradient, value by
+// value -> so: 17 x 17 64 -> 64 at 32 x 32, 8 images 937/1255 -> 625/627, 31 x 31 16 -> 32 at 64 x 64, 4 images 1059/2506 -> 558/720).
+struct Fetch { bool a, b, wide; };
+static Fetch fetch_of(int mode, int dtype, const ConvGeom& g, const void* a, const void* b) {
+    Fetch f{whole_chunks(dtype, mode == 0 ? g.cin : g.cout, a), whole_chunks(dtype, g.cin, b), false};
+    if (mode == 0) f.a = f.b = f.a && f.b;
+    f.wide = mode != 2 && f.a && g.k > 16;
+    return f;
+}
+struct Product { int M, N, K; };
+static Product product_of(int mode, const ConvGeom& g) {
+    // (a strided layer's K splits over the parity classes of the input: the longest class has ceil(k / stride)^2 positions)
+    const int taps = (g.k + g.stride - 1) / g.stride;
+    if (mode == 0) return {g.n * g.ho * g.wo, g.cout, g.k * g.k * g.cin};
+    if (mode == 1) return {g.n * g.h * g.w, g.cin, taps * taps * g.cout};
+    return {g.cout, g.k * g.k * g.cin, g.n * g.ho * g.wo};
+}
+static simt::Plan plan_of(int mode, int dtype, const ConvGeom& g, const Fetch& f) {
+    const Product p = product_of(mode, g);
+    return simt::plan(mode, dtype_size(dtype), p.M, p.N, p.K, f.a && f.b, f.wide);
+}
+static int simt_conv(int mode, int dtype, const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, const Fetch& f,
+                     const simt::Plan& p, cudaStream_t st, const SgdUpdate& upd = SgdUpdate(), float* sums = nullptr) {
+    const Product m = product_of(mode, g);
+    return dtype == CKPT_DTYPE_BF16 ? simt::launch<__nv_bfloat16>(mode, g, a, b, out, bias, relu, m.M, m.N, m.K, f.a, f.b, p, upd, st, sums)
+                                    : simt::launch<float>(mode, g, a, b, out, bias, relu, m.M, m.N, m.K, f.a, f.b, p, upd, st, sums);
 }
 
 int simt_conv_fwd(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, const float* bias, int relu, void* stream) {
     if (!bias && !relu && small_conv_supported(dtype, g) && g.cout % 64 == 0) return small_conv_fwd(g, x, w, z, stream);
-    const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
-    const bool v = g.k <= 16 && whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
-    return simt_conv(0, dtype, g, x, w, z, bias, relu, M, N, K, v, v, simt::plan(0, dtype_size(dtype), M, N, K, v), (cudaStream_t)stream);
+    const Fetch f = fetch_of(0, dtype, g, x, w);
+    return simt_conv(0, dtype, g, x, w, z, bias, relu, f, plan_of(0, dtype, g, f), (cudaStream_t)stream);
 }
 int simt_conv_fwd_stats(int dtype, const ConvGeom& g, const void* x, const void* w, void* z, float* partial, int* blocks, void* stream) {
-    const int M = g.n * g.ho * g.wo, N = g.cout, K = g.k * g.k * g.cin;
-    const bool v = g.k <= 16 && whole_chunks(dtype, g.cin, x) && whole_chunks(dtype, g.cin, w);
-    const simt::Plan p = simt::plan(0, dtype_size(dtype), M, N, K, v);
-    const int64_t tile = simt::kShapes[0][p.tile].m, rows = (M + tile - 1) / tile * p.cluster;
+    const Fetch f = fetch_of(0, dtype, g, x, w);
+    const simt::Plan p = plan_of(0, dtype, g, f);
+    const int64_t tile = simt::kShapes[0][p.tile].m, rows = (product_of(0, g).M + tile - 1) / tile * p.cluster;
     *blocks = 0;
     // (the first layer's kernel of its own gathers none; more partial rows than the scratch region is sized for neither)
     if ((small_conv_supported(dtype, g) && g.cout % 64 == 0) || rows > BN_MAX_BLOCKS) return simt_conv_fwd(dtype, g, x, w, z, nullptr, 0, stream);
     *blocks = (int)rows;
-    return simt_conv(0, dtype, g, x, w, z, nullptr, 0, M, N, K, v, v, p, (cudaStream_t)stream, SgdUpdate(), partial);
+    return simt_conv(0, dtype, g, x, w, z, nullptr, 0, f, p, (cudaStream_t)stream, SgdUpdate(), partial);
 }
 int simt_conv_dgrad(int dtype, const ConvGeom& g, const void* dz, const void* w, void* dx, void* stream) {
-    // (a strided layer's K splits over the parity classes of the input: the longest class has ceil(k / stride)^2 positions)
-    const int taps = (g.k + g.stride - 1) / g.stride;
-    const int M = g.n * g.h * g.w, N = g.cin, K = taps * taps * g.cout;
-    const bool va = g.k <= 16 && whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, w);
-    return simt_conv(1, dtype, g, dz, w, dx, nullptr, 0, M, N, K, va, vb, simt::plan(1, dtype_size(dtype), M, N, K, va && vb), (cudaStream_t)stream);
+    const Fetch f = fetch_of(1, dtype, g, dz, w);
+    return simt_conv(1, dtype, g, dz, w, dx, nullptr, 0, f, plan_of(1, dtype, g, f), (cudaStream_t)stream);
 }
 
-int simt_selftest_plan(const ConvGeom& g, int dtype, int mode, bool chunks, int32_t* plan) {
-    const int taps = mode == 1 ? (g.k + g.stride - 1) / g.stride : g.k, in = g.n * g.h * g.w, out = g.n * g.ho * g.wo;
-    const simt::Plan p = mode == 0 ? simt::plan(0, dtype_size(dtype), out, g.cout, taps * taps * g.cin, chunks)
-                       : mode == 1 ? simt::plan(1, dtype_size(dtype), in, g.cin, taps * taps * g.cout, chunks)
-                                   : simt::plan(2, dtype_size(dtype), g.cout, taps * taps * g.cin, out, chunks);
+int simt_selftest_plan(const ConvGeom& g, int dtype, int mode, bool aligned, int32_t* plan) {
+    const void* const operand = aligned ? nullptr : (const void*)4;
+    const Fetch f = fetch_of(mode, dtype, g, operand, operand);
+    const simt::Plan p = plan_of(mode, dtype, g, f);
     const simt::TileShape& s = simt::kShapes[mode][p.tile];
     plan[0] = s.m; plan[1] = s.n; plan[2] = p.cluster; plan[3] = p.slices; plan[4] = p.k_per_slice; plan[5] = s.held[dtype == CKPT_DTYPE_BF16];
+    plan[6] = (f.a ? 1 : 0) | (f.b ? 2 : 0) | (f.wide ? 4 : 0);
     return CKPT_OK;
 }
 
 int64_t simt_wgrad_scratch_bytes(int dtype, const ConvGeom& g) {
-    const int M = g.cout, N = g.k * g.k * g.cin, K = g.n * g.ho * g.wo;
-    const int slices = std::max(simt::plan(2, dtype_size(dtype), M, N, K, true).slices, simt::plan(2, dtype_size(dtype), M, N, K, false).slices);
-    return slices <= 1 ? 0 : (int64_t)slices * M * N * (int64_t)sizeof(float);
+    const Product m = product_of(2, g);
+    const int slices = std::max(plan_of(2, dtype, g, {true, true, false}).slices, plan_of(2, dtype, g, {false, false, false}).slices);
+    return slices <= 1 ? 0 : (int64_t)slices * m.M * m.N * (int64_t)sizeof(float);
 }
 int simt_conv_wgrad(int dtype, const ConvGeom& g, const void* dz, const void* x, float* dw, void* scratch, int64_t scratch_bytes, void* stream,
                     const SgdUpdate& upd) {
-    const int M = g.cout, N = g.k * g.k * g.cin, K = g.n * g.ho * g.wo;
-    const bool va = whole_chunks(dtype, g.cout, dz), vb = whole_chunks(dtype, g.cin, x);
-    const simt::Plan p = simt::plan(2, dtype_size(dtype), M, N, K, va && vb);
-    const int64_t elems = (int64_t)M * N;
+    const Fetch f = fetch_of(2, dtype, g, dz, x);
+    const simt::Plan p = plan_of(2, dtype, g, f);
+    const Product m = product_of(2, g);
+    const int64_t elems = (int64_t)m.M * m.N;
     if (p.slices > 1 && (!scratch || scratch_bytes < p.slices * elems * 4)) { set_error("wgrad scratch too small"); return CKPT_E_WORKSPACE; }
-    int rc = simt_conv(2, dtype, g, dz, x, p.slices > 1 ? scratch : dw, nullptr, 0, M, N, K, va, vb, p, (cudaStream_t)stream,
-                       p.slices > 1 ? SgdUpdate() : upd);
+    int rc = simt_conv(2, dtype, g, dz, x, p.slices > 1 ? scratch : dw, nullptr, 0, f, p, (cudaStream_t)stream, p.slices > 1 ? SgdUpdate() : upd);
     if (rc || p.slices <= 1) return rc;
     return slice_sum((const float*)scratch, dw, elems, p.slices, stream, upd);
 }

@@ -9,10 +9,10 @@ SHAPES = [ck.ConvShape(n, h, w, cin, cout, k, s, k // 2) for (n, h, w), (cin, co
     ((1, 5, 5), (4, 32, 32), (9, 37, 11), (32, 16, 16), (16, 112, 112)), ((3, 64), (16, 16), (64, 64), (96, 300), (512, 512)), (1, 3, 7), (1, 2))]
 
 
-@pytest.mark.parametrize("dtype,mode,chunks", list(itertools.product((ck.DTYPE_F32, ck.DTYPE_BF16), (0, 1, 2), (0, 1))))
-def test_plan_covers_the_reduction(dtype, mode, chunks):
+@pytest.mark.parametrize("dtype,mode,aligned", list(itertools.product((ck.DTYPE_F32, ck.DTYPE_BF16), (0, 1, 2), (0, 1))))
+def test_plan_covers_the_reduction(dtype, mode, aligned):
     for s in SHAPES:
-        p = ck.selftest_simt_plan(s, dtype, mode, chunks)
+        p = ck.selftest_simt_plan(s, dtype, mode, aligned)
         ho, wo = (s.h + 2 * s.pad - s.k) // s.stride + 1, (s.w + 2 * s.pad - s.k) // s.stride + 1
         reduction = (s.k ** 2 * s.c_in, (-(-s.k // s.stride)) ** 2 * s.c_out, s.n * ho * wo)[mode]
         parts = p["cluster"] * p["slices"]
@@ -22,7 +22,17 @@ def test_plan_covers_the_reduction(dtype, mode, chunks):
         assert (p["slices"] - 1) * p["cluster"] * p["length"] < reduction, (p, reduction)
         if mode == 2 and p["slices"] > 1:
             assert p["slices"] * s.c_out * s.k ** 2 * s.c_in * 4 <= ck.conv2d_scratch_bytes(s, dtype)
-        assert chunks or min(p["rows"], p["columns"]) <= 64
+        assert p["fetch"] == 3 or min(p["rows"], p["columns"]) <= 64
+
+
+@pytest.mark.parametrize("k,cin,cout,forward,dgrad,wgrad", [(16, 64, 64, 3, 3, 3), (17, 64, 64, 7, 7, 3), (31, 16, 24, 7, 7, 3), (21, 64, 6, 7, 2, 2), (21, 6, 64, 0, 5, 1)])
+def test_wide_filters_are_fetched_in_chunks(k, cin, cout, forward, dgrad, wgrad):
+    for dtype in (ck.DTYPE_F32, ck.DTYPE_BF16):
+        shape = ck.ConvShape(3, 40, 33, cin, cout, k, 1, k // 2)
+        assert [ck.selftest_simt_plan(shape, dtype, m, 1)["fetch"] for m in (0, 1, 2)] == [forward, dgrad, wgrad]
+        assert [ck.selftest_simt_plan(shape, dtype, m, 0)["fetch"] for m in (0, 1, 2)] == [0, 0, 0]
+        if k > 16:
+            assert all(ck.selftest_simt_plan(shape, dtype, m, 1)["rows"] == 64 for m in (0, 1) if (forward, dgrad)[m] & 4)
 
 
 def test_plan_counts_on_what_the_kernels_are_compiled_for():
