@@ -399,7 +399,8 @@ CKPT_API int ckpt_conv2d_wgrad(const ckpt_conv_shape* s, int dtype, int impl, co
  * chain runs them (the forward step d_i = f_i(d_{i-1}, w_i) of Eq. (1) up to the point where d_i is
  * stored): z = conv(x, w) and stats[0..4c) as for ckpt_bn_relu_forward, computed over the stored
  * (rounded) z.  Where the tensor-core kernel for the shape is a persistent one, the per-channel sums
- * are gathered in its epilogue and z is not read again; otherwise two kernels run.
+ * are gathered in its epilogue and z is not read again; otherwise two kernels run.  (A step on the CUDA cores gathers
+ * them in the epilogue too, in another order of additions than the separate kernel here.)
  * scratch: max(ckpt_conv2d_scratch_bytes, ckpt_bn_scratch_bytes(n*h_out*w_out, c_out)) bytes.
  * fused (host, optional): set to 1 when the sums came from the convolution's epilogue, else 0. */
 CKPT_API int ckpt_conv2d_bn_statistics(const ckpt_conv_shape* s, int dtype, const void* x, const void* w, void* z,

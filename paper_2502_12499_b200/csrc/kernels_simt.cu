@@ -1420,7 +1420,7 @@ __global__ void __launch_bounds__(256) maxpool3_arg_act_kernel(const __nv_bfloat
 }
 // Gradient of a 2 x 2 quad of inputs (rows 2a, 2a + 1; columns 2b, 2b + 1) from the recorded positions: an even row belongs
 // to window a only (its middle row), an odd one to windows a (last row) and a + 1 (first row).  With `act` the producer's
-// batch-norm backward sums (sum g, sum g*z over the values its ReLU passes) go to `partial` as in the 2x2 kernel.
+// batch-norm backward sums (sum g, sum g*z over the values its ReLU passes) go to `partial`, a row pair per block.
 template <bool SUMS>
 __global__ void __launch_bounds__(256) maxpool3_bwd_kernel(const uint8_t* arg, const __nv_bfloat16* dy, __nv_bfloat16* dx,
                                                            int64_t items, int h, int w, int c, int ho, int wo, const __nv_bfloat16* z,

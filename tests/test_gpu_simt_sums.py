@@ -34,3 +34,45 @@ def test_statistics_of_convolution(dtype, cin, c, batch, h, w):
     for (ui, name, _), g in zip(runner.flat, grads):
         want = ref["grads"][ui][name]
         assert max_rel_err(g.reshape(want.shape), want) <= tol, (ui, name)
+
+
+MAX_PARTIAL_ROWS = 148 * 8
+
+
+@pytest.mark.parametrize("dtype,cin,c,batch,h,w,shared,separate", [
+    ("f32", 16, 16, 4, 32, 32, False, False), ("f32", 3, 5, 2, 7, 9, False, False), ("f32", 128, 128, 2, 8, 8, True, False), ("f32", 64, 33, 1, 5, 5, True, False),
+    ("f32", 64, 64, 3, 150, 150, False, False), ("f32", 3, 64, 2, 200, 200, False, True), ("bf16", 20, 36, 2, 6, 10, True, False)])
+def test_statistics_against_float64(dtype, cin, c, batch, h, w, shared, separate):
+    """Mean and inverse deviation that a step saves against float64 ones of the z it stores: reductions shared by a cluster or not, and
+    more partial rows than the scratch region holds, which take a pass of their own.  A sum of float32 values in short
+    chains is within 2^-24 of its terms' root sum of squares a level, a dozen levels in all: 2^-24 * sqrt(12) = 2.1e-7 of the deviation; the
+    mean's own place in float32 (2^-24 of it) and the inverse's rounding come to that."""
+    import torch
+    shape = ck.ConvShape(batch, h, w, cin, c, 3, 1, 1)
+    code, store = (ck.DTYPE_BF16, torch.bfloat16) if dtype == "bf16" else (ck.DTYPE_F32, torch.float32)
+    plan = ck.selftest_simt_plan(shape, code, 0, 1)
+    assert (plan["cluster"] > 1) == shared, plan
+    assert (-(-batch * h * w // plan["rows"]) * plan["cluster"] > MAX_PARTIAL_ROWS) == separate, plan
+    spec = dict(units=[wl.conv_unit(cin, c), {"kind": "avgpool"}], input_hwc=(h, w, cin), batch=batch, dtype=dtype, loss="sum", name="stats")
+    params = wl.make_params(spec, seed=31, bn_affine="random")
+    x, _ = wl.make_batch(spec, seed=32)
+    runner = StepRunner(spec, params)
+    ck.launch_log(True)
+    runner.run(ck.POLICY_STORE_ALL, None, x + np.float32(0.25) if dtype == "f32" else x, None)
+    kernels = ck.launch_log_read()
+    ck.launch_log(False)
+    assert ("batch-norm statistics" in kernels) == separate, kernels
+    z = torch.empty((batch, h, w, c), dtype=store, device="cuda")
+    xd = torch.from_numpy(x + np.float32(0.25) if dtype == "f32" else x).cuda().to(store)
+    ck.conv2d_forward(shape, code, 0, xd, torch.from_numpy(params[0]["w"]).cuda().to(store), z)        # as the step stores it
+    mean = z.double().mean((0, 1, 2))
+    inv = (z.double().var((0, 1, 2), unbiased=False) + 1e-5).rsqrt()
+    # the saved rows [mean | inverse deviation | ...] lie in the workspace: where all of the means and inverses come close
+    words = runner.workspace[:runner.workspace.numel() // 4 * 4].view(torch.float32)
+    want = torch.cat((mean, inv)).float()
+    found = [i for i in torch.nonzero((words[:-2 * c] - want[0]).abs() < 1e-4 * (1 / inv[0]).float()).flatten().tolist()
+             if bool(((words[i:i + 2 * c] - want).abs() <= 1e-4 * torch.cat((1 / inv, inv)).float()).all())]
+    assert len(found) == 1, found
+    got = words[found[0]:found[0] + 2 * c].double()
+    assert ((got[:c] - mean).abs() * inv <= 2.1e-7 + 2.0 ** -24 * mean.abs() * inv).all()
+    assert ((got[c:] / inv - 1).abs() <= 2.1e-7 + 2.0 ** -24).all()
