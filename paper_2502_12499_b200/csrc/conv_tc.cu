@@ -3590,7 +3590,10 @@ bool wgrad_short_chains(const ConvGeom& g) { return (g.cin % 64 || g.cout % 64) 
 // CTAs win: fitted to 900 plans of 31 layers within 5 %, the choice 2.3 % behind the best in the mean (us with the slice sum, the
 // rules for long reductions -> this: 3x3 512 -> 512 at 7 x 6, 21 images 16.7 -> 11.8, 256 -> 512 at 4 x 4, 128 images 22.2 -> 11.7,
 // 1x1 2048 -> 512 at 7 x 7, 32 images 20.5 -> 10.9, 1024 -> 256 at 13 x 11, 21 images 12.2 -> 10.5; error against float64 in 1e-7
-// of the norm 3.9 -> 1.8, 3.9 -> 2.0, 3.8 -> 2.2, 3.3 -> 1.9).  From 4096 pixels on the plain chains are ahead by 1-10 %.
+// of the norm 3.4 -> 1.5, 3.9 -> 2.0, 3.8 -> 2.2, 3.3 -> 1.9).  From 4096 pixels on the plain chains are ahead by 1-10 %.
+// Ragged channel counts, whose chains are of 64 pixels, keep slices of at most four: the more chains a slice adds up one after another,
+// the further off it is (0.67 -> 0.73 at 96 -> 48, 3 images of 10 x 10, in one slice; us 7.2 -> 7.2, at most 13.8 -> 16.4, 96 -> 384 at
+// 13 x 13, 13 images).
 bool wgrad_short_plan(const ConvGeom& g, WgradParams* p, int* slices, int sms) {
     const int64_t pixels = (int64_t)g.n * g.ho * g.wo;
     if (pixels <= 256 || pixels >= 4096) return false;
@@ -3605,6 +3608,7 @@ bool wgrad_short_plan(const ConvGeom& g, WgradParams* p, int* slices, int sms) {
         const int tiles_w = (g.wo + tw - 1) / tw, tiles_h = (g.ho + th - 1) / th, tiles_n = (g.n + tn - 1) / tn, total = tiles_w * tiles_h * tiles_n;
         for (int want = 1; want <= total && (want == 1 || groups * co_tiles * want <= sms); ++want) {
             const int per = (total + want - 1) / want, s = (total + per - 1) / per;
+            if (wgrad_short_chains(g) && per * px > 4 * 16 * kChain) continue;
             const double ctas = (double)groups * co_tiles * s, rounds = std::ceil(ctas / sms), bytes = (2.0 + nb) * px * 128.0;
             const double stage = std::max(113.0 + px / 16 * 4.4 * std::max(1.0, nb / 2.0), bytes / std::min(43.0, 5870.0 / std::min<double>(ctas, sms)));
             const double t = 3160.0 + rounds * (per * stage + 760.0 * nb) + 9.5 * ctas * nb + (s > 1 ? 4300.0 + 8.9e-4 * s * elems : 0.0);
