@@ -44,9 +44,11 @@ MAX_PARTIAL_ROWS = 148 * 8
     ("f32", 64, 64, 3, 150, 150, False, False), ("f32", 3, 64, 2, 200, 200, False, True), ("bf16", 20, 36, 2, 6, 10, True, False)])
 def test_statistics_against_float64(dtype, cin, c, batch, h, w, shared, separate):
     """Mean and inverse deviation that a step saves against float64 ones of the z it stores: reductions shared by a cluster or not, and
-    more partial rows than the scratch region holds, which take a pass of their own.  A sum of float32 values in short
-    chains is within 2^-24 of its terms' root sum of squares a level, a dozen levels in all: 2^-24 * sqrt(12) = 2.1e-7 of the deviation; the
-    mean's own place in float32 (2^-24 of it) and the inverse's rounding come to that."""
+    more partial rows than the scratch region holds, which take a pass of their own.  In the root mean square over channels: an inverse
+    rounded to float32 is off by 2.5e-8 of itself, a mean of up to half a deviation by 1.2e-8 of the deviation; two thirds of that again are
+    left for the sums.  A tree of float32 additions of N values is off by 2^-24 * 0.58 * sqrt(levels * N) deviations, a dozen levels at most:
+    1.2e-7 / sqrt(N) of the deviation in the mean, which counts where N is small.  (Measured on 4,000 values and more: 2.5e-8 and 0.7e-8;
+    one float32 chain over 67,500 values would be off by 4e-8 of the deviation.)"""
     import torch
     shape = ck.ConvShape(batch, h, w, cin, c, 3, 1, 1)
     code, store = (ck.DTYPE_BF16, torch.bfloat16) if dtype == "bf16" else (ck.DTYPE_F32, torch.float32)
@@ -74,5 +76,5 @@ def test_statistics_against_float64(dtype, cin, c, batch, h, w, shared, separate
              if bool(((words[i:i + 2 * c] - want).abs() <= 1e-4 * torch.cat((1 / inv, inv)).float()).all())]
     assert len(found) == 1, found
     got = words[found[0]:found[0] + 2 * c].double()
-    assert ((got[:c] - mean).abs() * inv <= 2.1e-7 + 2.0 ** -24 * mean.abs() * inv).all()
-    assert ((got[c:] / inv - 1).abs() <= 2.1e-7 + 2.0 ** -24).all()
+    assert ((got[:c] - mean) * inv).square().mean().sqrt() <= 2e-8 + 1.2e-7 / (batch * h * w) ** 0.5
+    assert (got[c:] / inv - 1).square().mean().sqrt() <= 4e-8 + 1.2e-7 / (batch * h * w) ** 0.5
