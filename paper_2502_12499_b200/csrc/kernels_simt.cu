@@ -1163,7 +1163,8 @@ __global__ void __launch_bounds__(256, 2) maxpool2x2_bn_sums_kernel(const T* z, 
                 if (w0 + u * hop < p.windows) win[u].load(p, z, dy, (uint32_t)(w0 + u * hop), ch);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                // (the windows of a step are added up before they join the running sums, which are two floats each)
+                // (the windows of a step join the running sums, two floats each, one by one in float32; in bfloat16, whose products
+                // are exact and values few bits, added up)
                 float t0[C], t1[C];
 #pragma unroll
                 for (int i = 0; i < C; ++i) t0[i] = t1[i] = 0.f;
@@ -1181,10 +1182,15 @@ __global__ void __launch_bounds__(256, 2) maxpool2x2_bn_sums_kernel(const T* z, 
 #pragma unroll
                     for (int q = 0; q < 4; ++q) at |= win[u].z[q][j] & take[q];
 #pragma unroll
-                    for (int i = 0; i < C; ++i) { t0[i] += W::value(g, i); t1[i] = fmaf(W::value(g, i), W::value(at, i), t1[i]); }
+                    for (int i = 0; i < C; ++i) {
+                        t0[i] += W::value(g, i); t1[i] = fmaf(W::value(g, i), W::value(at, i), t1[i]);
+                        if (C == 1) { carry_sum(s0[j * C + i], t0[i]); carry_sum(s1[j * C + i], t1[i]); t0[i] = t1[i] = 0.f; }
+                    }
                 }
+                if (C > 1) {
 #pragma unroll
-                for (int i = 0; i < C; ++i) { carry_sum(s0[j * C + i], t0[i]); carry_sum(s1[j * C + i], t1[i]); }
+                    for (int i = 0; i < C; ++i) { carry_sum(s0[j * C + i], t0[i]); carry_sum(s1[j * C + i], t1[i]); }
+                }
             }
         }
     }
