@@ -1,9 +1,16 @@
 """Kernels that start under the tail of the one before them: operations queued back to back, each on what the one before
 wrote, leave the bits that they leave with the device idle between them."""
+import os
+import subprocess
+import sys
+
+import numpy as np
 import pytest
 
 from paper_2502_12499_b200 import binding as ck
-from tests.gpu_util import torch_dtype
+from paper_2502_12499_b200 import workloads as wl
+from tests.conftest import ROOT
+from tests.gpu_util import to_dev, torch_dtype
 
 pytestmark = pytest.mark.gpu
 
@@ -99,3 +106,50 @@ def test_kernels_with_tensor_memory_follow_one_another(n, h, w, cin, cout, k, st
         for a, b in zip(walk(False), want):
             assert torch.equal(a, b)
     ck.op_status()
+
+
+def small_chains():
+    """First layer, stem, both poolings, fully connected units, residual blocks with and without a stride, units of finer granularity and
+    convolutions on the CUDA cores."""
+    conv = {"kind": "conv", "cin": 64, "cout": 64, "k": 3, "stride": 1, "pad": 1}
+    plain = [dict(conv, cin=3), conv, conv, {"kind": "avgpool"}, {"kind": "fc", "cin": 64, "cout": 10, "relu": False}]
+    return [wl.vgg16_chain(4, hw=(32, 32), dtype="bf16", widths=(64, 64, 128, 128, 128), fc_width=64, classes=10, name="vgg"),
+            wl.split_units(wl.vgg16_chain(2, hw=(32, 64), dtype="bf16", widths=(48, 48, 72, 64, 64), fc_width=72, classes=10, name="vgg_fine"))[0],
+            wl.resnet_chain([1, 2, 1, 1], 3, hw=(72, 64), dtype="bf16", base=64, classes=10, name="resnet"),
+            wl.vgg16_chain(2, hw=(32, 32), dtype="f32", widths=(8, 16, 24, 32, 32), fc_width=24, classes=10, name="vgg_f32"),
+            dict(units=plain, input_hwc=(16, 16, 3), batch=4, dtype="bf16", loss="softmax_ce", name="plain_bf16")]
+
+
+def gradients_of_steps(recorded):
+    """Losses and gradients of each chain's planned step with early free: {chain: [arrays]}."""
+    import torch
+    out = {}
+    for spec in small_chains():
+        chain = ck.Chain(spec)
+        chain.set_graph(recorded)
+        d = chain.sizes()
+        mask, peak = ck.plan(ck.ALGO_DYNAMIC_N, d)
+        params, grads, _ = ck.upload_params(chain, wl.make_params(spec, seed=41, bn_affine="random"))
+        x, labels = wl.make_batch(spec, seed=42)
+        x, labels = to_dev(x, chain.dtype), torch.from_numpy(labels).cuda()
+        arena, workspace = (torch.empty(n, dtype=torch.uint8, device="cuda") for n in (peak, chain.workspace_bytes()))
+        for _ in range(4 if recorded else 2):
+            for g in grads:
+                g.fill_(float("nan"))
+            arena.fill_(0xFF)
+            report = ck.train_step(chain, mask, ck.POLICY_DYNAMIC, x, labels, params, grads, arena, workspace)
+        assert bool(report["replayed"]) == recorded
+        out[spec["name"]] = [np.float64(report["loss"])] + [g.cpu().numpy() for g in grads]
+    return out
+
+
+def test_recorded_and_queued_steps_against_one_launch_at_a_time(tmp_path):
+    """The same steps in a process whose launches are waited for one by one, queued here, and replayed from a recording: the same bits."""
+    program = "import sys; sys.path.insert(0, %r)\nfrom tests import test_gpu_overlap as t\nimport numpy as np\n" % ROOT
+    program += "np.savez(%r, **{'%%s %%d' %% (n, i): a for n, arrays in t.gradients_of_steps(False).items() for i, a in enumerate(arrays)})" % str(tmp_path / "one.npz")
+    subprocess.run([sys.executable, "-c", program], check=True, timeout=300, cwd=ROOT, env=dict(os.environ, CUDA_LAUNCH_BLOCKING="1"))
+    want = np.load(tmp_path / "one.npz")
+    for recorded in (False, True):
+        for name, arrays in gradients_of_steps(recorded).items():
+            for i, a in enumerate(arrays):
+                assert np.isfinite(a).all() and np.array_equal(a, want["%s %d" % (name, i)]), (name, i, recorded)
