@@ -7,15 +7,15 @@ checkpoints, loss, backward with segment recomputation, all weight gradients.  T
 dynamic planner's (Algorithm 6) and the schedule is Algorithm 4.  With N > 1 (torchrun) every
 rank runs an independent replica on its own batch: the step has no exchange between GPUs.
 
-The top-level fields of the JSON line are those of the headline workload (--config, default the VGG-16-shaped
-chain at batch 64).  At N = 1 the line also carries `configs`: the same measurements for every bf16 benchmark
-configuration (VGG-16 b64, ResNet-50 b128, ResNet-152 b256, the 1000-unit chain b32) - checkpointed and
-store-all (Algorithm 1) step times and the recompute overhead between them, end-to-end throughput from pinned
+Prints one short JSON line (rank 0): the headline workload (--config, default the VGG-16-shaped chain at batch 64) and, at
+N = 1, `configs_ms`: step times of every bf16 benchmark configuration (VGG-16 b64, ResNet-50 b128, ResNet-152 b256, the
+1000-unit chain b32).  The full record goes to --details FILE, or to stderr as one JSON line:
+for each configuration checkpointed and store-all (Algorithm 1) step times, end-to-end throughput from pinned
 host batches, device footprint (arena + workspace + parameters) under the plan and under store-all, planner times,
 and the roofline of its kernels: forward, dgrad and wgrad convolution mixes and the launch-weighted batch-norm
 and pooling bandwidth.  `--only` restricts the run to the headline workload.
 
-Prints one JSON line (rank 0).  `--impl reference` times the CPU oracle instead, on rank 0 only.
+`--impl reference` times the CPU oracle instead, on rank 0 only.
 """
 import argparse
 import json
@@ -375,6 +375,7 @@ def main():
     ap.add_argument("--config", type=int, default=2, help="headline workload: benchmark configuration 2..5")
     ap.add_argument("--only", action="store_true", help="measure the headline workload only (no `configs` map)")
     ap.add_argument("--regions", type=int, default=3, help="timed regions per measurement; the median is reported")
+    ap.add_argument("--details", default="", help="file for the full record (default: one line on stderr)")
     ap.add_argument("--batch", type=int, default=0, help="override the batch size (debugging only)")
     ap.add_argument("--cpu-batch", type=int, default=2)
     ap.add_argument("--steps-cpu", type=int, default=3)
@@ -463,9 +464,34 @@ def main():
             line["configs"] = {k: {kk: vv for kk, vv in v.items() if kk != "clocks"} for k, v in configs.items()}
         if not args.no_cpu_baseline and world == 1:
             line["cpu_baseline"] = run_reference(spec, min(spec["batch"], args.cpu_batch), steps=args.steps_cpu)
-        print(json.dumps(line))
+        record = json.dumps(line)
+        if args.details:
+            with open(args.details, "w") as fh:
+                fh.write(record + "\n")
+        else:
+            print(record, file=sys.stderr)
+        print(json.dumps(result_line(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
+
+
+def result_line(record):
+    """The short form of a record, for whoever sees the last 1,500 characters of the output."""
+    def short(v):
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return float("%.6g" % v) if isinstance(v, float) else v
+
+    line = {k: short(record[k]) for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                                          "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "peak_bytes", "predicted_bytes",
+                                          "recompute_overhead_pct")}
+    if "roofline" in record:
+        line["roofline"] = {k: short(record["roofline"][k]) for k in ("bound", "achieved", "peak", "unit", "frac")}
+    if "configs" in record:
+        line["configs_ms"] = {name: short(c["ms_per_step"]) for name, c in record["configs"].items()}
+    if "cpu_baseline" in record:
+        line["cpu_baseline"] = {k: short(record["cpu_baseline"][k]) for k in ("value", "unit", "cores", "kind")}
+    return line
 
 
 def headline_roofline(r, peaks):
