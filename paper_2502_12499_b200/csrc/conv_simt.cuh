@@ -34,6 +34,7 @@ namespace simt {
 
 constexpr int kStages = 4;
 constexpr int kChain = 64;         // additions in a row (see the kernel)
+enum class Form { CHAINS, WIDE, ONE_CHAIN };
 
 template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
@@ -86,6 +87,8 @@ struct Tile {
     static constexpr int by_registers = TM * TN >= 64 ? 256 / threads : TM * TN >= 32 ? (sizeof(T) == 4 ? 4 : 3) : TM * TN >= 16 ? 5 : 7;
     static constexpr int by_memory = 228 * 1024 / (smem + 1024);
     static constexpr int held = by_registers < by_memory ? by_registers : by_memory;
+    static constexpr int held_values = MODE == 2 && TM * TN >= 32 && held < 4 ? 4 : held;      // operands fetched value by value (shapes 2, 4 and 6)
+    static constexpr int held_one = TM * TN >= 32 ? (sizeof(T) == 4 ? 5 : 4) : TM * TN >= 16 ? (sizeof(T) == 4 ? 6 : 5) : 8;      // a chain at most
 };
 
 // A position along K of modes 0 and 1: channel within a filter position, and the filter position as (row, column) indices.
@@ -117,15 +120,18 @@ struct Pixel {
 // gridDim.z = slices * cluster; slice z of the reduction starts at z * k_per_slice (a multiple of BK).
 // Mode 1 with a stride: the input pixels fall into stride x stride parity classes, each reached by every stride-th filter
 // row and column only; a block works on one class (classes follow one another in blockIdx.x) and its K covers just those.
-// WIDE (modes 0, 1, chunks of A): filters of more than 16 rows, whose places outside the tensor are found by coordinates instead.
-template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB, bool WIDE>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN), (Tile<T, MODE, BM, BN, TM, TN>::held))
+// FORM (modes 0, 1): WIDE, chunks of A through filters of more than 16 rows, whose places outside the tensor are found by coordinates;
+// ONE_CHAIN, value by value, a reduction of one chain at most per CTA, without the registers of a second set of sums (us, with
+// them -> so: 3 -> 64 3x3 at 224 x 224, 16 images, float32 166 -> 147, 3 -> 64 1x1 at 40 x 40, 20 images, bfloat16 11.9 -> 7.8).
+template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB, Form FORM>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), (FORM == Form::ONE_CHAIN ? Tile<T, MODE, BM, BN, TM, TN>::held_one : VA && VB ? Tile<T, MODE, BM, BN, TM, TN>::held : Tile<T, MODE, BM, BN, TM, TN>::held_values))
 conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bias,
                  int relu, int M, int N, int K, int k_per_slice, int cluster, SgdUpdate upd, float* sums) {
     previous_grid_done();
     next_grid_may_start();
     using L = Tile<T, MODE, BM, BN, TM, TN>;
     constexpr int NT = L::threads, V = L::V, BK = L::BK;
+    constexpr bool WIDE = FORM == Form::WIDE, ONE = FORM == Form::ONE_CHAIN;
     extern __shared__ __align__(16) uint8_t smem[];
     T* const stages = reinterpret_cast<T*>(smem);
     const int tid = threadIdx.x;
@@ -312,17 +318,20 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
     auto n_of = [&](int j) { return L::b_k ? tx + j * TX : (j / GN) * (TX * GN) + tx * GN + j % GN; };
     // chains of kChain products, added up: the error of one float32 chain grows with the square root of its length (in 1e-7 of
     // the result's norm, a chain for the whole reduction -> this: 128 -> 128 3x3 at 28 x 28 6.0 -> 1.6, 512 -> 512 4.3 -> 1.7)
-    float acc[TM][TN], total[TM][TN];
+    float acc[TM][TN], total[ONE ? 1 : TM][ONE ? 1 : TN];
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = total[i][j] = 0.f;
+        for (int j = 0; j < TN; ++j) acc[i][j] = total[ONE ? 0 : i][ONE ? 0 : j] = 0.f;
     auto close_chain = [&] {
+        if constexpr (!ONE) {
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < TN; ++j) { total[i][j] += acc[i][j]; acc[i][j] = 0.f; }
+                for (int j = 0; j < TN; ++j) { total[i][j] += acc[i][j]; acc[i][j] = 0.f; }
+        }
     };
+    auto sum_of = [&](int i, int j) { return ONE ? acc[i][j] : total[ONE ? 0 : i][ONE ? 0 : j]; };
 
 #pragma unroll 1
     for (int p = 0; p < kStages - 1; ++p) {
@@ -339,10 +348,10 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
         const T* const as_ = stages + (size_t)(step % kStages) * (L::a_elems + L::b_elems);
         const T* const bs_ = as_ + L::a_elems;
         // Whole steps unrolled, so that shared-memory reads run ahead of the FMAs (float32, at equal plans, us: 3x3 64 -> 64 at 112 x 112,
-        // 16 images, forward / input gradient 418/438 with groups of four one at a time, 405/423 so).  Eight by eight blocks have no
-        // registers for more than four groups, 128 x 32 tiles of float32 outputs spill.  In mode 2 the fragments of one k at a time:
+        // 16 images, forward / input gradient 418/438 with groups of four one at a time, 405/423 so).  Eight by eight blocks and values
+        // fetched through registers have none left for more than four groups, 128 x 32 tiles of float32 outputs spill.  In mode 2 the fragments of one k at a time:
         // 64 x 64 tiles 3 % faster than with four fetched in front.
-#pragma unroll (TM * TN >= 64 ? 4 : sizeof(T) == 4 && MODE == 0 && BM == 4 * BN ? 1 : BK / 4)
+#pragma unroll (TM * TN >= 64 || !(VA && VB) ? 4 : sizeof(T) == 4 && MODE == 0 && BM == 4 * BN ? 1 : BK / 4)
         for (int k4 = 0; k4 < BK; k4 += 4) {
             if (MODE == 0 && !VA && k_begin + step * BK + k4 >= k_end) break;
             float a[TM][L::a_k ? 4 : 1];
@@ -424,7 +433,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < TN; ++j) store(m0 + m_of(i), n0 + n_of(j), total[i][j], blockIdx.z);
+            for (int j = 0; j < TN; ++j) store(m0 + m_of(i), n0 + n_of(j), sum_of(i, j), blockIdx.z);
         if (MODE == 0 && sums) {
             __syncthreads();                                  // every stage has been read
 #pragma unroll
@@ -432,7 +441,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
                 float s = 0.f, q = 0.f;
 #pragma unroll
                 for (int i = 0; i < TM; ++i)
-                    if (m0 + m_of(i) < M) add(total[i][j], s, q);
+                    if (m0 + m_of(i) < M) add(sum_of(i, j), s, q);
                 red[(ty * BN + n_of(j)) * 2] = s;
                 red[(ty * BN + n_of(j)) * 2 + 1] = q;
             }
@@ -448,7 +457,7 @@ conv_gemm_kernel(ConvGeom g, const T* A, const T* B, void* out, const float* bia
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) tile[m_of(i) * BN + n_of(j)] = total[i][j];
+        for (int j = 0; j < TN; ++j) tile[m_of(i) * BN + n_of(j)] = sum_of(i, j);
     cl.sync();
     const int rank = (int)cl.block_rank(), share = BM * BN / cluster;
     static_assert(NT % BN == 0, "a thread keeps its column of the tile");

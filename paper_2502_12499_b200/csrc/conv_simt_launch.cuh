@@ -5,11 +5,11 @@
 namespace ckpt {
 namespace simt {
 
-template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB, bool WIDE = false>
+template <typename T, int MODE, int BM, int BN, int TM, int TN, bool VA, bool VB, Form FORM = Form::CHAINS>
 static int go(const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K, const Plan& p,
               const SgdUpdate& upd, cudaStream_t st, float* sums) {
     using L = Tile<T, MODE, BM, BN, TM, TN>;
-    auto kernel = conv_gemm_kernel<T, MODE, BM, BN, TM, TN, VA, VB, WIDE>;
+    auto kernel = conv_gemm_kernel<T, MODE, BM, BN, TM, TN, VA, VB, FORM>;
     if (L::smem > 48 * 1024) {
         static DeviceFlags ready;
         if (int bad = allow_shared_memory(ready, {(const void*)kernel}, L::smem)) return bad;
@@ -41,11 +41,14 @@ static int go(const ConvGeom& g, const void* a, const void* b, void* out, const 
 template <typename T, int MODE, bool VA, bool VB>
 static int pick(const ConvGeom& g, const void* a, const void* b, void* out, const float* bias, int relu, int M, int N, int K, const Plan& p,
                 const SgdUpdate& upd, cudaStream_t st, float* sums) {
+    const bool one = MODE != 2 && !VA && !VB && p.k_per_slice <= kChain && (p.tile == 2 || p.tile == 4 || p.tile == 6);
 #define CKPT_CASE(I, BM, BN, TM, TN)                                                                                   \
     if constexpr ((VA && VB) || I == 2 || I == 4 || I == 6)                                                            \
-        if (p.tile == I && !p.wide) return go<T, MODE, BM, BN, TM, TN, VA, VB>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);    \
+        if (p.tile == I && !p.wide && !one) return go<T, MODE, BM, BN, TM, TN, VA, VB>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);    \
     if constexpr (MODE != 2 && VA && (I == 2 || (VB && I == 3) || I == 4 || I == 6))                                   \
-        if (p.tile == I && p.wide) return go<T, MODE, BM, BN, TM, TN, VA, VB, true>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);
+        if (p.tile == I && p.wide) return go<T, MODE, BM, BN, TM, TN, VA, VB, Form::WIDE>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);    \
+    if constexpr (MODE != 2 && !VA && !VB && (I == 2 || I == 4 || I == 6))                                              \
+        if (p.tile == I && one) return go<T, MODE, BM, BN, TM, TN, VA, VB, Form::ONE_CHAIN>(g, a, b, out, bias, relu, M, N, K, p, upd, st, sums);
     if constexpr (MODE == 2) { CKPT_SIMT_TILES_W(CKPT_CASE) } else { CKPT_SIMT_TILES(CKPT_CASE) }
 #undef CKPT_CASE
     set_error("CUDA-core convolution: no such tile");

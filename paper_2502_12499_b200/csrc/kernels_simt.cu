@@ -61,8 +61,10 @@ namespace simt {
 // us, float32, forward / dgrad / wgrad, one share per shape and no view of how many CTAs an SM holds -> this: 128 -> 128 at 8 x 8,
 // 32 images 51/52/36 -> 29/28/22, 256 -> 256 3x3 stride 2 at 28 x 28, 16 images 165/320/148 -> 125/206/100, 1x1 64 -> 256 at 56 x 56, 8 images
 // 33/39/63 -> 31/32/42.
-struct TileShape { int m, n, held[2]; };         // held: float32, bfloat16
-#define CKPT_SHAPE(MODE, BM, BN, TM, TN) {BM, BN, {Tile<float, MODE, BM, BN, TM, TN>::held, Tile<__nv_bfloat16, MODE, BM, BN, TM, TN>::held}},
+struct TileShape { int m, n, held[2], held_values[2]; };         // held: float32, bfloat16
+#define CKPT_SHAPE(MODE, BM, BN, TM, TN)                                                                                     \
+    {BM, BN, {Tile<float, MODE, BM, BN, TM, TN>::held, Tile<__nv_bfloat16, MODE, BM, BN, TM, TN>::held},                     \
+     {Tile<float, MODE, BM, BN, TM, TN>::held_values, Tile<__nv_bfloat16, MODE, BM, BN, TM, TN>::held_values}},
 #define CKPT_SHAPE0(I, BM, BN, TM, TN) CKPT_SHAPE(0, BM, BN, TM, TN)
 #define CKPT_SHAPE1(I, BM, BN, TM, TN) CKPT_SHAPE(1, BM, BN, TM, TN)
 #define CKPT_SHAPE2(I, BM, BN, TM, TN) CKPT_SHAPE(2, BM, BN, TM, TN)
@@ -80,11 +82,12 @@ static const ModeCost kCost[2][3] = {            // float32, bfloat16; modes
     {{{{0.65, 26}, {0.92, 76}, {0.72, 49}, {0.65, 50}, {0.68, 35}, {0.68, 44}, {0.45, 19}}, 1410, 1850, 29.0, 0, 0},
      {{{0.49, 14}, {0.63, 70}, {0.86, 64}, {0.66, 52}, {0.73, 40}, {0.61, 42}, {0.45, 20}}, 870, 2000, 28.8, 0, 0},
      {{{0.60, 10}, {0.79, 65}, {0.72, 39}, {0.55, 42}, {0.57, 25}, {0.51, 34}, {0.41, 21}}, 40, 2550, 16.4, 2300, 0.84}}};
+static double sms_in_reach(int cluster) { return 148.0 - (cluster > 1 ? 1.5 * cluster : 0.0); }
 static double clocks_of_chunks(int mode, int value_bytes, int t, double ctas, int per, int cluster, int slices, double outputs) {
     const ModeCost& c = kCost[value_bytes == 2][mode];
     const TileShape& s = kShapes[mode][t];
     const int held = s.held[value_bytes == 2];
-    const double load = std::ceil(ctas / (148.0 - (cluster > 1 ? 1.5 * cluster : 0.0)));
+    const double load = std::ceil(ctas / sms_in_reach(cluster));
     const double fma = (double)s.m * s.n / 128.0 / c.tile[t].share, rounds = std::floor(load / held), rest = load - rounds * held;
     double clk = rounds * (per * (fma * held + c.tile[t].wait) + c.round);
     if (rest > 0) clk += per * (fma * rest + c.tile[t].wait) + c.round;
@@ -98,12 +101,13 @@ static double clocks_of_chunks(int mode, int value_bytes, int t, double ctas, in
 // 2200 clocks per step of 16 whatever its tile - four warps do not hide their addresses and reads - so that its long reduction
 // wants more CTAs, also such a number of slices as rounds to fewer (us, 3 -> 256, 28 images of 13 x 49 float32 87 -> 34,
 // 5 -> 20 at 28 x 28 69 -> 16, 3 -> 64 1x1 at 40 x 40, 20 images 67 -> 18, bfloat16 65 -> 21).
-static double clocks_of_values(int mode, int t, int bm, int bn, double load, int per, int cluster, int slices, double outputs) {
+static double clocks_of_values(int mode, int value_bytes, int t, int bm, int bn, double ctas, int per, int cluster, int slices, double outputs) {
     static const double share[7] = {0.85, 0.8, 0.7, 0.6, 0.5, 0.4, 0.35};
     // CTAs per SM; one or two of 128 threads do not hide the latency of their shared-memory reads
+    const double load = std::ceil(ctas / 148.0);
     const double hidden = load < 2 ? 0.6 : load < 3 ? 0.8 : 1.0;
     double clk = load * ((double)bm * bn * per / (128.0 * share[t] * hidden) + 300.0);
-    if (mode == 2) clk = std::max(clk, 140.0 * per);
+    if (mode == 2) clk = std::max(clk, 140.0 * per * std::ceil(std::ceil(ctas / sms_in_reach(cluster)) / kShapes[mode][t].held_values[value_bytes == 2]));
     clk += 2000.0;
     if (cluster > 1) clk += 1000.0 + load * bm * bn / 32.0;
     if (slices > 1) clk += 4000.0 + (double)slices * outputs * 8.0 / 2500.0;
@@ -128,7 +132,7 @@ Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors, bool wid
                 }
                 const double ctas = (double)(tiles * cluster * slices), outputs = (double)M * N;
                 const double clk = vectors ? clocks_of_chunks(mode, value_bytes, t, ctas, per, cluster, slices, outputs)
-                                           : clocks_of_values(mode, t, bm, bn, std::ceil(ctas / 148.0), per, cluster, slices, outputs);
+                                           : clocks_of_values(mode, value_bytes, t, bm, bn, ctas, per, cluster, slices, outputs);
                 if (clk < best_t) { best_t = clk; best = Plan{t, cluster, slices, per, wide}; }
             }
         }
