@@ -82,13 +82,14 @@ static const ModeCost kCost[2][3] = {            // float32, bfloat16; modes
     {{{{0.65, 26}, {0.92, 76}, {0.72, 49}, {0.65, 50}, {0.68, 35}, {0.68, 44}, {0.45, 19}}, 1410, 1850, 29.0, 0, 0},
      {{{0.49, 14}, {0.63, 70}, {0.86, 64}, {0.66, 52}, {0.73, 40}, {0.61, 42}, {0.45, 20}}, 870, 2000, 28.8, 0, 0},
      {{{0.60, 10}, {0.79, 65}, {0.72, 39}, {0.55, 42}, {0.57, 25}, {0.51, 34}, {0.41, 21}}, 40, 2550, 16.4, 2300, 0.84}}};
-static double sms_in_reach(int cluster) { return 148.0 - (cluster > 1 ? 1.5 * cluster : 0.0); }
-static double clocks_of_chunks(int mode, int value_bytes, int t, double ctas, int per, int cluster, int slices, double outputs) {
+static int sms_in_reach(int cluster) { return 148 - (cluster > 1 ? 3 * cluster / 2 : 0); }
+static int per_sm(int64_t ctas, int sms) { return (int)((ctas + sms - 1) / sms); }      // (whole numbers throughout: a chain's creation runs this some thousand times)
+static double clocks_of_chunks(int mode, int value_bytes, int t, int64_t ctas, int per, int cluster, int slices, double outputs) {
     const ModeCost& c = kCost[value_bytes == 2][mode];
     const TileShape& s = kShapes[mode][t];
     const int held = s.held[value_bytes == 2];
-    const double load = std::ceil(ctas / sms_in_reach(cluster));
-    const double fma = (double)s.m * s.n / 128.0 / c.tile[t].share, rounds = std::floor(load / held), rest = load - rounds * held;
+    const int load = per_sm(ctas, sms_in_reach(cluster)), rounds = load / held, rest = load % held;
+    const double fma = (double)s.m * s.n / 128.0 / c.tile[t].share;
     double clk = rounds * (per * (fma * held + c.tile[t].wait) + c.round);
     if (rest > 0) clk += per * (fma * rest + c.tile[t].wait) + c.round;
     if (cluster == 2 && load <= 2) clk *= 1.1;                // (a pair may come to share an SM while others have none: 9-16 % more, measured)
@@ -101,13 +102,13 @@ static double clocks_of_chunks(int mode, int value_bytes, int t, double ctas, in
 // 2200 clocks per step of 16 whatever its tile - four warps do not hide their addresses and reads - so that its long reduction
 // wants more CTAs, also such a number of slices as rounds to fewer (us, 3 -> 256, 28 images of 13 x 49 float32 87 -> 34,
 // 5 -> 20 at 28 x 28 69 -> 16, 3 -> 64 1x1 at 40 x 40, 20 images 67 -> 18, bfloat16 65 -> 21).
-static double clocks_of_values(int mode, int value_bytes, int t, int bm, int bn, double ctas, int per, int cluster, int slices, double outputs) {
+static double clocks_of_values(int mode, int value_bytes, int t, int bm, int bn, int64_t ctas, int per, int cluster, int slices, double outputs) {
     static const double share[7] = {0.85, 0.8, 0.7, 0.6, 0.5, 0.4, 0.35};
     // CTAs per SM; one or two of 128 threads do not hide the latency of their shared-memory reads
-    const double load = std::ceil(ctas / 148.0);
+    const int load = per_sm(ctas, 148);
     const double hidden = load < 2 ? 0.6 : load < 3 ? 0.8 : 1.0;
     double clk = load * ((double)bm * bn * per / (128.0 * share[t] * hidden) + 300.0);
-    if (mode == 2) clk = std::max(clk, 140.0 * per * std::ceil(std::ceil(ctas / sms_in_reach(cluster)) / kShapes[mode][t].held_values[value_bytes == 2]));
+    if (mode == 2) clk = std::max(clk, 140.0 * per * per_sm(per_sm(ctas, sms_in_reach(cluster)), kShapes[mode][t].held_values[value_bytes == 2]));
     clk += 2000.0;
     if (cluster > 1) clk += 1000.0 + load * bm * bn / 32.0;
     if (slices > 1) clk += 4000.0 + (double)slices * outputs * 8.0 / 2500.0;
@@ -130,7 +131,8 @@ Plan plan(int mode, int value_bytes, int M, int N, int K, bool vectors, bool wid
                     if (vectors || mode != 2) continue;
                     slices = (int)((K + (int64_t)per * cluster - 1) / ((int64_t)per * cluster));      // rounding up leaves fewer
                 }
-                const double ctas = (double)(tiles * cluster * slices), outputs = (double)M * N;
+                const int64_t ctas = tiles * cluster * slices;
+                const double outputs = (double)M * N;
                 const double clk = vectors ? clocks_of_chunks(mode, value_bytes, t, ctas, per, cluster, slices, outputs)
                                            : clocks_of_values(mode, value_bytes, t, bm, bn, ctas, per, cluster, slices, outputs);
                 if (clk < best_t) { best_t = clk; best = Plan{t, cluster, slices, per, wide}; }
