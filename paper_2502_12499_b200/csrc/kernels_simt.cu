@@ -101,7 +101,8 @@ static double clocks_of_chunks(int mode, int value_bytes, int t, int64_t ctas, i
 // cluster costs its exchange, further slices a launch and a pass over the partial sums.  Such a weight gradient takes a CTA some
 // 2200 clocks per step of 16 whatever its tile - four warps do not hide their addresses and reads - so that its long reduction
 // wants more CTAs, also such a number of slices as rounds to fewer (us, 3 -> 256, 28 images of 13 x 49 float32 87 -> 34,
-// 5 -> 20 at 28 x 28 69 -> 16, 3 -> 64 1x1 at 40 x 40, 20 images 67 -> 18, bfloat16 65 -> 21).
+// 5 -> 20 at 28 x 28 69 -> 16, 3 -> 64 1x1 at 40 x 40, 20 images 67 -> 18, bfloat16 65 -> 21) - as many as an SM holds, or the steps
+// count for each round of the grid (7x7 stride 2 3 -> 64 at 200 x 168, 21 images 213 -> 150).
 static double clocks_of_values(int mode, int value_bytes, int t, int bm, int bn, int64_t ctas, int per, int cluster, int slices, double outputs) {
     static const double share[7] = {0.85, 0.8, 0.7, 0.6, 0.5, 0.4, 0.35};
     // CTAs per SM; one or two of 128 threads do not hide the latency of their shared-memory reads
